@@ -42,7 +42,7 @@ extern "C" {
 
 /* Precision of the structure-factor sum (Sec. 2, the structure-factor sum). */
 #define XRD_FP64 0          /* every step in FP64 */
-#define XRD_FP32_PHASE64 1  /* phase h.x+k.y+l.z formed and reduced mod 1 in FP64, the rest in FP32 */
+#define XRD_FP32_PHASE64 1  /* phase h.x+k.y+l.z formed and reduced mod 1 to 53 fractional bits, the rest in FP32 */
 #define XRD_FP32_PHASEFIX 2 /* coordinates in 32-bit fixed point, phase reduced mod 1 exactly in integers, the rest in FP32 */
 
 typedef struct xrd_handle xrd_handle;

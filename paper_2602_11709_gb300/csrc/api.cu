@@ -89,7 +89,7 @@ size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 // Byte offsets of every array in the caller's workspace.
 struct Layout {
     size_t geo, refl_cnt, run_cnt, refl_off, tile_off, order, atom_bad, cls_list, tile_tab, npk, nfm, fam_soff,
-        flags, coef32, atom32, atom64, astep, imax, cdd, atomr;
+        flags, coef32, atom32, atomx, astep, imax, cdd, atomr;
     size_t q, key, runs, I, Eb, cand_r, cand_s, g_bkt, g_flag, g_pstart, g_psum, g_fcnt;
     size_t st_q, st_I, st_foff, st_key, st_mult;
     size_t parts, oparts, pf, pf_rec, fkg, pf_sfk;
@@ -118,7 +118,7 @@ Layout layout(int64_t n, int64_t natoms, int zmax, int64_t R, bool pg = false)
     L.flags = take(kFlagBytes);
     L.coef32 = take(sizeof(xrd::Coef32) * (zmax + 1));
     L.atom32 = take(sizeof(xrd::Atom32) * natoms);
-    L.atom64 = take(sizeof(xrd::Atom64) * natoms);
+    L.atomx = take(sizeof(xrd::AtomX) * natoms);
     L.astep = take(8 * natoms);
     L.imax = take(4 * n);
     L.cdd = take(sizeof(float4) * 4 * (zmax + 1));
@@ -154,7 +154,7 @@ Layout layout(int64_t n, int64_t natoms, int zmax, int64_t R, bool pg = false)
 // Workspace of the broadened-pattern / gradient path: the geometry prefix of
 // the pattern layout plus the per-reflection state kept for the backward pass.
 struct LayoutG {
-    size_t geo, refl_cnt, run_cnt, refl_off, tile_off, order, atom_bad, tile_tab, flags, coef32, atom32, atom64,
+    size_t geo, refl_cnt, run_cnt, refl_off, tile_off, order, atom_bad, tile_tab, flags, coef32, atom32, atomx,
         astep;
     size_t q, key, runs, Fx, Ig, tb, td, perm, U, V, aorder, parts, oparts;
     size_t total;
@@ -175,7 +175,7 @@ LayoutG layout_grad(int64_t n, int64_t natoms, int zmax, int64_t R)
     L.flags = take(kFlagBytes);
     L.coef32 = take(sizeof(xrd::Coef32) * (zmax + 1));
     L.atom32 = take(sizeof(xrd::Atom32) * natoms);
-    L.atom64 = take(sizeof(xrd::Atom64) * natoms);
+    L.atomx = take(sizeof(xrd::AtomX) * natoms);
     L.astep = take(8 * natoms);
     L.tile_tab = take(8 * (R / kRunsPerTileHost + n + 1));
     L.q = take(8 * R);
@@ -303,7 +303,7 @@ xrd::GeomArgs geom_args(const xrd_batch* b, const xrd_opts* o, const Layout& L, 
     g.geo = (xrd::Geo*)(ws + L.geo);
     g.coef32 = (xrd::Coef32*)(ws + L.coef32);
     g.atom32 = (xrd::Atom32*)(ws + L.atom32);
-    g.atom64 = (xrd::Atom64*)(ws + L.atom64);
+    g.atomx = o->precision == XRD_FP32_PHASEFIX ? nullptr : (xrd::AtomX*)(ws + L.atomx);
     g.refl_cnt = (int64_t*)(ws + L.refl_cnt);
     g.run_cnt = (int64_t*)(ws + L.run_cnt);
     g.runs = (int*)(ws + L.runs);
@@ -372,8 +372,9 @@ int xrd_create(xrd_handle** h, int device)
     if (e != cudaSuccess) { xrd_destroy(p); return XRD_ECUDA; }
     p->ttab = xrd::init_tables(0);  // device tables (2-theta, re-evaluation), once per handle, legacy stream
     p->rtab = xrd::init_refine_tables(0);
+    const bool fx = xrd::init_fx_tables(0);
     e = cudaStreamSynchronize(0);
-    if (e != cudaSuccess || !p->ttab || !p->rtab.sc || !p->rtab.ex) { xrd_destroy(p); return XRD_ECUDA; }
+    if (e != cudaSuccess || !p->ttab || !p->rtab.sc || !p->rtab.ex || !fx) { xrd_destroy(p); return XRD_ECUDA; }
     *h = p;
     return XRD_OK;
 }
@@ -618,7 +619,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     sa.coef32 = ga.coef32;
     sa.coef = b->coef;
     sa.atom32 = ga.atom32;
-    sa.atom64 = ga.atom64;
+    sa.atomx = ga.atomx;
     sa.q = ga.q;
     sa.key = ga.key;
     if (o->precision == XRD_FP64) sa.I = (double*)(ws + L.I);
@@ -1078,7 +1079,6 @@ static void launch_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, c
     ga.geo = (xrd::Geo*)(ws + L.geo);
     ga.coef32 = (xrd::Coef32*)(ws + L.coef32);
     ga.atom32 = (xrd::Atom32*)(ws + L.atom32);
-    ga.atom64 = (xrd::Atom64*)(ws + L.atom64);
     ga.refl_cnt = (int64_t*)(ws + L.refl_cnt);
     ga.run_cnt = (int64_t*)(ws + L.run_cnt);
     ga.runs = (int*)(ws + L.runs);
@@ -1128,7 +1128,7 @@ static void launch_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, c
     sa.coef32 = ga.coef32;
     sa.coef = b->coef;
     sa.atom32 = ga.atom32;
-    sa.atom64 = ga.atom64;
+    sa.atomx = ga.atomx;
     sa.q = ga.q;
     sa.key = ga.key;
     if (grad) {

@@ -11,6 +11,7 @@
 // its own (no fused multiply-add), so the set of reflections on the sphere
 // boundary is decided exactly as a plain FP64 evaluation of the same order.
 #include "xrd_dd.cuh"
+#include "xrd_fx.cuh"
 #include "xrd_internal.cuh"
 #include "xrd_launch.h"
 
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
                                                const double* __restrict__ frac, const int16_t* __restrict__ Zin,
                                                const double* __restrict__ occ, const double* __restrict__ Bf, int zmax,
                                                Geo* __restrict__ geo, int set_geo, int* __restrict__ atom_bad,
-                                               Atom32* __restrict__ a32, Atom64* __restrict__ a64,
+                                               Atom32* __restrict__ a32, AtomX* __restrict__ ax,
                                                float2* __restrict__ astep, AtomR* __restrict__ ar,
                                                const float4* __restrict__ sctab)
 {
@@ -190,8 +191,7 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
             r.lo = -INFINITY;
             r.src = (int)i;
             a32[a0 + i] = r;
-            Atom64 d{};
-            a64[a0 + i] = d;
+            if (ax) ax[a0 + i] = AtomX{};
             if (astep) astep[a0 + i] = make_float2(1.f, 0.f);
             if (ar) {
                 AtomR e{};
@@ -247,9 +247,22 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
                 dd_sincos_turn((unsigned long long)r.Z << 32, sctab, cz, sz);
                 astep[a0 + pos] = make_float2(cz.hi + cz.lo, sz.hi + sz.lo);
             }
-            Atom64 d;
-            d.x = x; d.y = y; d.z = w; d.B = bb; d.occ = o; d.zz = z; d.pad = 0;
-            a64[a0 + pos] = d;
+            if (ax) {  // 64-bit fixed point with a signed low word, B log2(e) in fixed point
+                AtomX d;
+                const double v[3] = {x, y, w};
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const unsigned long long F = fix64(v[c]);
+                    d.hi[c] = (uint32_t)((F + 0x80000000ull) >> 32);
+                    d.lo[c] = (int32_t)(uint32_t)F;
+                }
+                const FxNum nb = fx_log2e(bb);
+                d.bm = nb.e == kFxSlow ? fx_as_bits(bb) : nb.m;
+                d.be = nb.e;
+                d.z = z;
+                d.occ = o;
+                ax[a0 + pos] = d;
+            }
             if (ar) {  // the accurate re-evaluation's record: 64-bit fixed point, two-float occ and B
                 AtomR e;
                 e.X = fix64(x);
@@ -1199,7 +1212,7 @@ void launch_atoms(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
     if (a.n_struct > 0)
         launch_k(pdl, k_atoms, a.n_struct, 128, st, a.atom_off, a.n_atoms, a.frac, a.Z, a.occ, a.B, a.zmax, a.geo,
-                 a.atoms_set_geo, a.atom_bad, a.atom32, a.atom64, a.runs_mode ? a.astep : (float2*)nullptr, a.atomr,
+                 a.atoms_set_geo, a.atom_bad, a.atom32, a.atomx, a.runs_mode ? a.astep : (float2*)nullptr, a.atomr,
                  a.sctab);
 }
 

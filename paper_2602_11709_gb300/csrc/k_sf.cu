@@ -15,8 +15,10 @@
 // The pattern variants form sin/cos on the FMA pipe from the exact phase
 // (sincos_turn32) and use the SFU for exp2 (MUFU.EX2); the gradient variant
 // uses the SFU for sin/cos too (MUFU.SIN/COS). FP64 arithmetic runs at
-// about 1/64 of the FP32 rate here, so the phase is reduced either in FP64
-// (XRD_FP32_PHASE64) or exactly in 32-bit integers (XRD_FP32_PHASEFIX).
+// about 1/64 of the FP32 rate here, so the phase is formed and reduced mod 1 in integers: from coordinates in 32-bit
+// fixed point (XRD_FP32_PHASEFIX), or in 53-bit fixed point, the resolution of an FP64 phase (XRD_FP32_PHASE64: three
+// more integer products a term; formed in FP64, four operations a term at 1.7 a clock and SM, it made the kernel take
+// 471 us on 1024 cells of 1 to 64 atoms; now about 80 us). The XRD_FP64 variant is k_sf64.cu.
 #include "xrd_internal.cuh"
 #include "xrd_launch.h"
 
@@ -60,6 +62,10 @@ __device__ __forceinline__ float fprime_of(const Coef32& c, float s2)
     return acc;
 }
 
+// Signed low word of a 64-bit fixed-point coordinate, rounded to its upper 21 bits: with |h| <= 511 the sum of
+// three index times low-word products stays below 2^31.
+__device__ __forceinline__ int low21(int32_t lo) { return (lo >> 11) + ((lo >> 10) & 1); }
+
 // The reflections of one lane in a tile: RUNS: one run of `len` reflections
 // consecutive in l from `first` (step 1); otherwise up to RB reflections from
 // `first` with a step of 32 (a tile of 32 RB consecutive reflections), `len` of
@@ -73,7 +79,7 @@ __device__ __forceinline__ float fprime_of(const Coef32& c, float s2)
 // e^{i(k+1)t} = 2 cos t e^{ikt} - e^{i(k-1)t} (two operations instead of four;
 // rounding grows by a few ulp over a run of four): one sin/cos pair per run
 // instead of per reflection. Otherwise every reflection's phase is formed exactly (integer
-// phase) or in FP64 (XRD_FP32_PHASE64).
+// phase; XRD_FP32_PHASE64 with the coordinates' low words too).
 //
 // Pattern variants (not GRAD): sin and cos come from the FMA pipe
 // (sincos_turn32, five times more accurate than the SFU's), F is summed in FP32
@@ -90,7 +96,7 @@ __device__ __forceinline__ float fprime_of(const Coef32& c, float s2)
 // GRAD also accumulates dF/ds^2 = sum_j occ_j exp(-B_j s^2)(f_j' - B_j f_j) e^{i phi_j}.
 template <int PREC, bool GRAD, int kSfRB, bool RUNS>
 __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, int64_t j0, int64_t j1, Atom32* sat,
-                              float2* sstep, const Coef32* scoef, bool staged)
+                              float2* sstep, int4* slo, const Coef32* scoef, bool staged)
 {
     constexpr float ln2 = 0.69314718055994531f;
     constexpr int step = RUNS ? 1 : 32;
@@ -124,6 +130,13 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
             for (int i = lane; i < nc; i += 32) {
                 sat[i] = a.atom32[c0 + i];
                 if (kRotate) sstep[i] = a.astep[c0 + i];
+                if (PREC == XRD_FP32_PHASE64) {
+                    const AtomX d = a.atomx[c0 + i];
+                    sat[i].X = d.hi[0];
+                    sat[i].Y = d.hi[1];
+                    sat[i].Z = d.hi[2];
+                    slo[i] = make_int4(low21(d.lo[0]), low21(d.lo[1]), low21(d.lo[2]), 0);
+                }
             }
             __syncwarp();
         }
@@ -139,7 +152,7 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
                 }
             }
             float cs = 0.f, sn = 0.f, cz = 1.f, sz = 0.f, tcz = 2.f, cp = 0.f, sp = 0.f;
-            double dx = 0.0, dy = 0.0, dz = 0.0;
+            int xl = 0, yl = 0, zl = 0;  // low words of the coordinates (XRD_FP32_PHASE64)
             if (kRotate) {
                 const uint32_t P = uh[0] * at.X + uk[0] * at.Y + ul[0] * at.Z;
                 if (ACC) sincos_turn32(P, sn, cs);
@@ -149,18 +162,16 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
                 sz = st.y;
                 tcz = cz + cz;  // exact
             } else if (PREC == XRD_FP32_PHASE64) {
-                const Atom64 d = a.atom64[c0 + jj];
-                dx = d.x; dy = d.y; dz = d.z;
+                const int4 lo = slo[jj];
+                xl = lo.x; yl = lo.y; zl = lo.z;
             }
             const bool fold = ACC && ((jj & kFoldMask) == kFoldMask || jj == nc - 1);  // uniform
 #pragma unroll
             for (int i = 0; i < kSfRB; i++) {
                 if (!kRotate) {
-                    uint32_t P;
-                    if (PREC == XRD_FP32_PHASEFIX)
-                        P = uh[i] * at.X + uk[i] * at.Y + ul[i] * at.Z;
-                    else
-                        P = fix32(fma((double)(int)uh[i], dx, fma((double)(int)uk[i], dy, (double)(int)ul[i] * dz)));
+                    uint32_t P = uh[i] * at.X + uk[i] * at.Y + ul[i] * at.Z;
+                    if (PREC == XRD_FP32_PHASE64)  // the low words' sum, below 2^31, rounded into the high words'
+                        P += (uint32_t)(((int)uh[i] * xl + (int)uk[i] * yl + (int)ul[i] * zl + (1 << 20)) >> 21);
                     if (ACC) sincos_turn32(P, sn, cs);
                     else __sincosf((float)(int32_t)P * kTwoPiOver2p32, &sn, &cs);
                 }
@@ -237,46 +248,6 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
     return imax;
 }
 
-// FP64 path: the lane's reflections one after another, every term in FP64.
-template <int kSfRB>
-__device__ void sf_tile_fp64(const SfArgs& a, int64_t first, int step, int len, int64_t j0, int64_t j1)
-{
-    for (int i = 0; i < kSfRB; i++) {
-        const bool act = i < len;
-        const int64_t r = first + (int64_t)step * (act ? i : 0);
-        const double q = a.q[r];
-        const uint32_t key = a.key[r];
-        const int h = hkl_h(key), k = hkl_k(key), l = hkl_l(key);
-        const double s2 = q * 0.25;
-        double Fr = 0.0, Fi = 0.0, f = 0.0;
-        int zc = -1;
-        for (int64_t j = j0; j < j1; j++) {
-            const Atom64 at = a.atom64[j];
-            if (at.zz != zc) {
-                zc = at.zz;
-                const double* c = a.coef + 8 * zc;
-                const double sum = c[0] * exp(-c[1] * s2) + c[2] * exp(-c[3] * s2) + c[4] * exp(-c[5] * s2) +
-                                   c[6] * exp(-c[7] * s2);
-                f = (double)zc - kFScale * s2 * sum;
-            }
-            double phi = fma((double)h, at.x, fma((double)k, at.y, (double)l * at.z));
-            phi -= rint(phi);
-            double sn, cs;
-            sincospi(2.0 * phi, &sn, &cs);
-            const double w = at.occ * f * exp(-at.B * s2);
-            Fr = fma(w, cs, Fr);
-            Fi = fma(w, sn, Fi);
-        }
-        const double X = (a.lambda * a.lambda * 0.25) * q;  // sin^2 theta
-        const double c2 = 1.0 - 2.0 * X;                     // cos 2theta
-        const double lp = (1.0 + c2 * c2) / (X * sqrt(fmax(1.0 - X, kCos90Sq)));
-        if (act) {
-            a.I[r] = (Fr * Fr + Fi * Fi) * lp;
-            if (a.F) a.F[r] = make_float2((float)Fr, (float)Fi);
-        }
-    }
-}
-
 // Persistent CTAs; every warp takes tiles of 32 runs (one per lane) from a
 // queue in largest-first order (tiles of the structures with the most atoms
 // first). A structure's atoms stay staged in the warp's shared memory while its
@@ -284,23 +255,21 @@ __device__ void sf_tile_fp64(const SfArgs& a, int64_t first, int step, int len, 
 // Register caps: 64 for the integer-phase variant with 2 reflections per lane
 // (32 resident warps per SM), about 85 for the other FP32 variants (24 warps).
 template <int PREC, bool GRAD, int RB, int WARPS, bool RUNS>
-__global__ void __launch_bounds__(32 * WARPS, PREC == XRD_FP64
-                                                  ? 1
-                                                  : ((PREC == XRD_FP32_PHASEFIX && !GRAD && RB == 2) ? 32 / WARPS
-                                                                                                     : 24 / WARPS))
+__global__ void __launch_bounds__(32 * WARPS,
+                                  (PREC == XRD_FP32_PHASEFIX && !GRAD && RB == 2) ? 32 / WARPS : 24 / WARPS)
     k_sf(const SfArgs a)
 {
     pdl_enter();
     constexpr int kSfThreads = 32 * WARPS;
     __shared__ Atom32 sat[WARPS][kSfChunk];
-    __shared__ float2 sstep[WARPS][kSfChunk];
+    __shared__ float2 sstep[RUNS ? WARPS : 1][RUNS ? kSfChunk : 1];
+    __shared__ int4 slo[PREC == XRD_FP32_PHASE64 ? WARPS : 1][PREC == XRD_FP32_PHASE64 ? kSfChunk : 1];
     extern __shared__ Coef32 scoef[];  // [zmax + 1]
     if (*a.abort_flag) return;
     const int ntiles = a.tile_off[a.n_struct];
-    if (PREC != XRD_FP64) {
-        for (int z = threadIdx.x; z <= a.zmax; z += kSfThreads) scoef[z] = a.coef32[z];
-        __syncthreads();
-    }
+    if ((int)blockIdx.x >= ntiles) return;  // the CTAs before this one already have a tile each
+    for (int z = threadIdx.x; z <= a.zmax; z += kSfThreads) scoef[z] = a.coef32[z];
+    __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int staged_s = -1;  // structure whose atoms (one chunk at most) are in sat[w]
     for (;;) {
@@ -330,18 +299,15 @@ __global__ void __launch_bounds__(32 * WARPS, PREC == XRD_FP64
             len = (int)max(min((re - first + 31) / 32, (int64_t)RB), (int64_t)0);
         }
         if (len == 0) first = rbase;  // keep the lane's (ignored) loads inside the array
-        if (PREC == XRD_FP64) {
-            sf_tile_fp64<RB>(a, first, RUNS ? 1 : 32, len, j0, j1);
-        } else {
-            const bool one_chunk = j1 - j0 <= kSfChunk;
-            float m = sf_tile_fp32<PREC, GRAD, RB, RUNS>(a, s, first, len, j0, j1, sat[w], sstep[w], scoef,
-                                                         one_chunk && s == staged_s);
-            staged_s = one_chunk ? s : -1;
-            if (!GRAD && a.imax) {  // the structure's largest reflection intensity (I >= 0: integer order)
+        const bool one_chunk = j1 - j0 <= kSfChunk;
+        float m = sf_tile_fp32<PREC, GRAD, RB, RUNS>(a, s, first, len, j0, j1, sat[w], sstep[RUNS ? w : 0],
+                                                     slo[PREC == XRD_FP32_PHASE64 ? w : 0], scoef,
+                                                     one_chunk && s == staged_s);
+        staged_s = one_chunk ? s : -1;
+        if (!GRAD && a.imax) {  // the structure's largest reflection intensity (I >= 0: integer order)
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if (lane == 0 && m > 0.f) atomicMax(a.imax + s, __float_as_uint(m));
-            }
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0 && m > 0.f) atomicMax(a.imax + s, __float_as_uint(m));
         }
     }
 }
@@ -351,7 +317,7 @@ static void launch_sf_shape(const SfArgs& a, cudaStream_t st, bool pdl)
 {
     // persistent grid: as many CTAs as fit on the SMs at once (cached per device and zmax)
     static int cache_per_sm[64] = {}, cache_zmax[64] = {};
-    const size_t smem = PREC == XRD_FP64 ? 0 : sizeof(Coef32) * (size_t)(a.zmax + 1);
+    const size_t smem = sizeof(Coef32) * (size_t)(a.zmax + 1);
     int dev = 0;
     cudaGetDevice(&dev);
     const bool cached = dev >= 0 && dev < 64 && cache_per_sm[dev] > 0 && cache_zmax[dev] == a.zmax;
@@ -384,7 +350,7 @@ void launch_sf(const SfArgs& a, cudaStream_t st, bool pdl)
         return;
     }
     switch (a.precision) {
-    case XRD_FP64: launch_sf_prec<XRD_FP64, false>(a, st, pdl); break;
+    case XRD_FP64: launch_sf64(a, st, pdl); break;
     case XRD_FP32_PHASE64: launch_sf_prec<XRD_FP32_PHASE64, false>(a, st, pdl); break;
     default:
         if (a.runs_mode) {

@@ -67,10 +67,17 @@ struct __align__(16) Atom32 {
     float zf;          // element number as a float (f(s) = Z + ...)
 };
 
-// Atom record for the FP64 loops and the FP64 phase.
-struct __align__(16) Atom64 {
-    double x, y, z, B, occ;
-    int32_t zz, pad;
+// Atom record for the FP64 loop and the FP64-accurate phase, element-sorted like Atom32: coordinates in 64-bit
+// fixed point as hi 2^32 + lo with a signed low word (an index times a coordinate is then one 32-bit and one
+// widening 32-bit product), B log2(e) as a 64-bit significand and an exponent (xrd_fx.cuh; be = kFxSlow: bm holds
+// the bits of B instead), the occupancy.
+struct __align__(16) AtomX {
+    uint32_t hi[3];
+    int32_t lo[3];
+    int32_t z;   // element number
+    int32_t be;
+    uint64_t bm;
+    double occ;
 };
 
 // f(s) = Z + s^2 sum_i a'_i 2^(bl_i s^2) with a'_i = -41.78214 a_i, bl_i = -b_i log2(e).

@@ -25,7 +25,7 @@ struct GeomArgs {
     Geo* geo;
     Coef32* coef32;
     Atom32* atom32;
-    Atom64* atom64;
+    AtomX* atomx;    // records of XRD_FP64 and XRD_FP32_PHASE64 (nullptr: not written)
     float2* astep;   // [atoms] exp(2 pi i z) of each element-sorted atom
     int64_t* refl_cnt;
     int64_t* run_cnt;  // [n_struct] runs of each structure
@@ -71,7 +71,7 @@ struct SfArgs {
     const Coef32* coef32;
     const double* coef;
     const Atom32* atom32;
-    const Atom64* atom64;
+    const AtomX* atomx;
     const double* q;
     const uint32_t* key;
     double* I;   // per reflection intensity |F|^2 LP (one Friedel half-space member), XRD_FP64
@@ -276,6 +276,8 @@ void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st);  // out: device [3], zeroed
 void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_sf(const SfArgs& a, cudaStream_t st, bool pdl);
+void launch_sf64(const SfArgs& a, cudaStream_t st, bool pdl);  // the XRD_FP64 variant
+bool init_fx_tables(cudaStream_t st);  // its tables, in device memory
 RefineTables init_refine_tables(cudaStream_t st);  // fills the tables, returns their device addresses
 void launch_refine(const RefineArgs& a, cudaStream_t st, bool pdl);
 size_t post_smem_bytes(int cap);

@@ -1,0 +1,54 @@
+"""The FP64 structure factor (fixed-point exp and sin/cos) and the FP64-accurate phase against the oracle, at the
+edges of their forms: atom counts around the staging chunk, coordinates outside [0, 1), occupancies other than 1,
+and coefficients that the fixed-point exponential covers, saturates on or leaves to the library's exp."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_11709_gb300 import synth
+
+from parity import compare_batch
+
+pytestmark = pytest.mark.gpu
+
+
+def _batch(rng, counts):
+    b = synth.concat([synth.random_cell(rng, n, edge=(3.0, 7.0)) for n in counts])
+    b.frac = rng.uniform(-3.0, 3.0, b.frac.shape)
+    b.occ = rng.choice([0.0, 0.25, 1.0, 1.0, 1.75], b.n_atoms)
+    b.occ[b.atom_off[:-1]] = 1.0  # no structure without scattering
+    return b
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_phase64"])
+@pytest.mark.parametrize("form", ["plain", "B_zero_and_large", "b_zero_and_large"])
+def test_forms(gpu_lib, prec, form):
+    rng = np.random.default_rng(20)
+    b = _batch(rng, [1, 31, 32, 33, 64, 65, 127, 129])
+    if form == "B_zero_and_large":
+        b.B[::3] = 0.0
+        b.B[1::5] = 3000.0
+    elif form == "b_zero_and_large":
+        b.coef[::2, 0, 1] = 0.0
+        b.coef[1::3, 1, 1] = 5e4
+        b.coef[::5, 2] = 0.0
+    o = synth.Opts(rel_cutoff=0.0, scaled=0)
+    got = gpu_lib.compute(b, o, prec)
+    compare_batch(got, oracle.pattern_batch(b, o), prec, o.rel_cutoff, o.scaled)
+
+
+@pytest.mark.parametrize("form", ["B_negative", "b_negative", "b_beyond_range"])
+def test_library_exp_forms(gpu_lib, form):
+    """Exponents that grow or lie outside the fixed-point range take the library's exp, atom by atom."""
+    rng = np.random.default_rng(21)
+    b = _batch(rng, [1, 33, 40])
+    if form == "B_negative":
+        b.B[::4] = -0.7
+    elif form == "b_negative":
+        b.coef[::2, 3, 1] = -0.3
+    else:
+        b.coef[::2, 3, 1] = 1e-310
+        b.coef[1::2, 2, 1] = 1e305
+    o = synth.Opts(rel_cutoff=0.0, scaled=0)
+    got = gpu_lib.compute(b, o, "fp64")
+    compare_batch(got, oracle.pattern_batch(b, o), "fp64", o.rel_cutoff, o.scaled)
