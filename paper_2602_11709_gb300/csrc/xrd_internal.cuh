@@ -234,20 +234,28 @@ __device__ __forceinline__ float ex2_approx(float x)
 // rounded to FP32; approximation error below 2.3e-9) are rotated back by q quarter turns. About
 // 2e-8 RMS and 1e-7 largest absolute error, five times below the SFU's sin/cos, whose error
 // dominated the FP32 structure factor.
+constexpr float kSinC[3] = {-0.16666650772094727f, 0.00833197869360447f, -0.00019495634478516877f};
+constexpr float kCosC[4] = {-0.5f, 0.04166662320494652f, -0.0013886763481423259f, 2.439044874336105e-05f};
+
+// (sin, cos)(a + q pi/2) from those of a: q = 1: (cos, -sin), 2: (-sin, -cos), 3: (-cos, sin)
+__device__ __forceinline__ void turn_quadrant(uint32_t q, float sa, float ca, float& s, float& c)
+{
+    const bool swap = q & 1u;
+    const float s1 = swap ? ca : sa, c1 = swap ? sa : ca;
+    s = __int_as_float(__float_as_int(s1) ^ (int)((q & 2u) << 30));
+    c = __int_as_float(__float_as_int(c1) ^ (int)(((q + 1u) & 2u) << 30));
+}
+
 __device__ __forceinline__ void sincos_turn32(uint32_t P, float& s, float& c)
 {
     const uint32_t q = (P + 0x20000000u) >> 30;
     const float a = (float)(int32_t)(P - (q << 30)) * 1.4629180792671596e-09f;  // 2 pi / 2^32
     const float a2 = a * a;
-    const float ps = fmaf(fmaf(-0.00019495634478516877f, a2, 0.00833197869360447f), a2, -0.16666650772094727f);
+    const float ps = fmaf(fmaf(kSinC[2], a2, kSinC[1]), a2, kSinC[0]);
     const float sa = fmaf(a * a2, ps, a);
-    const float pc = fmaf(fmaf(fmaf(2.439044874336105e-05f, a2, -0.0013886763481423259f), a2, 0.04166662320494652f),
-                          a2, -0.5f);
+    const float pc = fmaf(fmaf(fmaf(kCosC[3], a2, kCosC[2]), a2, kCosC[1]), a2, kCosC[0]);
     const float ca = fmaf(a2, pc, 1.f);
-    const bool swap = q & 1u;  // (sin, cos)(a + q pi/2): q = 1: (cos, -sin), 2: (-sin, -cos), 3: (-cos, sin)
-    const float s1 = swap ? ca : sa, c1 = swap ? sa : ca;
-    s = __int_as_float(__float_as_int(s1) ^ (int)((q & 2u) << 30));
-    c = __int_as_float(__float_as_int(c1) ^ (int)(((q + 1u) & 2u) << 30));
+    turn_quadrant(q, sa, ca, s, c);
 }
 
 // Positive normal double -> two floats, q = qh + ql to about 2^-47 relative,
