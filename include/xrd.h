@@ -355,9 +355,8 @@ int xrd_set_sf_shape(xrd_handle* h, int tile, int warps, int runs);
  */
 int xrd_set_point_group(xrd_handle* h, const int32_t* ops, int n_ops);
 
-/* Launch shape of the enumeration kernels (256 by default): 64, 128 or 256 threads per CTA
- * with one warp per structure (the CTA's whole block takes the few structures above 1024
- * columns or 4096 reflections), or 512 or 1024 threads with one CTA per structure.
+/* Threads per CTA of the enumeration kernels: 64, 128, 256 (the default), 512 or 1024. Every warp takes
+ * one structure, or one part of a structure with many (h, k) columns, at a time.
  * Neither the order of the enumerated reflections nor the pattern changes with it. */
 int xrd_set_enum_threads(xrd_handle* h, int threads);
 

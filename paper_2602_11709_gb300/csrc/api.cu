@@ -23,7 +23,7 @@ struct xrd_handle {
     const xrd::TTab* ttab = nullptr;  // 2-theta table on the handle's device
     int sf_rb = 4, sf_warps = 2;        // structure-factor launch shape (xrd_autotune)
     int sf_runs = 0;                    // lanes take runs consecutive in l (integer phase only)
-    int enum_threads = 256;             // threads per structure of the enumeration kernels (xrd_autotune)
+    int enum_threads = 256;             // threads per CTA of the enumeration kernels (xrd_autotune)
     // side streams for the concurrent post-processing size classes (fork/join by events)
     cudaStream_t side[xrd::kPostStreams - 1] = {};
     cudaEvent_t fork = nullptr, join[xrd::kPostStreams - 1] = {};
@@ -43,11 +43,12 @@ namespace {
 constexpr int kRunsPerTileHost = xrd::kRunsPerTile;  // structure-factor tile: 32 runs (one per lane)
 // flags area, zeroed at the start of every call: flag words (see GeomArgs::abort_flag), the
 // structure-factor work counters (3 x 64 bit) at byte kWorkOffset, the re-evaluation's
-// reflection count (64 bit) at kRefinedOffset, the enumeration claims at int 26 and the post
+// reflection count (64 bit) at kRefinedOffset, the enumeration claims and parts at ints 26 to 28 and the post
 // class counts and work counters at ints kFlagClsCnt and kFlagClsNext
 constexpr int kFlagBytes = 256;
 constexpr int kWorkOffset = 64;
 constexpr int kRefinedOffset = 96;
+constexpr int kQueryParts = 16384;  // enumeration parts of a reflection count outside a call
 constexpr int kStages = 9;
 constexpr int kSfStage = 5;      // index of the structure-factor stage
 constexpr int kRefineStage = 6;  // index of the re-evaluation stage
@@ -317,6 +318,9 @@ xrd::GeomArgs geom_args(const xrd_batch* b, const xrd_opts* o, const Layout& L, 
     g.cls_list = (int*)(ws + L.cls_list);
     g.abort_flag = (int*)(ws + L.flags);
     g.enum_ctr = g.abort_flag + 26;
+    g.part_tab = (int2*)(ws + L.st_q);  // free until the post-processing
+    g.part_cnt = (int2*)(ws + L.st_I);
+    g.part_cap = (int)std::min<int64_t>(cap_refl, INT32_MAX / 2);
     g.totals = totals;
     g.status = status;
     g.q = (double*)(ws + L.q);
@@ -372,9 +376,9 @@ int xrd_create(xrd_handle** h, int device)
     if (e != cudaSuccess) { xrd_destroy(p); return XRD_ECUDA; }
     p->ttab = xrd::init_tables(0);  // device tables (2-theta, re-evaluation), once per handle, legacy stream
     p->rtab = xrd::init_refine_tables(0);
-    const bool fx = xrd::init_fx_tables(0);
+    xrd::init_fx_tables(0);
     e = cudaStreamSynchronize(0);
-    if (e != cudaSuccess || !p->ttab || !p->rtab.sc || !p->rtab.ex || !fx) { xrd_destroy(p); return XRD_ECUDA; }
+    if (e != cudaSuccess || !p->ttab || !p->rtab.sc || !p->rtab.ex) { xrd_destroy(p); return XRD_ECUDA; }
     *h = p;
     return XRD_OK;
 }
@@ -445,7 +449,7 @@ static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* 
     const int64_t n = b->n_struct;
     cnt.assign(n, 0);
     if (n == 0) return XRD_OK;
-    const size_t need = al(sizeof(xrd::Geo) * n) + al(8 * n) + al(16);
+    const size_t need = al(sizeof(xrd::Geo) * n) + al(8 * n) + al(16) + 2 * al(8 * kQueryParts);
     if (h->qbuf_bytes < need) {
         if (h->qbuf) cudaFree(h->qbuf);
         h->qbuf = nullptr;
@@ -464,6 +468,11 @@ static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* 
     a.geo = (xrd::Geo*)((char*)h->qbuf + L.geo);
     a.refl_cnt = (int64_t*)((char*)h->qbuf + L.refl_cnt);
     a.enum_ctr = (int*)((char*)h->qbuf + L.refl_cnt + al(8 * n));  // the counting kernel's claim counter
+    a.part_tab = (int2*)((char*)a.enum_ctr + al(16));
+    a.part_cnt = (int2*)((char*)a.part_tab + al(8 * kQueryParts));
+    a.part_cap = kQueryParts;
+    a.enum_threads = 256;
+    a.sms = h->sms;
     cudaMemsetAsync(a.enum_ctr, 0, 16, st);
     xrd::launch_count_only(a, st);
     cudaError_t e = cudaMemcpyAsync(cnt.data(), a.refl_cnt, 8 * n, cudaMemcpyDeviceToHost, st);
@@ -555,6 +564,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     ga.sctab = h->rtab.sc;
     ga.runs_mode = runs;
     ga.enum_threads = h->enum_threads;
+    ga.sms = h->sms;
     ga.out_flags = out->flags;
     const bool refine = h->refine && o->precision != XRD_FP64;
 
@@ -916,8 +926,7 @@ int xrd_autotune(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const xrd
     h->sf_rb = brb;
     h->sf_warps = bw;
     h->sf_runs = bruns;
-    // then the enumeration's launch shape with that shape: one warp per structure (64-256 threads
-    // per CTA) for many small structures, one CTA of 512 or 1024 threads per structure for large ones
+    // then the threads per CTA of the enumeration with that shape
     const int keep_et = h->enum_threads;
     float best_et = 1e30f;
     int bet = keep_et;
@@ -1067,6 +1076,7 @@ static void launch_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, c
     ga.rb = rb;
     ga.runs_mode = grad ? 0 : runs;
     ga.enum_threads = grad ? 256 : h->enum_threads;
+    ga.sms = h->sms;
     radii(o, ga.r2min, ga.r2max, ga.rmax);
     ga.cap_refl = cap_refl;
     ga.lattice = b->lattice;
@@ -1092,6 +1102,9 @@ static void launch_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, c
     ga.tile_tab = (int2*)(ws + L.tile_tab);
     ga.abort_flag = (int*)(ws + L.flags);
     ga.enum_ctr = ga.abort_flag + 26;
+    ga.part_tab = (int2*)(ws + L.Fx);  // 16 bytes a reflection, free until the structure factor
+    ga.part_cnt = ga.part_tab + cap_refl;
+    ga.part_cap = (int)std::min<int64_t>(cap_refl, INT32_MAX / 2);
     ga.totals = totals;
     ga.status = status;
     ga.q = (double*)(ws + L.q);

@@ -41,7 +41,7 @@ __device__ __forceinline__ double cosd(double deg)
 // pointers are given.
 template <int LANES>
 __global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, Geo* __restrict__ geo,
-                       unsigned* __restrict__ imax, int32_t* __restrict__ flags)
+                       unsigned* __restrict__ imax, int32_t* __restrict__ flags, const EnumParts ep)
 {
     pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -95,7 +95,6 @@ __global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, G
             }
             const double v = ok ? __ddiv_rn(Cj, det) : 0.0;
             g.gs[j] = v;
-            if (j >= 3) g.g2[j - 3] = 2.0 * v;  // exact
             const float v32 = ok ? __double2float_rn(v) : 0.f;
             g.gf[j] = v32;
             g.gl[j] = ok ? __double2float_rn(v - (double)v32) : 0.f;
@@ -118,6 +117,20 @@ __global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, G
             g.K = K;
             g.L = L;
             g.status = st;
+            // the enumeration's parts of a structure with many columns (k_count, k_emit)
+            int pbase = -1;
+            const int ncol = H < 0 ? 0 : (K + 1) + H * (2 * K + 1);
+            if (ncol > ep.cols) {
+                const int np = (ncol + ep.cols - 1) / ep.cols, b = atomicAdd(ep.ctr, np);
+                const bool room = b >= 0 && b <= ep.cap - np;
+                if (room) pbase = b;
+                for (int i = 0; i < np && b >= 0 && b + i < ep.cap; i++) ep.tab[b + i] = make_int2(room ? s : -1, i);
+                if (room) {
+                    ep.cnt[s] = 0;
+                    if (ep.run_cnt) ep.run_cnt[s] = 0;
+                }
+            }
+            g.pbase = pbase;
         }
     }
 }
@@ -125,8 +138,7 @@ __global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, G
 // 8 lanes per structure up to this many structures (latency-bound), one above (throughput-bound)
 constexpr int kPrepWideMax = 8192;
 
-static void prep_launch(bool pdl, const double* lattice, int n, double rmax, Geo* geo, unsigned* imax,
-                        int32_t* flags, cudaStream_t st);
+static int enum_part_cols(int n_struct);
 
 // f(s) coefficients in the form the FP32 loops use (exp2 with the scale folded
 // in) and, for the accurate re-evaluation, (a_i, b_i) as two floats each
@@ -403,53 +415,6 @@ __device__ __forceinline__ void column_hk(const Geo& g, int c, int& h, int& k)
 // within the structure) << 3 | length.
 __device__ __forceinline__ int runs_of(int n, int rb) { return (n + rb - 1) / rb; }
 
-// Exclusive block scan of one (x, y) pair per thread, with the block totals.
-// tmp: 66 ints of shared memory; the caller synchronises before reusing it.
-__device__ __forceinline__ void block_scan_pair(int x, int y, int* tmp, int& ex, int& ey, int& tx, int& ty)
-{
-    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ix = warp_incl_scan(x), iy = warp_incl_scan(y);
-    if (lane == 31) {
-        tmp[w] = ix;
-        tmp[33 + w] = iy;
-    }
-    __syncthreads();
-    if (w == 0) {
-        const int sx = lane < nw ? tmp[lane] : 0, sy = lane < nw ? tmp[33 + lane] : 0;
-        const int px = warp_incl_scan(sx), py = warp_incl_scan(sy);
-        if (lane < nw) {
-            tmp[lane] = px - sx;
-            tmp[33 + lane] = py - sy;
-        }
-        if (lane == 31) {
-            tmp[32] = px;
-            tmp[65] = py;
-        }
-    }
-    __syncthreads();
-    ex = tmp[w] + ix - x;
-    ey = tmp[33 + w] + iy - y;
-    tx = tmp[32];
-    ty = tmp[65];
-}
-
-// Launch shapes of counting and emission (enum_threads): with 64, 128 or 256
-// threads per CTA every warp takes one structure at a time, claimed from a
-// counter, so the fixed cost of a structure (the loads of its cell, the
-// scans) is a warp's, not a CTA's, and a small structure's columns fill a
-// warp's lanes; with 512 or 1024 threads every structure has a CTA of its own
-// (batches of large cells).
-constexpr int kEnumMaxThreads = 1024;
-constexpr int kWarpModeMaxThreads = 256;
-constexpr int kWarpRecInts = 2 * 33 + 8 * 32;  // one warp's chunk of 32 column records
-
-__host__ __device__ inline bool enum_per_warp(int threads) { return threads <= kWarpModeMaxThreads; }
-__host__ __device__ inline int enum_cta_ints(int threads) { return 2 * (threads + 1) + 8 * threads; }
-size_t enum_smem_bytes(int threads)
-{
-    return 4 * ((enum_per_warp(threads) ? (threads / 32) * kWarpRecInts : 0) + enum_cta_ints(threads));
-}
-
 // The exact comparison of a candidate within the FP32 error bound of a sphere
 // surface, kept out of line so that the rare FP64 evaluation is a branch, not
 // work that every caller does.
@@ -482,178 +447,167 @@ __device__ __forceinline__ int warp_sum_int(int v)
     return v;
 }
 
-// Reflection (and, with rb > 0, run) counts per structure. With one warp per
-// structure the warps claim structures from a counter (ctr, zero at launch),
-// so a CTA is not held by its slowest structure; every structure, however
-// many columns it has, is counted by one warp.
+// Work of the enumeration kernels: one warp per item. A structure of more than part_cols columns is split into
+// parts of part_cols columns, which k_prep lists (GeomArgs::part_tab; Geo.pbase: the structure's first part) with
+// room for part_cap parts; a structure that finds no room, or has fewer columns, is one item. A warp takes a part in
+// about the time of part_cols / 32 steps of 32 columns, so a batch of few large cells, or one cell, fills the part.
+// Measured with one warp or one CTA a structure before: the 50 A cell of 679 000 reflections 0.25 ms to count and
+// 1.53 ms to emit, 256 cells of 15-40 A 0.13 and 1.37 ms.
+// Items are claimed from a counter, the parts first: kClaim structures (or one part) at a time.
+constexpr int kEnumMaxThreads = 1024;
+constexpr int kClaimWide = 4;         // structures a claim takes in a batch of at least kWideBatch structures
+constexpr int kWideBatch = 2048;      // enough structures to fill the GPU by themselves:
+constexpr int kPartColsWide = 512;    // only the longest are split; below, every chunk of 32 columns is an item, since
+constexpr int kPartColsNarrow = 32;   // a warp's chunks are a serial chain of about 5 us each
+static int enum_part_cols(int n_struct) { return n_struct >= kWideBatch ? kPartColsWide : kPartColsNarrow; }
+
+struct EnumItems {
+    int nparts, n_struct, claim;
+    int* ctr;
+    // claims the next items: first is the first of n items (parts: 0 .. nparts - 1, then structures); n = 0 at the end
+    __device__ __forceinline__ int next(int& n) const
+    {
+        const int lane = threadIdx.x & 31;
+        int v = 0;
+        if (lane == 0) v = atomicAdd(ctr, 1);
+        v = __shfl_sync(0xffffffffu, v, 0);
+        if (v < nparts) {
+            n = 1;
+            return v;
+        }
+        const int s0 = (v - nparts) * claim;
+        n = max(0, min(claim, n_struct - s0));
+        return nparts + s0;
+    }
+};
+
+__device__ __forceinline__ EnumItems enum_items(int n_struct, const int* part_ctr, int part_cap, int* ctr)
+{
+    return EnumItems{min(*part_ctr, part_cap), n_struct, n_struct >= kWideBatch ? kClaimWide : 1, ctr};
+}
+
+// The structure and the columns [c0, c1) of an item; false where there is nothing to do (a structure that its
+// parts cover, a slot of a structure that found no room)
+__device__ __forceinline__ bool enum_item(const Geo* __restrict__ geo, const int2* __restrict__ part_tab, int nparts,
+                                          int part_cols, int item, int& s, int& part, Geo& g, int& c0, int& c1)
+{
+    part = -1;
+    s = item - nparts;
+    if (item < nparts) {
+        const int2 t = part_tab[item];
+        s = t.x;
+        part = t.y;
+        if (s < 0) return false;
+    }
+    g = geo[s];
+    const int ncol = n_columns(g);
+    c0 = 0;
+    c1 = ncol;
+    if (part >= 0) {
+        c0 = part * part_cols;
+        c1 = min(c0 + part_cols, ncol);
+    } else if (g.pbase >= 0) {
+        return false;
+    }
+    return true;
+}
+
+// Reflection (and, with RUNS, run) counts per structure, and of every part (k_prep has zeroed the counts of a
+// structure in parts). ctr: zero at launch.
 template <bool RUNS>
 __global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict__ geo, int n_struct, double r2min,
                                                            double r2max, float r2minf, float r2maxf, int rb,
                                                            int64_t* __restrict__ cnt, int64_t* __restrict__ run_cnt,
-                                                           int* __restrict__ ctr)
+                                                           int* __restrict__ ctr, const int* __restrict__ part_ctr,
+                                                           const int2* __restrict__ part_tab,
+                                                           int2* __restrict__ part_cnt, int part_cap, int part_cols)
 {
     pdl_enter();
-    __shared__ int tmp[66];
-    const int nt = blockDim.x, lane = threadIdx.x & 31;
-    if (enum_per_warp(nt)) {
-        for (;;) {
-            int s = 0;
-            if (lane == 0) s = atomicAdd(ctr, 1);
-            s = __shfl_sync(0xffffffffu, s, 0);
-            if (s >= n_struct) break;
-            const Geo g = geo[s];
-            const int ncol = n_columns(g);
+    const int lane = threadIdx.x & 31;
+    const EnumItems items = enum_items(n_struct, part_ctr, part_cap, ctr);
+    for (;;) {
+        int m;
+        const int first = items.next(m);
+        if (m == 0) break;
+        for (int it = first; it < first + m; it++) {
+            int s, part, c0, c1;
+            Geo g;
+            if (!enum_item(geo, part_tab, items.nparts, part_cols, it, s, part, g, c0, c1)) continue;
             int local = 0, local_runs = 0;
-            for (int c = lane; c < ncol; c += 32) {
-                int h, k, m, mr;
-                column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, m, mr);
-                local += m;
-                local_runs += mr;
+            for (int c = c0 + lane; c < c1; c += 32) {
+                int h, k, n, nr;
+                column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, n, nr);
+                local += n;
+                local_runs += nr;
             }
             local = warp_sum_int(local);
             if (RUNS) local_runs = warp_sum_int(local_runs);
-            if (lane == 0) {
+            if (lane != 0) continue;
+            if (part < 0) {
                 cnt[s] = local;
                 if (RUNS && run_cnt) run_cnt[s] = local_runs;
+            } else {
+                part_cnt[it] = make_int2(local, local_runs);
+                atomicAdd((unsigned long long*)(cnt + s), (unsigned long long)local);
+                if (RUNS && run_cnt) atomicAdd((unsigned long long*)(run_cnt + s), (unsigned long long)local_runs);
             }
         }
-        return;
-    }
-    const int sb = blockIdx.x;  // one CTA per structure
-    if (sb >= n_struct) return;
-    const Geo g = geo[sb];
-    const int ncol = n_columns(g);
-    int local = 0, local_runs = 0;
-    for (int c = threadIdx.x; c < ncol; c += nt) {
-        int h, k, m, mr;
-        column_counts(g, geo[sb].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, m, mr);
-        local += m;
-        local_runs += mr;
-    }
-    int ex, ey, tx, ty;
-    block_scan_pair(local, local_runs, tmp, ex, ey, tx, ty);
-    if (threadIdx.x == 0) {
-        cnt[sb] = tx;
-        if (RUNS && run_cnt) run_cnt[sb] = ty;
     }
 }
 
-// Column records of one chunk of columns, for the flat emission: offsets, the
-// l interval and gap, (h, k), and the column's |g|^2 as a polynomial in l,
-// q(l) = t + u l + G*33 l^2 with t = G*11 h^2 + G*22 k^2 + 2 G*12 hk and
-// u = 2 G*13 h + 2 G*23 k in two-float arithmetic (about 1e-14 relative).
-struct ChunkCols {
-    int* off;   // [m + 1] exclusive reflection offsets within the chunk
-    int* roff;  // [m + 1] exclusive run offsets
-    int* a;     // first l
-    int* c;     // first l of the inner gap (INT_MAX: none)
-    int* gap;   // its length
-    int* hk;    // (h << 16) | (k & 0xffff)
-    float *th, *tl, *uh, *ul;
+// Record of a non-empty column of a chunk: its |g|^2 as a polynomial in l, q(l) = t + u l + G*33 l^2 with
+// t = G*11 h^2 + G*22 k^2 + 2 G*12 hk and u = 2 G*13 h + 2 G*23 k in two-float arithmetic (about 1e-14 relative),
+// and where its reflections and runs go.
+struct __align__(16) ColRec {
+    float th, tl, uh, ul;
+    int a_off;      // first l minus the column's offset within the chunk
+    int c, gap;     // first l of the inner gap (INT_MAX: none), its length
+    uint32_t key0;  // the packed key of (h, k, 0)
+    int off, roff;  // offset of the column's reflections and runs within the chunk
+    int n, n1;      // its reflections, and those below the gap
 };
 
-__device__ __forceinline__ ChunkCols chunk_cols(int* b, int m)
+__device__ __forceinline__ ColRec column_rec(const Geo& g, const ColSpan& sp, int h, int k, int n, int off, int roff)
 {
-    ChunkCols cc;
-    cc.off = b;
-    cc.roff = b + (m + 1);
-    int* r = b + 2 * (m + 1);
-    cc.a = r;
-    cc.c = r + m;
-    cc.gap = r + 2 * m;
-    cc.hk = r + 3 * m;
-    cc.th = (float*)(r + 4 * m);
-    cc.tl = (float*)(r + 5 * m);
-    cc.uh = (float*)(r + 6 * m);
-    cc.ul = (float*)(r + 7 * m);
-    return cc;
-}
-
-__device__ __forceinline__ void put_col(const ChunkCols& cc, int i, const Geo& g, const ColSpan& sp, int h, int k)
-{
-    cc.a[i] = sp.a;
-    cc.c[i] = sp.c <= sp.d ? sp.c : INT_MAX;
-    cc.gap[i] = sp.c <= sp.d ? sp.d - sp.c + 1 : 0;
-    cc.hk[i] = (h << 16) | (k & 0xffff);
+    ColRec r;
     const F2 G11{g.gf[0], g.gl[0]}, G22{g.gf[1], g.gl[1]}, G12{2.f * g.gf[3], 2.f * g.gl[3]};
     const F2 G13{2.f * g.gf[4], 2.f * g.gl[4]}, G23{2.f * g.gf[5], 2.f * g.gl[5]};
     const F2 t = f2_add(f2_add(f2_mul_int(G11, (float)(h * h)), f2_mul_int(G22, (float)(k * k))),
                         f2_mul_int(G12, (float)(h * k)));
     const F2 u = f2_add(f2_mul_int(G13, (float)h), f2_mul_int(G23, (float)k));
-    cc.th[i] = t.hi;
-    cc.tl[i] = t.lo;
-    cc.uh[i] = u.hi;
-    cc.ul[i] = u.lo;
+    r.th = t.hi;
+    r.tl = t.lo;
+    r.uh = u.hi;
+    r.ul = u.lo;
+    r.a_off = sp.a - off;
+    r.c = sp.c <= sp.d ? sp.c : INT_MAX;
+    r.gap = sp.c <= sp.d ? sp.d - sp.c + 1 : 0;
+    r.key0 = hkl_pack(h, k, 0);
+    r.off = off;
+    r.roff = roff;
+    r.n = n;
+    r.n1 = sp.first_part();
+    return r;
 }
 
-// Writes the chunk's reflections (and runs): thread t of nt takes positions t,
-// t + nt, ...; each finds its column by bisection over the m offsets, so the
-// writes of consecutive threads are consecutive.
-template <bool RUNS>
-__device__ __forceinline__ void emit_chunk(const F2 g33, const ChunkCols& cc, int m, int tot, int rtot, int t, int nt,
-                                           int rb, int64_t base, int64_t cap, int done, int done_runs,
-                                           double* __restrict__ q, uint32_t* __restrict__ key, int* __restrict__ runs)
-{
-    for (int p = t; p < tot; p += nt) {
-        int lo = 0, hi = m - 1;  // last column with off <= p
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (cc.off[mid] <= p) lo = mid;
-            else hi = mid - 1;
-        }
-        const int hk = cc.hk[lo];
-        int l = cc.a[lo] + (p - cc.off[lo]);
-        if (l >= cc.c[lo]) l += cc.gap[lo];
-        const int64_t pos = done + p;
-        if (pos < cap) {
-            const float fl = (float)l;
-            const F2 v = f2_add(f2_add(F2{cc.th[lo], cc.tl[lo]}, f2_mul_int(g33, fl * fl)),
-                                f2_mul_int(F2{cc.uh[lo], cc.ul[lo]}, fl));
-            q[base + pos] = f2d_fast(v.hi) + f2d_fast(v.lo);
-            key[base + pos] = hkl_pack(hk >> 16, (int)(short)(hk & 0xffff), l);
-        }
-    }
-    if (RUNS) {
-        for (int p = t; p < rtot; p += nt) {
-            int lo = 0, hi = m - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (cc.roff[mid] <= p) lo = mid;
-                else hi = mid - 1;
-            }
-            const int n = cc.off[lo + 1] - cc.off[lo];
-            const int n1 = cc.gap[lo] > 0 ? cc.c[lo] - cc.a[lo] : n;
-            const int j = p - cc.roff[lo], r1 = runs_of(n1, rb);
-            const int first = j < r1 ? j * rb : n1 + (j - r1) * rb;
-            const int len = j < r1 ? min(rb, n1 - j * rb) : min(rb, n - n1 - (j - r1) * rb);
-            const int64_t rpos = done_runs + p;
-            if (rpos < cap) runs[base + rpos] = ((done + cc.off[lo] + first) << 3) | len;
-        }
-    }
-}
-
-// The structure's entries of the structure-factor tile table from tile_off[s]:
-// (s, first run) of each tile of 32 runs (rb > 0), or (s, first reflection)
-// of each tile of tile_refl reflections.
-__device__ __forceinline__ void write_tiles(int s, int rb, int tile_refl, int64_t units, const int* __restrict__ tile_off,
+// The item's entries of the structure-factor tile table from tile_off[s]: (s, first run) of each tile of 32 runs
+// (runs), or (s, first reflection) of each tile of tile_refl reflections; entries t, t + nt, ...
+__device__ __forceinline__ void write_tiles(int s, bool runs, int tile_refl, int64_t units, const int* __restrict__ tile_off,
                                             int2* __restrict__ tile_tab, int t, int nt)
 {
-    const int per = rb > 0 ? kRunsPerTile : tile_refl;
+    const int per = runs ? kRunsPerTile : tile_refl;
     const int ntl = (int)((units + per - 1) / per), t0 = tile_off[s];
     for (int i = t; i < ntl; i += nt) tile_tab[t0 + i] = make_int2(s, i * per);
 }
 
 // Writes |g|^2 and the packed (h, k, l) of every reflection of each structure
-// (and its runs, rb > 0) from refl_off[s], and its tile-table entries. The
-// columns are taken 32 (one warp) or blockDim (the CTA) at a time: each thread
-// finds its column's span, a scan places the columns, and the warp or CTA then
-// writes the chunk's reflections and runs as one flat, coalesced range. The
+// (and its runs) from refl_off[s], and its tile-table entries. A warp takes an item's
+// columns 32 at a time: each lane finds its column's span, a scan places the columns, the non-empty ones leave their
+// records in shared memory, and the warp writes the chunk's reflections as one flat, coalesced range. Which column
+// owns position p0 + lane comes from one bit per column start in [p0, p0 + 32), gathered by a warp-wide OR: the
+// owner is the number of starts at or below the position (a bisection over 32 offsets cost five dependent
+// shared-memory loads per reflection). A reflection that starts a run writes the run's entry. The
 // output order is the column order above, l ascending, whatever the launch shape.
-// With one warp per structure the warps claim structures from ctr[0]; given the
-// post-processing size-class lists (cls_list, cls_cnt), the structures above
-// kPostCap6 reflections (the two largest classes) are left to whole CTAs,
-// which claim them from ctr[1] once the warps are done. ctr: zero at launch.
-// Dynamic shared memory: enum_smem_bytes(blockDim).
 template <bool RUNS>
 __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict__ geo, int n_struct, double r2min,
                                                           double r2max, float r2minf, float r2maxf, int rb,
@@ -662,108 +616,88 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict_
                                                           const int* __restrict__ abort_flag, double* __restrict__ q,
                                                           uint32_t* __restrict__ key, int* __restrict__ runs,
                                                           const int* __restrict__ tile_off, int2* __restrict__ tile_tab,
-                                                          int* __restrict__ ctr, const int* __restrict__ cls_list,
-                                                          const int* __restrict__ cls_cnt)
+                                                          int* __restrict__ ctr, const int* __restrict__ part_ctr,
+                                                          const int2* __restrict__ part_tab,
+                                                          const int2* __restrict__ part_cnt, int part_cap, int part_cols)
 {
     pdl_enter();
-    extern __shared__ int esm[];
-    __shared__ int tmp[66];
-    __shared__ int s_big;
+    extern __shared__ __align__(16) unsigned char esm[];
     if (*abort_flag) return;
-    const int nt = blockDim.x, t = threadIdx.x;
-    const bool per_warp = enum_per_warp(nt);
-    const int w = t >> 5, lane = t & 31;
-    const int64_t big_min = cls_list ? kPostCap6 : INT64_MAX;
-    int nbig = 0;
-    if (per_warp) {
-        const ChunkCols cc = chunk_cols(esm + enum_cta_ints(nt) + w * kWarpRecInts, 32);
-        for (;;) {
-            int s = 0;
-            if (lane == 0) s = atomicAdd(ctr, 1);
-            s = __shfl_sync(0xffffffffu, s, 0);
-            if (s >= n_struct) break;
+    const int lane = threadIdx.x & 31;
+    ColRec* const rec = (ColRec*)esm + 32 * (threadIdx.x >> 5);
+    const unsigned le = 0xffffffffu >> (31 - lane);
+    const EnumItems items = enum_items(n_struct, part_ctr, part_cap, ctr);
+    for (;;) {
+        int nit;
+        const int first = items.next(nit);
+        if (nit == 0) break;
+        for (int it = first; it < first + nit; it++) {
+            int s, part, c_lo, c_hi;
+            Geo g;
+            if (!enum_item(geo, part_tab, items.nparts, part_cols, it, s, part, g, c_lo, c_hi)) continue;
             const int64_t base = refl_off[s], cap = refl_off[s + 1] - base;
-            if (tile_tab) write_tiles(s, rb, tile_refl, rb > 0 ? run_cnt[s] : cap, tile_off, tile_tab, lane, 32);
-            if (cap <= 0 || cap > big_min) continue;
-            const Geo g = geo[s];
+            int done = 0, done_runs = 0;  // the structure's reflections and runs before this chunk
+            {
+                const int np = part < 0 ? 1 : (n_columns(g) + part_cols - 1) / part_cols;
+                if (tile_tab)
+                    write_tiles(s, RUNS, tile_refl, RUNS ? run_cnt[s] : cap, tile_off, tile_tab,
+                                32 * max(part, 0) + lane, 32 * np);
+                if (part > 0) {
+                    for (int i = lane; i < part; i += 32) {
+                        const int2 v = part_cnt[g.pbase + i];
+                        done += v.x;
+                        done_runs += v.y;
+                    }
+                    done = warp_sum_int(done);
+                    if (RUNS) done_runs = warp_sum_int(done_runs);
+                }
+            }
+            if (cap <= 0) continue;
             const F2 g33{g.gf[2], g.gl[2]};
-            const int ncol = n_columns(g);
-            int done = 0, done_runs = 0;
-            for (int c0 = 0; c0 < ncol; c0 += 32) {
+            for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
                 const int c = c0 + lane;
-                int m = 0, mr = 0;
-                if (c < ncol) {
-                    int h, k;
-                    const ColSpan sp =
-                        column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, m, mr);
-                    put_col(cc, lane, g, sp, h, k);
-                }
-                const int im = warp_incl_scan(m), imr = RUNS ? warp_incl_scan(mr) : 0;
-                cc.off[lane] = im - m;
-                if (RUNS) cc.roff[lane] = imr - mr;
+                int h = 0, k = 0, n = 0, nr = 0;
+                ColSpan sp{1, 0, 1, 0};
+                if (c < c_hi)
+                    sp = column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, n, nr);
+                const int im = warp_incl_scan(n), imr = RUNS ? warp_incl_scan(nr) : 0;
+                const int off = im - n;
+                const unsigned full = __ballot_sync(0xffffffffu, n > 0);
+                if (n > 0) rec[__popc(full & le) - 1] = column_rec(g, sp, h, k, n, off, imr - nr);
                 const int tot = __shfl_sync(0xffffffffu, im, 31);
-                const int rtot = RUNS ? __shfl_sync(0xffffffffu, imr, 31) : 0;
-                if (lane == 0) {
-                    cc.off[32] = tot;
-                    cc.roff[32] = rtot;
-                }
                 __syncwarp();
-                emit_chunk<RUNS>(g33, cc, 32, tot, rtot, lane, 32, rb, base, cap, done, done_runs, q, key, runs);
+                int started = 0;  // non-empty columns that start before p0
+                for (int p0 = 0; p0 < tot; p0 += 32) {
+                    const int d = off - p0;
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, (n > 0 && d >= 0 && d < 32) ? 1u << d : 0u);
+                    const ColRec r = rec[max(started + __popc(starts & le) - 1, 0)];
+                    started += __popc(starts);
+                    const int p = p0 + lane;
+                    if (p >= tot) continue;
+                    int l = r.a_off + p;
+                    if (l >= r.c) l += r.gap;
+                    const int64_t pos = done + p;
+                    if (pos < cap) {
+                        const float fl = (float)l;
+                        const F2 v = f2_add(f2_add(F2{r.th, r.tl}, f2_mul_int(g33, fl * fl)),
+                                            f2_mul_int(F2{r.uh, r.ul}, fl));
+                        q[base + pos] = f2d_fast(v.hi) + f2d_fast(v.lo);
+                        key[base + pos] = r.key0 + l;
+                    }
+                    if (RUNS) {
+                        const bool above = p - r.off >= r.n1;  // past the inner gap
+                        const int j = p - r.off - (above ? r.n1 : 0), nn = above ? r.n - r.n1 : r.n1;
+                        const int jr = j / rb;
+                        if (jr * rb == j) {
+                            const int64_t rpos = done_runs + r.roff + (above ? runs_of(r.n1, rb) : 0) + jr;
+                            if (rpos < cap) runs[base + rpos] = ((done + p) << 3) | min(rb, nn - j);
+                        }
+                    }
+                }
                 done += tot;
-                done_runs += rtot;
+                if (RUNS) done_runs += __shfl_sync(0xffffffffu, imr, 31);
                 __syncwarp();  // the records are read before the next chunk rewrites them
             }
-        }
-        if (!cls_list) return;
-        nbig = cls_cnt[kPostFlatClass - 1] + cls_cnt[kPostFlatClass];
-        if (nbig == 0) return;
-    }
-    const ChunkCols cc = chunk_cols(esm, nt);
-    for (int it = 0;; it++) {  // the structures taken by the whole CTA
-        int sb;
-        if (per_warp) {
-            __syncthreads();  // s_big and the chunk records are free
-            if (t == 0) s_big = atomicAdd(ctr + 1, 1);
-            __syncthreads();
-            const int j = s_big;
-            if (j >= nbig) break;
-            const int n5 = cls_cnt[kPostFlatClass];  // the largest class first
-            sb = j < n5 ? cls_list[(int64_t)kPostFlatClass * n_struct + j]
-                        : cls_list[(int64_t)(kPostFlatClass - 1) * n_struct + (j - n5)];
-        } else {
-            if (it > 0) break;
-            sb = blockIdx.x;  // one CTA per structure
-            if (sb >= n_struct) break;
-        }
-        const int64_t base = refl_off[sb], capb = refl_off[sb + 1] - base;
-        if (!per_warp && tile_tab) write_tiles(sb, rb, tile_refl, rb > 0 ? run_cnt[sb] : capb, tile_off, tile_tab, t, nt);
-        if (capb <= 0) continue;
-        const Geo g = geo[sb];
-        const F2 g33{g.gf[2], g.gl[2]};
-        const int ncol = n_columns(g);
-        int done = 0, done_runs = 0;
-        for (int c0 = 0; c0 < ncol; c0 += nt) {
-            const int c = c0 + t;
-            int m = 0, mr = 0;
-            if (c < ncol) {
-                int h, k;
-                const ColSpan sp =
-                    column_counts(g, geo[sb].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, m, mr);
-                put_col(cc, t, g, sp, h, k);
-            }
-            int ex, ey, tx, ty;
-            block_scan_pair(m, mr, tmp, ex, ey, tx, ty);
-            cc.off[t] = ex;
-            cc.roff[t] = ey;
-            if (t == 0) {
-                cc.off[nt] = tx;
-                cc.roff[nt] = ty;
-            }
-            __syncthreads();
-            emit_chunk<RUNS>(g33, cc, nt, tx, ty, t, nt, rb, base, capb, done, done_runs, q, key, runs);
-            done += tx;
-            done_runs += ty;
-            __syncthreads();  // the chunk's records are read; the next chunk rewrites them
         }
     }
 }
@@ -1146,12 +1080,19 @@ static void launch_k(bool pdl, void (*k)(P...), dim3 grid, dim3 block, cudaStrea
     else k<<<grid, block, 0, st>>>(static_cast<P>(args)...);
 }
 
-static void prep_launch(bool pdl, const double* lattice, int n, double rmax, Geo* geo, unsigned* imax,
-                        int32_t* flags, cudaStream_t st)
+static EnumParts enum_parts(const GeomArgs& a)
 {
+    return EnumParts{a.enum_ctr + kPartCtr, enum_part_cols(a.n_struct), a.part_cap, a.part_tab, a.refl_cnt, a.run_cnt};
+}
+
+static void prep_launch(bool pdl, const GeomArgs& a, cudaStream_t st)
+{
+    const int n = a.n_struct;
     if (n <= kPrepWideMax)  // 4 structures per CTA
-        launch_k(pdl, k_prep<8>, (n + 3) / 4, 32, st, lattice, n, rmax, geo, imax, flags);
-    else launch_k(pdl, k_prep<1>, (n + 127) / 128, 128, st, lattice, n, rmax, geo, imax, flags);
+        launch_k(pdl, k_prep<8>, (n + 3) / 4, 32, st, a.lattice, n, a.rmax, a.geo, a.imax, a.out_flags, enum_parts(a));
+    else
+        launch_k(pdl, k_prep<1>, (n + 127) / 128, 128, st, a.lattice, n, a.rmax, a.geo, a.imax, a.out_flags,
+                 enum_parts(a));
 }
 
 // Structure-factor work of the last call (for xrd_work_counts): terms = sum of
@@ -1200,7 +1141,7 @@ void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st)
 
 void launch_prep(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
-    if (a.n_struct > 0) prep_launch(pdl, a.lattice, a.n_struct, a.rmax, a.geo, a.imax, a.out_flags, st);
+    if (a.n_struct > 0) prep_launch(pdl, a, st);
 }
 
 void launch_coef(const GeomArgs& a, cudaStream_t st, bool pdl)
@@ -1234,27 +1175,35 @@ size_t order_parts_bytes(int64_t n)
     return nch > 2 ? (size_t)4 * kOrderBins * nch : 0;
 }
 
-void launch_count_only(const GeomArgs& a, cudaStream_t st)
+// CTAs of the enumeration: what fits on the SMs at once, or fewer where even one part per 32 columns and one
+// structure per warp would leave CTAs without an item
+static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
 {
-    const int n = a.n_struct;
-    if (n <= 0) return;
-    prep_launch(false, a.lattice, n, a.rmax, a.geo, (unsigned*)nullptr, (int32_t*)nullptr, st);
-    launch_pdl(k_count<false>, (n + 7) / 8, 256, 0, st, a.geo, n, a.r2min,
-               a.r2max, (float)a.r2min, (float)a.r2max, 0, a.refl_cnt, (int64_t*)nullptr, a.enum_ctr);
+    const int nt = a.enum_threads;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    const int64_t most = ((int64_t)a.n_struct + a.part_cap + nt / 32 - 1) / (nt / 32);
+    return (int)min((int64_t)a.sms * per_sm, max(most, (int64_t)1));
 }
 
-static int enum_grid(const GeomArgs& a)
+static void count_launch(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
-    const int per = enum_per_warp(a.enum_threads) ? a.enum_threads / 32 : 1;  // structures per CTA
-    return (a.n_struct + per - 1) / per;
+    const auto k = a.runs_mode ? k_count<true> : k_count<false>;
+    launch_k(pdl, k, enum_grid(a, (const void*)k, 0), a.enum_threads, st, a.geo, a.n_struct, a.r2min, a.r2max,
+             (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, a.refl_cnt, a.run_cnt, a.enum_ctr,
+             a.enum_ctr + kPartCtr, a.part_tab, a.part_cnt, a.part_cap, enum_part_cols(a.n_struct));
+}
+
+void launch_count_only(const GeomArgs& a, cudaStream_t st)
+{
+    if (a.n_struct <= 0) return;
+    prep_launch(false, a, st);
+    count_launch(a, st, true);
 }
 
 void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
-    if (a.n_struct > 0)
-        launch_k(pdl, a.runs_mode ? k_count<true> : k_count<false>, enum_grid(a), a.enum_threads, st, a.geo,
-                 a.n_struct, a.r2min, a.r2max,
-                 (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, a.refl_cnt, a.run_cnt, a.enum_ctr);
+    if (a.n_struct > 0) count_launch(a, st, pdl);
 }
 
 int scan_chunks(int n) { return (n + kScanItems * kScanThreads - 1) / (kScanItems * kScanThreads); }
@@ -1279,19 +1228,17 @@ void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl)
 void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
     if (a.n_struct <= 0) return;
-    auto k = a.runs_mode ? k_emit<true> : k_emit<false>;
-    const size_t smem = enum_smem_bytes(a.enum_threads);
-    if (pdl)
-        launch_pdl(k, enum_grid(a), a.enum_threads, smem, st, a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min,
-                   (float)a.r2max, a.runs_mode ? a.rb : 0, 32 * a.rb, (const int64_t*)a.refl_off,
-                   (const int64_t*)a.run_cnt, (const int*)a.abort_flag, a.q, a.key, a.runs, (const int*)a.tile_off,
-                   a.tile_tab, a.enum_ctr + 1, (const int*)a.cls_list, (const int*)(a.abort_flag + kFlagClsCnt));
-    else
-        k<<<enum_grid(a), a.enum_threads, smem, st>>>(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min,
-                                                       (float)a.r2max, a.runs_mode ? a.rb : 0, 32 * a.rb,
-                                                       a.refl_off, a.run_cnt, a.abort_flag, a.q, a.key, a.runs,
-                                                       a.tile_off, a.tile_tab, a.enum_ctr + 1, a.cls_list,
-                                                       a.abort_flag + kFlagClsCnt);
+    const auto k = a.runs_mode ? k_emit<true> : k_emit<false>;
+    const size_t smem = sizeof(ColRec) * (size_t)a.enum_threads;
+    const int grid = enum_grid(a, (const void*)k, smem);
+    auto go = [&](auto launch) {
+        launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, 32 * a.rb,
+               (const int64_t*)a.refl_off, (const int64_t*)a.run_cnt, (const int*)a.abort_flag, a.q, a.key, a.runs,
+               (const int*)a.tile_off, a.tile_tab, a.enum_ctr + 1, (const int*)(a.enum_ctr + kPartCtr),
+               (const int2*)a.part_tab, (const int2*)a.part_cnt, a.part_cap, enum_part_cols(a.n_struct));
+    };
+    if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });
+    else go([&](auto... v) { k<<<grid, a.enum_threads, smem, st>>>(v...); });
 }
 
 }  // namespace xrd

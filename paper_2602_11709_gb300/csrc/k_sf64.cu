@@ -9,8 +9,6 @@
 // point, and FP64 keeps the products and the sums: four operations per term, plus two per element run.
 // Measured, 1024 cells of 1 to 64 atoms (1.03 M reflections, 35 M terms): 7.27 ms with the library's functions, 0.88 ms
 // here (ALU pipe 50 %, FP64 pipe 39 %, 2.3 instructions a clock); the whole call 7.40 -> 1.15 ms.
-#include <cmath>
-
 #include "xrd_fx.cuh"
 #include "xrd_internal.cuh"
 #include "xrd_launch.h"
@@ -23,72 +21,63 @@ constexpr int kSf64Chunk = 32;  // atoms staged per warp at a time
 static __device__ uint64_t g_fx_exp[kFxExpN];
 static __device__ ulonglong2 g_fx_sc[kFxScN + 1];
 
-// ---- tables, formed once on the host in double-double (error-free sums and FMA products) ----
+// ---- tables, formed once per handle in double-double (error-free sums and FMA products) ----
 
-namespace {
 struct HD {
     double h, l;
 };
-HD hd_add(HD a, HD b)
+__device__ __forceinline__ HD hd_fast(double h, double l)
 {
-    const double s = a.h + b.h, bb = s - a.h;
-    const double e = ((a.h - (s - bb)) + (b.h - bb)) + (a.l + b.l);
-    const double h = s + e;
-    return HD{h, e - (h - s)};
+    const double s = __dadd_rn(h, l);
+    return HD{s, __dsub_rn(l, __dsub_rn(s, h))};
 }
-HD hd_mul(HD a, HD b)
+__device__ __forceinline__ HD hd_add(HD a, HD b)
 {
-    const double p = a.h * b.h;
-    const double e = std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h);
-    const double h = p + e;
-    return HD{h, e - (h - p)};
+    const double s = __dadd_rn(a.h, b.h), bb = __dsub_rn(s, a.h);
+    const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, bb)), __dsub_rn(b.h, bb));
+    return hd_fast(s, __dadd_rn(e, __dadd_rn(a.l, b.l)));
 }
-HD hd_div(HD a, double n)  // n a small integer
+__device__ __forceinline__ HD hd_mul(HD a, HD b)
 {
-    const double h = a.h / n, r = std::fma(-h, n, a.h) + a.l;
-    const double l = r / n, s = h + l;
-    return HD{s, l - (s - h)};
+    const double p = __dmul_rn(a.h, b.h);
+    return hd_fast(p, __dadd_rn(__fma_rn(a.h, b.h, -p), __fma_rn(a.h, b.l, __dmul_rn(a.l, b.h))));
+}
+__device__ __forceinline__ HD hd_div(HD a, double n)  // n a small integer
+{
+    const double h = __ddiv_rn(a.h, n);
+    return hd_fast(h, __ddiv_rn(__dadd_rn(__fma_rn(-h, n, a.h), a.l), n));
 }
 // a >= 0 in units of 2^-bits, rounded
-uint64_t hd_fixed(HD a, int bits)
+__device__ uint64_t hd_fixed(HD a, int bits)
 {
-    const double sc = std::ldexp(1.0, bits), v = a.h * sc, f = std::floor(v);
-    return (uint64_t)f + (uint64_t)(int64_t)std::rint((v - f) + a.l * sc);
+    const double sc = scalbn(1.0, bits), v = a.h * sc, f = floor(v);
+    return (uint64_t)f + (uint64_t)__double2ll_rn((v - f) + a.l * sc);
 }
 
-struct FxTables {
-    uint64_t ex[kFxExpN];
-    ulonglong2 sc[kFxScN + 1];
-    FxTables()
-    {
-        const HD ln2{0.6931471805599453, 2.3190468138462996e-17}, pi2{1.5707963267948966, 6.123233995736766e-17};
-        for (int j = 0; j < kFxExpN; j++) {
-            const HD x = hd_mul(ln2, HD{-j / (double)kFxExpN, 0.0});
-            HD t{1.0, 0.0}, s = t;
-            for (int k = 1; k <= 24; k++) s = hd_add(s, t = hd_div(hd_mul(t, x), k));
-            ex[j] = j ? hd_fixed(s, 64) : ~0ull;
-        }
-        for (int j = 0; j <= kFxScN; j++) {
-            const HD x = hd_mul(pi2, HD{j / (double)kFxScN, 0.0});
-            HD t{1.0, 0.0}, c = t, s{0.0, 0.0};
-            for (int k = 1; k <= 30; k++) {
-                t = hd_div(hd_mul(t, x), k);
-                const HD v = k & 2 ? HD{-t.h, -t.l} : t;
-                if (k & 1) s = hd_add(s, v);
-                else c = hd_add(c, v);
-            }
-            sc[j] = make_ulonglong2(j == kFxScN ? 0ull : hd_fixed(c, 62), hd_fixed(s, 62));
-        }
+__global__ void k_fx_init()
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kFxExpN) {  // 2^(-i / kFxExpN) by the series of exp
+        const HD x = hd_mul(HD{0.6931471805599453, 2.3190468138462996e-17}, HD{-i / (double)kFxExpN, 0.0});
+        HD t{1.0, 0.0}, s = t;
+        for (int k = 1; k <= 24; k++) s = hd_add(s, t = hd_div(hd_mul(t, x), k));
+        g_fx_exp[i] = i ? hd_fixed(s, 64) : ~0ull;
+        return;
     }
-};
-}  // namespace
-
-bool init_fx_tables(cudaStream_t st)
-{
-    static const FxTables t;
-    return cudaMemcpyToSymbolAsync(g_fx_exp, t.ex, sizeof(t.ex), 0, cudaMemcpyHostToDevice, st) == cudaSuccess &&
-           cudaMemcpyToSymbolAsync(g_fx_sc, t.sc, sizeof(t.sc), 0, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    const int j = i - kFxExpN;
+    if (j > kFxScN) return;
+    const HD x = hd_mul(HD{1.5707963267948966, 6.123233995736766e-17}, HD{j / (double)kFxScN, 0.0});
+    HD t{1.0, 0.0}, c = t, s{0.0, 0.0};
+    for (int k = 1; k <= 30; k++) {
+        t = hd_div(hd_mul(t, x), k);
+        const HD v = k & 2 ? HD{-t.h, -t.l} : t;
+        if (k & 1) s = hd_add(s, v);
+        else c = hd_add(c, v);
+    }
+    g_fx_sc[j] = make_ulonglong2(j == kFxScN ? 0ull : hd_fixed(c, 62), hd_fixed(s, 62));
 }
+
+void init_fx_tables(cudaStream_t st) { k_fx_init<<<(kFxExpN + kFxScN + 1 + 31) / 32, 32, 0, st>>>(); }
 
 // ---- f(s) of one element: Z - 41.78214 s^2 sum_i a_i exp(-b_i s^2) ----
 

@@ -47,11 +47,11 @@ constexpr int kFlagClsCnt = 32, kFlagClsNext = 48, kFlagPfBar = 4;
 // Per-structure geometry written by k_prep (step S0).
 struct Geo {
     double gs[6];  // reciprocal metric G* stored as (11, 22, 33, 12, 13, 23)
-    double g2[3];  // 2 G*12, 2 G*13, 2 G*23 (exact doubles of the off-diagonal terms)
     float gf[6];   // G* rounded to FP32, for the enumeration filter
     float gl[6];   // G* - gf (the low words of a two-float G*; off-diagonals doubled in hi and lo below)
     int H, K, L;   // enumeration box |h| <= H ...
     int status;    // XRD_OK or XRD_EINVAL
+    int pbase;     // first enumeration part of a structure counted and emitted in parts (-1: in one piece)
     int hex;       // 1: hexagonal cell (alpha, beta within 5 deg of 90, gamma within 5 deg of 120,
                    // |a - b| < 0.01 A): families by Miller-Bravais indices
 };

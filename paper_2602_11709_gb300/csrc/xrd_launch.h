@@ -11,7 +11,8 @@ namespace xrd {
 struct GeomArgs {
     int n_struct, zmax, rb;  // rb: reflections a structure-factor lane takes (2 or 4)
     int runs_mode;           // 1: tiles of 32 runs of <= rb reflections consecutive in l; 0: tiles of 32 rb reflections
-    int enum_threads;        // threads per structure of k_count / k_emit (64, 128 or 256; the same for both)
+    int enum_threads;        // threads per CTA of k_count / k_emit (64 to 1024; the same for both)
+    int sms;                 // SMs of the device
     int64_t n_atoms;
     double r2min, r2max, rmax;
     int64_t cap_refl;
@@ -46,12 +47,26 @@ struct GeomArgs {
     uint32_t* key;
     long long* parts;  // chunk sums of the multi-block scan (nullptr: single-block scan)
     int* oparts;       // [chunks][4096] bin counts of the multi-block order (nullptr: one-block order)
-    int* enum_ctr;     // flags[26..28]: structure claims of counting, of emission's warps and of its CTAs
+    int* enum_ctr;     // flags[26..28]: claims of counting and of emission, parts listed (kPartCtr)
+    int2* part_tab;    // [part_cap] (structure, part) of each enumeration part, by k_prep
+    int2* part_cnt;    // [part_cap] its reflections and runs, by k_count
+    int part_cap;
     const float4* sctab;  // [256] cos and sin of 2 pi k / 256 as two floats (the re-evaluation's table)
     unsigned* imax;    // [n_struct] largest reflection intensity slot, zeroed by k_prep (or nullptr)
     int32_t* out_flags;  // [n_struct] caller's flag words, written by k_prep (or nullptr)
     float4* cdd;       // [(zmax + 1) * 4] (a, b) coefficients as two floats, by k_coef (or nullptr)
     AtomR* atomr;      // [atoms] records of the accurate re-evaluation, by k_atoms (or nullptr)
+};
+
+constexpr int kPartCtr = 2;  // index of the part counter within enum_ctr
+
+// What k_prep needs to list the enumeration parts of the structures with more than `cols` columns.
+struct EnumParts {
+    int* ctr;
+    int cols, cap;
+    int2* tab;
+    int64_t* cnt;      // reflection and run counts: zeroed for the structures in parts
+    int64_t* run_cnt;  // (or nullptr)
 };
 
 struct SfArgs {
@@ -277,7 +292,7 @@ void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st);  
 void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_sf(const SfArgs& a, cudaStream_t st, bool pdl);
 void launch_sf64(const SfArgs& a, cudaStream_t st, bool pdl);  // the XRD_FP64 variant
-bool init_fx_tables(cudaStream_t st);  // its tables, in device memory
+void init_fx_tables(cudaStream_t st);  // fills its tables
 RefineTables init_refine_tables(cudaStream_t st);  // fills the tables, returns their device addresses
 void launch_refine(const RefineArgs& a, cudaStream_t st, bool pdl);
 size_t post_smem_bytes(int cap);
