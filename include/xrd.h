@@ -145,11 +145,10 @@ typedef struct {
 
 /*
  * Create a handle bound to CUDA device `device`. Returns XRD_OK or
- * XRD_ECUDA/XRD_EINVAL. The handle owns eight non-blocking side streams: the
- * nine post-processing size classes of xrd_pattern_batch (the largest as flat
- * device-wide passes) run on them and the caller's stream concurrently,
+ * XRD_ECUDA/XRD_EINVAL. The handle owns one non-blocking side stream, on which
+ * xrd_pattern_batch packs the atoms of a large batch beside the enumeration,
  * forked from and joined back into the caller's stream by events (so a
- * capture of the call on the caller's stream takes them in as branches).
+ * capture of the call on the caller's stream takes it in as a branch).
  */
 int xrd_create(xrd_handle** h, int device);
 /* Destroy a handle (NULL is ignored). */

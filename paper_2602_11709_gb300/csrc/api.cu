@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -24,11 +25,9 @@ struct xrd_handle {
     int sf_rb = 4, sf_warps = 2;        // structure-factor launch shape (xrd_autotune)
     int sf_runs = 0;                    // lanes take runs consecutive in l (integer phase only)
     int enum_threads = 256;             // threads per CTA of the enumeration kernels (xrd_autotune)
-    // side streams for the concurrent post-processing size classes (fork/join by events)
-    cudaStream_t side[xrd::kPostStreams - 1] = {};
-    cudaEvent_t fork = nullptr, join[xrd::kPostStreams - 1] = {};
-    // the input-only front (coefficients, atom packing, largest-first order) runs on side[0]
-    // beside the enumeration: forked by front, joined by order_done and atoms_done
+    // the input-only front of a large batch (coefficients, atom packing, largest-first order) runs on the side
+    // stream beside the enumeration: forked by front, joined by order_done and atoms_done
+    cudaStream_t side = nullptr;
     cudaEvent_t front = nullptr, order_done = nullptr, atoms_done = nullptr;
     unsigned long long* wbuf = nullptr;  // device [3]: xrd_work_counts result
     xrd::RefineTables rtab{};            // tables of the accurate re-evaluation on the handle's device
@@ -336,6 +335,26 @@ xrd::GeomArgs geom_args(const xrd_batch* b, const xrd_opts* o, const Layout& L, 
 }  // namespace
 
 namespace xrd {
+int resident_ctas(const void* kernel, int threads, size_t smem)
+{
+    struct Entry {
+        const void* kernel;
+        int device, threads;
+        size_t smem;
+        int ctas;
+    };
+    static std::mutex mu;
+    static std::vector<Entry> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Entry& e : known)
+        if (e.kernel == kernel && e.device == dev && e.threads == threads && e.smem == smem) return e.ctas;
+    int ctas = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, threads, smem) != cudaSuccess || ctas < 1) return 1;
+    known.push_back(Entry{kernel, dev, threads, smem, ctas});
+    return ctas;
+}
 int handle_device(const xrd_handle* h) { return h ? h->device : -1; }
 int set_error(xrd_handle* h, int code, const char* msg)
 {
@@ -363,12 +382,7 @@ int xrd_create(xrd_handle** h, int device)
         e = cudaEventCreate(&p->ev[i]);
         if (e != cudaSuccess) { xrd_destroy(p); return XRD_ECUDA; }
     }
-    for (int i = 0; i < xrd::kPostStreams - 1; i++) {
-        e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join[i], cudaEventDisableTiming);
-        if (e != cudaSuccess) { xrd_destroy(p); return XRD_ECUDA; }
-    }
-    e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
+    e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->front, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->order_done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->atoms_done, cudaEventDisableTiming);
@@ -389,11 +403,7 @@ void xrd_destroy(xrd_handle* h)
     DeviceGuard g(h->device);
     for (int i = 0; i < kEvents; i++)
         if (h->ev[i]) cudaEventDestroy(h->ev[i]);
-    for (int i = 0; i < xrd::kPostStreams - 1; i++) {
-        if (h->side[i]) cudaStreamDestroy(h->side[i]);
-        if (h->join[i]) cudaEventDestroy(h->join[i]);
-    }
-    if (h->fork) cudaEventDestroy(h->fork);
+    if (h->side) cudaStreamDestroy(h->side);
     for (cudaEvent_t ev : {h->front, h->order_done, h->atoms_done})
         if (ev) cudaEventDestroy(ev);
     if (h->qbuf) cudaFree(h->qbuf);
@@ -584,28 +594,32 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     const bool pdl = prof != 1;  // programmatic launches where no stage event separates two kernels
     cudaMemsetAsync(ws + L.flags, 0, kFlagBytes, st);
     mark();
-    // the input-only front beside the enumeration: order (needed by the scan), then
-    // coefficients and atoms (needed by the structure factor)
-    cudaStream_t side = h->side[0];
+    // the input-only front: in one launch for a small batch; else order (needed by the scan), coefficients and atoms
+    // (needed by the structure factor) on a side stream, beside the enumeration
     ga.atoms_set_geo = 0;
-    cudaEventRecord(h->front, st);
-    cudaStreamWaitEvent(side, h->front, 0);
-    xrd::launch_order(ga, side, false);
-    cudaEventRecord(h->order_done, side);
-    xrd::launch_coef(ga, side, true);
-    xrd::launch_atoms(ga, side, true);
-    cudaEventRecord(h->atoms_done, side);
-    xrd::launch_prep(ga, st, false);
+    const bool fused = xrd::front_fused((int)n, b->n_atoms);
+    if (fused) {
+        xrd::launch_front(ga, st);
+    } else {
+        cudaEventRecord(h->front, st);
+        cudaStreamWaitEvent(h->side, h->front, 0);
+        xrd::launch_order(ga, h->side, false);
+        cudaEventRecord(h->order_done, h->side);
+        xrd::launch_coef(ga, h->side, true);
+        xrd::launch_atoms(ga, h->side, true);
+        cudaEventRecord(h->atoms_done, h->side);
+        xrd::launch_prep(ga, st, false);
+    }
     mark();
     mark();  // the atom packing stage runs on the side stream: nothing on this one
     xrd::launch_count(ga, st, pdl);
     mark();
-    cudaStreamWaitEvent(st, h->order_done, 0);
-    xrd::launch_scan_refl(ga, st, false);
+    if (!fused) cudaStreamWaitEvent(st, h->order_done, 0);
+    xrd::launch_scan_refl(ga, st, fused && pdl);
     mark();
     xrd::launch_emit(ga, st, pdl);
     mark();
-    cudaStreamWaitEvent(st, h->atoms_done, 0);
+    if (!fused) cudaStreamWaitEvent(st, h->atoms_done, 0);
 
     xrd::SfArgs sa{};
     sa.n_struct = (int)n;
@@ -642,7 +656,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
         sa.tau = kRefineTau;
         sa.imax = ga.imax;
     }
-    xrd::launch_sf(sa, st, false);
+    xrd::launch_sf(sa, st, fused && prof == 0);
     mark();
     if (refine) {
         xrd::RefineArgs ra{};
@@ -748,19 +762,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
         pa.refl_I = out->refl_I;
     }
     if (pg) xrd::launch_pg_keys(pa, (unsigned long long*)(ws + L.fkg), st);
-    {  // the size classes run concurrently: fork to the side streams, join back
-        cudaStream_t cs[xrd::kPostStreams] = {st};
-        cudaEventRecord(h->fork, st);
-        for (int i = 1; i < xrd::kPostStreams; i++) {
-            cs[i] = h->side[i - 1];
-            cudaStreamWaitEvent(cs[i], h->fork, 0);
-        }
-        xrd::launch_post(pa, cs);
-        for (int i = 1; i < xrd::kPostStreams; i++) {
-            cudaEventRecord(h->join[i - 1], cs[i]);
-            cudaStreamWaitEvent(st, h->join[i - 1], 0);
-        }
-    }
+    xrd::launch_post(pa, cap_refl, st, prof == 0);
     mark();
 
     xrd::CompactArgs ca{};
@@ -785,7 +787,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     ca.st_mult = pa.st_mult;
     ca.out_abort = ga.abort_flag + 1;
     ca.out = *out;
-    xrd::launch_compact(ca, st);
+    xrd::launch_compact(ca, st, prof == 0 && fused);
     mark();
     h->recorded = prof;
     cudaError_t e = cudaGetLastError();
@@ -1062,7 +1064,7 @@ static xrd::GradArgs grad_args(xrd_handle* h, const xrd_batch* b, const xrd_grid
 // Geometry and structure factors of the broadened and augmented paths, one
 // stream: grad = true keeps strided tiles and stores F, dF/ds^2 and I for the
 // adjoint; grad = false runs the tuned pattern shape and stores I only.
-static void launch_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const LayoutG& L, char* ws,
+static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const LayoutG& L, char* ws,
                          int64_t cap_refl, int32_t* status, int64_t* totals, cudaStream_t st, bool grad)
 {
     const int64_t n = b->n_struct;
@@ -1174,7 +1176,7 @@ int xrd_pattern_broadened(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
     const LayoutG L = layout_grad(n, b->n_atoms, b->zmax, cap_refl);
-    launch_front(h, b, o, L, ws, cap_refl, status, totals, st, true);
+    profile_front(h, b, o, L, ws, cap_refl, status, totals, st, true);
     xrd::GradArgs gr = grad_args(h, b, grid, W, sigma, o, L, ws);
     gr.y = y;
     xrd::launch_broaden(gr, st);
@@ -1216,7 +1218,7 @@ int xrd_pattern_augmented(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
     const LayoutG L = layout_grad(n, b->n_atoms, b->zmax, cap_refl);
-    launch_front(h, b, o, L, ws, cap_refl, status, totals, st, false);
+    profile_front(h, b, o, L, ws, cap_refl, status, totals, st, false);
     xrd::AugArgs a{};
     a.n_struct = (int)n;
     a.n_pts = grid->n_pts;

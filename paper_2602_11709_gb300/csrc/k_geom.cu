@@ -40,11 +40,10 @@ __device__ __forceinline__ double cosd(double deg)
 // structure-factor pass) and writes its flag word (bit 0: hexagonal) when the
 // pointers are given.
 template <int LANES>
-__global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, Geo* __restrict__ geo,
-                       unsigned* __restrict__ imax, int32_t* __restrict__ flags, const EnumParts ep)
+__device__ __forceinline__ void prep_thread(int t, const double* __restrict__ lattice, int n, double rmax,
+                                            Geo* __restrict__ geo, unsigned* __restrict__ imax,
+                                            int32_t* __restrict__ flags, const EnumParts& ep)
 {
-    pdl_enter();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int s_raw = t / LANES, lane = t % LANES;
     const bool live = s_raw < n;
     if (LANES == 1 && !live) return;
@@ -135,6 +134,14 @@ __global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, G
     }
 }
 
+template <int LANES>
+__global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, Geo* __restrict__ geo,
+                       unsigned* __restrict__ imax, int32_t* __restrict__ flags, const EnumParts ep)
+{
+    pdl_enter();
+    prep_thread<LANES>(blockIdx.x * blockDim.x + threadIdx.x, lattice, n, rmax, geo, imax, flags, ep);
+}
+
 // 8 lanes per structure up to this many structures (latency-bound), one above (throughput-bound)
 constexpr int kPrepWideMax = 8192;
 
@@ -143,9 +150,9 @@ static int enum_part_cols(int n_struct);
 // f(s) coefficients in the form the FP32 loops use (exp2 with the scale folded
 // in) and, for the accurate re-evaluation, (a_i, b_i) as two floats each
 // (cdd[4 z + i] = (a hi, a lo, b hi, b lo); skipped when cdd is null).
-__global__ void k_coef(const double* __restrict__ coef, int zmax, Coef32* __restrict__ c32, float4* __restrict__ cdd)
+__device__ __forceinline__ void coef_block(const double* __restrict__ coef, int zmax, Coef32* __restrict__ c32,
+                                           float4* __restrict__ cdd)
 {
-    pdl_enter();
     for (int z = threadIdx.x; z <= zmax; z += blockDim.x) {
         Coef32 c;
         for (int i = 0; i < 4; i++) {
@@ -162,9 +169,21 @@ __global__ void k_coef(const double* __restrict__ coef, int zmax, Coef32* __rest
     }
 }
 
+__global__ void k_coef(const double* __restrict__ coef, int zmax, Coef32* __restrict__ c32, float4* __restrict__ cdd)
+{
+    pdl_enter();
+    coef_block(coef, zmax, c32, cdd);
+}
+
 // Validate and pack the atoms of one structure, sorted by element (stable:
 // ties keep their input order) so that f(s) is evaluated once per element run.
-__global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_off, int64_t n_atoms,
+constexpr int kAtomThreads = 128;
+struct AtomShared {
+    int off[kZmaxLimit + 1];
+    int pos[kAtomThreads];
+    int bad;
+};
+__device__ __forceinline__ void atoms_block(int s, AtomShared& sh, const int64_t* __restrict__ atom_off, int64_t n_atoms,
                                                const double* __restrict__ frac, const int16_t* __restrict__ Zin,
                                                const double* __restrict__ occ, const double* __restrict__ Bf, int zmax,
                                                Geo* __restrict__ geo, int set_geo, int* __restrict__ atom_bad,
@@ -172,16 +191,12 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
                                                float2* __restrict__ astep, AtomR* __restrict__ ar,
                                                const float4* __restrict__ sctab)
 {
-    pdl_enter();
-    __shared__ int off[kZmaxLimit + 1];
-    __shared__ int zs[128];
-    __shared__ int bad;
-    const int s = blockIdx.x;
+    int* const off = sh.off;
     int64_t a0 = atom_off[s], na = atom_off[s + 1] - a0;
     const bool range_ok = a0 >= 0 && na >= 0 && atom_off[s + 1] <= n_atoms && na <= (1 << 30);
     if (!range_ok) { a0 = 0; na = 0; }
     for (int i = threadIdx.x; i <= kZmaxLimit; i += blockDim.x) off[i] = 0;
-    if (threadIdx.x == 0) bad = !range_ok;
+    if (threadIdx.x == 0) sh.bad = !range_ok;
     __syncthreads();
     for (int64_t i = threadIdx.x; i < na; i += blockDim.x) {
         const int z = Zin[a0 + i];
@@ -189,12 +204,12 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
         const bool ok = z >= 0 && z <= zmax && isfinite(x) && isfinite(y) && isfinite(w) && occ[a0 + i] >= 0.0 &&
                         isfinite(occ[a0 + i]) &&
                         isfinite(Bf[a0 + i]) && fabs(x) < 262144.0 && fabs(y) < 262144.0 && fabs(w) < 262144.0;
-        if (!ok) atomicOr(&bad, 1);
+        if (!ok) atomicOr(&sh.bad, 1);
         else atomicAdd(&off[z], 1);
     }
     __syncthreads();
-    if (threadIdx.x == 0) atom_bad[s] = bad;
-    if (bad) {
+    if (threadIdx.x == 0) atom_bad[s] = sh.bad;
+    if (sh.bad) {
         // neutral records (weight 0, element 0) keep the structure-factor kernel's reads in bounds;
         // the structure reports XRD_EINVAL and gets no peaks
         if (threadIdx.x == 0 && set_geo) geo[s].status = XRD_EINVAL;
@@ -231,16 +246,28 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
         }
     }
     __syncthreads();
-    // stable placement, one chunk of blockDim atoms at a time
+    // stable placement, one chunk of blockDim atoms at a time: the first warp ranks the chunk's atoms among those of
+    // their element, 32 at a time, and advances the elements' offsets; then every thread packs its atom
     for (int64_t base = 0; base < na; base += blockDim.x) {
         const int64_t i = base + threadIdx.x;
         const int z = i < na ? (int)Zin[a0 + i] : -1;
-        zs[threadIdx.x] = z;
+        sh.pos[threadIdx.x] = z;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const int lane = threadIdx.x;
+            for (int c = 0; c < (int)blockDim.x && base + c < na; c += 32) {
+                const int zz = sh.pos[c + lane];
+                const unsigned peers = __match_any_sync(0xffffffffu, zz);
+                const int first = zz >= 0 ? off[zz] : 0;
+                __syncwarp();
+                if (zz >= 0 && lane == __ffs(peers) - 1) off[zz] = first + __popc(peers);
+                __syncwarp();
+                sh.pos[c + lane] = first + __popc(peers & ((1u << lane) - 1u));
+            }
+        }
         __syncthreads();
         if (i < na) {
-            int before = 0;
-            for (int t = 0; t < (int)threadIdx.x; t++) before += zs[t] == z;
-            const int pos = off[z] + before;
+            const int pos = sh.pos[threadIdx.x];
             const double x = frac[3 * (a0 + i)], y = frac[3 * (a0 + i) + 1], w = frac[3 * (a0 + i) + 2];
             const double o = occ[a0 + i], bb = Bf[a0 + i];
             Atom32 r;
@@ -289,10 +316,22 @@ __global__ void __launch_bounds__(128) k_atoms(const int64_t* __restrict__ atom_
                 ar[a0 + pos] = e;
             }
         }
-        __syncthreads();  // every read of off[] for this chunk is done
-        if (i < na) atomicAdd(&off[z], 1);
-        __syncthreads();
+        __syncthreads();  // the positions are read before the next chunk's
     }
+}
+
+__global__ void __launch_bounds__(kAtomThreads) k_atoms(const int64_t* __restrict__ atom_off, int64_t n_atoms,
+                                                        const double* __restrict__ frac,
+                                                        const int16_t* __restrict__ Zin, const double* __restrict__ occ,
+                                                        const double* __restrict__ Bf, int zmax, Geo* __restrict__ geo,
+                                                        int set_geo, int* __restrict__ atom_bad, Atom32* __restrict__ a32,
+                                                        AtomX* __restrict__ ax, float2* __restrict__ astep,
+                                                        AtomR* __restrict__ ar, const float4* __restrict__ sctab)
+{
+    pdl_enter();
+    __shared__ AtomShared sh;
+    atoms_block(blockIdx.x, sh, atom_off, n_atoms, frac, Zin, occ, Bf, zmax, geo, set_geo, atom_bad, a32, ax, astep, ar,
+                sctab);
 }
 
 // |g|^2 in the fixed order ((G11 hh + G22 kk) + G33 ll) + 2 ((G12 hk + G13 hl) + G23 kl).
@@ -976,12 +1015,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_final(const int64_t*
 // block, warp-aggregated shared-memory atomics, so structures of one bin keep
 // the order of their warp. It depends on the input only and runs beside the
 // enumeration.
-__global__ void __launch_bounds__(kScanThreads) k_order(const int64_t* __restrict__ atom_off, int n,
-                                                        int* __restrict__ order)
+__device__ __forceinline__ void order_block(const int64_t* __restrict__ atom_off, int n, int* __restrict__ order,
+                                            int* bins, int* tmp)
 {
-    pdl_enter();
-    __shared__ int bins[kOrderBins];
-    __shared__ int tmp[66];
     const int nt = blockDim.x, tid = threadIdx.x, CH = kScanItems * nt;
     for (int b = tid; b < kOrderBins; b += nt) bins[b] = 0;
     __syncthreads();
@@ -1010,6 +1046,48 @@ __global__ void __launch_bounds__(kScanThreads) k_order(const int64_t* __restric
             const int slot = warp_aggregated_slot(bins, b[u], i < n);
             if (i < n) order[slot] = i;
         }
+    }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_order(const int64_t* __restrict__ atom_off, int n,
+                                                        int* __restrict__ order)
+{
+    pdl_enter();
+    __shared__ int bins[kOrderBins];
+    __shared__ int tmp[66];
+    order_block(atom_off, n, order, bins, tmp);
+}
+
+// The whole input-only front of a small batch in one launch: block 0 forms the coefficients and the largest-first
+// order, the next blocks the cells (16 structures each), the others pack the atoms of one structure each. One launch
+// instead of four on two streams: a small batch is bound by its chain of launches. Taken up to kFrontMax structures of
+// kFrontAtoms atoms on average; beyond, packing the atoms takes longer than counting the reflections, and the two
+// run side by side on two streams instead.
+struct FrontArgs {
+    GeomArgs g;
+    EnumParts ep;
+    int prep_blocks;
+};
+__global__ void __launch_bounds__(kAtomThreads) k_front(const FrontArgs f)
+{
+    pdl_enter();
+    __shared__ union {
+        AtomShared at;
+        struct {
+            int bins[kOrderBins], tmp[66];
+        } ord;
+    } sh;
+    const GeomArgs& g = f.g;
+    const int b = blockIdx.x;
+    if (b == 0) {
+        coef_block(g.coef, g.zmax, g.coef32, g.cdd);
+        order_block(g.atom_off, g.n_struct, g.order, sh.ord.bins, sh.ord.tmp);
+    } else if (b <= f.prep_blocks) {
+        prep_thread<8>((b - 1) * kAtomThreads + threadIdx.x, g.lattice, g.n_struct, g.rmax, g.geo, g.imax, g.out_flags,
+                       f.ep);
+    } else {
+        atoms_block(b - 1 - f.prep_blocks, sh.at, g.atom_off, g.n_atoms, g.frac, g.Z, g.occ, g.B, g.zmax, g.geo, 0,
+                    g.atom_bad, g.atom32, g.atomx, g.runs_mode ? g.astep : nullptr, g.atomr, g.sctab);
     }
 }
 
@@ -1139,6 +1217,16 @@ void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st)
                                                                    a.work, out);
 }
 
+constexpr int kFrontMax = 2048, kFrontAtoms = 128;
+bool front_fused(int n_struct, int64_t n_atoms) { return n_struct <= kFrontMax && n_atoms <= (int64_t)n_struct * kFrontAtoms; }
+
+void launch_front(const GeomArgs& a, cudaStream_t st)
+{
+    if (a.n_struct <= 0) return;
+    FrontArgs f{a, enum_parts(a), (8 * a.n_struct + kAtomThreads - 1) / kAtomThreads};
+    k_front<<<1 + f.prep_blocks + a.n_struct, kAtomThreads, 0, st>>>(f);
+}
+
 void launch_prep(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
     if (a.n_struct > 0) prep_launch(pdl, a, st);
@@ -1152,7 +1240,7 @@ void launch_coef(const GeomArgs& a, cudaStream_t st, bool pdl)
 void launch_atoms(const GeomArgs& a, cudaStream_t st, bool pdl)
 {
     if (a.n_struct > 0)
-        launch_k(pdl, k_atoms, a.n_struct, 128, st, a.atom_off, a.n_atoms, a.frac, a.Z, a.occ, a.B, a.zmax, a.geo,
+        launch_k(pdl, k_atoms, a.n_struct, kAtomThreads, st, a.atom_off, a.n_atoms, a.frac, a.Z, a.occ, a.B, a.zmax, a.geo,
                  a.atoms_set_geo, a.atom_bad, a.atom32, a.atomx, a.runs_mode ? a.astep : (float2*)nullptr, a.atomr,
                  a.sctab);
 }
@@ -1180,8 +1268,7 @@ size_t order_parts_bytes(int64_t n)
 static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
 {
     const int nt = a.enum_threads;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nt, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    const int per_sm = resident_ctas(kernel, nt, smem);
     const int64_t most = ((int64_t)a.n_struct + a.part_cap + nt / 32 - 1) / (nt / 32);
     return (int)min((int64_t)a.sms * per_sm, max(most, (int64_t)1));
 }

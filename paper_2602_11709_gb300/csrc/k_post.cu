@@ -15,6 +15,9 @@
 // The anchor rule is sequential, so it is split: a reflection whose gap to its
 // predecessor is >= tol always opens a peak (a definite start); the short runs
 // between definite starts are resolved one thread per run.
+#include <atomic>
+#include <type_traits>
+
 #include "xrd_internal.cuh"
 #include "xrd_launch.h"
 #include "xrd_post.cuh"
@@ -343,24 +346,24 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, co
 // variants also stage the intensities there, in the second half of the
 // peak-sum area (FP32 peak sums use the first half).
 template <int CAP, int NT, bool FI>
-__global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const PostArgs a, int cls)
+__global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const PostArgs a, int c_lo, int c_hi, bool first)
 {
     static_assert(CAP > 0, "the largest class runs as the flat passes");
-    pdl_enter();
+    pdl_chain_enter(first);
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int tmp[66];
     __shared__ double dtmp[32];
     __shared__ int claim;
-    if (*a.abort_flag) return;
-    const int cnt = a.cls_cnt[cls];
-    const int* __restrict__ list = a.cls_list + (int64_t)cls * a.n_struct;
-    for (;;) {
+    for (; !*a.abort_flag;) {
         __syncthreads();  // the previous structure is done with shared memory and claim
-        if (threadIdx.x == 0) claim = atomicAdd(a.cls_next + cls, 1);
+        if (threadIdx.x == 0) {
+            int li = atomicAdd(a.cls_next + c_lo, 1), c = c_hi;  // the larger classes first
+            while (c >= c_lo && li >= a.cls_cnt[c]) li -= a.cls_cnt[c--];
+            claim = c >= c_lo ? a.cls_list[(int64_t)c * a.n_struct + li] : -1;
+        }
         __syncthreads();
-        const int li = claim;
-        if (li >= cnt) break;
-        const int s = list[li];
+        const int s = claim;
+        if (s < 0) break;
         const int64_t base = a.refl_off[s];
         const int n = (int)(a.refl_off[s + 1] - base);
         if (a.atom_bad && a.atom_bad[s]) {  // an invalid atom: no peaks, the structure reports XRD_EINVAL
@@ -399,6 +402,7 @@ __global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const Pos
             post_structure<uint16_t, FI>(a, s, base, n, sq, sk, sI, perm, bkt, flag, pst, psum, fcnt, tmp, dtmp);
         }
     }
+    pdl_chain_exit();
 }
 
 // Exclusive scans of kept peaks and families per structure (single block),
@@ -598,41 +602,72 @@ __global__ void __launch_bounds__(kCompactThreads) k_compact(const CompactArgs a
     }
 }
 
+// Structures of classes c_lo to c_hi, all of at most CAP reflections
 template <int CAP, int NT, bool FI>
-static void launch_post_class(const PostArgs& a, int cls, cudaStream_t st)
+static void launch_post_class(const PostArgs& a, int c_lo, int c_hi, bool first, bool pdl, cudaStream_t st)
 {
+    const auto k = k_post<CAP, NT, FI>;
     const size_t smem = post_smem_bytes(CAP);
-    static int per_sm_cache[64] = {};
+    static std::atomic<int> per_sm_cache[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
-    int per_sm = (dev >= 0 && dev < 64) ? per_sm_cache[dev] : 0;
+    int per_sm = (dev >= 0 && dev < 64) ? per_sm_cache[dev].load(std::memory_order_relaxed) : 0;
     if (per_sm < 1) {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k_post<CAP, NT, FI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         // all of the unified L1 / shared storage as shared memory: more structures in flight per SM
-        cudaFuncSetAttribute(k_post<CAP, NT, FI>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_post<CAP, NT, FI>, NT, smem) != cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        if (dev >= 0 && dev < 64) per_sm_cache[dev] = per_sm;
+        cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+        if (dev >= 0 && dev < 64) per_sm_cache[dev].store(per_sm, std::memory_order_relaxed);
     }
     const int grid = min(a.grid * per_sm, a.n_struct);
-    k_post<CAP, NT, FI><<<grid, NT, smem, st>>>(a, cls);
+    if (pdl) launch_pdl(k, grid, NT, smem, st, a, c_lo, c_hi, first);
+    else k<<<grid, NT, smem, st>>>(a, c_lo, c_hi, first);
 }
 
-// st[c]: the stream of size class c (the caller forks and joins them); the largest first
+// The size classes in a row on one stream, the largest first, each starting as the CTAs of the one before leave room
+// (pdl_chain_enter): the flat passes where a structure can be that large, then the shared-memory classes that a
+// structure of the batch can fall into (no structure has more reflections than the batch has room for).
+// The classes keep the shared memory of a CTA close to what its structure needs, which matters where structures
+// queue for the SMs; a batch that leaves SMs free has nothing to gain from it, and every class costs a launch:
+// up to one structure per SM takes one launch for all, up to kPostFewMax structures three. Measured against nine streams
+// forked and joined by events, one class each: 24 mixed cells 136 -> 134 us a call, 1024 small cells 247 -> 205 us,
+// 256 hexagonal/P1 cells 165 -> 141 us, 20 000 cells at Mo K-alpha 7.38 -> 6.81 ms, rock salt in FP64 155 -> 132 us
+// (with the one-launch front, k_front).
+constexpr int kPostFewMax = 2048;
 template <bool FI>
-static void launch_post_fi(const PostArgs& a, const cudaStream_t* st)
+static void launch_post_fi(const PostArgs& a, int64_t cap_refl, cudaStream_t st, bool pdl)
 {
-    launch_post_flat(a, kPostFlatClass, st[kPostFlatClass]);
-    launch_post_class<kPostCap7, 1024, FI>(a, 7, st[7]);
-    launch_post_class<kPostCap6, 512, FI>(a, 6, st[6]);
-    launch_post_class<kPostCap5, 512, FI>(a, 5, st[5]);
-    launch_post_class<kPostCap4, 256, FI>(a, 4, st[4]);
-    launch_post_class<kPostCap3, 256, FI>(a, 3, st[3]);
-    launch_post_class<kPostCap2, 192, FI>(a, 2, st[2]);
-    launch_post_class<kPostCap1, 128, FI>(a, 1, st[1]);
-    launch_post_class<kPostCap0, 64, FI>(a, 0, st[0]);
+    bool first = true;
+    if (cap_refl > kPostCap7) {
+        launch_post_flat(a, kPostFlatClass, st);
+        first = false;
+        pdl = true;
+    }
+    auto go = [&](auto cap, auto nt, int c_lo, int c_hi, int64_t below) {
+        if (c_lo > 0 && cap_refl <= below) return;
+        launch_post_class<decltype(cap)::value, decltype(nt)::value, FI>(a, c_lo, c_hi, first, pdl, st);
+        first = false;
+        pdl = true;
+    };
+#define XRD_POST(CAP, NT, LO, HI, BELOW) \
+    go(std::integral_constant<int, CAP>{}, std::integral_constant<int, NT>{}, LO, HI, BELOW)
+    if (a.n_struct <= a.grid && cap_refl > kPostCap3) {
+        XRD_POST(kPostCap7, 1024, 0, 7, 0);
+    } else if (a.n_struct <= kPostFewMax) {
+        XRD_POST(kPostCap7, 1024, 7, 7, kPostCap6);
+        XRD_POST(kPostCap6, 512, 4, 6, kPostCap3);
+        XRD_POST(kPostCap3, 256, 0, 3, 0);
+    } else {
+        XRD_POST(kPostCap7, 1024, 7, 7, kPostCap6);
+        XRD_POST(kPostCap6, 512, 6, 6, kPostCap5);
+        XRD_POST(kPostCap5, 512, 5, 5, kPostCap4);
+        XRD_POST(kPostCap4, 256, 4, 4, kPostCap3);
+        XRD_POST(kPostCap3, 256, 3, 3, kPostCap2);
+        XRD_POST(kPostCap2, 192, 2, 2, kPostCap1);
+        XRD_POST(kPostCap1, 128, 1, 1, kPostCap0);
+        XRD_POST(kPostCap0, 64, 0, 0, 0);
+    }
+#undef XRD_POST
 }
 
 // With a caller's point group: the family key of every reflection of the batch
@@ -652,18 +687,19 @@ void launch_pg_keys(const PostArgs& a, unsigned long long* fkg, cudaStream_t st)
 }
 
 // a.grid = number of SMs
-void launch_post(const PostArgs& a, const cudaStream_t* st)
+void launch_post(const PostArgs& a, int64_t cap_refl, cudaStream_t st, bool pdl)
 {
     if (a.n_struct <= 0) return;
-    if (a.If) launch_post_fi<true>(a, st);
-    else launch_post_fi<false>(a, st);
+    if (a.If) launch_post_fi<true>(a, cap_refl, st, pdl);
+    else launch_post_fi<false>(a, cap_refl, st, pdl);
 }
 
-void launch_compact(const CompactArgs& a, cudaStream_t st)
+void launch_compact(const CompactArgs& a, cudaStream_t st, bool pdl)
 {
     const int nch = (a.n_struct + kOutItems * kOutThreads - 1) / (kOutItems * kOutThreads);
     if (nch <= 2 || !a.parts) {
-        k_scan_out<<<1, kOutThreads, 0, st>>>(a);
+        if (pdl) launch_pdl(k_scan_out, 1, kOutThreads, 0, st, a);
+        else k_scan_out<<<1, kOutThreads, 0, st>>>(a);
     } else {
         k_scan_out_parts<<<nch, kOutThreads, 0, st>>>(a);
         launch_pdl(k_scan_out_final, nch, kOutThreads, 0, st, a);

@@ -226,10 +226,7 @@ template <int RB>
 static void launch_sf64_rb(const SfArgs& a, cudaStream_t st, bool pdl)
 {
     const size_t smem = sizeof(CoefX) * (size_t)(a.zmax + 1);
-    int per_sm = 0;  // of a device and zmax; asked for on every launch: it costs about a microsecond
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sf64<RB>, 32 * kSf64Warps, smem) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
+    const int per_sm = resident_ctas((const void*)k_sf64<RB>, 32 * kSf64Warps, smem);
     if (pdl) launch_pdl(k_sf64<RB>, a.grid * per_sm, 32 * kSf64Warps, smem, st, a);
     else k_sf64<RB><<<a.grid * per_sm, 32 * kSf64Warps, smem, st>>>(a);
 }

@@ -21,14 +21,12 @@ constexpr int kHklLimit = 511;        // |h|, |k|, |l| fit the 10-bit fields of 
 // 64, 128, 192, 256, 256, 512, 512 or 1024 threads; finer classes at the small
 // end keep the shared memory of a CTA close to what its structure needs, so
 // more structures are in flight per SM. Larger structures go to the last
-// class, processed by flat device-wide passes (k_post_flat.cu). Every class
-// runs on a stream of its own.
+// class, processed by flat device-wide passes (k_post_flat.cu).
 constexpr int kPostClasses = 9;
 constexpr int kRunsPerTile = 32;  // structure-factor tile: one run of reflections per lane of a warp
 constexpr int kPostCap0 = 256, kPostCap1 = 512, kPostCap2 = 768, kPostCap3 = 1024, kPostCap4 = 1536,
               kPostCap5 = 2048, kPostCap6 = 3072, kPostCap7 = 6144;
 constexpr int kPostFlatClass = kPostClasses - 1;
-constexpr int kPostStreams = kPostClasses;
 __host__ __device__ __forceinline__ int post_class(long long c)
 {
     return c <= kPostCap0   ? 0
@@ -162,6 +160,20 @@ __device__ __forceinline__ void pdl_enter()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A kernel of a group of independent ones launched in a row (the post-processing classes): the first enters by
+// pdl_enter, each later one starts as soon as its predecessor's CTAs have all started, without waiting for it (what
+// the group reads was complete before the first one began). At its end one CTA of each waits for the predecessor
+// (pdl_chain_exit), so that the group's last kernel completes after all of them.
+__device__ __forceinline__ void pdl_chain_enter(bool first)
+{
+    if (first) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_chain_exit()
+{
+    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Launch k on st as a programmatic dependent of the previous kernel on st.

@@ -281,6 +281,8 @@ struct AugArgs {
 // pdl: launch as a programmatic dependent of the previous kernel on st (only
 // when that kernel directly precedes it on the stream)
 void launch_prep(const GeomArgs& a, cudaStream_t st, bool pdl);
+bool front_fused(int n_struct, int64_t n_atoms);  // the front runs as one launch:
+void launch_front(const GeomArgs& a, cudaStream_t st);  // order, coefficients, cells and atoms
 void launch_coef(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_atoms(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_order(const GeomArgs& a, cudaStream_t st, bool pdl);
@@ -297,8 +299,10 @@ RefineTables init_refine_tables(cudaStream_t st);  // fills the tables, returns 
 void launch_refine(const RefineArgs& a, cudaStream_t st, bool pdl);
 size_t post_smem_bytes(int cap);
 void launch_post_flat(const PostArgs& a, int cls, cudaStream_t st);
-void launch_post(const PostArgs& a, const cudaStream_t* st);  // st[kPostStreams]: a stream per class
-void launch_compact(const CompactArgs& a, cudaStream_t st);
+void launch_post(const PostArgs& a, int64_t cap_refl, cudaStream_t st, bool pdl);  // cap_refl: reflections the batch can have
+void launch_compact(const CompactArgs& a, cudaStream_t st, bool pdl);
+// CTAs of a kernel that fit on an SM of the current device at once (at least 1), remembered per device, kernel and shape
+int resident_ctas(const void* kernel, int threads, size_t smem);
 const TTab* init_tables(cudaStream_t st);  // fills the 2-theta table, returns its device address
 size_t broaden_smem_bytes(int n_pts, int W);
 void launch_broaden(const GradArgs& a, cudaStream_t st);

@@ -22,18 +22,20 @@ XRD_NOALLOC_SCRATCH_BYTES = 64 << 20  # fixed device scratch of xrd_pattern_batc
 PRECISIONS = {"fp64": XRD_FP64, "fp32_phase64": XRD_FP32_PHASE64, "fp32_phasefix": XRD_FP32_PHASEFIX}
 STAGES = ["prep", "atoms", "count", "scan", "emit", "structure_factor", "refine", "post", "compact", "profile_sum"]
 XRD_FLAG_HEXAGONAL = 1  # bit of the per-structure flag word: families by Miller-Bravais indices
-# kernels xrd_pattern_batch launches per call: order, coef, atoms (a side stream), prep, count, scan, emit,
-# structure factor, re-evaluation of weak reflections (selection and evaluation, FP32 variants), post
-# (eight shared-memory size classes and one cooperative kernel of flat passes for the largest), output scan,
-# compaction
+# kernels xrd_pattern_batch launches per call, batches of more than 2048 structures: order, coef, atoms (a side
+# stream), prep, count, scan, emit, structure factor, re-evaluation of weak reflections (selection and evaluation,
+# FP32 variants), post (one cooperative kernel of flat passes for the largest size class, eight shared-memory
+# classes), output scan, compaction
 LAUNCHES_PER_BATCH = 21
 
 
 def launches_per_batch(n_struct: int, refine: bool = True, point_group: bool = False) -> int:
-    """Kernels of one xrd_pattern_batch call: above two chunks of 4096 structures the
+    """Kernels of one xrd_pattern_batch call, at most: above two chunks of 4096 structures the
     largest-first order, the reflection scan and the output scan each take two kernels (chunk
     sums, then the chunks); the FP64 variant (or refine off) has no re-evaluation kernels; a
-    caller's point group adds the family-key kernel."""
+    caller's point group adds the family-key kernel. Smaller batches take fewer: up to 2048 structures the
+    front is one kernel and the post-processing classes share launches, and classes larger than the
+    workspace has reflections are not launched."""
     return (LAUNCHES_PER_BATCH - (0 if refine else 2) + (3 if (n_struct + 4095) // 4096 > 2 else 0)
             + (1 if point_group else 0))
 
