@@ -24,6 +24,7 @@ struct xrd_handle {
     const xrd::TTab* ttab = nullptr;  // 2-theta table on the handle's device
     int sf_rb = 4, sf_warps = 2;        // structure-factor launch shape (xrd_autotune)
     int sf_runs = 0;                    // lanes take runs consecutive in l (integer phase only)
+    bool sf_chosen = false;             // the shape was chosen (xrd_set_sf_shape, xrd_autotune): keep it
     int enum_threads = 256;             // threads per CTA of the enumeration kernels (xrd_autotune)
     // the input-only front of a large batch (coefficients, atom packing, largest-first order) runs on the side
     // stream beside the enumeration: forked by front, joined by order_done and atoms_done
@@ -42,7 +43,7 @@ namespace {
 constexpr int kRunsPerTileHost = xrd::kRunsPerTile;  // structure-factor tile: 32 runs (one per lane)
 // flags area, zeroed at the start of every call: flag words (see GeomArgs::abort_flag), the
 // structure-factor work counters (3 x 64 bit) at byte kWorkOffset, the re-evaluation's
-// reflection count (64 bit) at kRefinedOffset, the enumeration claims and parts at ints 26 to 28 and the post
+// reflection count (64 bit) at kRefinedOffset, the enumeration's counters at ints 26 to 29 and the post
 // class counts and work counters at ints kFlagClsCnt and kFlagClsNext
 constexpr int kFlagBytes = 256;
 constexpr int kWorkOffset = 64;
@@ -239,9 +240,20 @@ int check_opts(xrd_handle* h, const xrd_opts* o)
     return XRD_OK;
 }
 
-// launch shape of the structure-factor kernel for this call
-void sf_shape(const xrd_handle* h, const xrd_opts* o, int& rb, int& warps, int& runs)
+// Launch shape of the structure-factor kernel for this call. Where nobody has chosen one, strided tiles (whose results
+// do not depend on their size): FP64 lanes take one reflection (they would take several one after another); FP32
+// lanes take four, which share an atom's loads and a packed instruction's halves, or two where tiles of 128 would fill
+// less than half of the resident warps (12 of 24 per SM) and the longest tile sets the time. 24 mixed cells (140 tiles
+// of 128) 30.3 us with four, 21.8 us with two; 256 hexagonal/P1 cells 24.2 and 20.2; 1024 small cells (8500 tiles)
+// 65.2 and 69.2. Rock salt in FP64 (3 tiles of 128): 45 us with four, 20 us with one.
+void sf_shape(const xrd_handle* h, const xrd_opts* o, int64_t cap_refl, int& rb, int& warps, int& runs)
 {
+    if (o->tile == -1 && !h->sf_chosen) {
+        rb = o->precision == XRD_FP64 ? 1 : (cap_refl / 128 < (int64_t)12 * h->sms ? 2 : 4);
+        warps = 2;
+        runs = 0;
+        return;
+    }
     rb = o->tile == 64 ? 2 : (o->tile == 128 ? 4 : h->sf_rb);
     warps = (o->precision == XRD_FP32_PHASEFIX) ? h->sf_warps : 2;
     runs = (o->precision == XRD_FP32_PHASEFIX && o->tile == -1 && rb == 4) ? h->sf_runs : 0;
@@ -569,7 +581,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     char* ws = (char*)workspace;
     const Layout L = layout(n, b->n_atoms, b->zmax, cap_refl, pg);
     int rb, warps, runs;
-    sf_shape(h, o, rb, warps, runs);
+    sf_shape(h, o, cap_refl, rb, warps, runs);
     xrd::GeomArgs ga = geom_args(b, o, L, ws, cap_refl, out->totals, out->status, rb);
     ga.sctab = h->rtab.sc;
     ga.runs_mode = runs;
@@ -597,7 +609,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     // the input-only front: in one launch for a small batch; else order (needed by the scan), coefficients and atoms
     // (needed by the structure factor) on a side stream, beside the enumeration
     ga.atoms_set_geo = 0;
-    const bool fused = xrd::front_fused((int)n, b->n_atoms);
+    const bool fused = n > 0 && xrd::front_fused((int)n, b->n_atoms);
     if (fused) {
         xrd::launch_front(ga, st);
     } else {
@@ -612,10 +624,12 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     }
     mark();
     mark();  // the atom packing stage runs on the side stream: nothing on this one
-    xrd::launch_count(ga, st, pdl);
+    xrd::launch_count(ga, st, pdl, fused);
     mark();
-    if (!fused) cudaStreamWaitEvent(st, h->order_done, 0);
-    xrd::launch_scan_refl(ga, st, fused && pdl);
+    if (!fused) {  // else the counting kernel's last CTA has scanned
+        cudaStreamWaitEvent(st, h->order_done, 0);
+        xrd::launch_scan_refl(ga, st, false);
+    }
     mark();
     xrd::launch_emit(ga, st, pdl);
     mark();
@@ -671,6 +685,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
         ra.cref = (float)(o->rel_cutoff > 0.0 ? o->rel_cutoff : kRefineFloorNoCut);
         ra.abort_flag = ga.abort_flag;
         ra.nref = (unsigned long long*)(ws + L.flags + kRefinedOffset);
+        ra.cap_refl = cap_refl;
         ra.cand_r = (int64_t*)(ws + L.cand_r);
         ra.cand_s = (int*)(ws + L.cand_s);
         ra.refl_off = ga.refl_off;
@@ -874,6 +889,7 @@ int xrd_set_sf_shape(xrd_handle* h, int tile, int warps, int runs)
     h->sf_rb = tile / 32;
     h->sf_warps = warps;
     h->sf_runs = runs;
+    h->sf_chosen = true;
     return XRD_OK;
 }
 
@@ -888,6 +904,8 @@ int xrd_autotune(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const xrd
     const int nshape = all ? 9 : 2;
     const int keep_rb = h->sf_rb, keep_w = h->sf_warps, keep_runs = h->sf_runs;
     const int keep_prof = h->profiling;
+    const bool keep_chosen = h->sf_chosen;
+    h->sf_chosen = true;
     xrd_opts oo = o ? *o : xrd_opts{};
     oo.tile = -1;
     float best = 1e30f;
@@ -910,12 +928,14 @@ int xrd_autotune(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const xrd
             const int rc = xrd_pattern_batch(h, b, &oo, out, workspace, ws_bytes, stream);
             if (rc != XRD_OK) {
                 h->sf_rb = keep_rb; h->sf_warps = keep_w; h->sf_runs = keep_runs; h->profiling = keep_prof;
+                h->sf_chosen = keep_chosen;
                 return finish(rc);
             }
             float ms[kStages];
             const int m = xrd_stage_times(h, ms, kStages);
             if (m < 0) {
                 h->sf_rb = keep_rb; h->sf_warps = keep_w; h->sf_runs = keep_runs; h->profiling = keep_prof;
+                h->sf_chosen = keep_chosen;
                 return finish(-m);
             }
             // the stages the shape changes: count, scan, emit (runs are built there), structure factor;
@@ -1074,7 +1094,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.n_atoms = b->n_atoms;
     ga.sctab = h->rtab.sc;
     int rb, warps, runs;
-    sf_shape(h, o, rb, warps, runs);
+    sf_shape(h, o, cap_refl, rb, warps, runs);
     ga.rb = rb;
     ga.runs_mode = grad ? 0 : runs;
     ga.enum_threads = grad ? 256 : h->enum_threads;
@@ -1118,7 +1138,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     xrd::launch_coef(ga, st, true);
     xrd::launch_atoms(ga, st, true);
     xrd::launch_order(ga, st, true);
-    xrd::launch_count(ga, st, true);
+    xrd::launch_count(ga, st, true, false);
     xrd::launch_scan_refl(ga, st, true);
     xrd::launch_emit(ga, st, true);
     xrd::SfArgs sa{};

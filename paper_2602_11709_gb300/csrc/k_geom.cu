@@ -551,49 +551,6 @@ __device__ __forceinline__ bool enum_item(const Geo* __restrict__ geo, const int
     return true;
 }
 
-// Reflection (and, with RUNS, run) counts per structure, and of every part (k_prep has zeroed the counts of a
-// structure in parts). ctr: zero at launch.
-template <bool RUNS>
-__global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict__ geo, int n_struct, double r2min,
-                                                           double r2max, float r2minf, float r2maxf, int rb,
-                                                           int64_t* __restrict__ cnt, int64_t* __restrict__ run_cnt,
-                                                           int* __restrict__ ctr, const int* __restrict__ part_ctr,
-                                                           const int2* __restrict__ part_tab,
-                                                           int2* __restrict__ part_cnt, int part_cap, int part_cols)
-{
-    pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const EnumItems items = enum_items(n_struct, part_ctr, part_cap, ctr);
-    for (;;) {
-        int m;
-        const int first = items.next(m);
-        if (m == 0) break;
-        for (int it = first; it < first + m; it++) {
-            int s, part, c0, c1;
-            Geo g;
-            if (!enum_item(geo, part_tab, items.nparts, part_cols, it, s, part, g, c0, c1)) continue;
-            int local = 0, local_runs = 0;
-            for (int c = c0 + lane; c < c1; c += 32) {
-                int h, k, n, nr;
-                column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, n, nr);
-                local += n;
-                local_runs += nr;
-            }
-            local = warp_sum_int(local);
-            if (RUNS) local_runs = warp_sum_int(local_runs);
-            if (lane != 0) continue;
-            if (part < 0) {
-                cnt[s] = local;
-                if (RUNS && run_cnt) run_cnt[s] = local_runs;
-            } else {
-                part_cnt[it] = make_int2(local, local_runs);
-                atomicAdd((unsigned long long*)(cnt + s), (unsigned long long)local);
-                if (RUNS && run_cnt) atomicAdd((unsigned long long*)(run_cnt + s), (unsigned long long)local_runs);
-            }
-        }
-    }
-}
-
 // Record of a non-empty column of a chunk: its |g|^2 as a polynomial in l, q(l) = t + u l + G*33 l^2 with
 // t = G*11 h^2 + G*22 k^2 + 2 G*12 hk and u = 2 G*13 h + 2 G*23 k in two-float arithmetic (about 1e-14 relative),
 // and where its reflections and runs go.
@@ -755,10 +712,11 @@ constexpr int kOrderBins = 4096;
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 
+template <int BINS = kOrderBins>
 __device__ __forceinline__ int order_bin(const int64_t* __restrict__ atom_off, int s)
 {
     const long long na = atom_off[s + 1] - atom_off[s];
-    return kOrderBins - 1 - (int)min(max(na, 0LL), (long long)(kOrderBins - 1));
+    return BINS - 1 - (int)min(max(na, 0LL), (long long)(BINS - 1));
 }
 
 // Rank of this lane among the lanes of its warp with the same key, and the
@@ -776,19 +734,42 @@ __device__ __forceinline__ int warp_aggregated_slot(int* ctr, int key, bool acti
     return base + __popc(peers & ((1u << lane) - 1u));
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __restrict__ cnt,
-                                                            const int64_t* __restrict__ run_cnt,
-                                                            const Geo* __restrict__ geo, int n, int tile_refl,
-                                                            int64_t cap_refl, int64_t* __restrict__ refl_off,
-                                                            int* __restrict__ tile_off, const int* __restrict__ order,
-                                                            int* __restrict__ cls_list, int* __restrict__ abort_flag,
-                                                            int64_t* __restrict__ totals, int32_t* __restrict__ status,
-                                                            unsigned long long* __restrict__ work)
+struct ScanArgs {
+    const int64_t* run_cnt;
+    int tile_refl;
+    int64_t cap_refl;
+    int64_t* refl_off;
+    int* tile_off;
+    const int* order;
+    int* cls_list;
+    int* abort_flag;
+    int64_t* totals;
+    int32_t* status;
+    unsigned long long* work;
+};
+struct ScanShared {
+    long long ws[33];
+    int ccnt[kPostClasses];
+};
+
+// buf: kScanItems * blockDim long longs of shared memory. The counts are read past the L1 cache: the CTA that runs
+// this may be one of the kernel that wrote them.
+__device__ __forceinline__ void scan_refl_block(const int64_t* cnt, const Geo* __restrict__ geo, int n,
+                                                const ScanArgs& sa, ScanShared& sh, long long* buf)
 {
-    pdl_enter();
-    __shared__ long long ws[33];
-    __shared__ __align__(16) long long buf[kScanItems * kScanThreads];
-    __shared__ int ccnt[kPostClasses];
+    const int64_t* const run_cnt = sa.run_cnt;
+    const int tile_refl = sa.tile_refl;
+    const int64_t cap_refl = sa.cap_refl;
+    int64_t* const refl_off = sa.refl_off;
+    int* const tile_off = sa.tile_off;
+    const int* const order = sa.order;
+    int* const cls_list = sa.cls_list;
+    int* const abort_flag = sa.abort_flag;
+    int64_t* const totals = sa.totals;
+    int32_t* const status = sa.status;
+    unsigned long long* const work = sa.work;
+    long long* const ws = sh.ws;
+    int* const ccnt = sh.ccnt;
     const int nt = blockDim.x, tid = threadIdx.x, CH = kScanItems * nt;
     long long tot;
     // 1. reflection offsets in structure order, and the status of each structure
@@ -799,7 +780,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __res
 #pragma unroll
         for (int u = 0; u < kScanItems; u++) {
             const int i = base + u * nt + tid;
-            v[u] = i < n ? cnt[i] : 0;
+            v[u] = i < n ? __ldcg((const long long*)cnt + i) : 0;
             st[u] = i < n ? geo[i].status : XRD_OK;
         }
         chunk_scan<kScanItems>(v, buf, ws, &tot);
@@ -835,10 +816,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __res
         long long c[kScanItems];
 #pragma unroll
         for (int u = 0; u < kScanItems; u++) {
-            c[u] = sv[u] >= 0 ? cnt[sv[u]] : 0;
+            c[u] = sv[u] >= 0 ? __ldcg((const long long*)cnt + sv[u]) : 0;
             // tiles of 32 runs, or of tile_refl reflections
             v[u] = sv[u] < 0 ? 0 : (tile_refl > 0 ? (c[u] + tile_refl - 1) / tile_refl
-                                                  : (run_cnt[sv[u]] + kRunsPerTile - 1) / kRunsPerTile);
+                                                  : (__ldcg((const long long*)run_cnt + sv[u]) + kRunsPerTile - 1) / kRunsPerTile);
         }
         chunk_scan<kScanItems>(v, buf, ws, &tot);
 #pragma unroll
@@ -868,6 +849,71 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __res
         totals[3] = nbad;
         *abort_flag = over;
     }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __restrict__ cnt,
+                                                            const Geo* __restrict__ geo, int n, const ScanArgs sa)
+{
+    pdl_enter();
+    __shared__ ScanShared sh;
+    __shared__ __align__(16) long long buf[kScanItems * kScanThreads];
+    scan_refl_block(cnt, geo, n, sa, sh, buf);
+}
+
+// Reflection (and, with RUNS, run) counts per structure, and of every part (k_prep has zeroed the counts of a
+// structure in parts). ctr: zero at launch. done: CTAs finished (zero at launch), or null: no scan.
+template <bool RUNS>
+__global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict__ geo, int n_struct, double r2min,
+                                                           double r2max, float r2minf, float r2maxf, int rb,
+                                                           int64_t* __restrict__ cnt, int64_t* __restrict__ run_cnt,
+                                                           int* __restrict__ ctr, const int* __restrict__ part_ctr,
+                                                           const int2* __restrict__ part_tab,
+                                                           int2* __restrict__ part_cnt, int part_cap, int part_cols,
+                                                           const ScanArgs scan, int* __restrict__ done)
+{
+    pdl_enter();
+    const int lane = threadIdx.x & 31;
+    const EnumItems items = enum_items(n_struct, part_ctr, part_cap, ctr);
+    for (;;) {
+        int m;
+        const int first = items.next(m);
+        if (m == 0) break;
+        for (int it = first; it < first + m; it++) {
+            int s, part, c0, c1;
+            Geo g;
+            if (!enum_item(geo, part_tab, items.nparts, part_cols, it, s, part, g, c0, c1)) continue;
+            int local = 0, local_runs = 0;
+            for (int c = c0 + lane; c < c1; c += 32) {
+                int h, k, n, nr;
+                column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, n, nr);
+                local += n;
+                local_runs += nr;
+            }
+            local = warp_sum_int(local);
+            if (RUNS) local_runs = warp_sum_int(local_runs);
+            if (lane != 0) continue;
+            if (part < 0) {
+                cnt[s] = local;
+                if (RUNS && run_cnt) run_cnt[s] = local_runs;
+            } else {
+                part_cnt[it] = make_int2(local, local_runs);
+                atomicAdd((unsigned long long*)(cnt + s), (unsigned long long)local);
+                if (RUNS && run_cnt) atomicAdd((unsigned long long*)(run_cnt + s), (unsigned long long)local_runs);
+            }
+        }
+    }
+    if (!done) return;
+    // the CTA that finishes last scans the counts (a launch less in a small batch's chain)
+    extern __shared__ __align__(16) long long scan_buf[];
+    __shared__ ScanShared sh;
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    scan_refl_block(cnt, geo, n_struct, scan, sh, scan_buf);
 }
 
 // Multi-block form of k_scan_refl for batches of more than two chunks (one
@@ -1015,30 +1061,31 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_final(const int64_t*
 // block, warp-aggregated shared-memory atomics, so structures of one bin keep
 // the order of their warp. It depends on the input only and runs beside the
 // enumeration.
+template <int BINS>
 __device__ __forceinline__ void order_block(const int64_t* __restrict__ atom_off, int n, int* __restrict__ order,
                                             int* bins, int* tmp)
 {
     const int nt = blockDim.x, tid = threadIdx.x, CH = kScanItems * nt;
-    for (int b = tid; b < kOrderBins; b += nt) bins[b] = 0;
+    for (int b = tid; b < BINS; b += nt) bins[b] = 0;
     __syncthreads();
     for (int base = 0; base < n; base += CH) {
         int b[kScanItems];
 #pragma unroll
         for (int u = 0; u < kScanItems; u++) {
             const int i = base + u * nt + tid;
-            b[u] = i < n ? order_bin(atom_off, i) : 0;
+            b[u] = i < n ? order_bin<BINS>(atom_off, i) : 0;
         }
 #pragma unroll
         for (int u = 0; u < kScanItems; u++) warp_aggregated_slot(bins, b[u], base + u * nt + tid < n);
     }
     __syncthreads();
-    block_excl_scan(bins, kOrderBins, tmp);
+    block_excl_scan(bins, BINS, tmp);
     for (int base = 0; base < n; base += CH) {
         int b[kScanItems];
 #pragma unroll
         for (int u = 0; u < kScanItems; u++) {
             const int i = base + u * nt + tid;
-            b[u] = i < n ? order_bin(atom_off, i) : 0;
+            b[u] = i < n ? order_bin<BINS>(atom_off, i) : 0;
         }
 #pragma unroll
         for (int u = 0; u < kScanItems; u++) {
@@ -1055,14 +1102,15 @@ __global__ void __launch_bounds__(kScanThreads) k_order(const int64_t* __restric
     pdl_enter();
     __shared__ int bins[kOrderBins];
     __shared__ int tmp[66];
-    order_block(atom_off, n, order, bins, tmp);
+    order_block<kOrderBins>(atom_off, n, order, bins, tmp);
 }
 
-// The whole input-only front of a small batch in one launch: block 0 forms the coefficients and the largest-first
-// order, the next blocks the cells (16 structures each), the others pack the atoms of one structure each. One launch
+// The whole input-only front of a small batch in one launch: block 0 forms the largest-first order, block 1 the
+// coefficients, the next blocks the cells (16 structures each), the others pack the atoms of one structure each. One launch
 // instead of four on two streams: a small batch is bound by its chain of launches. Taken up to kFrontMax structures of
 // kFrontAtoms atoms on average; beyond, packing the atoms takes longer than counting the reflections, and the two
 // run side by side on two streams instead.
+constexpr int kFrontBins = 512;  // atom counts above this share a bin: the order only balances the load
 struct FrontArgs {
     GeomArgs g;
     EnumParts ep;
@@ -1074,19 +1122,20 @@ __global__ void __launch_bounds__(kAtomThreads) k_front(const FrontArgs f)
     __shared__ union {
         AtomShared at;
         struct {
-            int bins[kOrderBins], tmp[66];
+            int bins[kFrontBins], tmp[66];
         } ord;
     } sh;
     const GeomArgs& g = f.g;
     const int b = blockIdx.x;
     if (b == 0) {
+        order_block<kFrontBins>(g.atom_off, g.n_struct, g.order, sh.ord.bins, sh.ord.tmp);
+    } else if (b == 1) {
         coef_block(g.coef, g.zmax, g.coef32, g.cdd);
-        order_block(g.atom_off, g.n_struct, g.order, sh.ord.bins, sh.ord.tmp);
-    } else if (b <= f.prep_blocks) {
-        prep_thread<8>((b - 1) * kAtomThreads + threadIdx.x, g.lattice, g.n_struct, g.rmax, g.geo, g.imax, g.out_flags,
+    } else if (b <= 1 + f.prep_blocks) {
+        prep_thread<8>((b - 2) * kAtomThreads + threadIdx.x, g.lattice, g.n_struct, g.rmax, g.geo, g.imax, g.out_flags,
                        f.ep);
     } else {
-        atoms_block(b - 1 - f.prep_blocks, sh.at, g.atom_off, g.n_atoms, g.frac, g.Z, g.occ, g.B, g.zmax, g.geo, 0,
+        atoms_block(b - 2 - f.prep_blocks, sh.at, g.atom_off, g.n_atoms, g.frac, g.Z, g.occ, g.B, g.zmax, g.geo, 0,
                     g.atom_bad, g.atom32, g.atomx, g.runs_mode ? g.astep : nullptr, g.atomr, g.sctab);
     }
 }
@@ -1224,7 +1273,7 @@ void launch_front(const GeomArgs& a, cudaStream_t st)
 {
     if (a.n_struct <= 0) return;
     FrontArgs f{a, enum_parts(a), (8 * a.n_struct + kAtomThreads - 1) / kAtomThreads};
-    k_front<<<1 + f.prep_blocks + a.n_struct, kAtomThreads, 0, st>>>(f);
+    k_front<<<2 + f.prep_blocks + a.n_struct, kAtomThreads, 0, st>>>(f);
 }
 
 void launch_prep(const GeomArgs& a, cudaStream_t st, bool pdl)
@@ -1273,24 +1322,36 @@ static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
     return (int)min((int64_t)a.sms * per_sm, max(most, (int64_t)1));
 }
 
-static void count_launch(const GeomArgs& a, cudaStream_t st, bool pdl)
+static ScanArgs scan_args(const GeomArgs& a)
+{
+    return ScanArgs{a.run_cnt, a.runs_mode ? 0 : 32 * a.rb, a.cap_refl, a.refl_off, a.tile_off, a.order, a.cls_list,
+                    a.abort_flag, a.totals, a.status, a.work};
+}
+
+static void count_launch(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan)
 {
     const auto k = a.runs_mode ? k_count<true> : k_count<false>;
-    launch_k(pdl, k, enum_grid(a, (const void*)k, 0), a.enum_threads, st, a.geo, a.n_struct, a.r2min, a.r2max,
-             (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, a.refl_cnt, a.run_cnt, a.enum_ctr,
-             a.enum_ctr + kPartCtr, a.part_tab, a.part_cnt, a.part_cap, enum_part_cols(a.n_struct));
+    const size_t smem = scan ? sizeof(long long) * kScanItems * (size_t)a.enum_threads : 0;
+    const int grid = enum_grid(a, (const void*)k, smem);
+    auto go = [&](auto launch) {
+        launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, a.refl_cnt,
+               a.run_cnt, a.enum_ctr, (const int*)(a.enum_ctr + kPartCtr), (const int2*)a.part_tab, a.part_cnt,
+               a.part_cap, enum_part_cols(a.n_struct), scan_args(a), scan ? a.enum_ctr + kDoneCtr : (int*)nullptr);
+    };
+    if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });
+    else go([&](auto... v) { k<<<grid, a.enum_threads, smem, st>>>(v...); });
 }
 
 void launch_count_only(const GeomArgs& a, cudaStream_t st)
 {
     if (a.n_struct <= 0) return;
     prep_launch(false, a, st);
-    count_launch(a, st, true);
+    count_launch(a, st, true, false);
 }
 
-void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl)
+void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan)
 {
-    if (a.n_struct > 0) count_launch(a, st, pdl);
+    if (a.n_struct > 0) count_launch(a, st, pdl, scan);
 }
 
 int scan_chunks(int n) { return (n + kScanItems * kScanThreads - 1) / (kScanItems * kScanThreads); }
@@ -1300,9 +1361,7 @@ void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl)
     const int nch = scan_chunks(a.n_struct);
     const int tile_refl = a.runs_mode ? 0 : 32 * a.rb;
     if (nch <= 2 || !a.parts) {  // one block walks the chunks
-        launch_k(pdl, k_scan_refl, 1, kScanThreads, st, a.refl_cnt, a.run_cnt, a.geo, a.n_struct, tile_refl,
-                 a.cap_refl, a.refl_off, a.tile_off, (const int*)a.order, a.cls_list, a.abort_flag, a.totals,
-                 a.status, a.work);
+        launch_k(pdl, k_scan_refl, 1, kScanThreads, st, a.refl_cnt, a.geo, a.n_struct, scan_args(a));
         return;
     }
     launch_k(pdl, k_scan_refl_parts, nch, kScanThreads, st, a.refl_cnt, a.run_cnt, a.geo, a.n_struct, tile_refl,

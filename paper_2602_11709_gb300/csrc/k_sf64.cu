@@ -233,7 +233,8 @@ static void launch_sf64_rb(const SfArgs& a, cudaStream_t st, bool pdl)
 
 void launch_sf64(const SfArgs& a, cudaStream_t st, bool pdl)
 {
-    if (a.rb == 2) launch_sf64_rb<2>(a, st, pdl);
+    if (a.rb == 1) launch_sf64_rb<1>(a, st, pdl);
+    else if (a.rb == 2) launch_sf64_rb<2>(a, st, pdl);
     else launch_sf64_rb<4>(a, st, pdl);
 }
 

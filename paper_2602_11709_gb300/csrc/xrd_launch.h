@@ -47,7 +47,7 @@ struct GeomArgs {
     uint32_t* key;
     long long* parts;  // chunk sums of the multi-block scan (nullptr: single-block scan)
     int* oparts;       // [chunks][4096] bin counts of the multi-block order (nullptr: one-block order)
-    int* enum_ctr;     // flags[26..28]: claims of counting and of emission, parts listed (kPartCtr)
+    int* enum_ctr;     // flags[26..29]: claims of counting and of emission, parts listed (kPartCtr), CTAs of counting done
     int2* part_tab;    // [part_cap] (structure, part) of each enumeration part, by k_prep
     int2* part_cnt;    // [part_cap] its reflections and runs, by k_count
     int part_cap;
@@ -58,7 +58,7 @@ struct GeomArgs {
     AtomR* atomr;      // [atoms] records of the accurate re-evaluation, by k_atoms (or nullptr)
 };
 
-constexpr int kPartCtr = 2;  // index of the part counter within enum_ctr
+constexpr int kPartCtr = 2, kDoneCtr = 3;  // indices within enum_ctr
 
 // What k_prep needs to list the enumeration parts of the structures with more than `cols` columns.
 struct EnumParts {
@@ -117,6 +117,7 @@ struct RefineArgs {
     float cref;   // cutoff fraction (the floor of the guarantee), relative to the largest reflection M
     const int* abort_flag;
     unsigned long long* nref;     // reflections re-evaluated: the candidate list's length (zeroed per call)
+    int64_t cap_refl;             // reflections the batch can have
     int64_t* cand_r;              // [reflections] candidate list: reflection index
     int* cand_s;                  // [reflections] and its structure
     const int64_t* refl_off;
@@ -287,7 +288,7 @@ void launch_coef(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_atoms(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_order(const GeomArgs& a, cudaStream_t st, bool pdl);
 size_t order_parts_bytes(int64_t n);  // bytes of GeomArgs::oparts for n structures (0: one-block order)
-void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl);
+void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan);  // scan: and launch_scan_refl's work
 void launch_count_only(const GeomArgs& a, cudaStream_t st);
 void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st);  // out: device [3], zeroed

@@ -1,0 +1,35 @@
+"""Merged peaks of many members against the oracle: cubic, hexagonal and orthorhombic cells, where equal and nearly
+equal |g| make peaks of 1 to over 100 Friedel-unique members (one thread, a warp's lanes, or more than a warp holds),
+and tolerances that make runs of close reflections split at an anchor."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_11709_gb300 import adapter, synth
+
+from parity import compare_batch
+
+pytestmark = pytest.mark.gpu
+
+
+def _cells():
+    rng = np.random.default_rng(5)
+    lat = [[7.0] * 3 + [90.0] * 3, [4.1] * 3 + [90.0] * 3, [5.0, 5.0, 8.0, 90.0, 90.0, 120.0], [6.0, 6.0, 6.002, 90.0, 90.0, 90.0],
+           [11.0] * 3 + [90.0] * 3]
+    b = synth.concat([synth.random_cell(rng, 1 + i) for i in range(len(lat))])
+    b.lattice = np.array(lat)
+    return b
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_phasefix"])
+@pytest.mark.parametrize("tol", [1e-5, 0.02, 0.3])
+@pytest.mark.parametrize("group", [None, "mmm"])
+def test_many_members(gpu_lib, prec, tol, group):
+    b = _cells()
+    o = synth.Opts(tt_max=100.0, tt_tol=tol, rel_cutoff=1e-4)
+    if group:
+        o.point_group = adapter.laue_group_ops(group)
+    ref = oracle.pattern_batch(b, o)
+    assert max(len(p) and int(np.diff(f).max()) for p, f in zip(ref["peak_tt"], ref["peak_fam_off"])) >= (2 if tol > 1e-4 else 1)
+    got = gpu_lib.compute(b, o, prec)
+    compare_batch(got, ref, prec, o.rel_cutoff, o.scaled)
