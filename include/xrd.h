@@ -268,7 +268,8 @@ typedef struct {
  *   PV(u) = eta (2 / (pi w)) / (1 + x^2) + (1 - eta) (2 / w) sqrt(ln 2 / pi) 2^(-x^2),
  *           x = 2 u / w, w = fwhm (area-normalised pseudo-Voigt),
  * then, with noise_z, y[s][k] += sigma sqrt(max(y[s][k], 0)) z[s][k]. The
- * Lorentzian is summed over every grid point (no window); a reflection's
+ * Lorentzian is summed over every grid point (no window), beyond 256 points by
+ * interpolation of a run's sum (below 1e-7 of it); a reflection's
  * Gaussian is skipped only on runs of 256 consecutive grid points where it
  * stays below 2^-40 of its peak (x^2 >= 40). grid.fwhm is ignored; grid.n_pts <= 2^22
  * and every 2-theta in [tt_min, tt_max] lies within 2^22 dt of t0.

@@ -403,6 +403,7 @@ int xrd_create(xrd_handle** h, int device)
     p->ttab = xrd::init_tables(0);  // device tables (2-theta, re-evaluation), once per handle, legacy stream
     p->rtab = xrd::init_refine_tables(0);
     xrd::init_fx_tables(0);
+    xrd::init_aug_tables(0);
     e = cudaStreamSynchronize(0);
     if (e != cudaSuccess || !p->ttab || !p->rtab.sc || !p->rtab.ex) { xrd_destroy(p); return XRD_ECUDA; }
     *h = p;
@@ -1241,6 +1242,7 @@ int xrd_pattern_augmented(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     profile_front(h, b, o, L, ws, cap_refl, status, totals, st, false);
     xrd::AugArgs a{};
     a.n_struct = (int)n;
+    a.sms = h->sms;
     a.n_pts = grid->n_pts;
     a.t0 = grid->t0;
     a.dt = grid->dt;

@@ -8,19 +8,28 @@
 //   then y_k += sigma sqrt(max(y_k, 0)) z_k.
 //
 // k_aug_order lists the structures by reflection count, largest first.
-// k_aug_sum gives each CTA 1024 grid points of one structure (kAugPts
+// k_aug_sum gives each warp 256 grid points of one structure (kAugPts
 // consecutive points per thread) and streams all of the structure's reflections
 // through shared memory, turning each into a record as it is staged: its grid
 // cell b, the offset d of 2theta within the cell scaled by s = 2 dt / w, and the
-// Lorentzian and Gaussian amplitudes. The Lorentzian has no window: every
-// (point, reflection) pair costs half a reciprocal (MUFU, one per pair of
-// points) and about five FP32 operations. The Gaussian is evaluated by a warp
-// only for the reflections that reach its points with x^2 < 40 (a test made
-// once per reflection while staging).
+// Lorentzian and Gaussian amplitudes. The Lorentzian has no window, but beyond
+// kAugNear points from the middle of the warp's points a reflection's Lorentzian is
+// smooth over them: those reflections are summed at kAugNodes of the points only
+// (the Chebyshev-Lobatto points of the interval, rounded to the grid) and the sum is interpolated to all
+// 256 by its polynomial through the nodes. At the least distance that errs by 7e-8 of the Lorentzian at the worst
+// point, whatever the width (the poles of a Lorentzian lie at its 2theta, half a width off the real axis), about an
+// FP32 rounding, and by rho^-16, rho = r + sqrt(r^2 - 1), r = distance / 127.5, farther out. The Gaussian and the near
+// Lorentzians (an eighth of the reflections on 4096 points) are evaluated at every point; the Gaussian only for the reflections that reach
+// the warp's points with x^2 < 40.
+// What bounds it: instruction issue and the reciprocals, 2.2 instructions a clock (the CTAs also wait at the barriers
+// around the staging): per reflection and warp about 2.5 instructions for a far one, 36 for a near Lorentzian and 30 for
+// a Gaussian. 1024 cells of 1 to 64 atoms, 4096 points: 755 us with every (point, reflection) pair evaluated by
+// itself, 282 us now; summing the tails once per node instead of in every point's long sum also took the error of the
+// patterns from 4.6e-6 to 2e-7 of their norm.
 //
 // Precision: x = (k - b) s - d s with k - b an exact integer in FP32 (|k|, |b| <
 // 2^22); for s <= 1 the points after a thread's first take x + j s (absolute
-// error a few ulp of kAugPts s there); sums are FP32 in reflection order.
+// error a few ulp of kAugPts s there); sums are FP32.
 #include <cmath>
 
 #include "xrd_internal.cuh"
@@ -29,11 +38,10 @@
 namespace xrd {
 
 constexpr int kAugPts = 8;                       // consecutive grid points per thread
-constexpr int kAugThreads = 1024 / kAugPts;
-constexpr int kAugSpan = kAugThreads * kAugPts;  // grid points per CTA
-constexpr int kAugWarps = kAugThreads / 32;
+constexpr int kAugBlock = 32 * kAugPts;          // points of a warp
+constexpr int kAugNodes = 16;                    // of them, the interpolation's
+constexpr float kAugNear = 256.f;                // grid points from the warp's middle within which every point is summed
 constexpr int kAugBuckets = 128;                 // reflection-count buckets of the largest-first order
-constexpr int kAugChunk = 1024;                  // reflections staged in shared memory at a time
 
 __device__ __forceinline__ float rcp_approx(float x)
 {
@@ -144,132 +152,236 @@ __device__ __forceinline__ float4 aug_record(const AugArgs& a, const AugStruct& 
     return make_float4(-(float)(int)fb, -(float)((pos - fb) * (double)c.sc), A * c.cl, A * c.cg);
 }
 
-// Lorentzian part of m staged reflections at a thread's kAugPts consecutive
-// points (branch-free body; the unrolled iterations overlap). x at the thread's
+// Lorentzian part of one reflection at a thread's kAugPts consecutive
+// points, two points to a packed FP32 operation. x at the thread's
 // first point is exact up to rounding ((k - b) is an exact integer in FP32).
 // EXACT computes every point the same way; otherwise x_j = x_0 + j s in one fma
 // (absolute error a few ulp of kAugPts s: used for s <= 1, i.e. fwhm >= 2 dt).
+// acc[j] holds points 2 j + 1 and 2 j, in this order.
 template <bool EXACT>
-__device__ __forceinline__ void aug_lorentz(const float4* __restrict__ st, int m, float kf, float sc,
-                                            float (&acc)[kAugPts])
+__device__ __forceinline__ void aug_lorentz(const float4 R, float kf, float sc, float2 (&acc)[kAugPts / 2])
 {
-#pragma unroll 4
-    for (int i = 0; i < m; i++) {
-        const float4 R = st[i];  // (-b, -d s, Lorentzian amplitude, Gaussian amplitude)
-        const float m0 = kf + R.x;
-        float x[kAugPts];
+    // R = (-b, -d s, Lorentzian amplitude, Gaussian amplitude)
+    const float m0 = kf + R.x;
+    const float2 s2 = make_float2(sc, sc), one = make_float2(1.f, 1.f);
+    const float x0 = fmaf(m0, sc, R.y);
+    // one reciprocal per pair of points: 1/d0 = d1 / (d0 d1). d <= 1 + 2^58 (2^9 grid steps of at most 1e6 in x):
+    // d0 d1 does not overflow
 #pragma unroll
-        for (int j = 0; j < kAugPts; j++)
-            x[j] = EXACT ? fmaf(m0 + (float)j, sc, R.y) : (j ? fmaf((float)j, sc, x[0]) : fmaf(m0, sc, R.y));
-        // one reciprocal per pair of points: 1/d0 = d1 / (d0 d1). d <= 1 + 2^86 (2^23 grid
-        // steps of at most 1e6 in x), so d0 d1 only overflows where both d exceed 2^42
-        // (both terms below 2^-42 of the reflection's peak), and then both become 0.
-#pragma unroll
-        for (int j = 0; j < kAugPts; j += 2) {
-            const float d0 = fmaf(x[j], x[j], 1.f), d1 = fmaf(x[j + 1], x[j + 1], 1.f);
-            const float r = R.z * rcp_approx(d0 * d1);
-            acc[j] = fmaf(d1, r, acc[j]);
-            acc[j + 1] = fmaf(d0, r, acc[j + 1]);
-        }
+    for (int j = 0; j < kAugPts; j += 2) {
+        const float2 x = EXACT ? __ffma2_rn(make_float2(m0 + (float)j, m0 + (float)(j + 1)), s2, make_float2(R.y, R.y))
+                               : __ffma2_rn(make_float2((float)j, (float)(j + 1)), s2, make_float2(x0, x0));
+        const float2 d = __ffma2_rn(x, x, one);
+        const float r = R.z * rcp_approx(d.x * d.y);
+        acc[j / 2] = __ffma2_rn(d, make_float2(r, r), acc[j / 2]);
     }
 }
 
-// Gaussian part of the staged reflections that reach this warp's points (bit i
-// of near[i / 32], set where |x| at the warp's centre is below half the warp's
-// span in x plus sqrt(40)), in reflection order.
-__device__ __forceinline__ void aug_gauss(const float4* __restrict__ st, const uint32_t* __restrict__ near, int m,
-                                          float kf, float sc, float (&acc)[kAugPts])
+// Gaussian part of one reflection at a thread's points
+__device__ __forceinline__ void aug_gauss(const float4 R, float kf, float sc, float2 (&acc)[kAugPts / 2])
 {
-    for (int w = 0; w < (m + 31) >> 5; w++) {
-        uint32_t bits = near[w];
-        while (bits) {
-            const int i = 32 * w + __ffs(bits) - 1;
-            bits &= bits - 1;
-            const float4 R = st[i];
-            const float m0 = kf + R.x;
+    const float m0 = kf + R.x;
 #pragma unroll
-            for (int j = 0; j < kAugPts; j++) {
-                const float x = fmaf(m0 + (float)j, sc, R.y);
-                acc[j] = fmaf(R.w, ex2_approx(-x * x), acc[j]);
-            }
-        }
+    for (int j = 0; j < kAugPts; j += 2) {
+        const float2 x = __ffma2_rn(make_float2(m0 + (float)(j + 1), m0 + (float)j), make_float2(sc, sc), make_float2(R.y, R.y));
+        const float2 x2 = __fmul2_rn(x, x);
+        acc[j / 2] = __ffma2_rn(make_float2(R.w, R.w), make_float2(ex2_approx(-x2.x), ex2_approx(-x2.y)), acc[j / 2]);
     }
 }
 
-__global__ void __launch_bounds__(kAugThreads) k_aug_sum(const AugArgs a, int nblk)
+// The interpolation's nodes, as offsets from a warp's first point: Chebyshev-Lobatto points of [0, 255], rounded.
+static __constant__ int c_aug_node[kAugNodes] = {0, 3, 11, 24, 42, 64, 88, 114, 141, 167, 191, 213, 231, 244, 252, 255};
+static __device__ float4 g_aug_w[kAugBlock][kAugNodes / 4];  // weight of each node's sum at each point
+
+// Lagrange's basis on the nodes, in FP64
+__global__ void k_aug_init()
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= kAugBlock) return;
+    float w[kAugNodes];
+    for (int j = 0; j < kAugNodes; j++) {
+        double v = 1.0;
+        for (int i = 0; i < kAugNodes; i++)
+            if (i != j) v *= (double)(k - c_aug_node[i]) / (double)(c_aug_node[j] - c_aug_node[i]);
+        w[j] = (float)v;
+    }
+    for (int j = 0; j < kAugNodes / 4; j++) g_aug_w[k][j] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+}
+
+void init_aug_tables(cudaStream_t st) { k_aug_init<<<kAugBlock / 32, 32, 0, st>>>(); }
+
+// Staging order: the reflections of a chunk by the half block (128 points) that holds their 2theta, in the CTA's
+// 2 WARPS half blocks, one more on either side and the two outer rests, by a stable counting sort. The half blocks
+// of the reflections within kAugNear of a warp's middle are then four in a row: the near reflections are one range of
+// the chunk and the far ones the two ranges beside it, with no test per reflection.
+template <int WARPS>
+struct AugStage {
+    static constexpr int kThreads = 32 * WARPS, kChunk = 2 * kThreads, kGroups = kChunk / 32, kBins = 2 * WARPS + 4;
+    float4 rec[kChunk];
+    float2 b[kChunk / 2], ds[kChunk / 2], al[kChunk / 2];  // the far sum's operands, two reflections a load
+    int cnt[kGroups][kBins + 1];  // of each 32 reflections, per bin; then the place of their first
+    int start[kBins + 1];
+    float4 node[WARPS][kAugNodes / 4];
+    AugStruct cs;
+};
+
+// Resident warps: 32 per SM (48 would spill registers).
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 32 / WARPS) k_aug_sum(const AugArgs a, int nblk)
 {
     pdl_enter();
-    __shared__ float4 st[kAugChunk];
-    __shared__ uint32_t near[kAugWarps][kAugChunk / 32];  // reflections whose Gaussian reaches warp w
-    __shared__ AugStruct cs;
+    using S = AugStage<WARPS>;
+    __shared__ S sh;
     const int ib = blockIdx.x / nblk;
     const int s = a.aorder[ib];
-    const int k0 = (blockIdx.x - ib * nblk) * kAugSpan;
+    const int k0 = (blockIdx.x - ib * nblk) * WARPS * kAugBlock;
     if (threadIdx.x == 0) {
         bool bad;
-        cs = aug_struct(a, s, bad);
+        sh.cs = aug_struct(a, s, bad);
         if (bad && k0 == 0) {  // flagged once, by the structure's first CTA
             a.status[s] = XRD_EINVAL;
             atomicAdd((unsigned long long*)&a.totals[3], 1ull);
         }
     }
     __syncthreads();
-    const AugStruct c = cs;
-    const int kt = k0 + kAugPts * (int)threadIdx.x;  // this thread's first grid point
-    const float kf = (float)kt;
-    float acc[kAugPts];
+    const AugStruct& c = sh.cs;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4;
+    const int kw = k0 + kAugBlock * warp;   // this warp's first grid point
+    const int kt = kw + kAugPts * lane;     // this thread's first grid point
+    const float kf = (float)kt, sc = c.sc;
+    const bool lor = c.lor, gau = c.gau;
+    float2 acc[kAugPts / 2];
 #pragma unroll
-    for (int j = 0; j < kAugPts; j++) acc[j] = 0.f;
-    // warp w's points: k0 + 256 w .. k0 + 256 w + 255; none can reach x^2 < 40 when |x| at
-    // their centre exceeds half their span in x plus sqrt(40) (with margin)
-    const float kc0 = (float)k0 + 0.5f * (float)(32 * kAugPts - 1);
-    const float reach = fmaf(0.5f * (float)(32 * kAugPts - 1), c.sc, 6.5f) * 1.0001f;
-    const int warp = threadIdx.x >> 5;
+    for (int j = 0; j < kAugPts / 2; j++) acc[j] = make_float2(0.f, 0.f);
+    // none of the warp's points is within x^2 < 40 when |x| at their middle exceeds half their span in x plus sqrt(40)
+    // (with margin); where that can be beyond kAugNear the Gaussians of the whole chunk are tested
+    const float kc = (float)kw + 0.5f * (float)(kAugBlock - 1);
+    const float reach = fmaf(0.5f * (float)(kAugBlock - 1), sc, 6.5f) * 1.0001f;
+    const bool wide_gauss = reach >= (kAugNear - 2.f) * sc;
+    const float knode = (float)(kw + c_aug_node[lane & 15]);  // the two halves of the warp take two reflections each at a time
+    const float2 kn2 = make_float2(knode, knode), sc2 = make_float2(sc, sc), one = make_float2(1.f, 1.f);
+    float2 far = make_float2(0.f, 0.f);
     const int64_t base = c.n ? a.refl_off[s] : 0;
-    for (int c0 = 0; c0 < c.n; c0 += kAugChunk) {
-        const int m = min(kAugChunk, c.n - c0);
+    for (int c0 = 0; c0 < c.n; c0 += S::kChunk) {
+        const int m = min((int)S::kChunk, c.n - c0);
+        float4 R[2];
+        int bin[2], rank[2];
+        __syncthreads();  // the previous chunk is done with
+        for (int i = threadIdx.x; i < S::kGroups * (S::kBins + 1); i += S::kThreads) (&sh.cnt[0][0])[i] = 0;
         __syncthreads();
-        // whole warps stage 32 consecutive reflections each, so a ballot is one word of near[w]
-        for (int i = threadIdx.x; i < ((m + 31) & ~31); i += kAugThreads) {
-            float4 R = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i < m) {
-                R = aug_record(a, c, base + c0 + i);
-                st[i] = R;
-            }
 #pragma unroll
-            for (int w = 0; w < kAugWarps; w++) {
-                const float kcw = kc0 + (float)(32 * kAugPts * w);
-                const bool nr = i < m && c.gau && fabsf(fmaf(kcw + R.x, c.sc, R.y)) < reach;
-                const uint32_t bal = __ballot_sync(0xffffffffu, nr);
-                if ((threadIdx.x & 31) == 0) near[w][i >> 5] = bal;
+        for (int u = 0; u < 2; u++) {
+            const int g = warp + u * WARPS, i = 32 * g + lane;
+            R[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            bin[u] = S::kBins;  // past the end: no reflection
+            if (i < m) {
+                R[u] = aug_record(a, c, base + c0 + i);
+                bin[u] = min(max((((int)-R[u].x - k0) >> 7) + 2, 0), S::kBins - 1);
+            }
+            const unsigned peers = __match_any_sync(0xffffffffu, bin[u]);
+            rank[u] = __popc(peers & ((1u << lane) - 1u));
+            if (rank[u] == 0) sh.cnt[g][bin[u]] = __popc(peers);
+        }
+        __syncthreads();
+        for (int b = threadIdx.x; b <= S::kBins; b += S::kThreads) {  // places within the bin
+            int run = 0;
+            for (int g = 0; g < S::kGroups; g++) {
+                const int v = sh.cnt[g][b];
+                sh.cnt[g][b] = run;
+                run += v;
+            }
+            sh.start[b] = run;
+        }
+        __syncthreads();
+        if (warp == 0) {  // bins in their order
+            int carry = 0;
+            for (int b0 = 0; b0 <= S::kBins; b0 += 32) {
+                const int v = b0 + lane <= S::kBins ? sh.start[b0 + lane] : 0;
+                const int inc = warp_incl_scan(v);
+                if (b0 + lane <= S::kBins) sh.start[b0 + lane] = carry + inc - v;
+                carry += __shfl_sync(0xffffffffu, inc, 31);
             }
         }
         __syncthreads();
-        if (c.lor) {
-            if (c.sc <= 1.f) aug_lorentz<false>(st, m, kf, c.sc, acc);
-            else aug_lorentz<true>(st, m, kf, c.sc, acc);
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int at = sh.start[bin[u]] + sh.cnt[warp + u * WARPS][bin[u]] + rank[u];
+            sh.rec[at] = R[u];
+            ((float*)sh.b)[at] = R[u].x;
+            ((float*)sh.ds)[at] = R[u].y;
+            ((float*)sh.al)[at] = R[u].z;
         }
-        if (c.gau) aug_gauss(st, near[warp], m, kf, c.sc, acc);
+        __syncthreads();
+        if (kw >= a.n_pts) continue;  // uniform in the warp
+        const int n0 = sh.start[2 * warp + 1], n1 = sh.start[2 * warp + 5];  // the near reflections
+        if (lor) {
+            auto far_pair = [&](int i, float2 A) {  // reflections 2 i and 2 i + 1 at this lane's node
+                const float2 x = __ffma2_rn(__fadd2_rn(kn2, sh.b[i]), sc2, sh.ds[i]);
+                const float2 d = __ffma2_rn(x, x, one);
+                far = __ffma2_rn(A, make_float2(rcp_approx(d.x), rcp_approx(d.y)), far);
+            };
+            auto far_range = [&](int lo, int hi) {  // [lo, hi), the halves of the warp on alternate pairs
+                const int p0 = lo >> 1, p1 = (hi + 1) >> 1;  // pairs; the first and the last may reach past the range
+                for (int i = p0 + half; i < p1; i += 2) {
+                    float2 A = sh.al[i];
+                    if (2 * i < lo) A.x = 0.f;
+                    if (2 * i + 1 >= hi) A.y = 0.f;
+                    far_pair(i, A);
+                }
+            };
+            far_range(0, n0);
+            far_range(n1, m);
+            if (sc <= 1.f)
+                for (int i = n0; i < n1; i++) aug_lorentz<false>(sh.rec[i], kf, sc, acc);
+            else
+                for (int i = n0; i < n1; i++) aug_lorentz<true>(sh.rec[i], kf, sc, acc);
+        }
+        if (gau) {
+            const int g0 = wide_gauss ? 0 : n0, g1 = wide_gauss ? m : n1;
+            for (int i0 = g0; i0 < g1; i0 += 32) {
+                const int i = min(i0 + lane, g1 - 1);
+                unsigned b = __ballot_sync(0xffffffffu, i0 + lane < g1 && fabsf(fmaf(kc + sh.rec[i].x, sc, sh.rec[i].y)) < reach);
+                for (; b; b &= b - 1) aug_gauss(sh.rec[i0 + __ffs(b) - 1], kf, sc, acc);
+            }
+        }
     }
-    const bool noise = c.valid && a.noise_z != nullptr;
+    float f = far.x + far.y;
+    f += __shfl_xor_sync(0xffffffffu, f, 16);
+    if (lane < kAugNodes) ((float*)sh.node[warp])[lane] = f;
+    __syncwarp();
+    if (kw >= a.n_pts) return;
+    const bool valid = c.valid, noise = valid && a.noise_z != nullptr;
     float* __restrict__ yo = a.y + (int64_t)s * a.n_pts;
     const float* __restrict__ zo = noise ? a.noise_z + (int64_t)s * a.n_pts : nullptr;
 #pragma unroll
     for (int j = 0; j < kAugPts; j++) {
         const int k = kt + j;
         if (k >= a.n_pts) break;
-        float v = acc[j];
+        float v = j & 1 ? acc[j / 2].x : acc[j / 2].y;
+        if (lor) {
+            float f = 0.f;
+#pragma unroll
+            for (int q = 0; q < kAugNodes / 4; q++) {
+                const float4 w = g_aug_w[kAugPts * lane + j][q], n = sh.node[warp][q];
+                f = fmaf(w.x, n.x, fmaf(w.y, n.y, fmaf(w.z, n.z, fmaf(w.w, n.w, f))));
+            }
+            v += f;
+        }
         if (noise) v = fmaf(c.sig * sqrtf(fmaxf(v, 0.f)), zo[k], v);
-        yo[k] = c.valid ? v : 0.f;
+        yo[k] = valid ? v : 0.f;
     }
 }
 
+// CTAs of 8 warps (2048 points share a staging), or of 4 for shorter grids and where the wider ones would not fill the
+// SMs twice. 16 warps a CTA took the same time on 4096 points.
 void launch_aug(const AugArgs& a, cudaStream_t st)
 {
     if (a.n_struct <= 0) return;
-    const int nblk = (a.n_pts + kAugSpan - 1) / kAugSpan;
     launch_pdl(k_aug_order, 1, 1024, 0, st, a);
-    launch_pdl(k_aug_sum, (unsigned)((int64_t)a.n_struct * nblk), kAugThreads, 0, st, a, nblk);
+    const int wide = (a.n_pts + 8 * kAugBlock - 1) / (8 * kAugBlock), narrow = (a.n_pts + 4 * kAugBlock - 1) / (4 * kAugBlock);
+    if (a.n_pts > 4 * kAugBlock && (int64_t)a.n_struct * wide >= 2 * a.sms)
+        launch_pdl(k_aug_sum<8>, (unsigned)((int64_t)a.n_struct * wide), 256, 0, st, a, wide);
+    else launch_pdl(k_aug_sum<4>, (unsigned)((int64_t)a.n_struct * narrow), 128, 0, st, a, narrow);
 }
 
 }  // namespace xrd

@@ -256,7 +256,7 @@ struct GradArgs {
 };
 
 struct AugArgs {
-    int n_struct, n_pts;
+    int n_struct, n_pts, sms;
     double t0, dt, inv_dt;
     float l2h, l2l;  // lambda^2 / 4 as two floats
     const TTab* ttab;
@@ -308,6 +308,7 @@ const TTab* init_tables(cudaStream_t st);  // fills the 2-theta table, returns i
 size_t broaden_smem_bytes(int n_pts, int W);
 void launch_broaden(const GradArgs& a, cudaStream_t st);
 void launch_grad(const GradArgs& a, cudaStream_t st);
+void init_aug_tables(cudaStream_t st);  // fills the interpolation's table
 void launch_aug(const AugArgs& a, cudaStream_t st);   // per-reflection amplitudes, then the profile sums
 
 // handle accessors for entry points defined outside api.cu
