@@ -45,12 +45,13 @@ class BroadenedPattern(torch.autograd.Function):
         db = _device_batch(frac_c, B_c, lat_c, fixed)
         co = xrd.make_opts(opts, "fp32_phasefix")
         cg = xrd.make_grid(grid)
+        n = db.n_struct
+        # the call writes all of these; allocated before the counting, while the device still has work
+        y = torch.empty(n, int(grid.n_pts), dtype=torch.float32, device=frac.device)
+        status = torch.empty(n, dtype=torch.int32, device=frac.device)
+        totals = torch.empty(4, dtype=torch.int64, device=frac.device)
         sz = handle.query_sizes(db, co)
         ws = xrd.workspace(sz.ws_grad_bytes, frac.device)
-        n = db.n_struct
-        y = torch.empty(n, int(grid.n_pts), dtype=torch.float32, device=frac.device)
-        status = torch.zeros(n, dtype=torch.int32, device=frac.device)
-        totals = torch.zeros(4, dtype=torch.int64, device=frac.device)
         handle.pattern_broadened(db, co, cg, y, status, totals, ws)
         ctx.state = (db, co, cg, ws, handle, status)
         ctx.dtypes = (frac.dtype, B.dtype, lattice.dtype)

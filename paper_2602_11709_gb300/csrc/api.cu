@@ -30,7 +30,7 @@ struct xrd_handle {
     // stream beside the enumeration: forked by front, joined by order_done and atoms_done
     cudaStream_t side = nullptr;
     cudaEvent_t front = nullptr, order_done = nullptr, atoms_done = nullptr;
-    unsigned long long* wbuf = nullptr;  // device [3]: xrd_work_counts result
+    unsigned long long* wbuf = nullptr;  // device [8]: xrd_work_counts and xrd_query_sizes results
     xrd::RefineTables rtab{};            // tables of the accurate re-evaluation on the handle's device
     int8_t* pg = nullptr;                // device [kMaxPgOps][9]: the point group of the family mode
     int npg = 0;                         // its operations (0: families by permutation and sign)
@@ -187,8 +187,8 @@ LayoutG layout_grad(int64_t n, int64_t natoms, int zmax, int64_t R)
     L.tb = take(4 * R);
     L.td = take(4 * R);
     L.perm = take(4 * R);
-    L.U = take(4 * R);
-    L.V = take(4 * R);
+    L.U = take(8 * R);  // U, then V
+    L.V = L.U + 4 * R;
     L.aorder = take(4 * n);
     L.parts = take(scan_parts_bytes(n));
     L.oparts = take(xrd::order_parts_bytes(n));
@@ -464,14 +464,13 @@ int xrd_stage_times(xrd_handle* h, float* ms, int n)
     return m;
 }
 
-// Friedel-unique reflection count of every structure into cnt (host), on `st` (synchronised);
-// the scratch is the handle's own.
-static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cudaStream_t st,
-                             std::vector<int64_t>& cnt)
+// Friedel-unique reflection count of every structure (n_struct > 0), on `st` (synchronised): into cnt (host), or, with cnt NULL, their sum, largest and number
+// of tiles of tile_refl reflections into sums[0..2] (the counts stay on the device: their readback and the sums on the
+// host kept the GPU waiting). The scratch is the handle's own.
+static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cudaStream_t st, int64_t* cnt,
+                             int64_t* sums, int tile_refl)
 {
     const int64_t n = b->n_struct;
-    cnt.assign(n, 0);
-    if (n == 0) return XRD_OK;
     const size_t need = al(sizeof(xrd::Geo) * n) + al(8 * n) + al(16) + 2 * al(8 * kQueryParts);
     if (h->qbuf_bytes < need) {
         if (h->qbuf) cudaFree(h->qbuf);
@@ -497,8 +496,9 @@ static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* 
     a.enum_threads = 256;
     a.sms = h->sms;
     cudaMemsetAsync(a.enum_ctr, 0, 16, st);
-    xrd::launch_count_only(a, st);
-    cudaError_t e = cudaMemcpyAsync(cnt.data(), a.refl_cnt, 8 * n, cudaMemcpyDeviceToHost, st);
+    xrd::launch_count_only(a, cnt ? nullptr : h->wbuf + 4, tile_refl, st);
+    cudaError_t e = cnt ? cudaMemcpyAsync(cnt, a.refl_cnt, 8 * n, cudaMemcpyDeviceToHost, st)
+                        : cudaMemcpyAsync(sums, h->wbuf + 4, 24, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "reflection count");
     return XRD_OK;
@@ -512,11 +512,9 @@ int xrd_reflection_counts(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     if (rc) return rc;
     if ((rc = check_opts(h, o))) return rc;
     if (!counts && b->n_struct > 0) return fail(h, XRD_EINVAL, "counts is NULL");
+    if (b->n_struct == 0) return XRD_OK;
     DeviceGuard g(h->device);
-    std::vector<int64_t> cnt;
-    if ((rc = count_reflections(h, b, o, (cudaStream_t)stream, cnt))) return rc;
-    for (size_t i = 0; i < cnt.size(); i++) counts[i] = cnt[i];
-    return XRD_OK;
+    return count_reflections(h, b, o, (cudaStream_t)stream, counts, nullptr, 0);
 }
 
 int xrd_query_sizes(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, xrd_sizes* sizes, void* stream)
@@ -536,17 +534,12 @@ int xrd_query_sizes(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, xrd_si
         sizes->ws_grad_bytes = layout_grad(0, b->n_atoms, b->zmax, 0).total;
         return XRD_OK;
     }
-    std::vector<int64_t> cnt;
-    if ((rc = count_reflections(h, b, o, st, cnt))) return rc;
-    int64_t tot = 0, mx = 0, tiles = 0;
-    for (int64_t c : cnt) {
-        tot += c;
-        mx = c > mx ? c : mx;
-        tiles += (c + 32 * h->sf_rb - 1) / (32 * h->sf_rb);
-    }
+    int64_t sums[3] = {};  // reflections, the most of one structure, tiles
+    if ((rc = count_reflections(h, b, o, st, nullptr, sums, 32 * h->sf_rb))) return rc;
+    const int64_t tot = sums[0];
     sizes->n_refl = tot;
-    sizes->max_refl = mx;
-    sizes->n_tiles = tiles;
+    sizes->max_refl = sums[1];
+    sizes->n_tiles = sums[2];
     sizes->ws_bytes = layout(n, b->n_atoms, b->zmax, tot, h->npg > 0).total;
     sizes->ws_grad_bytes = layout_grad(n, b->n_atoms, b->zmax, tot).total;
     return XRD_OK;
@@ -1058,7 +1051,10 @@ static xrd::GradArgs grad_args(xrd_handle* h, const xrd_batch* b, const xrd_grid
     a.n_atoms = b->n_atoms;
     a.t0 = g->t0;
     a.dt = g->dt;
+    a.inv_dt = 1.0 / g->dt;
     a.sigma = sigma;
+    a.cg = (float)(1.4426950408889634f / (2.0 * sigma * sigma));
+    a.inv_s2 = (float)(1.0 / (sigma * sigma));
     a.l2d = o->lambda * o->lambda * 0.25;
     a.l2h = (float)a.l2d;
     a.l2l = (float)(a.l2d - (double)a.l2h);
@@ -1075,20 +1071,25 @@ static xrd::GradArgs grad_args(xrd_handle* h, const xrd_batch* b, const xrd_grid
     a.tb = (int*)(ws + L.tb);
     a.td = (float*)(ws + L.td);
     a.perm = (int*)(ws + L.perm);
+    a.sb = (int*)(ws + L.runs);      // no runs in this path
+    a.sda = (float2*)(ws + L.U);     // U and V: the backward pass's, free in the forward
     a.U = (float*)(ws + L.U);
     a.V = (float*)(ws + L.V);
     a.atom32 = (const xrd::Atom32*)(ws + L.atom32);
+    a.order = (const int*)(ws + L.order);
+    a.aorder = (const int*)(ws + L.aorder);
     a.coef32 = (const xrd::Coef32*)(ws + L.coef32);
     return a;
 }
 
 // Geometry and structure factors of the broadened and augmented paths, one
-// stream: grad = true keeps strided tiles and stores F, dF/ds^2 and I for the
-// adjoint; grad = false runs the tuned pattern shape and stores I only.
+// stream: with gr, strided tiles, and F, dF/ds^2, I and each reflection's grid cell are stored for
+// the profile and the adjoint; without, the tuned pattern shape, and I only.
 static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const LayoutG& L, char* ws,
-                         int64_t cap_refl, int32_t* status, int64_t* totals, cudaStream_t st, bool grad)
+                          int64_t cap_refl, int32_t* status, int64_t* totals, cudaStream_t st, const xrd::GradArgs* gr)
 {
     const int64_t n = b->n_struct;
+    const bool grad = gr != nullptr;
     xrd::GeomArgs ga{};
     ga.n_struct = (int)n;
     ga.zmax = b->zmax;
@@ -1121,7 +1122,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.tile_off = (int*)(ws + L.tile_off);
     ga.order = (int*)(ws + L.order);
     ga.atom_bad = (int*)(ws + L.atom_bad);
-    ga.atoms_set_geo = 1;  // atoms run before the enumeration here
+    ga.atoms_set_geo = 1;  // a structure with an invalid atom has no reflections here
     ga.tile_tab = (int2*)(ws + L.tile_tab);
     ga.abort_flag = (int*)(ws + L.flags);
     ga.enum_ctr = ga.abort_flag + 26;
@@ -1135,12 +1136,17 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.parts = (long long*)(ws + L.parts);
     ga.oparts = xrd::order_parts_bytes(n) ? (int*)(ws + L.oparts) : nullptr;
     cudaMemsetAsync(ws + L.flags, 0, kFlagBytes, st);
-    xrd::launch_prep(ga, st, false);
-    xrd::launch_coef(ga, st, true);
-    xrd::launch_atoms(ga, st, true);
-    xrd::launch_order(ga, st, true);
-    xrd::launch_count(ga, st, true, false);
-    xrd::launch_scan_refl(ga, st, true);
+    if (n > 0 && xrd::front_fused((int)n, b->n_atoms)) {
+        xrd::launch_front(ga, st);
+        xrd::launch_count(ga, st, true, true);  // structures with an invalid atom lose their status there
+    } else {
+        xrd::launch_prep(ga, st, false);
+        xrd::launch_coef(ga, st, true);
+        xrd::launch_atoms(ga, st, true);
+        xrd::launch_order(ga, st, true);
+        xrd::launch_count(ga, st, true, false);
+        xrd::launch_scan_refl(ga, st, true);
+    }
     xrd::launch_emit(ga, st, true);
     xrd::SfArgs sa{};
     sa.n_struct = (int)n;
@@ -1167,9 +1173,11 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     sa.atomx = ga.atomx;
     sa.q = ga.q;
     sa.key = ga.key;
+    sa.aorder = (int*)(ws + L.aorder);
     if (grad) {
         sa.Fx = (float4*)(ws + L.Fx);
         sa.Ig = (float*)(ws + L.Ig);
+        sa.cell = xrd::CellArgs{gr->t0, gr->dt, gr->inv_dt, gr->l2h, gr->l2l, gr->ttab, gr->n_pts, gr->W, gr->tb, gr->td};
     } else {
         sa.If = (float*)(ws + L.Ig);
     }
@@ -1197,8 +1205,8 @@ int xrd_pattern_broadened(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
     const LayoutG L = layout_grad(n, b->n_atoms, b->zmax, cap_refl);
-    profile_front(h, b, o, L, ws, cap_refl, status, totals, st, true);
     xrd::GradArgs gr = grad_args(h, b, grid, W, sigma, o, L, ws);
+    profile_front(h, b, o, L, ws, cap_refl, status, totals, st, &gr);
     gr.y = y;
     xrd::launch_broaden(gr, st);
     cudaError_t e = cudaGetLastError();
@@ -1239,7 +1247,7 @@ int xrd_pattern_augmented(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
     const LayoutG L = layout_grad(n, b->n_atoms, b->zmax, cap_refl);
-    profile_front(h, b, o, L, ws, cap_refl, status, totals, st, false);
+    profile_front(h, b, o, L, ws, cap_refl, status, totals, st, nullptr);
     xrd::AugArgs a{};
     a.n_struct = (int)n;
     a.sms = h->sms;
@@ -1263,7 +1271,7 @@ int xrd_pattern_augmented(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     a.po_r = aug->po_r;
     a.noise_z = aug->noise_z;
     a.noise_sigma = aug->noise_sigma;
-    a.aorder = (int*)(ws + L.aorder);
+    a.aorder = (const int*)(ws + L.aorder);
     a.status = status;
     a.totals = totals;
     a.y = y;

@@ -7,7 +7,7 @@
 //   PV(u) = eta (2 / (pi w)) / (1 + x^2) + (1 - eta) (2 / w) sqrt(ln 2 / pi) 2^(-x^2),  x = 2 u / w
 //   then y_k += sigma sqrt(max(y_k, 0)) z_k.
 //
-// k_aug_order lists the structures by reflection count, largest first.
+// The structures come in order of their reflection count, largest first (aorder, by the structure-factor kernel).
 // k_aug_sum gives each warp 256 grid points of one structure (kAugPts
 // consecutive points per thread) and streams all of the structure's reflections
 // through shared memory, turning each into a record as it is staged: its grid
@@ -41,39 +41,12 @@ constexpr int kAugPts = 8;                       // consecutive grid points per 
 constexpr int kAugBlock = 32 * kAugPts;          // points of a warp
 constexpr int kAugNodes = 16;                    // of them, the interpolation's
 constexpr float kAugNear = 256.f;                // grid points from the warp's middle within which every point is summed
-constexpr int kAugBuckets = 128;                 // reflection-count buckets of the largest-first order
 
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-// Structures by reflection count, largest first (buckets of a quarter octave),
-// so that the CTAs of the largest structures start first. One CTA.
-__global__ void __launch_bounds__(1024) k_aug_order(const AugArgs a)
-{
-    pdl_enter();
-    __shared__ int cnt[kAugBuckets];
-    for (int i = threadIdx.x; i < kAugBuckets; i += blockDim.x) cnt[i] = 0;
-    __syncthreads();
-    auto bucket = [&](int s) {
-        const int64_t R = a.refl_off[s + 1] - a.refl_off[s];
-        return R <= 0 ? 0 : min(kAugBuckets - 1, 1 + (int)(4.f * log2f((float)R)));
-    };
-    for (int s = threadIdx.x; s < a.n_struct; s += blockDim.x) atomicAdd(&cnt[bucket(s)], 1);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int b = kAugBuckets - 1; b >= 0; b--) {
-            const int c = cnt[b];
-            cnt[b] = acc;
-            acc += c;
-        }
-    }
-    __syncthreads();
-    for (int s = threadIdx.x; s < a.n_struct; s += blockDim.x) a.aorder[atomicAdd(&cnt[bucket(s)], 1)] = s;
 }
 
 // Per-structure constants of the profile sum (all zero for a structure that is
@@ -193,22 +166,20 @@ __device__ __forceinline__ void aug_gauss(const float4 R, float kf, float sc, fl
 static __constant__ int c_aug_node[kAugNodes] = {0, 3, 11, 24, 42, 64, 88, 114, 141, 167, 191, 213, 231, 244, 252, 255};
 static __device__ float4 g_aug_w[kAugBlock][kAugNodes / 4];  // weight of each node's sum at each point
 
-// Lagrange's basis on the nodes, in FP64
+// Lagrange's basis on the nodes, in FP64: thread j of block k the weight of node j at point k
 __global__ void k_aug_init()
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= kAugBlock) return;
-    float w[kAugNodes];
-    for (int j = 0; j < kAugNodes; j++) {
-        double v = 1.0;
-        for (int i = 0; i < kAugNodes; i++)
-            if (i != j) v *= (double)(k - c_aug_node[i]) / (double)(c_aug_node[j] - c_aug_node[i]);
-        w[j] = (float)v;
-    }
-    for (int j = 0; j < kAugNodes / 4; j++) g_aug_w[k][j] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+    const int k = blockIdx.x, j = threadIdx.x;
+    double num = 1.0, den = 1.0;
+    for (int i = 0; i < kAugNodes; i++)
+        if (i != j) {
+            num *= (double)(k - c_aug_node[i]);
+            den *= (double)(c_aug_node[j] - c_aug_node[i]);
+        }
+    ((float*)g_aug_w[k])[j] = (float)(num / den);
 }
 
-void init_aug_tables(cudaStream_t st) { k_aug_init<<<kAugBlock / 32, 32, 0, st>>>(); }
+void init_aug_tables(cudaStream_t st) { k_aug_init<<<kAugBlock, kAugNodes, 0, st>>>(); }
 
 // Staging order: the reflections of a chunk by the half block (128 points) that holds their 2theta, in the CTA's
 // 2 WARPS half blocks, one more on either side and the two outer rests, by a stable counting sort. The half blocks
@@ -377,7 +348,6 @@ __global__ void __launch_bounds__(32 * WARPS, 32 / WARPS) k_aug_sum(const AugArg
 void launch_aug(const AugArgs& a, cudaStream_t st)
 {
     if (a.n_struct <= 0) return;
-    launch_pdl(k_aug_order, 1, 1024, 0, st, a);
     const int wide = (a.n_pts + 8 * kAugBlock - 1) / (8 * kAugBlock), narrow = (a.n_pts + 4 * kAugBlock - 1) / (4 * kAugBlock);
     if (a.n_pts > 4 * kAugBlock && (int64_t)a.n_struct * wide >= 2 * a.sms)
         launch_pdl(k_aug_sum<8>, (unsigned)((int64_t)a.n_struct * wide), 256, 0, st, a, wide);

@@ -525,10 +525,11 @@ __device__ __forceinline__ EnumItems enum_items(int n_struct, const int* part_ct
     return EnumItems{min(*part_ctr, part_cap), n_struct, n_struct >= kWideBatch ? kClaimWide : 1, ctr};
 }
 
-// The structure and the columns [c0, c1) of an item; false where there is nothing to do (a structure that its
+// The structure and the columns [c0, c1) of an item (none where bad says so); false where there is nothing to do (a structure that its
 // parts cover, a slot of a structure that found no room)
 __device__ __forceinline__ bool enum_item(const Geo* __restrict__ geo, const int2* __restrict__ part_tab, int nparts,
-                                          int part_cols, int item, int& s, int& part, Geo& g, int& c0, int& c1)
+                                          int part_cols, int item, int& s, int& part, Geo& g, int& c0, int& c1,
+                                          const int* __restrict__ bad = nullptr)
 {
     part = -1;
     s = item - nparts;
@@ -548,6 +549,7 @@ __device__ __forceinline__ bool enum_item(const Geo* __restrict__ geo, const int
     } else if (g.pbase >= 0) {
         return false;
     }
+    if (bad && bad[s]) c1 = c0;  // a structure with an invalid atom has no reflections
     return true;
 }
 
@@ -746,6 +748,8 @@ struct ScanArgs {
     int64_t* totals;
     int32_t* status;
     unsigned long long* work;
+    const int* bad;  // structures with an invalid atom become invalid here (or nullptr)
+    unsigned long long* sums;  // not nullptr: no scan, but the counts' sum, largest and tiles into sums[0..2]
 };
 struct ScanShared {
     long long ws[33];
@@ -754,7 +758,7 @@ struct ScanShared {
 
 // buf: kScanItems * blockDim long longs of shared memory. The counts are read past the L1 cache: the CTA that runs
 // this may be one of the kernel that wrote them.
-__device__ __forceinline__ void scan_refl_block(const int64_t* cnt, const Geo* __restrict__ geo, int n,
+__device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restrict__ geo, int n,
                                                 const ScanArgs& sa, ScanShared& sh, long long* buf)
 {
     const int64_t* const run_cnt = sa.run_cnt;
@@ -782,6 +786,10 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, const Geo* _
             const int i = base + u * nt + tid;
             v[u] = i < n ? __ldcg((const long long*)cnt + i) : 0;
             st[u] = i < n ? geo[i].status : XRD_OK;
+            if (i < n && sa.bad && sa.bad[i]) {
+                st[u] = XRD_EINVAL;
+                geo[i].status = XRD_EINVAL;
+            }
         }
         chunk_scan<kScanItems>(v, buf, ws, &tot);
 #pragma unroll
@@ -851,8 +859,8 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, const Geo* _
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __restrict__ cnt,
-                                                            const Geo* __restrict__ geo, int n, const ScanArgs sa)
+__global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __restrict__ cnt, Geo* __restrict__ geo,
+                                                            int n, const ScanArgs sa)
 {
     pdl_enter();
     __shared__ ScanShared sh;
@@ -863,13 +871,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __res
 // Reflection (and, with RUNS, run) counts per structure, and of every part (k_prep has zeroed the counts of a
 // structure in parts). ctr: zero at launch. done: CTAs finished (zero at launch), or null: no scan.
 template <bool RUNS>
-__global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict__ geo, int n_struct, double r2min,
+__global__ void __launch_bounds__(kEnumMaxThreads) k_count(Geo* geo, int n_struct, double r2min,
                                                            double r2max, float r2minf, float r2maxf, int rb,
                                                            int64_t* __restrict__ cnt, int64_t* __restrict__ run_cnt,
                                                            int* __restrict__ ctr, const int* __restrict__ part_ctr,
                                                            const int2* __restrict__ part_tab,
                                                            int2* __restrict__ part_cnt, int part_cap, int part_cols,
-                                                           const ScanArgs scan, int* __restrict__ done)
+                                                           const ScanArgs scan, int* __restrict__ done,
+                                                           const int* __restrict__ bad)
 {
     pdl_enter();
     const int lane = threadIdx.x & 31;
@@ -881,7 +890,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict
         for (int it = first; it < first + m; it++) {
             int s, part, c0, c1;
             Geo g;
-            if (!enum_item(geo, part_tab, items.nparts, part_cols, it, s, part, g, c0, c1)) continue;
+            if (!enum_item(geo, part_tab, items.nparts, part_cols, it, s, part, g, c0, c1, bad)) continue;
             int local = 0, local_runs = 0;
             for (int c = c0 + lane; c < c1; c += 32) {
                 int h, k, n, nr;
@@ -903,7 +912,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict
         }
     }
     if (!done) return;
-    // the CTA that finishes last scans the counts (a launch less in a small batch's chain)
+    // the CTA that finishes last scans the counts (a launch less in a small batch's chain), or adds them up
     extern __shared__ __align__(16) long long scan_buf[];
     __shared__ ScanShared sh;
     __shared__ int last;
@@ -913,6 +922,22 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_count(const Geo* __restrict
     __syncthreads();
     if (!last) return;
     __threadfence();
+    if (scan.sums) {
+        long long sum = 0, most = 0, tiles = 0, t;
+        for (int i = threadIdx.x; i < n_struct; i += blockDim.x) {
+            const long long c = __ldcg((const long long*)cnt + i);
+            sum += c;
+            most = max(most, c);
+            tiles += (c + scan.tile_refl - 1) / scan.tile_refl;
+        }
+        block_prefix_ll(sum, sh.ws, &t);
+        if (threadIdx.x == 0) scan.sums[0] = t;
+        block_prefix_ll(tiles, sh.ws, &t);
+        if (threadIdx.x == 0) scan.sums[2] = t;
+        const unsigned long long m = block_max_u64(most, (unsigned long long*)sh.ws);
+        if (threadIdx.x == 0) scan.sums[1] = m;
+        return;
+    }
     scan_refl_block(cnt, geo, n_struct, scan, sh, scan_buf);
 }
 
@@ -1325,33 +1350,39 @@ static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
 static ScanArgs scan_args(const GeomArgs& a)
 {
     return ScanArgs{a.run_cnt, a.runs_mode ? 0 : 32 * a.rb, a.cap_refl, a.refl_off, a.tile_off, a.order, a.cls_list,
-                    a.abort_flag, a.totals, a.status, a.work};
+                    a.abort_flag, a.totals, a.status, a.work, a.atoms_set_geo ? a.atom_bad : nullptr, nullptr};
 }
 
-static void count_launch(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan)
+static void count_launch(const GeomArgs& a, const ScanArgs& sa, cudaStream_t st, bool pdl, bool last)
 {
     const auto k = a.runs_mode ? k_count<true> : k_count<false>;
-    const size_t smem = scan ? sizeof(long long) * kScanItems * (size_t)a.enum_threads : 0;
+    const size_t smem = last && !sa.sums ? sizeof(long long) * kScanItems * (size_t)a.enum_threads : 0;
     const int grid = enum_grid(a, (const void*)k, smem);
     auto go = [&](auto launch) {
         launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, a.refl_cnt,
                a.run_cnt, a.enum_ctr, (const int*)(a.enum_ctr + kPartCtr), (const int2*)a.part_tab, a.part_cnt,
-               a.part_cap, enum_part_cols(a.n_struct), scan_args(a), scan ? a.enum_ctr + kDoneCtr : (int*)nullptr);
+               a.part_cap, enum_part_cols(a.n_struct), sa, last ? a.enum_ctr + kDoneCtr : (int*)nullptr, sa.bad);
     };
     if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });
     else go([&](auto... v) { k<<<grid, a.enum_threads, smem, st>>>(v...); });
 }
 
-void launch_count_only(const GeomArgs& a, cudaStream_t st)
+void launch_count_only(const GeomArgs& a, unsigned long long* sums, int tile_refl, cudaStream_t st)
 {
     if (a.n_struct <= 0) return;
     prep_launch(false, a, st);
-    count_launch(a, st, true, false);
+    ScanArgs sa{};
+    sa.sums = sums;
+    sa.tile_refl = tile_refl;
+    count_launch(a, sa, st, true, sums != nullptr);
 }
 
 void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan)
 {
-    if (a.n_struct > 0) count_launch(a, st, pdl, scan);
+    if (a.n_struct <= 0) return;
+    ScanArgs sa = scan_args(a);
+    if (!scan) sa.bad = nullptr;  // k_atoms has marked them
+    count_launch(a, sa, st, pdl, scan);
 }
 
 int scan_chunks(int n) { return (n + kScanItems * kScanThreads - 1) / (kScanItems * kScanThreads); }

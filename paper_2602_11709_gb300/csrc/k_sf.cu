@@ -19,6 +19,8 @@
 // fixed point (XRD_FP32_PHASEFIX), or in 53-bit fixed point, the resolution of an FP64 phase (XRD_FP32_PHASE64: three
 // more integer products a term; formed in FP64, four operations a term at 1.7 a clock and SM, it made the kernel take
 // 471 us on 1024 cells of 1 to 64 atoms; now about 80 us). The XRD_FP64 variant is k_sf64.cu.
+#include <climits>
+
 #include "xrd_internal.cuh"
 #include "xrd_launch.h"
 
@@ -104,6 +106,27 @@ __device__ __forceinline__ float2 fprime_of(const CoefPair& c, float2 s2)
 // Signed low word of a 64-bit fixed-point coordinate, rounded to its upper 21 bits: with |h| <= 511 the sum of
 // three index times low-word products stays below 2^31.
 __device__ __forceinline__ int low21(int32_t lo) { return (lo >> 11) + ((lo >> 10) & 1); }
+
+// x / d correctly rounded, inv = 1 / d correctly rounded: Markstein's theorem (IBM J. Res. Dev. 34, 1990) makes one FMA
+// step from a quotient within an ulp the rounded one; the first step gets it there. Five FP64 operations.
+__device__ __forceinline__ double div_by(double x, double d, double inv)
+{
+    const double q0 = __dmul_rn(x, inv);
+    const double q1 = __fma_rn(__fma_rn(-q0, d, x), inv, q0);
+    return __fma_rn(__fma_rn(-q1, d, x), inv, q1);
+}
+
+// Grid cell b of 2theta and the position d within it, for the broadened profile (b = INT_MIN: no grid point within the
+// window). In this kernel, whose FP64 unit is idle.
+__device__ __forceinline__ void place(const CellArgs& c, int64_t r, double q)
+{
+    const double T = two_theta_q(q, c.l2h, c.l2l, c.ttab);
+    const double pos = div_by(T - c.t0, c.dt, c.inv_dt);
+    const double fb = floor(pos);
+    const bool off = fb < (double)(-c.W - 1) || fb > (double)(c.n_pts + c.W);
+    c.tb[r] = off ? INT_MIN : (int)fb;
+    c.td[r] = off ? 0.f : (float)(pos - fb);
+}
 
 // The reflections of one lane in a tile: RUNS: one run of `len` reflections
 // consecutive in l from `first` (step 1); otherwise up to RB reflections from
@@ -298,6 +321,7 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
         if (GRAD) {
             a.Fx[r] = make_float4(fr, fi, half(Gr, i), half(Gi, i));
             a.Ig[r] = I;
+            place(a.cell, r, a.q[r]);
         } else {
             a.If[r] = I;
             if (ACC && a.Eb) {
@@ -313,6 +337,32 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
         }
     }
     return imax;
+}
+
+// Structures by reflection count, largest first (buckets of a quarter octave), by one CTA beside the tiles of the
+// others: the profile kernels that follow give every structure a CTA and start with the largest. cnt: kCountBuckets
+// ints of shared memory. The order within a bucket is arbitrary; nothing but the load balance depends on it.
+constexpr int kCountBuckets = 128;
+__device__ void order_by_count(const SfArgs& a, int* cnt)
+{
+    for (int i = threadIdx.x; i < kCountBuckets; i += blockDim.x) cnt[i] = 0;
+    __syncthreads();
+    auto bucket = [&](int s) {
+        const int64_t R = a.refl_off[s + 1] - a.refl_off[s];
+        return R <= 0 ? 0 : min(kCountBuckets - 1, 1 + (int)(4.f * log2f((float)R)));
+    };
+    for (int s = threadIdx.x; s < a.n_struct; s += blockDim.x) atomicAdd(&cnt[bucket(s)], 1);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int acc = 0;
+        for (int b = kCountBuckets - 1; b >= 0; b--) {
+            const int c = cnt[b];
+            cnt[b] = acc;
+            acc += c;
+        }
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < a.n_struct; s += blockDim.x) a.aorder[atomicAdd(&cnt[bucket(s)], 1)] = s;
 }
 
 // Persistent CTAs; every warp takes tiles of 32 runs (one per lane) from a
@@ -334,6 +384,10 @@ __global__ void __launch_bounds__(32 * WARPS,
     __shared__ float2 sstep[RUNS ? WARPS : 1][RUNS ? kSfChunk : 1];
     __shared__ int4 slo[PREC == XRD_FP32_PHASE64 ? WARPS : 1][PREC == XRD_FP32_PHASE64 ? kSfChunk : 1];
     extern __shared__ CoefPair scoef[];  // [zmax + 1]
+    if (a.aorder && blockIdx.x == gridDim.x - 1) {
+        __shared__ int cnt[kCountBuckets];
+        order_by_count(a, cnt);
+    }
     if (*a.abort_flag) return;
     const int ntiles = a.tile_off[a.n_struct];
     if ((int)blockIdx.x >= ntiles) return;  // the CTAs before this one already have a tile each

@@ -42,11 +42,6 @@ __device__ __forceinline__ HD hd_mul(HD a, HD b)
     const double p = __dmul_rn(a.h, b.h);
     return hd_fast(p, __dadd_rn(__fma_rn(a.h, b.h, -p), __fma_rn(a.h, b.l, __dmul_rn(a.l, b.h))));
 }
-__device__ __forceinline__ HD hd_div(HD a, double n)  // n a small integer
-{
-    const double h = __ddiv_rn(a.h, n);
-    return hd_fast(h, __ddiv_rn(__dadd_rn(__fma_rn(-h, n, a.h), a.l), n));
-}
 // a >= 0 in units of 2^-bits, rounded
 __device__ uint64_t hd_fixed(HD a, int bits)
 {
@@ -56,11 +51,18 @@ __device__ uint64_t hd_fixed(HD a, int bits)
 
 __global__ void k_fx_init()
 {
+    constexpr int kTerms = 30;
+    __shared__ HD inv[kTerms + 1];  // 1 / k
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (threadIdx.x < kTerms) {
+        const double k = threadIdx.x + 1.0, h = __ddiv_rn(1.0, k);
+        inv[threadIdx.x + 1] = HD{h, __ddiv_rn(__fma_rn(-h, k, 1.0), k)};
+    }
+    __syncthreads();
     if (i < kFxExpN) {  // 2^(-i / kFxExpN) by the series of exp
         const HD x = hd_mul(HD{0.6931471805599453, 2.3190468138462996e-17}, HD{-i / (double)kFxExpN, 0.0});
         HD t{1.0, 0.0}, s = t;
-        for (int k = 1; k <= 24; k++) s = hd_add(s, t = hd_div(hd_mul(t, x), k));
+        for (int k = 1; k <= 24; k++) s = hd_add(s, t = hd_mul(hd_mul(t, x), inv[k]));
         g_fx_exp[i] = i ? hd_fixed(s, 64) : ~0ull;
         return;
     }
@@ -68,8 +70,8 @@ __global__ void k_fx_init()
     if (j > kFxScN) return;
     const HD x = hd_mul(HD{1.5707963267948966, 6.123233995736766e-17}, HD{j / (double)kFxScN, 0.0});
     HD t{1.0, 0.0}, c = t, s{0.0, 0.0};
-    for (int k = 1; k <= 30; k++) {
-        t = hd_div(hd_mul(t, x), k);
+    for (int k = 1; k <= kTerms; k++) {
+        t = hd_mul(hd_mul(t, x), inv[k]);
         const HD v = k & 2 ? HD{-t.h, -t.l} : t;
         if (k & 1) s = hd_add(s, v);
         else c = hd_add(c, v);

@@ -37,7 +37,8 @@ struct GeomArgs {
     int* order;      // [n_struct] structures by atom count, largest first
     int2* tile_tab;  // [tiles] (structure, first reflection) of each structure-factor tile
     int* atom_bad;   // [n_struct] 1 where an atom of the structure is invalid
-    int atoms_set_geo;  // k_atoms also marks such structures invalid in geo (only when it runs before k_count)
+    int atoms_set_geo;  // such structures become invalid in geo before the enumeration: by k_atoms, or after
+                        // k_front by k_count
     int* cls_list;   // [kPostClasses][n_struct] post-processing size classes (nullptr: not built)
     int* abort_flag; // flags[0]; flags[1] output abort, flags[2] tile queue, flags[4..6] flat-pass grid barrier, flags[26..28] enumeration
                      // claims, flags[kFlagClsCnt + c] class counts, flags[kFlagClsNext + c] class work counters
@@ -69,6 +70,16 @@ struct EnumParts {
     int64_t* run_cnt;  // (or nullptr)
 };
 
+// Gradient path: the grid on which the structure-factor kernel places each reflection (GradArgs' members)
+struct CellArgs {
+    double t0, dt, inv_dt;
+    float l2h, l2l;
+    const TTab* ttab;
+    int n_pts, W;
+    int* tb;
+    float* td;
+};
+
 struct SfArgs {
     int n_struct, precision, tile, grid, zmax;
     int rb, warps;  // launch shape: reflections per lane (2 or 4), warps per CTA (1, 2 or 4)
@@ -94,11 +105,13 @@ struct SfArgs {
     float2* F;   // optional per-reflection F (nullptr: not stored)
     float4* Fx;  // gradient path: (Re F, Im F, Re dF/ds^2, Im dF/ds^2) per reflection (nullptr otherwise)
     float* Ig;   // gradient path: |F|^2 LP per reflection
+    CellArgs cell;  // gradient path
     float* Eb;   // FP32 pattern variants: bound of the intensity's rounding error per reflection (or nullptr):
                  // LP dF (2 |F| + dF) with dF = eps_k sqrt(sum_j a_j^2), a_j = occ DW max(|f|, Z)
     int* Es;     // the structure of each reflection whose bound exceeds tau times its intensity (others: unset)
     float eps_k; // K times the relative error of one FP32 term (the bound of |dF| / sqrt(sum a_j^2))
     float tau;
+    int* aorder;     // [n_struct] structures by reflection count, largest first, for the profile kernels (or nullptr)
     unsigned* imax;  // FP32 pattern variants: [n_struct] bits of the largest reflection intensity (zeroed by k_prep)
 };
 
@@ -229,7 +242,8 @@ struct CompactArgs {
 struct GradArgs {
     int n_struct, n_pts, W;
     int64_t n_atoms;
-    double t0, dt, sigma, l2d;
+    double t0, dt, inv_dt, sigma, l2d;
+    float cg, inv_s2;  // log2(e) / (2 sigma^2) and 1 / sigma^2, formed in FP64 (a division per thread costs ten FP64 operations)
     float l2h, l2l;  // lambda^2 / 4 as two floats
     const TTab* ttab;
     const Geo* geo;
@@ -243,13 +257,17 @@ struct GradArgs {
     const float* Ig;   // |F|^2 LP
     int* tb;           // grid cell of each reflection's 2theta (INT_MIN: off the grid)
     float* td;         // position within the cell, [0, 1)
-    int* perm;         // per-reflection scratch
+    int* perm;         // per-reflection scratch of the forward pass: the order by cell, then
+    int* sb;           // the cell of each reflection in that order
+    float2* sda;       // and its position within the cell and twice its intensity
     float* y;          // [n_struct][n_pts]
     const float* dLdy; // [n_struct][n_pts]
     float* U;          // dL/dI LP Re F per reflection
     float* V;          // dL/dI LP Im F
     const Atom32* atom32;
     const Coef32* coef32;
+    const int* order;   // [n_struct] structures by atom count, largest first
+    const int* aorder;  // and by reflection count
     float* d_frac;
     float* d_B;
     float* d_lat;
@@ -273,7 +291,7 @@ struct AugArgs {
     const double* po_r;
     const float* noise_z;
     const double* noise_sigma;
-    int* aorder; // [n_struct] structures by reflection count, largest first
+    const int* aorder; // [n_struct] structures by reflection count, largest first
     int32_t* status;
     int64_t* totals;
     float* y;    // [n_struct][n_pts]
@@ -289,7 +307,8 @@ void launch_atoms(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_order(const GeomArgs& a, cudaStream_t st, bool pdl);
 size_t order_parts_bytes(int64_t n);  // bytes of GeomArgs::oparts for n structures (0: one-block order)
 void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan);  // scan: and launch_scan_refl's work
-void launch_count_only(const GeomArgs& a, cudaStream_t st);
+// counts only; with sums, also their sum, largest and tiles of tile_refl into sums[0..2]
+void launch_count_only(const GeomArgs& a, unsigned long long* sums, int tile_refl, cudaStream_t st);
 void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st);  // out: device [3], zeroed
 void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl);
