@@ -642,6 +642,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     sa.astep = ga.astep;
     sa.grid = h->sms;
     sa.lambda = o->lambda;
+    sa.l2f = (float)(o->lambda * o->lambda * 0.25);
     sa.atom_off = b->atom_off;
     sa.refl_off = ga.refl_off;
     sa.tile_off = ga.tile_off;
@@ -1161,6 +1162,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     sa.astep = ga.astep;
     sa.grid = h->sms;
     sa.lambda = o->lambda;
+    sa.l2f = (float)(o->lambda * o->lambda * 0.25);
     sa.atom_off = b->atom_off;
     sa.refl_off = ga.refl_off;
     sa.tile_off = ga.tile_off;

@@ -446,13 +446,14 @@ __device__ __forceinline__ void column_hk(const Geo& g, int c, int& h, int& k)
     k = r % nk - g.K;
 }
 
-// Runs: the structure-factor kernel gives each lane a run of at most rb
+// Runs: the structure-factor kernel gives each lane a run of at most kRunLen
 // reflections that are consecutive in l within one column, so that it can step
 // the phase factor exp(2 pi i g.x) from l to l + 1 by one complex rotation.
-// Each of a column's (at most two) contiguous parts is cut into runs of rb
+// Each of a column's (at most two) contiguous parts is cut into runs of kRunLen
 // from its first l, the last one shorter. Run entries: (first reflection
 // within the structure) << 3 | length.
-__device__ __forceinline__ int runs_of(int n, int rb) { return (n + rb - 1) / rb; }
+constexpr int kRunLen = 4;
+__device__ __forceinline__ int runs_of(int n) { return (n + kRunLen - 1) / kRunLen; }
 
 // The exact comparison of a candidate within the FP32 error bound of a sphere
 // surface, kept out of line so that the rare FP64 evaluation is a branch, not
@@ -465,7 +466,7 @@ __device__ __noinline__ int q_side_exact(const double* gs, int h, int k, int l, 
 
 // Reflections and runs of column c.
 __device__ __forceinline__ ColSpan column_counts(const Geo& g, const double* gsg, int c, double r2min, double r2max,
-                                                 float r2minf, float r2maxf, int rb, bool runs, int& h, int& k, int& n,
+                                                 float r2minf, float r2maxf, bool runs, int& h, int& k, int& n,
                                                  int& nr)
 {
     column_hk(g, c, h, k);
@@ -474,7 +475,7 @@ __device__ __forceinline__ ColSpan column_counts(const Geo& g, const double* gsg
     nr = 0;
     if (runs) {
         const int n1 = sp.first_part();
-        nr = runs_of(n1, rb) + runs_of(n - n1, rb);
+        nr = runs_of(n1) + runs_of(n - n1);
     }
     return sp;
 }
@@ -491,13 +492,14 @@ __device__ __forceinline__ int warp_sum_int(int v)
 // room for part_cap parts; a structure that finds no room, or has fewer columns, is one item. A warp takes a part in
 // about the time of part_cols / 32 steps of 32 columns, so a batch of few large cells, or one cell, fills the part.
 // Measured with one warp or one CTA a structure before: the 50 A cell of 679 000 reflections 0.25 ms to count and
-// 1.53 ms to emit, 256 cells of 15-40 A 0.13 and 1.37 ms.
+// 1.53 ms to emit, 256 cells of 15-40 A 0.13 and 1.37 ms; now 6 and 32 us, 17 and 106 us. 100 000 mixed cells in parts of
+// 512 columns 0.21 and 0.72 ms, of 128 columns 0.19 and 0.55 ms; 5000 of them 45 and 153 us, and 20 and 64 us.
 // Items are claimed from a counter, the parts first: kClaim structures (or one part) at a time.
 constexpr int kEnumMaxThreads = 1024;
-constexpr int kClaimWide = 4;         // structures a claim takes in a batch of at least kWideBatch structures
-constexpr int kWideBatch = 2048;      // enough structures to fill the GPU by themselves:
-constexpr int kPartColsWide = 512;    // only the longest are split; below, every chunk of 32 columns is an item, since
-constexpr int kPartColsNarrow = 32;   // a warp's chunks are a serial chain of about 5 us each
+constexpr int kClaimWide = 2;         // structures a claim takes in a batch of at least kWideBatch structures
+constexpr int kWideBatch = 2048;      // enough structures to fill the GPU by themselves: parts of four chunks, which
+constexpr int kPartColsWide = 128;    // bound the tail; below, every chunk of 32 columns is an item, since a warp's chunks
+constexpr int kPartColsNarrow = 32;   // are a serial chain of about 5 us each
 static int enum_part_cols(int n_struct) { return n_struct >= kWideBatch ? kPartColsWide : kPartColsNarrow; }
 
 struct EnumItems {
@@ -608,7 +610,7 @@ __device__ __forceinline__ void write_tiles(int s, bool runs, int tile_refl, int
 // output order is the column order above, l ascending, whatever the launch shape.
 template <bool RUNS>
 __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict__ geo, int n_struct, double r2min,
-                                                          double r2max, float r2minf, float r2maxf, int rb,
+                                                          double r2max, float r2minf, float r2maxf,
                                                           int tile_refl, const int64_t* __restrict__ refl_off,
                                                           const int64_t* __restrict__ run_cnt,
                                                           const int* __restrict__ abort_flag, double* __restrict__ q,
@@ -657,7 +659,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict_
                 int h = 0, k = 0, n = 0, nr = 0;
                 ColSpan sp{1, 0, 1, 0};
                 if (c < c_hi)
-                    sp = column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, n, nr);
+                    sp = column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, RUNS, h, k, n, nr);
                 const int im = warp_incl_scan(n), imr = RUNS ? warp_incl_scan(nr) : 0;
                 const int off = im - n;
                 const unsigned full = __ballot_sync(0xffffffffu, n > 0);
@@ -685,10 +687,9 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict_
                     if (RUNS) {
                         const bool above = p - r.off >= r.n1;  // past the inner gap
                         const int j = p - r.off - (above ? r.n1 : 0), nn = above ? r.n - r.n1 : r.n1;
-                        const int jr = j / rb;
-                        if (jr * rb == j) {
-                            const int64_t rpos = done_runs + r.roff + (above ? runs_of(r.n1, rb) : 0) + jr;
-                            if (rpos < cap) runs[base + rpos] = ((done + p) << 3) | min(rb, nn - j);
+                        if ((j & (kRunLen - 1)) == 0) {
+                            const int64_t rpos = done_runs + r.roff + (above ? runs_of(r.n1) : 0) + j / kRunLen;
+                            if (rpos < cap) runs[base + rpos] = ((done + p) << 3) | min(kRunLen, nn - j);
                         }
                     }
                 }
@@ -872,7 +873,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __res
 // structure in parts). ctr: zero at launch. done: CTAs finished (zero at launch), or null: no scan.
 template <bool RUNS>
 __global__ void __launch_bounds__(kEnumMaxThreads) k_count(Geo* geo, int n_struct, double r2min,
-                                                           double r2max, float r2minf, float r2maxf, int rb,
+                                                           double r2max, float r2minf, float r2maxf,
                                                            int64_t* __restrict__ cnt, int64_t* __restrict__ run_cnt,
                                                            int* __restrict__ ctr, const int* __restrict__ part_ctr,
                                                            const int2* __restrict__ part_tab,
@@ -894,7 +895,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_count(Geo* geo, int n_struc
             int local = 0, local_runs = 0;
             for (int c = c0 + lane; c < c1; c += 32) {
                 int h, k, n, nr;
-                column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, rb, RUNS, h, k, n, nr);
+                column_counts(g, geo[s].gs, c, r2min, r2max, r2minf, r2maxf, RUNS, h, k, n, nr);
                 local += n;
                 local_runs += nr;
             }
@@ -1359,7 +1360,7 @@ static void count_launch(const GeomArgs& a, const ScanArgs& sa, cudaStream_t st,
     const size_t smem = last && !sa.sums ? sizeof(long long) * kScanItems * (size_t)a.enum_threads : 0;
     const int grid = enum_grid(a, (const void*)k, smem);
     auto go = [&](auto launch) {
-        launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, a.refl_cnt,
+        launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.refl_cnt,
                a.run_cnt, a.enum_ctr, (const int*)(a.enum_ctr + kPartCtr), (const int2*)a.part_tab, a.part_cnt,
                a.part_cap, enum_part_cols(a.n_struct), sa, last ? a.enum_ctr + kDoneCtr : (int*)nullptr, sa.bad);
     };
@@ -1409,7 +1410,7 @@ void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl)
     const size_t smem = sizeof(ColRec) * (size_t)a.enum_threads;
     const int grid = enum_grid(a, (const void*)k, smem);
     auto go = [&](auto launch) {
-        launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.runs_mode ? a.rb : 0, 32 * a.rb,
+        launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, 32 * a.rb,
                (const int64_t*)a.refl_off, (const int64_t*)a.run_cnt, (const int*)a.abort_flag, a.q, a.key, a.runs,
                (const int*)a.tile_off, a.tile_tab, a.enum_ctr + 1, (const int*)(a.enum_ctr + kPartCtr),
                (const int2*)a.part_tab, (const int2*)a.part_cnt, a.part_cap, enum_part_cols(a.n_struct));

@@ -422,7 +422,9 @@ __device__ void pf_merge(const PostArgs& a, int cls, int B, int G)
                 a.refl_hkl[3 * o] = hkl_h(kv);
                 a.refl_hkl[3 * o + 1] = hkl_k(kv);
                 a.refl_hkl[3 * o + 2] = hkl_l(kv);
-                a.refl_tt[o] = two_theta_q(qv, a.l2h, a.l2l, a.ttab);
+                float qh, ql;
+                split_pos(qv, qh, ql);
+                a.refl_tt[o] = two_theta_out(qh, ql, a.l2h, a.l2l, a.ttab);
                 a.refl_I[o] = FI ? (double)rec[p].I : a.pf_rI[p];
             }
         }

@@ -307,7 +307,7 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
         }
     }
     auto half = [](const float2* v, int i) { return i & 1 ? v[i / 2].y : v[i / 2].x; };
-    const float l2 = (float)(a.lambda * a.lambda * 0.25);
+    const float l2 = a.l2f;
     float imax = 0.f;
 #pragma unroll
     for (int i = 0; i < kSfRB; i++) {

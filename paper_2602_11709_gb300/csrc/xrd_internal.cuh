@@ -346,18 +346,79 @@ __device__ __forceinline__ double two_theta_q(double q, float Lh, float Ll, cons
     return f2d_fast(T) + f2d_fast(v);
 }
 
+// two_theta_q for the outputs, where its last bits are free: the table index from an approximate arcsine (it may be off by
+// a small part of a step: the remainder u covers it), approximate division and square root in the closed form of u, and one
+// Newton step, which leaves the rounding of its FP32 residual (a second one does not lower it). About half the instructions; the error is the same, about 1e-8 degrees.
+// The table's angle and u are added as integers (2^-32 degrees, 1.2e-10 at most). q = qh + ql.
+__device__ __forceinline__ double two_theta_out(float qh, float ql, float Lh, float Ll, const TTab* __restrict__ tab)
+{
+    float Xh = qh * Lh;
+    float Xl = fmaf(qh, Lh, -Xh) + fmaf(qh, Ll, ql * Lh);
+    if (Xh > 1.f || (Xh == 1.f && Xl > 0.f)) {
+        Xh = 1.f;
+        Xl = 0.f;
+    }
+    const bool comp = Xh > 0.5f || (Xh == 0.5f && Xl > 0.f);
+    const float Yh = comp ? 1.f - Xh : Xh;  // exact for Xh in [0.5, 1]
+    const float Yl = comp ? -Xl : Xl;
+    const float Yf = fmaxf(Yh + Yl, 0.f);
+    // asin(x) / x in x^2 on [0, 1/2], fitted (least squares on Chebyshev nodes, error of asin below 7e-7)
+    const float x = Yf * rsqrtf(fmaxf(Yf, 1e-30f));
+    const float pa = fmaf(fmaf(fmaf(fmaf(fmaf(0.0963539108633995f, Yf, -0.02421635203063488f), Yf, 0.06088736653327942f), Yf,
+                                         0.0729263499379158f),
+                                    Yf, 0.16676093637943268f),
+                               Yf, 0.9999993443489075f);
+    const int j = min((int)fmaf(x * pa, (float)(4.0 * kTabN / kPi), 0.5f), kTabN);
+    int T = 0;  // 2theta = T steps of the table (45 / 512 degrees) + v
+    float v;
+    if (j <= 2) {
+        v = asinf(sqrtf(Yf)) * (float)(360.0 / kPi);
+    } else {
+        const TTab e = tab[j];
+        const float r = (Yh - e.Sh) + (Yl - e.Sl);
+        const float w = fmaf(4.f * e.Bc, r, e.A * e.A);
+        float u = __fdividef(4.f * r, e.A + w * rsqrtf(w));
+        const float u2 = u * u;
+        const float su = u - u * u2 * (1.f / 6.f);
+        const float cu = u2 * (0.5f - u2 * (1.f / 24.f));
+        const float fv = fmaf(e.A, su, fmaf(e.Bc, cu, -2.f * r));
+        u -= __fdividef(fv, fmaf(e.A, 1.f - 0.5f * u2, e.Bc * su));
+        T = j;
+        v = u * (float)(180.0 / kPi);
+    }
+    if (comp) {
+        T = 2 * kTabN - T;  // 180 degrees
+        v = -v;
+    }
+    // in 2^-40 degrees; |v| < 0.06, or 0.23 for j <= 2
+    const long long S = (long long)T * (45ll << 31) + (long long)__float2int_rn(v * 4294967296.f) * 256;
+    const double r = __longlong_as_double(0x4330000000000000ll | S) - 4503599627370496.0;
+    return S == 0 ? 0.0 : __hiloint2double(__double2hiint(r) - (40 << 20), __double2loint(r));
+}
+
 // d = 1/sqrt(q) for q > 0 in float range: an FP32 seed refined by one Newton
 // step whose residual 1 - q y0^2 is formed exactly in FP32 (q split into two
 // floats, y0^2 into two floats); about 1e-13 relative, one FP64 addition.
-__device__ __forceinline__ double inv_sqrt_df(double q)
+// The correction is added to the seed's bits as a double's, in units of 2^-48. q = qh + ql.
+__device__ __forceinline__ double inv_sqrt_df(float qh, float ql)
 {
-    float qh, ql;
-    split_pos(q, qh, ql);
     const float y0 = rsqrtf(qh);
     const float p = y0 * y0, pe = fmaf(y0, y0, -p);
     float r = fmaf(-qh, p, 1.f);
     r = fmaf(-qh, pe, fmaf(-ql, p, r));
-    return f2d_fast(y0) + f2d_fast(0.5f * y0 * r * fmaf(0.75f, r, 1.f));
+    const float c = 0.5f * r * fmaf(0.75f, r, 1.f);  // relative correction, below 2^-21
+    const uint32_t u = __float_as_uint(y0);
+    const float m = __uint_as_float((u & 0x7fffffu) | 0x3f800000u);  // y0's significand in [1, 2)
+    const long long bits = (long long)(((unsigned long long)u << 29) + (896ull << 52)) +
+                           16ll * __float2int_rn(m * c * 281474976710656.f);
+    return __longlong_as_double(bits);
+}
+
+// Float >= 0 (zero or normal) -> double; denormals become 0.
+__device__ __forceinline__ double f2d_nonneg(float x)
+{
+    const uint32_t u = __float_as_uint(x);
+    return u < 0x00800000u ? 0.0 : __longlong_as_double((long long)(((unsigned long long)u << 29) + (896ull << 52)));
 }
 
 // ---- block-wide primitives over generic pointers (shared or global memory) ----

@@ -85,6 +85,7 @@ struct SfArgs {
     int rb, warps;  // launch shape: reflections per lane (2 or 4), warps per CTA (1, 2 or 4)
     int runs_mode;  // lanes take runs (integer phase only) instead of strided reflections
     double lambda;
+    float l2f;      // lambda^2 / 4
     const int64_t* atom_off;
     const int64_t* refl_off;
     const int* tile_off;  // [n_struct + 1]: [n_struct] is the number of tiles

@@ -35,6 +35,10 @@ static __device__ __forceinline__ bool tt_close(double qa, double qb, float l2, 
     if (dbits(qb) <= dbits(qa)) return ttol > 0.f;  // equal |g|^2: a gap of 0
     if (ttol == INFINITY) return true;              // tol above 180 degrees: every gap is below it
     const float dqf = d2f_pos(qb - qa);
+    // sqrt qa + sqrt qb <= 2 sqrt qb and the cosines are at most 1: a gap beyond this bound (squared, no root) is one
+    // whatever the angle, as nearly every gap of a low-symmetry cell is
+    const float lhb = lh * dqf, tb = 4.0002f * ttol;
+    if (lhb * lhb > tb * tb * d2f_pos(qb)) return false;
     const float qaf = d2f_pos(qa), qbf = d2f_pos(qb);
     const float ua = fmaxf(fmaf(-l2, qaf, 1.f), 1e-30f), ub = fmaxf(fmaf(-l2, qbf, 1.f), 1e-30f);
     const float sq = qaf * rsqrtf(qaf) + qbf * rsqrtf(qbf);
