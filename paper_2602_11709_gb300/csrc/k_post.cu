@@ -43,7 +43,8 @@ __host__ __device__ constexpr int post_min_blocks(int cap, int nt)
 {
     const int b = (int)((228u * 1024u) / (post_smem_of((size_t)cap) + 2048u));
     const int t = 2048 / nt;
-    return b < 1 ? 1 : (b < t ? b : t);
+    const int r = b < 1 ? 1 : (b < t ? b : t);
+    return r * nt > 1280 ? 1280 / nt : r;
 }
 
 static __device__ TTab g_ttab[kTabN + 1];
@@ -135,7 +136,87 @@ __device__ void post_singles(const PostArgs& a, int s, int64_t base, int n, cons
     }
 }
 
-// A peak of more than 32 members (out of line: rare): its number of families, and their staging at family offset f0.
+// Sum of a peak's intensities (each half-space reflection stands for g and -g): the same operations whoever sums.
+__device__ __forceinline__ float peak_add(float sum, float v, bool first) { return first ? 2.f * v : fmaf(2.f, v, sum); }
+__device__ __forceinline__ double peak_add(double sum, double v, bool first) { return (first ? 0.0 : sum) + 2.0 * v; }
+
+// A peak of up to 32 C members at merge positions i0 .. i0 + m - 1, by a whole warp, C members to a lane: the members'
+// intensities summed in merge order (every lane gets the sum), and the families found by one round of comparisons
+// against each member in turn. A family leaves its representative (the largest packed key) and its size (from the
+// second family on) in the key and |g|^2 slots of the peak's member of its rank, by descending representative.
+// Returns the number of families.
+constexpr int kWarpPeak = 128;
+template <int C, typename PermT, bool FI, typename FK, typename T>
+__device__ __forceinline__ int merged_peak_body(FK fk, double* q, uint32_t* key, const PermT* perm, int i0, int m,
+                                                const float* Is, const double* I, T& sum)
+{
+    const int lane = threadIdx.x & 31;
+    int v[C], cnt[C], rank[C];
+    T Iv[C];
+    unsigned long long k[C];
+    uint32_t kv[C], rep[C];
+    bool lead[C];
+#pragma unroll
+    for (int c = 0; c < C; c++) {
+        const int i = 32 * c + lane, at = i0 + (i < m ? i : 0);
+        v[c] = perm[at];
+        if constexpr (FI) Iv[c] = Is[v[c]];
+        else Iv[c] = I[v[c]];
+        k[c] = fk(at);
+        kv[c] = key[v[c]];
+        lead[c] = i < m;
+        cnt[c] = 0;
+        rank[c] = 0;
+        rep[c] = 0;
+    }
+    sum = (T)0;
+#pragma unroll
+    for (int b = 0; b < C; b++) {
+        const int mb = min(32, m - 32 * b);
+        for (int j = 0; j < mb; j++) {
+            sum = peak_add(sum, __shfl_sync(0xffffffffu, Iv[b], j), b == 0 && j == 0);
+            const unsigned long long kj = __shfl_sync(0xffffffffu, k[b], j);
+            const uint32_t kvj = __shfl_sync(0xffffffffu, kv[b], j);
+#pragma unroll
+            for (int c = 0; c < C; c++)
+                if (kj == k[c]) {
+                    cnt[c]++;
+                    rep[c] = max(rep[c], kvj);
+                    lead[c] = lead[c] && 32 * b + j >= 32 * c + lane;
+                }
+        }
+    }
+    unsigned leaders[C];
+    int nf = 0;
+#pragma unroll
+    for (int b = 0; b < C; b++) {
+        leaders[b] = __ballot_sync(0xffffffffu, lead[b]);
+        nf += __popc(leaders[b]);
+        for (unsigned u = leaders[b]; u; u &= u - 1) {
+            const uint32_t r = __shfl_sync(0xffffffffu, rep[b], __ffs(u) - 1);
+#pragma unroll
+            for (int c = 0; c < C; c++) rank[c] += r > rep[c];
+        }
+    }
+    __syncwarp();  // every key is read
+#pragma unroll
+    for (int c = 0; c < C; c++)
+        if (lead[c]) {
+            const int slot = perm[i0 + rank[c]];
+            key[slot] = rep[c];
+            if (rank[c] > 0) q[slot] = __longlong_as_double(cnt[c]);
+        }
+    return nf;
+}
+// out of line: few peaks have more than 32 members
+template <typename PermT, bool FI, typename FK, typename T>
+__device__ __noinline__ int merged_peak_large(FK fk, double* q, uint32_t* key, const PermT* perm, int i0, int m,
+                                              const float* Is, const double* I, T& sum)
+{
+    return merged_peak_body<kWarpPeak / 32, PermT, FI>(fk, q, key, perm, i0, m, Is, I, sum);
+}
+
+// A peak of more than kWarpPeak members (out of line: rare): its number of families, and their staging at family offset f0.
 template <typename PermT>
 struct FamilyKeys {  // family key of the member at merge position i
     const unsigned long long* fkg;
@@ -264,21 +345,20 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
         post_singles<PermT, FI>(a, s, base, n, q, key, Is, perm, flag, pst, psum, tmp, dtmp);
         return;
     }
+    for (int i = tid; i < n; i += nt) pst[i] = flag[i];
+    __syncthreads();
     for (int i = tid; i < n; i += nt) {
-        if (!flag[i]) continue;
+        if (!flag[i] || i + 1 >= n || flag[i + 1]) continue;
         double qa = q[perm[i]];
-        pst[i] = 1;
-        int e = i + 1;  // end of the run: the next definite start
-        while (e < n && !flag[e]) e++;
+        int e = i + 2;  // end of the run: the next definite start, four flags at a time where they are aligned
+        while (e < n && !flag[e]) e += (e & 3) == 0 && e + 4 <= n && *(const uint32_t*)(flag + e) == 0u ? 4 : 1;
         // |g|^2 ascends, so a last member within the tolerance of the first one has all others within it too
-        const bool one = e - i == 1 || tt_close(qa, q[perm[e - 1]], l2, lh, ttol, lam, tol);
+        if (tt_close(qa, q[perm[e - 1]], l2, lh, ttol, lam, tol)) continue;
         for (int j = i + 1; j < e; j++) {
             const double qj = q[perm[j]];
-            if (!one && !tt_close(qa, qj, l2, lh, ttol, lam, tol)) {
+            if (!tt_close(qa, qj, l2, lh, ttol, lam, tol)) {
                 pst[j] = 1;
                 qa = qj;
-            } else {
-                pst[j] = 0;
             }
         }
     }
@@ -289,16 +369,13 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
         if ((i + 1 < n ? pst[i + 1] : np) != pst[i]) bkt[pst[i]] = i;
     if (tid == 0) {
         bkt[np] = n;
-        bkt[np + 1] = 0;  // merged peaks of 2 to 32 members (np < n here)
+        bkt[np + 1] = 0;  // merged peaks of 2 to kWarpPeak members (np < n here)
     }
     __syncthreads();
     // ---- per peak: merged intensity (each half-space reflection stands for g and -g) and families ----
-    // A peak of one member is its thread's; one of 2 to 32 members goes to a list (pst is free until the cutoff) that
-    // the warps work off, a lane per member: the members' intensities are summed in merge order, and the families
-    // are found by one round of comparisons against each member in turn. A family leaves its representative and its
-    // size (from the second family on) in the key and |g|^2 slots of the peak's member of its rank. One thread a peak
-    // took most of the structure's time where peaks have many members: rock salt (293 reflections, peaks of up to 24)
-    // 62 000 of 105 000 cycles, and 13 000 more in the staging.
+    // A peak of one member is its thread's; one of 2 to kWarpPeak members goes to a list (pst is free until the cutoff)
+    // that the warps work off (merged_peak). One thread a peak took most of the structure's time where peaks have many
+    // members: rock salt (293 reflections, peaks of up to 36) 62 000 of 105 000 cycles, and 13 000 more in the staging.
     // Peak sums are >= 0, so their maximum is taken through the bit patterns.
     using T = typename std::conditional<FI, float, double>::type;
     T* const ps = (T*)psum;
@@ -310,56 +387,30 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
         if constexpr (FI) return __float_as_uint(v);
         else return dbits(v);
     };
-    auto add = [](T sum, T v, bool first) -> T {  // the same operations whoever sums
-        if constexpr (FI) return first ? 2.f * v : fmaf(2.f, v, sum);
-        else return (first ? 0.0 : sum) + 2.0 * v;
-    };
     unsigned long long lmax = 0;
     for (int p = tid; p < np; p += nt) {
         const int i0 = bkt[p], i1 = bkt[p + 1], m = i1 - i0;
-        if (m > 1 && m <= 32) {
+        if (m > 1 && m <= kWarpPeak) {
             pst[atomicAdd(&bkt[np + 1], 1)] = p;
             continue;
         }
-        T sum = add((T)0, member_I(perm[i0]), true);
-        for (int i = i0 + 1; i < i1; i++) sum = add(sum, member_I(perm[i]), false);
+        T sum = peak_add((T)0, member_I(perm[i0]), true);
+        for (int i = i0 + 1; i < i1; i++) sum = peak_add(sum, member_I(perm[i]), false);
         ps[p] = sum;
         fcnt[p] = m == 1 ? 1 : large_count<PermT>(fk.fkg, key, perm, hex, i0, i1);
         lmax = max(lmax, bits_of(sum));
     }
     __syncthreads();
-    const int nmulti = bkt[np + 1], lane = tid & 31;
+    const int nmulti = bkt[np + 1];
     for (int li = tid >> 5; li < nmulti; li += nt >> 5) {
         const int p = pst[li], i0 = bkt[p], m = bkt[p + 1] - i0;
-        const bool live = lane < m;
-        const int v = perm[i0 + (live ? lane : 0)];
-        const T Iv = member_I(v);
-        const unsigned long long k = fk(i0 + (live ? lane : 0));
-        const uint32_t kv = key[v];
-        T sum = add((T)0, __shfl_sync(0xffffffffu, Iv, 0), true);
-        bool lead = live;
-        int cnt = 0, rank = 0;
-        uint32_t rep = 0;
-        for (int j = 0; j < m; j++) {
-            if (j > 0) sum = add(sum, __shfl_sync(0xffffffffu, Iv, j), false);
-            const bool same = __shfl_sync(0xffffffffu, k, j) == k;
-            const uint32_t kj = __shfl_sync(0xffffffffu, kv, j);
-            if (same) {
-                cnt++;
-                rep = max(rep, kj);
-                lead = lead && j >= lane;
-            }
-        }
-        const unsigned leaders = __ballot_sync(0xffffffffu, lead);
-        for (unsigned b = leaders; b; b &= b - 1) rank += __shfl_sync(0xffffffffu, rep, __ffs(b) - 1) > rep;
-        const int slot = __shfl_sync(0xffffffffu, v, rank & 31);
-        if (lead) {
-            key[slot] = rep;
-            if (rank > 0) q[slot] = __longlong_as_double(cnt);
-        }
-        if (lane == 0) {
+        T sum;
+        int nf;
+        if (m <= 32) nf = merged_peak_body<1, PermT, FI>(fk, q, key, perm, i0, m, Is, FI ? nullptr : a.I + base, sum);
+        else nf = merged_peak_large<PermT, FI>(fk, q, key, perm, i0, m, Is, FI ? nullptr : a.I + base, sum);
+        if ((tid & 31) == 0) {
             ps[p] = sum;
-            fcnt[p] = __popc(leaders);
+            fcnt[p] = nf;
             lmax = max(lmax, bits_of(sum));
         }
     }
@@ -395,7 +446,7 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
         const T v = ps[p];        // the largest peak maps to exactly 100
         ((T*)a.st_I)[o] = (a.scaled && imax > (T)0) ? (v == imax ? (T)100 : (T)100 * (v * inv_imax)) : v;
         a.st_foff[o] = f0;
-        if (m > 32) {
+        if (m > kWarpPeak) {
             large_families<PermT>(a, base, key, perm, hex, i0, i0 + m, f0);
             continue;
         }
