@@ -61,20 +61,28 @@ __device__ __forceinline__ float2 f_of(const CoefPair& c, float2 zf, float2 s2)
                       zf);
 }
 
-// sincos_turn32 of two phases, the polynomials packed (the same operations, so the same results)
-__device__ __forceinline__ void sincos2_turn32(uint32_t P0, uint32_t P1, float2& s, float2& c)
+// sin and cos of two phases in turns (t: phase plus an eighth of a turn), the polynomials packed
+__device__ __forceinline__ void sincos2_turn32(uint32_t t0, uint32_t t1, float2& s, float2& c)
 {
-    const uint32_t q0 = (P0 + 0x20000000u) >> 30, q1 = (P1 + 0x20000000u) >> 30;
-    const float2 a = __fmul2_rn(make_float2((float)(int32_t)(P0 - (q0 << 30)), (float)(int32_t)(P1 - (q1 << 30))),
-                                dup2(kTwoPiOver2p32));
+    const float2 a = __fmul2_rn(make_float2(turn_rest(t0), turn_rest(t1)), dup2(kTurnScale));
     const float2 a2 = __fmul2_rn(a, a);
     const float2 ps = __ffma2_rn(__ffma2_rn(dup2(kSinC[2]), a2, dup2(kSinC[1])), a2, dup2(kSinC[0]));
     const float2 sa = __ffma2_rn(__fmul2_rn(a, a2), ps, a);
     const float2 pc =
         __ffma2_rn(__ffma2_rn(__ffma2_rn(dup2(kCosC[3]), a2, dup2(kCosC[2])), a2, dup2(kCosC[1])), a2, dup2(kCosC[0]));
     const float2 ca = __ffma2_rn(a2, pc, dup2(1.f));
-    turn_quadrant(q0, sa.x, ca.x, s.x, c.x);
-    turn_quadrant(q1, sa.y, ca.y, s.y, c.y);
+    turn_quadrant(t0, sa.x, ca.x, s.x, c.x);
+    turn_quadrant(t1, sa.y, ca.y, s.y, c.y);
+}
+
+__device__ __forceinline__ void sincos_turn32(uint32_t t, float& s, float& c)
+{
+    const float a = turn_rest(t) * kTurnScale, a2 = a * a;
+    const float ps = fmaf(fmaf(kSinC[2], a2, kSinC[1]), a2, kSinC[0]);
+    const float sa = fmaf(a * a2, ps, a);
+    const float pc = fmaf(fmaf(fmaf(kCosC[3], a2, kCosC[2]), a2, kCosC[1]), a2, kCosC[0]);
+    const float ca = fmaf(a2, pc, 1.f);
+    turn_quadrant(t, sa, ca, s, c);
 }
 
 // Lorentz-polarisation factor (1 + cos^2 2theta) / (sin^2 theta cos theta) with
@@ -143,11 +151,13 @@ __device__ __forceinline__ void place(const CellArgs& c, int64_t r, double q)
 // instead of per reflection. Otherwise every reflection's phase is formed exactly (integer
 // phase; XRD_FP32_PHASE64 with the coordinates' low words too).
 //
-// The kernel is bound by instruction issue (about 76 % of the slots at 3 instructions a clock), so the FP32 work of two
+// The kernel is bound by instruction issue (about 77 % of the slots at 3 instructions a clock), so the FP32 work of two
 // reflections goes into one packed instruction wherever both halves are at hand: the polynomials of sin and cos, f(s),
 // the displacement factor's argument, the weights and the sums. The packed operations round each half as the scalar
-// ones do: the results are the same bits. 256 cells of 200-2000 atoms: 10.20 -> 9.41 ms with runs; 100 000 mixed
-// cells: 3.15 -> 2.93 ms.
+// ones do: the results are the same bits. 256 cells of 200-2000 atoms: 10.20 -> 9.11 ms with runs; 100 000 mixed
+// cells: 3.15 -> 2.85 ms. Fewer instructions alone do not make it faster: one packed sin/cos for two atoms of a run
+// costs the moves that it saves (2.99 ms), and with a branch of its own for equal elements 9 % fewer instructions ran
+// at 72 % (9.14 and 3.04 ms).
 //
 // Pattern variants (not GRAD): sin and cos come from the FMA pipe
 // (sincos_turn32, five times more accurate than the SFU's), F is summed in FP32
@@ -191,7 +201,7 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
     }
 #pragma unroll
     for (int p = 0; p < NP; p++) Fr[p] = Fi[p] = f[p] = Gr[p] = Gi[p] = fp[p] = Rh[p] = Rl[p] = Ih[p] = Il[p] = A2[p] = zero;
-    float zf = 0.f;
+    float zf = 0.f, fm = 0.f;  // fm, with runs: max(|f|, Z) of the first reflection
     constexpr bool kRotate = RUNS && PREC == XRD_FP32_PHASEFIX;
     constexpr int kFold = kRotate ? 16 : 8;  // block size of the two-float sum: 16 atoms with runs, else 8
     int zc = -1;
@@ -226,12 +236,13 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
                     for (int p = 0; p < NP; p++) {
                         f[p] = f_of(c, dup2(zf), s2[p]);
                         if (GRAD) fp[p] = fprime_of(c, s2[p]);
+                        if (kRotate && p == 0) fm = fmaxf(fabsf(f[0].x), zf);
                     }
                 }
                 float2 cs[NP], sn[NP];
                 if (kRotate) {  // the run's phase factors from its first one
                     float s0, co;
-                    sincos_turn32(uh[0] * at.X + uk[0] * at.Y + ul[0] * at.Z, s0, co);
+                    sincos_turn32(uh[0] * at.X + kEighthTurn + uk[0] * at.Y + ul[0] * at.Z, s0, co);
                     const float2 st = sstep[jj];
                     const float tcz = st.x + st.x;  // exact
                     cs[0].x = co;
@@ -254,7 +265,7 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
 #pragma unroll
                         for (int o = 0; o < 2; o++) {
                             const int i = 2 * p + o;
-                            P[o] = uh[i] * at.X + uk[i] * at.Y + ul[i] * at.Z;
+                            P[o] = uh[i] * at.X + (ACC ? kEighthTurn : 0u) + uk[i] * at.Y + ul[i] * at.Z;
                             if (PREC == XRD_FP32_PHASE64)  // the low words' sum, below 2^31, rounded into the high words'
                                 P[o] += (uint32_t)(((int)uh[i] * lo.x + (int)uk[i] * lo.y + (int)ul[i] * lo.z + (1 << 20)) >> 21);
                         }
@@ -275,7 +286,7 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
                     if (ACC) {
                         if (kRotate) {  // a run's reflections share one scale (s^2 nearly equal)
                             if (p == 0) {
-                                const float m = dw.x * fmaxf(fabsf(f[0].x), zf);
+                                const float m = dw.x * fm;
                                 A2[0].x = fmaf(m, m, A2[0].x);
                             }
                         } else {
@@ -370,12 +381,13 @@ __device__ void order_by_count(const SfArgs& a, int* cnt)
 // first). A structure's atoms stay staged in the warp's shared memory while its
 // consecutive tiles follow (when they fit one chunk).
 // Register caps: 64 for the integer-phase variant with 2 reflections per lane
-// (32 resident warps per SM), about 85 for the other FP32 variants (24 warps).
+// (32 resident warps per SM), 72 with runs (28 warps asked for, 26 fit beside the staged atoms: 2.85 ms on 100 000
+// mixed cells, 2.88 with 24), about 85 for the other FP32 variants (24 warps).
 template <int PREC, bool GRAD, int RB, int WARPS, bool RUNS>
 __global__ void __launch_bounds__(32 * WARPS,
                                   (PREC == XRD_FP32_PHASEFIX && !GRAD && RB == 2) ? 32 / WARPS
                                   : (PREC == XRD_FP32_PHASE64 && RB == 4)         ? 20 / WARPS
-                                                                                  : 24 / WARPS)
+                                                                                  : (RUNS ? 28 : 24) / WARPS)
     k_sf(const SfArgs a)
 {
     pdl_enter();

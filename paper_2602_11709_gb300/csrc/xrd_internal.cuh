@@ -249,25 +249,20 @@ __device__ __forceinline__ float ex2_approx(float x)
 constexpr float kSinC[3] = {-0.16666650772094727f, 0.00833197869360447f, -0.00019495634478516877f};
 constexpr float kCosC[4] = {-0.5f, 0.04166662320494652f, -0.0013886763481423259f, 2.439044874336105e-05f};
 
-// (sin, cos)(a + q pi/2) from those of a: q = 1: (cos, -sin), 2: (-sin, -cos), 3: (-cos, sin)
-__device__ __forceinline__ void turn_quadrant(uint32_t q, float sa, float ca, float& s, float& c)
-{
-    const bool swap = q & 1u;
-    const float s1 = swap ? ca : sa, c1 = swap ? sa : ca;
-    s = __int_as_float(__float_as_int(s1) ^ (int)((q & 2u) << 30));
-    c = __int_as_float(__float_as_int(c1) ^ (int)(((q + 1u) & 2u) << 30));
-}
+// The functions take t = P + 2^29 (an eighth of a turn more: the callers' products start from it): the quarter turn is
+// the top two bits of t, and the remainder 4 d (its sign bit in place) is 4 t with the sign bit turned over.
+constexpr uint32_t kEighthTurn = 0x20000000u;
+constexpr float kTurnScale = 0.25f * 1.4629180792671596e-09f;  // 2 pi / 2^34
+__device__ __forceinline__ float turn_rest(uint32_t t) { return (float)(int32_t)(4u * t + 0x80000000u); }
 
-__device__ __forceinline__ void sincos_turn32(uint32_t P, float& s, float& c)
+// (sin, cos)(a + q pi/2) from those of a: q = 1: (cos, -sin), 2: (-sin, -cos), 3: (-cos, sin). The signs are the top
+// bits of t and of t plus a quarter turn.
+__device__ __forceinline__ void turn_quadrant(uint32_t t, float sa, float ca, float& s, float& c)
 {
-    const uint32_t q = (P + 0x20000000u) >> 30;
-    const float a = (float)(int32_t)(P - (q << 30)) * 1.4629180792671596e-09f;  // 2 pi / 2^32
-    const float a2 = a * a;
-    const float ps = fmaf(fmaf(kSinC[2], a2, kSinC[1]), a2, kSinC[0]);
-    const float sa = fmaf(a * a2, ps, a);
-    const float pc = fmaf(fmaf(fmaf(kCosC[3], a2, kCosC[2]), a2, kCosC[1]), a2, kCosC[0]);
-    const float ca = fmaf(a2, pc, 1.f);
-    turn_quadrant(q, sa, ca, s, c);
+    const bool swap = t & 0x40000000u;
+    const float s1 = swap ? ca : sa, c1 = swap ? sa : ca;
+    s = __uint_as_float(__float_as_uint(s1) ^ (t & 0x80000000u));
+    c = __uint_as_float(__float_as_uint(c1) ^ ((t + 0x40000000u) & 0x80000000u));
 }
 
 // Positive normal double -> two floats, q = qh + ql to about 2^-47 relative,
