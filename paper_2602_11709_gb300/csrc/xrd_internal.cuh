@@ -394,7 +394,8 @@ __device__ __forceinline__ double two_theta_out(float qh, float ql, float Lh, fl
 // d = 1/sqrt(q) for q > 0 in float range: an FP32 seed refined by one Newton
 // step whose residual 1 - q y0^2 is formed exactly in FP32 (q split into two
 // floats, y0^2 into two floats); about 1e-13 relative, one FP64 addition.
-// The correction is added to the seed's bits as a double's, in units of 2^-48. q = qh + ql.
+// The correction is added to the seed's bits as a double's, in units of 2^-48 of its binade; where the sum leaves the
+// binade (d next to a power of two) the part beyond counts double below and half above. q = qh + ql.
 __device__ __forceinline__ double inv_sqrt_df(float qh, float ql)
 {
     const float y0 = rsqrtf(qh);
@@ -404,9 +405,11 @@ __device__ __forceinline__ double inv_sqrt_df(float qh, float ql)
     const float c = 0.5f * r * fmaf(0.75f, r, 1.f);  // relative correction, below 2^-21
     const uint32_t u = __float_as_uint(y0);
     const float m = __uint_as_float((u & 0x7fffffu) | 0x3f800000u);  // y0's significand in [1, 2)
-    const long long bits = (long long)(((unsigned long long)u << 29) + (896ull << 52)) +
-                           16ll * __float2int_rn(m * c * 281474976710656.f);
-    return __longlong_as_double(bits);
+    // the sum's significand less 1, in units of 2^-52
+    const long long f = (long long)((unsigned long long)(u & 0x7fffffu) << 29) +
+                        16ll * __float2int_rn(m * c * 281474976710656.f);
+    const long long beyond = f < 0 ? f : f >= (1ll << 52) ? ((1ll << 52) - f) >> 1 : 0;
+    return __longlong_as_double((long long)((unsigned long long)((u >> 23) + 896u) << 52) + f + beyond);
 }
 
 // Float >= 0 (zero or normal) -> double; denormals become 0.

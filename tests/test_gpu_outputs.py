@@ -34,3 +34,19 @@ def test_two_theta_and_d(gpu_lib, edge, tt_max, refl):
             e = np.abs(got["refl_tt"][s] - 2.0 * np.degrees(np.arcsin(x)))
             assert np.all(e <= 2e-8 + 2e-12 / np.sqrt(np.maximum(1.0 - x * x, 1e-12)))
             np.testing.assert_allclose(d, 1.0 / np.sqrt(np.sort(q)), rtol=1e-12)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1.5])  # 1.5: no d at a power of two
+def test_d_next_to_a_power_of_two(gpu_lib, scale):
+    eps = np.linspace(-4e-7, 4e-7, 161)
+    rng = np.random.default_rng(5)
+    b = synth.concat([synth.random_cell(rng, 1) for _ in eps])
+    b.lattice[:, :3] = scale * 4.0 * (1.0 + eps)[:, None]  # cubic: d of (100), (200), (400) around 4, 2 and 1
+    b.lattice[:, 3:] = 90.0
+    o = synth.Opts(wavelength=0.71073, tt_max=60.0, rel_cutoff=0.0)
+    got = gpu_lib.compute(b, o, "fp64")
+    for s in range(len(eps)):
+        a, d = b.lattice[s, 0], got["peak_d"][s]
+        n = np.rint((a / d) ** 2)
+        assert {1.0, 4.0, 16.0} <= set(n)
+        np.testing.assert_allclose(d, a / np.sqrt(n), rtol=1e-12)
