@@ -37,14 +37,14 @@ size_t post_smem_bytes(int cap) { return post_smem_of((size_t)cap); }
 
 // CTAs per SM that the shared memory of a class allows (228 KB per SM; about
 // 2 KB more per CTA for the static arrays and the per-CTA reservation), at most
-// 2048 threads: the launch bounds ask the compiler to fit that many CTAs in the
-// register file too.
+// 1024 threads: the launch bounds ask the compiler to fit that many CTAs in the
+// register file too, and 64 registers a thread spill nothing. More threads gain nothing on large batches (100 000
+// mixed cells 6.89 ms, 6.87 with 1280 threads, 6.89 with 1536) and their spills cost on small ones (256 hexagonal/P1
+// cells 119, 124 and 133 us; 1024 small cells 190, 196 and 199 us).
 __host__ __device__ constexpr int post_min_blocks(int cap, int nt)
 {
     const int b = (int)((228u * 1024u) / (post_smem_of((size_t)cap) + 2048u));
-    const int t = 2048 / nt;
-    const int r = b < 1 ? 1 : (b < t ? b : t);
-    return r * nt > 1280 ? 1280 / nt : r;
+    return b < 1 ? 1 : b * nt > 1024 ? 1024 / nt : b;
 }
 
 static __device__ TTab g_ttab[kTabN + 1];
@@ -72,6 +72,27 @@ const TTab* init_tables(cudaStream_t st)
     return (const TTab*)p;
 }
 
+// The largest of all threads' values (bit patterns of floats >= 0), by one barrier; tmp: 32 words of shared memory,
+// free after the caller's next barrier.
+template <bool FI>
+__device__ __forceinline__ unsigned long long post_max(unsigned long long v, unsigned long long* tmp)
+{
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    auto warp_max = [](unsigned long long x) -> unsigned long long {
+        if constexpr (FI) {
+            return __reduce_max_sync(0xffffffffu, (unsigned)x);
+        } else {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x = max(x, (unsigned long long)__shfl_xor_sync(0xffffffffu, x, o));
+            return x;
+        }
+    };
+    v = warp_max(v);
+    if (lane == 0) tmp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return warp_max(lane < nw ? tmp[lane] : 0ull);
+}
+
 // The common case of a structure whose sorted reflections are all farther apart
 // than the tolerance: every reflection is a peak of one family (g and -g, so
 // multiplicity 2), and the merge runs, the peak-start scan and the family
@@ -96,7 +117,7 @@ __device__ void post_singles(const PostArgs& a, int s, int64_t base, int n, cons
             lmax = max(lmax, dbits(v));
         }
     }
-    const unsigned long long m = block_max_u64(lmax, (unsigned long long*)dtmp);
+    const unsigned long long m = post_max<FI>(lmax, (unsigned long long*)dtmp);
     if (FI) {
         imaxf = __uint_as_float((uint32_t)m);
         inv_imaxf = imaxf > 0.f ? 1.f / imaxf : 0.f;
@@ -106,13 +127,14 @@ __device__ void post_singles(const PostArgs& a, int s, int64_t base, int n, cons
     }
     const uint32_t thrf = __float_as_uint((float)a.cutoff * imaxf);
     const unsigned long long thr = dbits(a.cutoff * imax);
-    for (int p = tid; p < n; p += nt) {
-        const bool keep = a.cutoff == 0.0 || (FI ? __float_as_uint(((float*)psum)[p]) > thrf : dbits(psum[p]) > thr);
-        flag[p] = keep;
-        pst[p] = keep;
-    }
+    auto keep = [&](int p) -> int {
+        return a.cutoff == 0.0 || (FI ? __float_as_uint(((float*)psum)[p]) > thrf : dbits(psum[p]) > thr);
+    };
+    const int nk = block_scan_to(n, tmp, keep, [&](int p, int sum, int v) {
+        flag[p] = v;
+        pst[p] = sum;
+    });
     __syncthreads();
-    const int nk = block_excl_scan(pst, n, tmp);
     for (int p = tid; p < n; p += nt) {
         if (!flag[p]) continue;
         const int64_t o = base + pst[p];
@@ -268,16 +290,21 @@ __device__ __noinline__ void large_families(const PostArgs& a, int64_t base, con
 
 // FI: intensities are FP32 (the FP32 structure-factor variants) and peak sums,
 // cutoff and scaling run in FP32; otherwise FP64 throughout.
-// Is: the FP32 intensities of the structure (shared or global memory).
-template <typename PermT, bool FI>
-__device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, double* q, uint32_t* key,
-                               const float* Is, PermT* perm, int* bkt, uint8_t* flag, int* pst, double* psum, int* fcnt,
-                               int* tmp, double* dtmp)
+// hex: Miller-Bravais families. ahead(0), ahead(1): called once each by all threads, in this order, where the work in
+// between hides the latency of a global load.
+// The phases are short (a few elements a thread), so barriers and the latency of passes through shared memory bound
+// them: loading and counting are one pass, the flags are the peak starts, the peak list, the cutoff and the offsets come
+// out of the scans themselves, and the next structure is claimed meanwhile (16 barriers a structure; with a pass for
+// each of these, 25 barriers and the claim in the open, 100 000 mixed cells took 7.06 ms a call, now 6.89; 20 000 at
+// Mo K-alpha 6.31, now 6.17).
+template <typename PermT, bool FI, typename Ahead>
+__device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, bool hex, double* q, uint32_t* key,
+                               float* Is, PermT* perm, int* bkt, uint8_t* flag, int* pst, double* psum, int* fcnt,
+                               int* tmp, double* dtmp, Ahead ahead)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
     const float l2 = a.l2f, lh = a.lhf, ttol = a.ttol;
     const double lam = a.lambda, tol = a.tol;
-    const bool hex = a.geo[s].hex != 0;  // Miller-Bravais families
     // family key of the member at merge position i: the caller's point group (precomputed per
     // reflection), else permutation and sign (Miller-Bravais for a hexagonal cell)
     const FamilyKeys<PermT> fk{a.fkg ? a.fkg + base : nullptr, key, perm, hex};
@@ -292,7 +319,11 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
     for (int i = tid; i <= nb; i += nt) bkt[i] = 0;
     __syncthreads();
     for (int i = tid; i < n; i += nt) {
-        const float qf = d2f_pos(q[i]);
+        const double qi = a.q[base + i];
+        q[i] = qi;
+        key[i] = a.key[base + i];
+        if (FI) Is[i] = a.If[base + i];
+        const float qf = d2f_pos(qi);
         int b = (int)((qf * sqrtf(qf) - lo3) * scale);
         b = min(max(b, 0), nb - 1);
         bid[i] = b;
@@ -300,6 +331,7 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
     }
     __syncthreads();
     block_excl_scan(bkt, nb, tmp);
+    ahead(0);
     for (int i = tid; i < n; i += nt) perm1[atomicAdd(&bkt[bid[i]], 1)] = i;
     __syncthreads();
     // bkt[b] is now the end of bucket b; rank within the bucket gives the position
@@ -339,14 +371,14 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
     for (int i = tid; i < n; i += nt) {
         const bool start = (i == 0) || !tt_close(q[perm[i - 1]], q[perm[i]], l2, lh, ttol, lam, tol);
         flag[i] = start;
+        pst[i] = start;
         close_pair |= !start;
     }
+    ahead(1);
     if (!__syncthreads_or(close_pair)) {  // no two reflections within the tolerance: every one is a peak
         post_singles<PermT, FI>(a, s, base, n, q, key, Is, perm, flag, pst, psum, tmp, dtmp);
         return;
     }
-    for (int i = tid; i < n; i += nt) pst[i] = flag[i];
-    __syncthreads();
     for (int i = tid; i < n; i += nt) {
         if (!flag[i] || i + 1 >= n || flag[i + 1]) continue;
         double qa = q[perm[i]];
@@ -363,10 +395,10 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
         }
     }
     __syncthreads();
-    // peak starts -> peak ids (exclusive scan); bkt becomes the list of peak start positions
-    const int np = block_excl_scan(pst, n, tmp);
-    for (int i = tid; i < n; i += nt)
-        if ((i + 1 < n ? pst[i + 1] : np) != pst[i]) bkt[pst[i]] = i;
+    // bkt becomes the list of peak start positions
+    const int np = block_scan_to(n, tmp, [&](int i) { return pst[i]; }, [&](int i, int id, int start) {
+        if (start) bkt[id] = i;
+    });
     if (tid == 0) {
         bkt[np] = n;
         bkt[np + 1] = 0;  // merged peaks of 2 to kWarpPeak members (np < n here)
@@ -414,7 +446,7 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
             lmax = max(lmax, bits_of(sum));
         }
     }
-    const unsigned long long mbits = block_max_u64(lmax, (unsigned long long*)dtmp);
+    const unsigned long long mbits = post_max<FI>(lmax, (unsigned long long*)dtmp);
     T imax, inv_imax;
     unsigned long long thr;
     if constexpr (FI) {
@@ -424,24 +456,23 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
     } else {
         imax = __longlong_as_double((long long)mbits);
         thr = dbits(a.cutoff * imax);
-        if (tid == 0) dtmp[0] = imax > 0.0 ? 1.0 / imax : 0.0;
+        if (tid == 0) dtmp[32] = imax > 0.0 ? 1.0 / imax : 0.0;
         __syncthreads();
-        inv_imax = dtmp[0];
+        inv_imax = dtmp[32];
     }
-    // ---- cutoff, then compaction offsets of kept peaks and their families ----
-    for (int p = tid; p < np; p += nt) {
-        const bool keep = a.cutoff == 0.0 || bits_of(ps[p]) > thr;
-        flag[p] = keep;
-        pst[p] = keep;
-        if (!keep) fcnt[p] = 0;
-    }
+    // ---- cutoff and the offsets of kept peaks (upper half) and their families (at most 6144 each) ----
+    const int kf = block_scan_to(
+        np, tmp, [&](int p) { return a.cutoff == 0.0 || bits_of(ps[p]) > thr ? 1 << 16 | fcnt[p] : 0; },
+        [&](int p, int sum, int v) {
+            flag[p] = v != 0;
+            pst[p] = sum;
+        });
+    const int nk = kf >> 16, nf = kf & 0xffff;
     __syncthreads();
-    int nk, nf;
-    block_excl_scan2(pst, fcnt, np, tmp, nk, nf);
     for (int p = tid; p < np; p += nt) {
         if (!flag[p]) continue;
-        const int i0 = bkt[p], m = bkt[p + 1] - i0, f0 = fcnt[p];
-        const int64_t o = base + pst[p];
+        const int i0 = bkt[p], m = bkt[p + 1] - i0, f0 = pst[p] & 0xffff;
+        const int64_t o = base + (pst[p] >> 16);
         a.st_q[o] = q[perm[i0]];  // anchor |g|^2: 2-theta and d are formed during compaction
         const T v = ps[p];        // the largest peak maps to exactly 100
         ((T*)a.st_I)[o] = (a.scaled && imax > (T)0) ? (v == imax ? (T)100 : (T)100 * (v * inv_imax)) : v;
@@ -450,7 +481,7 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
             large_families<PermT>(a, base, key, perm, hex, i0, i0 + m, f0);
             continue;
         }
-        const int nfp = (p + 1 < np ? fcnt[p + 1] : nf) - f0;  // dropped peaks have no families
+        const int nfp = fcnt[p];
         int first = m;  // members of the first family: those of no other
         for (int r = nfp - 1; r >= 0; r--) {
             const int u = perm[i0 + r], c = r ? (int)__double_as_longlong(q[u]) : first;
@@ -465,8 +496,24 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, do
     }
 }
 
+// An asynchronous copy of N bytes (4 or 8, aligned) to shared memory, and the wait for the thread's copies
+template <int N>
+__device__ __forceinline__ void copy_async(void* to, const void* from)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from), "n"(N) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// A claimed structure: its extent in the reflection arrays, hexagonal, with an invalid atom
+struct PostClaim {
+    int64_t base, end;
+    int s, hex, bad;
+};
+
 // Persistent CTAs over one size class of structures (a list built by the scan
-// kernel, largest first), each CTA claiming the next structure from a counter.
+// kernel, largest first), each CTA claiming the next structure from a counter
+// while it works on the current one.
 // The structure's reflections live in shared memory (n <= CAP); the FP32
 // variants also stage the intensities there, in the second half of the
 // peak-sum area (FP32 peak sums use the first half).
@@ -476,37 +523,61 @@ __global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const Pos
     static_assert(CAP > 0, "the largest class runs as the flat passes");
     pdl_chain_enter(first);
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int tmp[66];
-    __shared__ double dtmp[32];
-    __shared__ int claim;
-    for (; !*a.abort_flag;) {
-        __syncthreads();  // the previous structure is done with shared memory and claim
-        if (threadIdx.x == 0) {
-            int li = atomicAdd(a.cls_next + c_lo, 1), c = c_hi;  // the larger classes first
-            while (c >= c_lo && li >= a.cls_cnt[c]) li -= a.cls_cnt[c--];
-            claim = c >= c_lo ? a.cls_list[(int64_t)c * a.n_struct + li] : -1;
-        }
-        __syncthreads();
-        const int s = claim;
+    __shared__ int tmp[32];
+    __shared__ double dtmp[33];
+    __shared__ PostClaim claims[2];
+    if (*a.abort_flag) {
+        pdl_chain_exit();
+        return;
+    }
+    // thread 0's claim of the next structure while the CTA works on the current one: the queue's counter, then the
+    // structure from its class's list (step 0), then its extent (1), each copied to shared memory without waiting for it
+    auto list = [&](int li, PostClaim& c) {
+        int cls = c_hi;  // the larger classes first
+        while (cls >= c_lo && li >= a.cls_cnt[cls]) li -= a.cls_cnt[cls--];
+        if (cls >= c_lo) copy_async<4>(&c.s, a.cls_list + (int64_t)cls * a.n_struct + li);
+        else c.s = -1;
+    };
+    auto extent = [&](PostClaim& c) {
+        copy_async_wait();
+        if (c.s < 0) return;
+        copy_async<8>(&c.base, a.refl_off + c.s);
+        copy_async<8>(&c.end, a.refl_off + c.s + 1);
+        copy_async<4>(&c.hex, &a.geo[c.s].hex);
+        if (a.atom_bad) copy_async<4>(&c.bad, a.atom_bad + c.s);
+        else c.bad = 0;
+    };
+    if (threadIdx.x == 0) {
+        list(atomicAdd(a.cls_next + c_lo, 1), claims[0]);
+        extent(claims[0]);
+        copy_async_wait();
+    }
+    for (int k = 0;; k ^= 1) {
+        __syncthreads();  // the previous structure is done with shared memory, the claim is written
+        const PostClaim cl = claims[k];
+        const int s = cl.s;
         if (s < 0) break;
-        const int64_t base = a.refl_off[s];
-        const int n = (int)(a.refl_off[s + 1] - base);
-        if (a.atom_bad && a.atom_bad[s]) {  // an invalid atom: no peaks, the structure reports XRD_EINVAL
+        const int64_t base = cl.base;
+        const int n = (int)(cl.end - base);
+        int li = 0;
+        if (threadIdx.x == 0) li = atomicAdd(a.cls_next + c_lo, 1);
+        auto ahead = [&](int step) {
+            if (threadIdx.x) return;
+            if (step == 0) list(li, claims[k ^ 1]);
+            else extent(claims[k ^ 1]);
+        };
+        if (cl.bad || n == 0) {
             if (threadIdx.x == 0) {
                 a.npk[s] = 0;
                 a.nfm[s] = 0;
-                if (a.status[s] == XRD_OK) {
+                if (cl.bad && a.status[s] == XRD_OK) {  // an invalid atom: no peaks, the structure reports XRD_EINVAL
                     a.status[s] = XRD_EINVAL;
                     atomicAdd((unsigned long long*)&a.totals[3], 1ull);
                 }
             }
-            continue;
-        }
-        if (n == 0) {
-            if (threadIdx.x == 0) { a.npk[s] = 0; a.nfm[s] = 0; }
-            continue;
-        }
-        {
+            ahead(0);
+            ahead(1);
+        } else {
             const size_t c = (size_t)CAP;
             unsigned char* p = smem;
             double* sq = (double*)p; p += align16(c * 8);
@@ -518,14 +589,10 @@ __global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const Pos
             double* psum = (double*)p; p += align16(c * 8);
             int* fcnt = (int*)p;
             float* sI = (float*)psum + c;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                sq[i] = a.q[base + i];
-                sk[i] = a.key[base + i];
-                if (FI) sI[i] = a.If[base + i];
-            }
-            __syncthreads();
-            post_structure<uint16_t, FI>(a, s, base, n, sq, sk, sI, perm, bkt, flag, pst, psum, fcnt, tmp, dtmp);
+            post_structure<uint16_t, FI>(a, s, base, n, cl.hex != 0, sq, sk, sI, perm, bkt, flag, pst, psum, fcnt, tmp,
+                                         dtmp, ahead);
         }
+        if (threadIdx.x == 0) copy_async_wait();
     }
     pdl_chain_exit();
 }

@@ -432,81 +432,36 @@ __device__ __forceinline__ int warp_incl_scan(int v)
     return v;
 }
 
-// Exclusive prefix sum of a[0..n) in place by the whole block; returns the
-// total. `tmp` is shared scratch of at least 33 ints. All threads must call.
-// In-place exclusive scan of a[0..n) in shared memory by the whole block; each
-// thread takes one contiguous segment, so the block synchronises three times
-// whatever n is. Returns the total. tmp: 33 ints of shared memory.
-__device__ __forceinline__ int block_excl_scan(int* a, int n, int* tmp)
+// Block-wide exclusive scan of get(i), i < n: put(i, sum of those before i, get(i)) for every i; returns the total. One
+// barrier, before the calls of put; the caller's next barrier frees tmp (32 ints of shared memory). get is called twice.
+template <typename Get, typename Put>
+__device__ __forceinline__ int block_scan_to(int n, int* tmp, Get get, Put put)
 {
     const int nt = blockDim.x, nw = (nt + 31) >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int seg = (n + nt - 1) / nt;
     const int i0 = min((int)threadIdx.x * seg, n), i1 = min(i0 + seg, n);
     int s = 0;
-    for (int i = i0; i < i1; i++) s += a[i];
+    for (int i = i0; i < i1; i++) s += get(i);
     const int inc = warp_incl_scan(s);
     if (lane == 31) tmp[w] = inc;
     __syncthreads();
-    if (w == 0) {
-        const int v = lane < nw ? tmp[lane] : 0;
-        const int si = warp_incl_scan(v);
-        if (lane < nw) tmp[lane] = si - v;
-        if (lane == 31) tmp[32] = si;
-    }
-    __syncthreads();
-    int run = tmp[w] + inc - s;
-    const int total = tmp[32];
+    const int t = lane < nw ? tmp[lane] : 0;
+    int run = __reduce_add_sync(0xffffffffu, lane < w ? t : 0) + inc - s;
+    const int total = __reduce_add_sync(0xffffffffu, t);
     for (int i = i0; i < i1; i++) {
-        const int v = a[i];
-        a[i] = run;
+        const int v = get(i);
+        put(i, run, v);
         run += v;
     }
-    __syncthreads();
     return total;
 }
 
-// Two exclusive scans of the same length at once (a and b); totals in ta, tb.
-// tmp: 66 ints of shared memory.
-__device__ __forceinline__ void block_excl_scan2(int* a, int* b, int n, int* tmp, int& ta, int& tb)
+// The exclusive scan of a in place (two barriers; tmp and a are free again on return)
+__device__ __forceinline__ int block_excl_scan(int* a, int n, int* tmp)
 {
-    const int nt = blockDim.x, nw = (nt + 31) >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int seg = (n + nt - 1) / nt;
-    const int i0 = min((int)threadIdx.x * seg, n), i1 = min(i0 + seg, n);
-    int sa = 0, sb = 0;
-    for (int i = i0; i < i1; i++) {
-        sa += a[i];
-        sb += b[i];
-    }
-    const int ia = warp_incl_scan(sa), ib = warp_incl_scan(sb);
-    if (lane == 31) {
-        tmp[w] = ia;
-        tmp[33 + w] = ib;
-    }
+    const int total = block_scan_to(n, tmp, [&](int i) { return a[i]; }, [&](int i, int sum, int) { a[i] = sum; });
     __syncthreads();
-    if (w == 0) {
-        const int va = lane < nw ? tmp[lane] : 0, vb = lane < nw ? tmp[33 + lane] : 0;
-        const int xa = warp_incl_scan(va), xb = warp_incl_scan(vb);
-        if (lane < nw) {
-            tmp[lane] = xa - va;
-            tmp[33 + lane] = xb - vb;
-        }
-        if (lane == 31) {
-            tmp[32] = xa;
-            tmp[65] = xb;
-        }
-    }
-    __syncthreads();
-    int ra = tmp[w] + ia - sa, rb = tmp[33 + w] + ib - sb;
-    ta = tmp[32];
-    tb = tmp[65];
-    for (int i = i0; i < i1; i++) {
-        const int va = a[i], vb = b[i];
-        a[i] = ra;
-        b[i] = rb;
-        ra += va;
-        rb += vb;
-    }
-    __syncthreads();
+    return total;
 }
 
 // Exclusive block-wide prefix of one 64-bit value per thread (two barriers;

@@ -33,3 +33,31 @@ def test_many_members(gpu_lib, prec, tol, group):
     assert max(len(p) and int(np.diff(f).max()) for p, f in zip(ref["peak_tt"], ref["peak_fam_off"])) >= (2 if tol > 1e-4 else 1)
     got = gpu_lib.compute(b, o, prec)
     compare_batch(got, ref, prec, o.rel_cutoff, o.scaled)
+
+
+@pytest.mark.parametrize("n", [60, 700, 2500])  # one launch, three, eight
+def test_invalid_and_empty_structures_between_others(gpu_lib, n):
+    """Structures with an invalid atom or without reflections in the size classes' queues: the others' outputs are
+    those of a batch without them, bit for bit."""
+    rng = np.random.default_rng(n)
+    o = synth.Opts(tt_max=60.0)
+    cells, good = [], []
+    for i in range(n):
+        b = synth.random_cell(rng, int(rng.integers(1, 9)))
+        b.lattice[0, :3] = rng.uniform(3.0, 25.0 if i % 10 == 0 else 10.0) * rng.uniform(0.9, 1.1, 3)
+        if i % 3 == 1:
+            b.frac[0, 0] = np.nan
+        elif i % 7 == 2:
+            b.lattice[0, :3] = 0.7
+        else:
+            good.append(i)
+        cells.append(b)
+    got = gpu_lib.compute(synth.concat(cells), o)
+    ref = gpu_lib.compute(synth.concat([cells[i] for i in good]), o)
+    want = np.where(np.arange(n) % 3 == 1, gpu_lib.XRD_EINVAL, 0)
+    assert np.array_equal(got["status"], want)
+    for k, i in enumerate(good):
+        for f in ("peak_tt", "peak_I", "peak_d", "peak_fam_off"):
+            assert np.array_equal(got[f][i], ref[f][k])
+    for i in set(range(n)) - set(good):
+        assert len(got["peak_tt"][i]) == 0
