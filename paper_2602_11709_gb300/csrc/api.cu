@@ -755,7 +755,8 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
         pa.pf_pst = (int*)(ws + L.cand_s);
         pa.pf_pj = (int*)(ws + L.Eb);
         pa.pf_kidx = (int*)(ws + L.cand_r);
-        pa.pf_fidx = pa.pf_kidx + (cap_refl + 1);
+        // 16-byte aligned; the area's rounding to 256 bytes leaves the room
+        pa.pf_fidx = pa.pf_kidx + ((cap_refl + 4) & ~(int64_t)3);
         pa.pf_rec = (xrd::PfRec*)(ws + L.pf_rec);
         pa.pf_rI = (double*)(ws + L.cand_r);  // until the kept-peak scan
     }

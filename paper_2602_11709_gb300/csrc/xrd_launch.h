@@ -203,7 +203,7 @@ struct PostArgs {
     unsigned long long* pf_smax;   // [n_struct] bits of each structure's largest peak sum
     int* pf_scal;                  // [4]: reflections of the class (V), its peaks
     long long* pf_parts;           // [2 kPfScanBlocksMax] segment sums of the scans
-    int* pf_pst;                   // [reflections + 1] peak starts, then peak ids
+    int* pf_pst;                   // [reflections + 1] peak ids
     int* pf_pj;                    // [reflections] structure (class-list position) of each peak
     int* pf_kidx;                  // [reflections + 1] kept-peak index of each peak
     int* pf_fidx;                  // [reflections + 1] family offset of each peak

@@ -61,3 +61,17 @@ def test_invalid_and_empty_structures_between_others(gpu_lib, n):
             assert np.array_equal(got[f][i], ref[f][k])
     for i in set(range(n)) - set(good):
         assert len(got["peak_tt"][i]) == 0
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_phasefix"])
+@pytest.mark.parametrize("n", [1, 2, 5])
+def test_flat_passes_any_counts(gpu_lib, prec, n):
+    """Structures above the shared-memory classes, whose counts leave every remainder of the scans' four elements."""
+    rng = np.random.default_rng(n)
+    b = synth.concat([synth.random_cell(rng, 2) for _ in range(n)])
+    b.lattice[:, :3] = 25.0 + 0.2 * np.arange(n)[:, None] + [0.0, 0.7, 1.3]
+    o = synth.Opts(tt_max=60.0, rel_cutoff=1e-3)
+    got = gpu_lib.compute(b, o, prec)
+    ref = oracle.pattern_batch(b, o)
+    assert got["sizes"]["n_refl"] > 6144 * n
+    compare_batch(got, ref, prec, o.rel_cutoff, o.scaled)
