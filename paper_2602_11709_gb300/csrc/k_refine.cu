@@ -140,21 +140,33 @@ __device__ void refine_one(const RefineArgs& a, int64_t r, int s, const float4* 
 
 
 // Selection: every candidate has E > tau I (the criterion is
-// E > tau max(I, c M)); for those few the structure-factor kernel has noted the
-// structure, whose floor c M decides.
-__device__ __forceinline__ bool refine_take(const RefineArgs& a, int64_t r, float E, float I, int& s)
+// E > tau max(I, c M)); for those few percent the structure-factor kernel has noted the
+// structure, whose floor c M decides. N reflections of a thread at a time, so that the structures' numbers, then their
+// floors, are read together (one after the other, a branch each, the selection took 179 us on 100 000 mixed cells, now
+// 147; with eight reflections 154). Bit j of the result takes reflection r(j), of structure s[j].
+template <int N, typename R>
+__device__ __forceinline__ unsigned refine_take(const RefineArgs& a, R r, const float* E, const float* I, int* s)
 {
-    if (!(E > 0.f && E > a.tau * I)) return false;
-    s = a.Es[r];
-    const float floorI = a.cref * __uint_as_float(a.imax[s]);
-    const bool bad = a.atom_bad && a.atom_bad[s];
-    return !bad && E > a.tau * fmaxf(I, floorI);
+    float floorI[N];
+    unsigned take = 0;
+#pragma unroll
+    for (int j = 0; j < N; j++) s[j] = E[j] > 0.f && E[j] > a.tau * I[j] ? a.Es[r(j)] : -1;
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        floorI[j] = s[j] >= 0 ? a.cref * __uint_as_float(a.imax[s[j]]) : 0.f;
+        if (s[j] >= 0 && a.atom_bad && a.atom_bad[s[j]]) s[j] = -1;
+    }
+#pragma unroll
+    for (int j = 0; j < N; j++)
+        if (s[j] >= 0 && E[j] > a.tau * fmaxf(I[j], floorI[j])) take |= 1u << j;
+    return take;
 }
 
 // A CTA collects its candidates in shared memory and appends them to the list
 // with one atomic per flush: candidates are rare (a fraction of a percent), and
 // one atomic per warp on the list's single counter had serialised.
-constexpr int kSelCap = 2048;  // shared-memory candidates per CTA; flushed above kSelCap - 4 kRefThreads
+constexpr int kSelChunk = 4 * kRefThreads;  // reflections a CTA takes at a time
+constexpr int kSelCap = 2048;               // shared-memory candidates per CTA; flushed above kSelCap - kSelChunk
 
 __global__ void __launch_bounds__(kRefThreads) k_refine_select(const RefineArgs a)
 {
@@ -179,12 +191,12 @@ __global__ void __launch_bounds__(kRefThreads) k_refine_select(const RefineArgs 
         if (threadIdx.x == 0) sn = 0;
         __syncthreads();
     };
-    // the CTA takes 4 kRefThreads consecutive reflections at a time, four per thread in one 16-byte
+    // the CTA takes kSelChunk consecutive reflections at a time, four per thread in one 16-byte
     // load of each array (both 256-byte aligned)
-    constexpr int kChunk = 4 * kRefThreads;
-    for (int64_t c0 = (int64_t)blockIdx.x * kChunk; c0 < total; c0 += (int64_t)gridDim.x * kChunk) {
+    for (int64_t c0 = (int64_t)blockIdx.x * kSelChunk; c0 < total; c0 += (int64_t)gridDim.x * kSelChunk) {
         const int64_t r4 = c0 + 4 * threadIdx.x;
         float E[4] = {0.f, 0.f, 0.f, 0.f}, I[4] = {0.f, 0.f, 0.f, 0.f};
+        int st[4];
         if (r4 + 4 <= total) {
             const float4 e4 = *reinterpret_cast<const float4*>(a.Eb + r4);
             const float4 i4 = *reinterpret_cast<const float4*>(a.If + r4);
@@ -197,17 +209,18 @@ __global__ void __launch_bounds__(kRefThreads) k_refine_select(const RefineArgs 
                     I[j] = a.If[r4 + j];
                 }
         }
+        const unsigned take = refine_take<4>(a, [&](int j) { return r4 + j; }, E, I, st);
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int st = 0;
-            if (r4 + j < total && refine_take(a, r4 + j, E[j], I[j], st)) {
+        for (int j = 0; j < 4; j++)
+            if (take >> j & 1u) {
                 const int slot = atomicAdd(&sn, 1);
                 sr[slot] = r4 + j;
-                ss[slot] = st;
+                ss[slot] = st[j];
             }
-        }
         __syncthreads();
-        if (sn > kSelCap - kChunk) flush();  // uniform: every thread reads sn after the barrier
+        const bool full = sn > kSelCap - kSelChunk;
+        __syncthreads();  // every thread has read sn before any adds to it again
+        if (full) flush();
     }
     __syncthreads();
     flush();
@@ -234,7 +247,7 @@ __global__ void __launch_bounds__(kRefThreads) k_refine_eval(const RefineArgs a)
 // Small batches: selection and evaluation in one launch. Each CTA of a grid with a thread per reflection selects among
 // its own and its warps evaluate what it found. Where the CTAs take one chunk each the launch saved is worth more
 // than the balance lost (24 mixed cells: 17.4 us as two kernels, 12.4 us as one; 256 hexagonal/P1 cells 14.4 and 9.2);
-// 100 000 mixed cells take 422 us as two kernels and 555 us as a persistent form of this one.
+// 100 000 mixed cells take 390 us as two kernels and 555 us as a persistent form of this one.
 
 __global__ void __launch_bounds__(kRefThreads) k_refine_small(const RefineArgs a)
 {
@@ -251,8 +264,9 @@ __global__ void __launch_bounds__(kRefThreads) k_refine_small(const RefineArgs a
     ssc[threadIdx.x] = a.sc[threadIdx.x];
     if (threadIdx.x < 64) sex[threadIdx.x] = a.ex[threadIdx.x];
     __syncthreads();
-    int st = 0;
-    if (r < total && refine_take(a, r, a.Eb[r], a.If[r], st)) {
+    int st = -1;
+    const float E = r < total ? a.Eb[r] : 0.f, I = r < total ? a.If[r] : 0.f;
+    if (refine_take<1>(a, [&](int) { return r; }, &E, &I, &st)) {
         const int slot = atomicAdd(&sn, 1);
         sr[slot] = r;
         ss[slot] = st;
