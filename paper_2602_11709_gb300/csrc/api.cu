@@ -651,6 +651,7 @@ int xrd_pattern_batch(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cons
     sa.abort_flag = ga.abort_flag;
     sa.coef32 = ga.coef32;
     sa.coef = b->coef;
+    sa.frac = b->frac;
     sa.atom32 = ga.atom32;
     sa.atomx = ga.atomx;
     sa.q = ga.q;

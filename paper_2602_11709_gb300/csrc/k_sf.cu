@@ -18,7 +18,8 @@
 // about 1/64 of the FP32 rate here, so the phase is formed and reduced mod 1 in integers: from coordinates in 32-bit
 // fixed point (XRD_FP32_PHASEFIX), or in 53-bit fixed point, the resolution of an FP64 phase (XRD_FP32_PHASE64: three
 // more integer products a term; formed in FP64, four operations a term at 1.7 a clock and SM, it made the kernel take
-// 471 us on 1024 cells of 1 to 64 atoms; now about 80 us). The XRD_FP64 variant is k_sf64.cu.
+// 471 us on 1024 cells of 1 to 64 atoms; now about 75 us; next to a rounding tie the FP64 phase is formed after all, so
+// that the results are the same bits). The XRD_FP64 variant is k_sf64.cu.
 #include <climits>
 
 #include "xrd_internal.cuh"
@@ -115,6 +116,20 @@ __device__ __forceinline__ float2 fprime_of(const CoefPair& c, float2 s2)
 // three index times low-word products stays below 2^31.
 __device__ __forceinline__ int low21(int32_t lo) { return (lo >> 11) + ((lo >> 10) & 1); }
 
+// The phase of XRD_FP32_PHASE64 is that of an FP64 evaluation, rounded to 2^-32 turns. The integer one errs by at most
+// 0.501 (|h| + |k| + |l|) in units of 2^-53 (the coordinates' rounding), the FP64 one by half an ulp of each of three
+// results, none above (|h| + |k| + |l|) times the largest coordinate. So both round alike unless the integer one is
+// within phase_margin times |h| + |k| + |l| of a tie (one term in 10^4), where the FP64 one is formed.
+__device__ __forceinline__ uint32_t phase_fp64(int h, int k, int l, const double* x)
+{
+    return fix32(fma((double)h, x[0], fma((double)k, x[1], (double)l * x[2])));
+}
+__device__ __forceinline__ int phase_margin(const double* x)
+{
+    const float m = fmaxf(fmaxf(__double2float_ru(fabs(x[0])), __double2float_ru(fabs(x[1]))), __double2float_ru(fabs(x[2])));
+    return (int)fminf(4.1f * fmaxf(m, 1.f) + 1.f, 1048576.f);
+}
+
 // x / d correctly rounded, inv = 1 / d correctly rounded: Markstein's theorem (IBM J. Res. Dev. 34, 1990) makes one FMA
 // step from a quotient within an ulp the rounded one; the first step gets it there. Five FP64 operations.
 __device__ __forceinline__ double div_by(double x, double d, double inv)
@@ -205,6 +220,10 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
     constexpr bool kRotate = RUNS && PREC == XRD_FP32_PHASEFIX;
     constexpr int kFold = kRotate ? 16 : 8;  // block size of the two-float sum: 16 atoms with runs, else 8
     int zc = -1;
+    int hkl1 = 0;  // the largest |h| + |k| + |l| of the lane's reflections
+    if (PREC == XRD_FP32_PHASE64)
+#pragma unroll
+        for (int i = 0; i < kSfRB; i++) hkl1 = max(hkl1, abs((int)uh[i]) + abs((int)uk[i]) + abs((int)ul[i]));
     for (int64_t c0 = j0; c0 < j1; c0 += kSfChunk) {
         const int nc = (int)min((int64_t)kSfChunk, j1 - c0);
         if (!staged) {
@@ -217,7 +236,8 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
                     at.X = d.hi[0];
                     at.Y = d.hi[1];
                     at.Z = d.hi[2];
-                    slo[i] = make_int4(low21(d.lo[0]), low21(d.lo[1]), low21(d.lo[2]), 0);
+                    slo[i] = make_int4(low21(d.lo[0]), low21(d.lo[1]), low21(d.lo[2]),
+                                       phase_margin(a.frac + 3 * (j0 + a.atom32[c0 + i].src)));
                 }
                 sat[i] = at;
             }
@@ -258,22 +278,34 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
                         sn[p].y = fmaf(tcz, sn[p].x, -sn[p - 1].y);
                     }
                 } else {
-                    const int4 lo = PREC == XRD_FP32_PHASE64 ? slo[jj] : make_int4(0, 0, 0, 0);
+                    uint32_t P[kSfRB];
+#pragma unroll
+                    for (int i = 0; i < kSfRB; i++)
+                        P[i] = uh[i] * at.X + (ACC ? kEighthTurn : 0u) + uk[i] * at.Y + ul[i] * at.Z;
+                    if (PREC == XRD_FP32_PHASE64) {  // the low words' sums, below 2^31, rounded into the high words'
+                        const int4 lo = slo[jj];
+                        const uint32_t near = min((uint32_t)hkl1 * (uint32_t)lo.w + 2u, 1u << 20);
+                        bool tie = false;
+#pragma unroll
+                        for (int i = 0; i < kSfRB; i++) {
+                            const int v = (int)uh[i] * lo.x + (int)uk[i] * lo.y + (int)ul[i] * lo.z + (1 << 20);
+                            P[i] += (uint32_t)(v >> 21);
+                            tie |= (((uint32_t)v + near) & 0x1fffffu) <= 2u * near;
+                        }
+                        if (tie) {  // the FP64 phase may round the other way
+                            const double* x = a.frac + 3 * (j0 + a.atom32[c0 + jj].src);
+#pragma unroll
+                            for (int i = 0; i < kSfRB; i++)
+                                P[i] = phase_fp64((int)uh[i], (int)uk[i], (int)ul[i], x) + kEighthTurn;
+                        }
+                    }
 #pragma unroll
                     for (int p = 0; p < NP; p++) {
-                        uint32_t P[2];
-#pragma unroll
-                        for (int o = 0; o < 2; o++) {
-                            const int i = 2 * p + o;
-                            P[o] = uh[i] * at.X + (ACC ? kEighthTurn : 0u) + uk[i] * at.Y + ul[i] * at.Z;
-                            if (PREC == XRD_FP32_PHASE64)  // the low words' sum, below 2^31, rounded into the high words'
-                                P[o] += (uint32_t)(((int)uh[i] * lo.x + (int)uk[i] * lo.y + (int)ul[i] * lo.z + (1 << 20)) >> 21);
-                        }
                         if (ACC) {
-                            sincos2_turn32(P[0], P[1], sn[p], cs[p]);
+                            sincos2_turn32(P[2 * p], P[2 * p + 1], sn[p], cs[p]);
                         } else {
-                            __sincosf((float)(int32_t)P[0] * kTwoPiOver2p32, &sn[p].x, &cs[p].x);
-                            __sincosf((float)(int32_t)P[1] * kTwoPiOver2p32, &sn[p].y, &cs[p].y);
+                            __sincosf((float)(int32_t)P[2 * p] * kTwoPiOver2p32, &sn[p].x, &cs[p].x);
+                            __sincosf((float)(int32_t)P[2 * p + 1] * kTwoPiOver2p32, &sn[p].y, &cs[p].y);
                         }
                     }
                 }

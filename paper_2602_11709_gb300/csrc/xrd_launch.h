@@ -93,6 +93,7 @@ struct SfArgs {
     const int64_t* run_cnt;  // [n_struct] runs of each structure
     const int* runs;      // [reflections] run entries, indexed from refl_off[s]
     const float2* astep;  // [atoms] exp(2 pi i z) of each element-sorted atom (the l + 1 step)
+    const double* frac;   // the caller's coordinates [atoms][3] (XRD_FP32_PHASE64)
     int* tile_counter;    // work-queue head, zeroed by the caller
     const int* abort_flag;
     const Coef32* coef32;

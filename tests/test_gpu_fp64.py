@@ -52,3 +52,19 @@ def test_library_exp_forms(gpu_lib, form):
     o = synth.Opts(rel_cutoff=0.0, scaled=0)
     got = gpu_lib.compute(b, o, "fp64")
     compare_batch(got, oracle.pattern_batch(b, o), "fp64", o.rel_cutoff, o.scaled)
+
+
+@pytest.mark.parametrize("bits", [20, 33, 34])  # phases in whole units of 2^-32 turns, at ties of them, at quarters
+def test_phase_as_fp64_rounds_it(gpu_lib, bits):
+    """XRD_FP32_PHASE64's integer phase rounds as the FP64 one. Coordinates shifted by 2^16 (their phases are exact in
+    FP64 too) leave nearly every term to the FP64 evaluation: the intensities are the same bits."""
+    rng = np.random.default_rng(bits)
+    b = synth.concat([synth.random_cell(rng, n, edge=(3.0, 4.0)) for n in (1, 7, 40, 129)])
+    b.frac = (2.0 * rng.integers(0, 2 ** (bits - 1), b.frac.shape) + 1.0) * 2.0 ** -bits
+    o = synth.Opts(tt_max=60.0, rel_cutoff=0.0, scaled=0)
+    one = gpu_lib.compute(b, o, "fp32_phase64")
+    b.frac = b.frac + 2.0 ** 16
+    two = gpu_lib.compute(b, o, "fp32_phase64")
+    for s in range(b.n_struct):
+        assert len(one["peak_I"][s]) > 10
+        assert np.array_equal(one["peak_I"][s], two["peak_I"][s])
