@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict_
 //  2. in the largest-first order (k_order), each structure's first tile and
 //     the post-processing size-class lists (post_class; within a class the
 //     order follows the chunks).
-// The tile table itself is written by k_emit, one CTA per structure.
+// The tile table itself is written by k_emit, each item its share of its structure's entries.
 constexpr int kOrderBins = 4096;
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
