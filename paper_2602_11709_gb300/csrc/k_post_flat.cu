@@ -699,7 +699,9 @@ template <bool FI>
 __global__ void __launch_bounds__(kPfThreads, kPfCtasPerSm) k_pf_fused(const PostArgs a, int cls)
 {
     pdl_enter();
-    if (*a.abort_flag) return;  // set before this launch: the same for every CTA
+    // both set before this launch: the same for every CTA. An empty class, the rule in small batches, takes no barrier
+    // (24 mixed cells 104 -> 101 us a call, 256 hexagonal/P1 cells 120 -> 117)
+    if (*a.abort_flag || a.cls_cnt[cls] == 0) return;
     const int B = blockIdx.x, G = gridDim.x;
     int* bar = a.pf_bar;
     const int extra = a.pf_bar_extra;
