@@ -4,11 +4,15 @@
 // lane operations per clock and SM), so the FP64 loop's exponentials and
 // phase factors are formed in integers: a table (1024 exponentials, 513 phase
 // factors of a quarter turn) and a short Taylor series, every product a 32 x 32
-// bit multiplication or three of them. Errors stay below one unit in the last
-// place of a double (exp: relative; sin and cos: 3e-18 absolute, so their
-// largest error is that of the final rounding to a double).
+// bit multiplication or three of them. exp(-x) errs by less than (1/2 + x/128)
+// 2^-53 of itself before it is rounded to a double (rounding x itself to a
+// double costs up to x 2^-53). sin and cos err by less than 6.5e-18 absolute
+// (3.7e-18 seen), a 17th of a rounding at 1, but not relative to themselves
+// next to a zero as the library's do: in a structure factor's sum the
+// rounding of the phase, which is exact here, weighed more.
 //
-// Host and device: tests compare both functions with a wider evaluation.
+// Host and device: tests/test_fx_host.py compares both functions, compiled for
+// the host, with a 60-digit evaluation.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -32,6 +36,16 @@ XRD_HD uint64_t fx_mulhi64(uint64_t a, uint64_t b)
 {
     const uint32_t ah = fx_hi32(a), al = (uint32_t)a, bh = fx_hi32(b), bl = (uint32_t)b;
     return (uint64_t)ah * bh + fx_mulhi(ah, bl) + fx_mulhi(al, bh);
+}
+XRD_HD uint64_t fx_umul64hi(uint64_t a, uint64_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    const uint32_t ah = fx_hi32(a), al = (uint32_t)a, bh = fx_hi32(b), bl = (uint32_t)b;
+    const uint64_t mid = (uint64_t)ah * bl + fx_mulhi(al, bl), low = (uint64_t)al * bh + (uint32_t)mid;
+    return (uint64_t)ah * bh + fx_hi32(mid) + fx_hi32(low);
+#endif
 }
 XRD_HD int fx_clz64(uint64_t x)  // x != 0
 {
@@ -65,11 +79,13 @@ XRD_HD uint64_t fx_as_bits(double d)
 constexpr int kFxExpN = 1024;  // 2^(-j / 1024), 64 fractional bits
 constexpr int kFxScN = 512;    // cos and sin of (j / 512) quarter turns, 62 fractional bits, j = 0 .. 512
 
-// A positive double as m 2^(e - 63), m in [2^63, 2^64); zero has m = 0.
+// A positive double as m 2^(e - 63), m in [2^63, 2^64). Zero has m = 0 and an exponent below any other's: fx_exp2_neg
+// takes a product's size from the exponents, and a product of zero is small whatever the other factor.
 struct FxNum {
     uint64_t m;
     int e;
 };
+constexpr int kFxZero = -4096;
 constexpr int kFxSlow = 1 << 20;  // exponent of an exponent coefficient that the fixed-point form does not cover
 
 // v >= 0 (a normal double, or zero)
@@ -81,20 +97,20 @@ XRD_HD FxNum fx_num(double v)
     r.m = ((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 11;
     if (v == 0.0) {
         r.m = 0;
-        r.e = 0;
+        r.e = kFxZero;
     }
     return r;
 }
 
 // b log2(e) for an exponent coefficient b >= 0, to about 2^-64 relative; e = kFxSlow where b is negative, not
 // finite or outside [2^-300, 2^300] (and not zero): the caller takes the library's exp there.
-__device__ __forceinline__ FxNum fx_log2e(double b)
+XRD_HD FxNum fx_log2e(double b)
 {
-    if (b == 0.0) return FxNum{0ull, 0};
+    if (b == 0.0) return FxNum{0ull, kFxZero};
     if (!(b >= 0x1p-300 && b <= 0x1p300)) return FxNum{0ull, kFxSlow};
     constexpr uint64_t L = 0xB8AA3B295C17F0BCull;  // log2(e) 2^63
     const FxNum n = fx_num(b);
-    const uint64_t hi = __umul64hi(n.m, L);  // in [0.72 2^62, 1.45 2^63): the product 2^(e - 62) / 2^64
+    const uint64_t hi = fx_umul64hi(n.m, L);  // in [0.72 2^62, 1.45 2^63): the product 2^(e - 62) / 2^64
     const uint64_t lo = n.m * L;
     if (hi >> 63) return FxNum{hi + (lo >> 63), n.e + 1};
     return FxNum{(hi << 1) | (lo >> 63), n.e};

@@ -68,3 +68,15 @@ def test_phase_as_fp64_rounds_it(gpu_lib, bits):
     for s in range(b.n_struct):
         assert len(one["peak_I"][s]) > 10
         assert np.array_equal(one["peak_I"][s], two["peak_I"][s])
+
+
+def test_zero_coefficients_at_large_s(gpu_lib):
+    """B = 0 and b = 0 where s^2 exceeds 1024: their exponentials are 1 at any angle and wavelength."""
+    rng = np.random.default_rng(22)
+    b = synth.concat([synth.random_cell(rng, n, edge=(1.5, 2.5)) for n in (1, 5, 33)])
+    b.B[:] = 0.0
+    b.coef[::2, 0, 1] = 0.0
+    o = synth.Opts(wavelength=0.0251, tt_min=107.0, tt_max=107.05, rel_cutoff=0.0, scaled=0)
+    ref = oracle.pattern_batch(b, o)
+    assert all(len(p) > 100 for p in ref["peak_tt"])
+    compare_batch(gpu_lib.compute(b, o, "fp64"), ref, "fp64", o.rel_cutoff, o.scaled)
