@@ -41,7 +41,7 @@ extern "C" {
 #define XRD_ETIMEOUT 4  /* a bounded device-side wait ran out */
 
 /* Precision of the structure-factor sum (Sec. 2, the structure-factor sum). */
-#define XRD_FP64 0          /* every step in FP64 */
+#define XRD_FP64 0          /* FP64 throughout; phases, sin, cos and exponentials in 64-bit fixed point, to FP64's accuracy */
 #define XRD_FP32_PHASE64 1  /* phase h.x+k.y+l.z formed and reduced mod 1 to 53 fractional bits, the rest in FP32 */
 #define XRD_FP32_PHASEFIX 2 /* coordinates in 32-bit fixed point, phase reduced mod 1 exactly in integers, the rest in FP32 */
 

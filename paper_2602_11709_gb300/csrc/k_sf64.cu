@@ -83,32 +83,28 @@ void init_fx_tables(cudaStream_t st) { k_fx_init<<<(kFxExpN + kFxScN + 1 + 31) /
 
 // ---- f(s) of one element: Z - 41.78214 s^2 sum_i a_i exp(-b_i s^2) ----
 
-// Coefficients of one element in fixed point: a_i = ai 2^(ae - 59) with the largest |a_i| below 2^(ae + 1), and
-// kf = -41.78214 2^(ae - 59), so that f = Z + (kf s^2) sum_i ai exp(-b_i s^2). slow: a coefficient outside the
-// fixed-point form (negative or huge b, not finite); f is then formed in FP64 with the library's exp.
+// Coefficients of one element in fixed point (fx_exp_sum). slow: one of them is outside the fixed-point form (negative
+// or huge b, denormal a, not finite); f is then formed in FP64 with the library's exp.
 struct CoefX {
     uint64_t bm[4];
-    int64_t ai[4];
-    int be[4];
-    double kf;
+    int64_t am[4];
+    int16_t be[4], ae[4];
     int slow, pad;
 };
 
 __device__ void coefx_of(const double* __restrict__ c, CoefX& o)
 {
-    double amax = 0.0;
     bool ok = true;
     for (int i = 0; i < 4; i++) {
+        const double a = c[2 * i];
         const FxNum b = fx_log2e(c[2 * i + 1]);
+        int e;
+        o.am[i] = fx_signed(a, e);
+        o.ae[i] = (int16_t)e;
         o.bm[i] = b.m;
-        o.be[i] = b.e;
-        ok = ok && b.e != kFxSlow && isfinite(c[2 * i]);
-        amax = fmax(amax, fabs(c[2 * i]));
+        o.be[i] = (int16_t)(b.e == kFxSlow ? 0 : b.e);
+        ok = ok && b.e != kFxSlow && (a == 0.0 || (fabs(a) >= 0x1p-300 && fabs(a) <= 0x1p300));
     }
-    ok = ok && amax <= 0x1p300;
-    const int ae = amax >= 0x1p-300 ? (int)(fx_as_bits(amax) >> 52) - 1023 : -300;
-    for (int i = 0; i < 4; i++) o.ai[i] = ok ? __double2ll_rn(scalbn(c[2 * i], 59 - ae)) : 0;
-    o.kf = scalbn(-kFScale, ae - 59);
     o.slow = !ok;
     o.pad = 0;
 }
@@ -124,17 +120,7 @@ __device__ __noinline__ double dw64_slow(double B, double s2) { return exp(-B * 
 
 __device__ __forceinline__ double f64_of(const CoefX& c, double zf, double s2, FxNum S, const uint64_t* __restrict__ ex)
 {
-    int64_t sum = 0;
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        int n;
-        const uint64_t m = fx_exp2_neg(c.bm[i], c.be[i], S.m, S.e, ex, n);
-        const int64_t ai = c.ai[i];
-        const uint64_t aa = ai < 0 ? (uint64_t)-ai : (uint64_t)ai;
-        const int64_t v = n < 64 ? (int64_t)(fx_mulhi64(aa, m) >> n) : 0;
-        sum += ai < 0 ? -v : v;
-    }
-    return fma(c.kf * s2, fx_to_double<0>(sum), zf);
+    return fma(-kFScale * s2, fx_exp_sum(c.am, c.ae, c.bm, c.be, S, ex), zf);
 }
 
 // h x + k y + l z mod 1 in 64-bit fixed point, exact for the record's coordinates

@@ -151,6 +151,46 @@ XRD_HD double fx_exp_double(uint64_t m, int n)
     return fx_as_double(((uint64_t)(1021 - n) << 52) + (m >> 11) + ((m >> 10) & 1ull));
 }
 
+// A normal double as am 2^(e - 60), |am| in [2^60, 2^61); zero has am = 0.
+XRD_HD int64_t fx_signed(double v, int& e)
+{
+    const FxNum n = fx_num(v < 0.0 ? -v : v);
+    e = n.e;
+    const int64_t am = (int64_t)(n.m >> 3);
+    return v < 0.0 ? -am : am;
+}
+
+// sum of four am_i 2^(ae_i - 60) exp(-b_i s2), the exponentials as in fx_exp2_neg, to 2^-58 of the largest term: terms
+// are aligned to that one, not to the largest coefficient, whose term may have decayed.
+XRD_HD double fx_exp_sum(const int64_t* am, const int16_t* ae, const uint64_t* bm, const int16_t* be, FxNum S,
+                         const uint64_t* __restrict__ tab)
+{
+    uint64_t v[4];
+    int e[4], top = -(1 << 20);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        int n;
+        const uint64_t m = fx_exp2_neg(bm[i], be[i], S.m, S.e, tab, n);
+        v[i] = fx_mulhi64(am[i] < 0 ? 0ull - (uint64_t)am[i] : (uint64_t)am[i], m);  // v 2^(ae - n - 60), below 2^61
+        e[i] = ae[i] - n;
+        if (v[i] != 0ull && e[i] > top) top = e[i];
+    }
+    int64_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int sh = top - e[i];
+        const int64_t w = v[i] != 0ull && sh < 64 ? (int64_t)(v[i] >> sh) : 0;
+        sum += am[i] < 0 ? -w : w;
+    }
+    if (sum == 0) return 0.0;
+    const uint64_t a = sum < 0 ? 0ull - (uint64_t)sum : (uint64_t)sum;
+    const int z = fx_clz64(a);
+    const int f = 1023 + 62 + top - 60 - z;  // exponent field less one: the significand's top bit carries into it
+    if (f < 0) return 0.0;                   // below 2^-1022
+    const uint64_t m = a << z;
+    return fx_as_double((sum < 0 ? 0x8000000000000000ull : 0ull) | (((uint64_t)f << 52) + (m >> 11) + ((m >> 10) & 1ull)));
+}
+
 // A signed fixed-point number with F fractional bits as a double (rounded to nearest)
 template <int F>
 XRD_HD double fx_to_double(int64_t v)

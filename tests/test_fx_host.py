@@ -24,6 +24,23 @@ extern "C" void host_exp(int n, const double* b, const double* s2, const uint64_
         out[i] = L.e == kFxSlow ? -1.0 : fx_exp_double(m[i], ex[i]);
     }
 }
+extern "C" void host_exp_sum(int n, const double* ab, const double* s2, const uint64_t* tab, double* out)
+{
+    for (int i = 0; i < n; i++) {
+        int64_t am[4];
+        uint64_t bm[4];
+        int16_t ae[4], be[4];
+        for (int j = 0; j < 4; j++) {
+            int e;
+            am[j] = fx_signed(ab[8 * i + 2 * j], e);
+            ae[j] = (int16_t)e;
+            const FxNum b = fx_log2e(ab[8 * i + 2 * j + 1]);
+            bm[j] = b.m;
+            be[j] = (int16_t)b.e;
+        }
+        out[i] = fx_exp_sum(am, ae, bm, be, fx_num(s2[i]), tab);
+    }
+}
 extern "C" void host_sincos(int n, const uint64_t* P, const uint64_t* tab, int64_t* c, int64_t* s)
 {
     for (int i = 0; i < n; i++) fx_sincos(P[i], (const ulonglong2*)tab, c[i], s[i]);
@@ -98,6 +115,32 @@ def test_exp(fx):
         assert g == (np.ldexp(float((int(m) + 1024) >> 11), 11 - 64 - int(n)) if m else 0.0)
     assert _exp(fx, [1.0, 1e80], [1e4, 1e80])[2].tolist() == [0.0, 0.0]
     assert _exp(fx, [-1.0, 1e200, 1e-200, np.inf, np.nan], 1.0)[2].tolist() == [-1.0] * 5  # left to the library's exp
+
+
+@pytest.mark.parametrize("form", ["positive", "signs", "spread", "zeros"])
+@pytest.mark.parametrize("s2", [0.01, 1.0, 10.0, 25.0, 100.0, 1500.0])
+def test_exp_sum(fx, form, s2):
+    """sum_i a_i exp(-b_i s^2) with every term's own relative error, as in FP64, also where those of the largest a_i have
+    decayed: the exponential's (1/2 + b s^2 / 128) 2^-53 and 2^-57 of the largest term each (two truncated products and
+    the alignment), then the rounding of the sum. Exponentials below 2^-1021 and sums below 2^-1022 are zero."""
+    rng = np.random.default_rng(5)
+    ab = np.stack([rng.uniform(0.5, 4.0, (300, 4)), rng.uniform(0.05, 50.0, (300, 4))], axis=2)
+    if form == "signs":
+        ab[:, :, 0] *= rng.choice([-1.0, 1.0], (300, 4))
+    elif form == "spread":
+        ab[:, :, 0] *= 10.0 ** rng.integers(-80, 80, (300, 4))
+    elif form == "zeros":
+        ab[np.arange(300), rng.integers(0, 4, 300), 0] = 0.0
+        ab[np.arange(300), rng.integers(0, 4, 300), 1] = 0.0
+    ab, s, out = np.ascontiguousarray(ab), np.full(300, s2), np.zeros(300)
+    fx.host_exp_sum(300, _p(ab), _p(s), _p(fx.exp_tab), _p(out))
+    for c, g in zip(ab, out):
+        y = [Decimal(float(b)) * Decimal(s2) for b in c[:, 1]]
+        t = [Decimal(float(a)) * (-v).exp() for a, v in zip(c[:, 0], y)]
+        lost = Decimal(2) ** -1022 + sum(abs(Decimal(float(a))) * Decimal(2) ** -1020 for a, v in zip(c[:, 0], y) if v > 707)
+        unit = Decimal(2) ** -53
+        bound = sum(abs(v) * (Decimal("0.5") + w / 128) * unit for v, w in zip(t, y)) + max(map(abs, t)) * unit / 4 + abs(sum(t)) * unit + lost
+        assert abs(Decimal(float(g)) - sum(t)) <= bound
 
 
 def test_sincos(fx):
