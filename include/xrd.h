@@ -298,8 +298,9 @@ int xrd_pattern_augmented(xrd_handle* h, const xrd_batch* batch, const xrd_opts*
  * factor; the minimum of four calls) with CUDA events, synchronising `stream`,
  * and keeps the fastest shape in the handle, then picks the enumeration
  * kernels' launch shape (xrd_set_enum_threads) the same way; later calls with opts.tile = -1 use
- * it. Writes the chosen tile, warps and runs (0 or 1) if the pointers are not
- * NULL. Returns after `stream` has been synchronised (every tuning call has
+ * it. XRD_FP64 has one shape (tiles of 32 reflections): for it only the
+ * enumeration is tuned and the handle's shape stays. Writes the handle's tile,
+ * warps and runs (0 or 1) if the pointers are not NULL. Returns after `stream` has been synchronised (every tuning call has
  * finished). Not capturable.
  */
 int xrd_autotune(xrd_handle* h, const xrd_batch* batch, const xrd_opts* opts, const xrd_pattern* out,
@@ -332,7 +333,8 @@ int xrd_unit_rates(xrd_handle* h, double* rates);
 
 /* Set the structure-factor launch shape directly (tile 64 or 128 reflections per
  * warp, 1, 2 or 4 warps per CTA; warps apply to XRD_FP32_PHASEFIX; runs = 1,
- * with tile 128 and XRD_FP32_PHASEFIX only, makes lanes take runs consecutive in l). */
+ * with tile 128 and XRD_FP32_PHASEFIX only, makes lanes take runs consecutive in l).
+ * XRD_FP64 calls take tiles of 32 reflections unless opts.tile says otherwise. */
 int xrd_set_sf_shape(xrd_handle* h, int tile, int warps, int runs);
 
 /*

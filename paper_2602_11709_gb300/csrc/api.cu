@@ -240,15 +240,16 @@ int check_opts(xrd_handle* h, const xrd_opts* o)
     return XRD_OK;
 }
 
-// Launch shape of the structure-factor kernel for this call. Where nobody has chosen one, strided tiles (whose results
-// do not depend on their size): FP64 lanes take one reflection (they would take several one after another); FP32
-// lanes take four, which share an atom's loads and a packed instruction's halves, or two where tiles of 128 would fill
+// Launch shape of the structure-factor kernel for this call. XRD_FP64 takes tiles of 32 reflections, one a lane, whatever
+// shape was chosen for the FP32 kernels (a lane would take several one after another: 1 to 2000 small cells 1.9 to 2.8
+// times as long with tiles of 128). Where nobody has chosen one, FP32 takes strided tiles (whose results do not depend
+// on their size): lanes take four reflections, which share an atom's loads and a packed instruction's halves, or two where tiles of 128 would fill
 // less than half of the resident warps (12 of 24 per SM) and the longest tile sets the time. 24 mixed cells (140 tiles
 // of 128) 30.3 us with four, 21.8 us with two; 256 hexagonal/P1 cells 24.2 and 20.2; 1024 small cells (8500 tiles)
 // 65.2 and 69.2. Rock salt in FP64 (3 tiles of 128): 45 us with four, 20 us with one.
 void sf_shape(const xrd_handle* h, const xrd_opts* o, int64_t cap_refl, int& rb, int& warps, int& runs)
 {
-    if (o->tile == -1 && !h->sf_chosen) {
+    if (o->tile == -1 && (o->precision == XRD_FP64 || !h->sf_chosen)) {
         rb = o->precision == XRD_FP64 ? 1 : (cap_refl / 128 < (int64_t)12 * h->sms ? 2 : 4);
         warps = 2;
         runs = 0;
@@ -898,11 +899,12 @@ int xrd_autotune(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, const xrd
     static const int shapes[9][3] = {{4, 2, 0}, {4, 1, 0}, {4, 4, 0}, {2, 2, 0}, {2, 1, 0},
                                      {2, 4, 0}, {4, 1, 1}, {4, 2, 1}, {4, 4, 1}};
     const bool all = o && o->precision == XRD_FP32_PHASEFIX;
-    const int nshape = all ? 9 : 2;
+    const bool fp64 = o && o->precision == XRD_FP64;  // has one shape (sf_shape): the handle keeps its own
+    const int nshape = all ? 9 : fp64 ? 0 : 2;
     const int keep_rb = h->sf_rb, keep_w = h->sf_warps, keep_runs = h->sf_runs;
     const int keep_prof = h->profiling;
     const bool keep_chosen = h->sf_chosen;
-    h->sf_chosen = true;
+    h->sf_chosen = keep_chosen || !fp64;
     xrd_opts oo = o ? *o : xrd_opts{};
     oo.tile = -1;
     float best = 1e30f;
