@@ -86,7 +86,7 @@ typedef struct {
 typedef struct {
     int64_t n_refl;       /* Friedel-unique reflections of the whole batch (each stands for g and -g) */
     int64_t max_refl;     /* largest Friedel-unique count of one structure */
-    int64_t n_tiles;      /* structure-factor tiles at the tuned tile size */
+    int64_t n_tiles;      /* structure-factor tiles at the tile size a call with ws_bytes takes (runs along l: as if strided) */
     size_t ws_bytes;      /* workspace bytes xrd_pattern_batch needs for this batch and these options */
     size_t ws_grad_bytes; /* workspace bytes xrd_pattern_broadened + xrd_pattern_grad need */
 } xrd_sizes;

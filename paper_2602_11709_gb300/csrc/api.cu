@@ -465,8 +465,8 @@ int xrd_stage_times(xrd_handle* h, float* ms, int n)
     return m;
 }
 
-// Friedel-unique reflection count of every structure (n_struct > 0), on `st` (synchronised): into cnt (host), or, with cnt NULL, their sum, largest and number
-// of tiles of tile_refl reflections into sums[0..2] (the counts stay on the device: their readback and the sums on the
+// Friedel-unique reflection count of every structure (n_struct > 0), on `st` (synchronised): into cnt (host), or, with cnt NULL, their sum, largest and the
+// numbers of tiles of tile_refl and of tile_refl / 2 reflections into sums[0..3] (the counts stay on the device: their readback and the sums on the
 // host kept the GPU waiting). The scratch is the handle's own.
 static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, cudaStream_t st, int64_t* cnt,
                              int64_t* sums, int tile_refl)
@@ -499,7 +499,7 @@ static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* 
     cudaMemsetAsync(a.enum_ctr, 0, 16, st);
     xrd::launch_count_only(a, cnt ? nullptr : h->wbuf + 4, tile_refl, st);
     cudaError_t e = cnt ? cudaMemcpyAsync(cnt, a.refl_cnt, 8 * n, cudaMemcpyDeviceToHost, st)
-                        : cudaMemcpyAsync(sums, h->wbuf + 4, 24, cudaMemcpyDeviceToHost, st);
+                        : cudaMemcpyAsync(sums, h->wbuf + 4, 32, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "reflection count");
     return XRD_OK;
@@ -535,13 +535,16 @@ int xrd_query_sizes(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, xrd_si
         sizes->ws_grad_bytes = layout_grad(0, b->n_atoms, b->zmax, 0).total;
         return XRD_OK;
     }
-    int64_t sums[3] = {};  // reflections, the most of one structure, tiles
-    if ((rc = count_reflections(h, b, o, st, nullptr, sums, 32 * h->sf_rb))) return rc;
+    int64_t sums[4] = {};  // reflections, the most of one structure, tiles
+    int rb_most, rb, warps, runs;
+    sf_shape(h, o, INT64_MAX, rb_most, warps, runs);  // the shape of the largest batches; small ones take half as many
+    if ((rc = count_reflections(h, b, o, st, nullptr, sums, 32 * rb_most))) return rc;
     const int64_t tot = sums[0];
     sizes->n_refl = tot;
     sizes->max_refl = sums[1];
-    sizes->n_tiles = sums[2];
     sizes->ws_bytes = layout(n, b->n_atoms, b->zmax, tot, h->npg > 0).total;
+    sf_shape(h, o, refl_capacity(n, b->n_atoms, b->zmax, sizes->ws_bytes, h->npg > 0), rb, warps, runs);
+    sizes->n_tiles = rb == rb_most ? sums[2] : sums[3];
     sizes->ws_grad_bytes = layout_grad(n, b->n_atoms, b->zmax, tot).total;
     return XRD_OK;
 }

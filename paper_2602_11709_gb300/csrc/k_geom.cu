@@ -750,7 +750,8 @@ struct ScanArgs {
     int32_t* status;
     unsigned long long* work;
     const int* bad;  // structures with an invalid atom become invalid here (or nullptr)
-    unsigned long long* sums;  // not nullptr: no scan, but the counts' sum, largest and tiles into sums[0..2]
+    unsigned long long* sums;  // not nullptr: no scan, but the counts' sum, largest, and tiles of tile_refl and of half as
+                               // many reflections into sums[0..3]
 };
 struct ScanShared {
     long long ws[33];
@@ -924,17 +925,20 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_count(Geo* geo, int n_struc
     if (!last) return;
     __threadfence();
     if (scan.sums) {
-        long long sum = 0, most = 0, tiles = 0, t;
+        long long sum = 0, most = 0, tiles = 0, half = 0, t;
         for (int i = threadIdx.x; i < n_struct; i += blockDim.x) {
             const long long c = __ldcg((const long long*)cnt + i);
             sum += c;
             most = max(most, c);
             tiles += (c + scan.tile_refl - 1) / scan.tile_refl;
+            half += (2 * c + scan.tile_refl - 1) / scan.tile_refl;
         }
         block_prefix_ll(sum, sh.ws, &t);
         if (threadIdx.x == 0) scan.sums[0] = t;
         block_prefix_ll(tiles, sh.ws, &t);
         if (threadIdx.x == 0) scan.sums[2] = t;
+        block_prefix_ll(half, sh.ws, &t);
+        if (threadIdx.x == 0) scan.sums[3] = t;
         const unsigned long long m = block_max_u64(most, (unsigned long long*)sh.ws);
         if (threadIdx.x == 0) scan.sums[1] = m;
         return;

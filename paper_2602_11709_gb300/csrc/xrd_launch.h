@@ -309,7 +309,7 @@ void launch_atoms(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_order(const GeomArgs& a, cudaStream_t st, bool pdl);
 size_t order_parts_bytes(int64_t n);  // bytes of GeomArgs::oparts for n structures (0: one-block order)
 void launch_count(const GeomArgs& a, cudaStream_t st, bool pdl, bool scan);  // scan: and launch_scan_refl's work
-// counts only; with sums, also their sum, largest and tiles of tile_refl into sums[0..2]
+// counts only; with sums, also their sum, largest, and tiles of tile_refl and of half as many reflections into sums[0..3]
 void launch_count_only(const GeomArgs& a, unsigned long long* sums, int tile_refl, cudaStream_t st);
 void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl);
 void launch_work(const GeomArgs& a, unsigned long long* out, cudaStream_t st);  // out: device [3], zeroed

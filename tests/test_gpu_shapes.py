@@ -42,3 +42,20 @@ def test_fp64_shape_stays(gpu_lib, chosen):
             assert got == _ceil(cnt, 64)
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_phase64", "fp32_phasefix"])
+@pytest.mark.parametrize("n", [1, 40, 1024])
+@pytest.mark.parametrize("shape", [None, (64, 2, 0), (128, 2, 0)])
+@pytest.mark.parametrize("tile", [-1, 64, 128])
+def test_sizes_tell_the_tiles_of_a_call(gpu_lib, prec, n, shape, tile):
+    xrd = gpu_lib
+    b, o = synth.small(n=n)
+    h = xrd.Handle(0)
+    try:
+        if shape:
+            h.set_sf_shape(*shape)
+        got, _, sz = _tiles(xrd, h, b, o, prec, tile)
+        assert sz.n_tiles == got
+    finally:
+        h.close()
