@@ -1129,6 +1129,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.refl_off = (int64_t*)(ws + L.refl_off);
     ga.tile_off = (int*)(ws + L.tile_off);
     ga.order = (int*)(ws + L.order);
+    ga.aorder = (int*)(ws + L.aorder);
     ga.atom_bad = (int*)(ws + L.atom_bad);
     ga.atoms_set_geo = 1;  // a structure with an invalid atom has no reflections here
     ga.tile_tab = (int2*)(ws + L.tile_tab);
@@ -1182,7 +1183,6 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     sa.atomx = ga.atomx;
     sa.q = ga.q;
     sa.key = ga.key;
-    sa.aorder = (int*)(ws + L.aorder);
     if (grad) {
         sa.Fx = (float4*)(ws + L.Fx);
         sa.Ig = (float*)(ws + L.Ig);

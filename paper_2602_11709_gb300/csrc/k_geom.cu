@@ -737,6 +737,13 @@ __device__ __forceinline__ int warp_aggregated_slot(int* ctr, int key, bool acti
     return base + __popc(peers & ((1u << lane) - 1u));
 }
 
+// Bins of the order by reflection count, largest first: a quarter octave each, the last for none.
+constexpr int kCountBins = 128;
+__device__ __forceinline__ int count_bin(long long r)
+{
+    return r <= 0 ? kCountBins - 1 : max(kCountBins - 2 - (int)(4.f * log2f((float)r)), 0);
+}
+
 struct ScanArgs {
     const int64_t* run_cnt;
     int tile_refl;
@@ -749,6 +756,8 @@ struct ScanArgs {
     int64_t* totals;
     int32_t* status;
     unsigned long long* work;
+    int* aorder;     // [n] the structures by reflection count, largest first (or nullptr); within a bin the order is
+                     // arbitrary: nothing but the load balance depends on it
     const int* bad;  // structures with an invalid atom become invalid here (or nullptr)
     unsigned long long* sums;  // not nullptr: no scan, but the counts' sum, largest, and tiles of tile_refl and of half as
                                // many reflections into sums[0..3]
@@ -756,7 +765,24 @@ struct ScanArgs {
 struct ScanShared {
     long long ws[33];
     int ccnt[kPostClasses];
+    int bins[kCountBins];
 };
+
+// Exclusive scan of the kCountBins bins by the first warp
+__device__ __forceinline__ void scan_count_bins(int* bins)
+{
+    if (threadIdx.x >= 32) return;
+    constexpr int per = kCountBins / 32;
+    int v[per], sum = 0;
+#pragma unroll
+    for (int j = 0; j < per; j++) sum += v[j] = bins[per * threadIdx.x + j];
+    int run = warp_incl_scan(sum) - sum;
+#pragma unroll
+    for (int j = 0; j < per; j++) {
+        bins[per * threadIdx.x + j] = run;
+        run += v[j];
+    }
+}
 
 // buf: kScanItems * blockDim long longs of shared memory. The counts are read past the L1 cache: the CTA that runs
 // this may be one of the kernel that wrote them.
@@ -777,8 +803,14 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restr
     long long* const ws = sh.ws;
     int* const ccnt = sh.ccnt;
     const int nt = blockDim.x, tid = threadIdx.x, CH = kScanItems * nt;
+    int* const aorder = sa.aorder;
+    int* const bins = sh.bins;
     long long tot;
-    // 1. reflection offsets in structure order, and the status of each structure
+    if (aorder) {
+        for (int b = tid; b < kCountBins; b += nt) bins[b] = 0;
+        __syncthreads();
+    }
+    // 1. reflection offsets in structure order, the status of each structure, and how many have how many reflections
     long long carry = 0, bad = 0;
     for (int base = 0; base < n; base += CH) {
         long long v[kScanItems];
@@ -792,6 +824,7 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restr
                 st[u] = XRD_EINVAL;
                 geo[i].status = XRD_EINVAL;
             }
+            if (aorder && i < n) atomicAdd(&bins[count_bin(v[u])], 1);
         }
         chunk_scan<kScanItems>(v, buf, ws, &tot);
 #pragma unroll
@@ -812,6 +845,7 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restr
     if (over)
         for (int i = tid; i < n; i += nt) status[i] = XRD_ECAPACITY;
     if (tid < kPostClasses) ccnt[tid] = 0;
+    if (aorder) scan_count_bins(bins);
     __syncthreads();
     // 2. tiles and size classes in the largest-first order
     long long tcarry = 0;
@@ -836,6 +870,7 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restr
         for (int u = 0; u < kScanItems; u++) {
             const int p = base + u * nt + tid;
             if (p < n) tile_off[sv[u]] = (int)(tcarry + v[u]);  // first tile of the structure
+            if (aorder && p < n) aorder[atomicAdd(&bins[count_bin(c[u])], 1)] = sv[u];
             if (!over && cls_list) {
                 const int k = post_class(c[u]);
                 const int slot = warp_aggregated_slot(ccnt, k, p < n);
@@ -963,13 +998,15 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_parts(const int64_t*
                                                                   const int64_t* __restrict__ run_cnt,
                                                                   const Geo* __restrict__ geo, int n, int tile_refl,
                                                                   const int* __restrict__ order,
-                                                                  long long* __restrict__ parts)
+                                                                  long long* __restrict__ parts,
+                                                                  int* __restrict__ oparts)
 {
     pdl_enter();
     __shared__ long long ws[33];
-    __shared__ int cc[kPostClasses];
+    __shared__ int cc[kPostClasses], bins[kCountBins];
     const int nt = blockDim.x, tid = threadIdx.x, base = blockIdx.x * kScanItems * nt;
     if (tid < kPostClasses) cc[tid] = 0;
+    if (tid < kCountBins) bins[tid] = 0;
     __syncthreads();
     long long refl = 0, bad = 0, tiles = 0;
 #pragma unroll
@@ -982,6 +1019,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_parts(const int64_t*
             const long long c = cnt[sv];
             tiles += tiles_of(run_cnt, sv, c, tile_refl);
             atomicAdd(&cc[post_class(c)], 1);
+            if (oparts) atomicAdd(&bins[count_bin(c)], 1);
         }
     }
     long long t;
@@ -991,6 +1029,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_parts(const int64_t*
     bad = t;
     block_prefix_ll(tiles, ws, &t);
     tiles = t;
+    if (oparts && tid < kCountBins) oparts[(int64_t)blockIdx.x * kOrderBins + tid] = bins[tid];
     if (tid == 0) {
         long long* o = parts + (int64_t)blockIdx.x * kScanPartWords;
         o[0] = refl;
@@ -1008,13 +1047,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_final(const int64_t*
                                                                   int* __restrict__ cls_list, int* __restrict__ abort_flag,
                                                                   int64_t* __restrict__ totals, int32_t* __restrict__ status,
                                                                   unsigned long long* __restrict__ work,
-                                                                  const long long* __restrict__ parts)
+                                                                  const long long* __restrict__ parts,
+                                                                  const int* __restrict__ oparts, int* __restrict__ aorder)
 {
     pdl_enter();
     __shared__ long long ws[33];
     __shared__ __align__(16) long long buf[kScanItems * kScanThreads];
     __shared__ long long pre[kScanPartWords], all[kScanPartWords];
-    __shared__ int ccnt[kPostClasses];
+    __shared__ int ccnt[kPostClasses], bins[kCountBins];
     const int nt = blockDim.x, tid = threadIdx.x, b = blockIdx.x, base = b * kScanItems * nt;
     const int nch = gridDim.x;
     if (tid < kScanPartWords) {  // sums of the chunks before this one, and of all chunks
@@ -1028,7 +1068,22 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_final(const int64_t*
         all[tid] = a;
     }
     if (tid < kPostClasses) ccnt[tid] = 0;
+    int before = 0;  // structures of this thread's bin in the chunks before this one
+    if (aorder && tid < kCountBins) {
+        int a = 0;
+        for (int c = 0; c < nch; c++) {
+            const int v = oparts[(int64_t)c * kOrderBins + tid];
+            before += c < b ? v : 0;
+            a += v;
+        }
+        bins[tid] = a;
+    }
     __syncthreads();
+    if (aorder) {
+        scan_count_bins(bins);
+        __syncthreads();
+        if (tid < kCountBins) bins[tid] += before;  // read after the scans below
+    }
     const long long total = all[0];
     const bool over = total > cap_refl;
     long long v[kScanItems], tot;
@@ -1064,6 +1119,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl_final(const int64_t*
     for (int u = 0; u < kScanItems; u++) {
         const int p = base + u * nt + tid;
         if (p < n) tile_off[sv[u]] = (int)(pre[2] + v[u]);
+        if (aorder && p < n) aorder[atomicAdd(&bins[count_bin(c[u])], 1)] = sv[u];
         if (!over && cls_list) {
             const int k = post_class(c[u]);
             const int slot = warp_aggregated_slot(ccnt, k, p < n);
@@ -1355,7 +1411,7 @@ static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
 static ScanArgs scan_args(const GeomArgs& a)
 {
     return ScanArgs{a.run_cnt, a.runs_mode ? 0 : 32 * a.rb, a.cap_refl, a.refl_off, a.tile_off, a.order, a.cls_list,
-                    a.abort_flag, a.totals, a.status, a.work, a.atoms_set_geo ? a.atom_bad : nullptr, nullptr};
+                    a.abort_flag, a.totals, a.status, a.work, a.aorder, a.atoms_set_geo ? a.atom_bad : nullptr, nullptr};
 }
 
 static void count_launch(const GeomArgs& a, const ScanArgs& sa, cudaStream_t st, bool pdl, bool last)
@@ -1401,10 +1457,10 @@ void launch_scan_refl(const GeomArgs& a, cudaStream_t st, bool pdl)
         return;
     }
     launch_k(pdl, k_scan_refl_parts, nch, kScanThreads, st, a.refl_cnt, a.run_cnt, a.geo, a.n_struct, tile_refl,
-             (const int*)a.order, a.parts);
+             (const int*)a.order, a.parts, a.aorder ? a.oparts : (int*)nullptr);
     launch_k(true, k_scan_refl_final, nch, kScanThreads, st, a.refl_cnt, a.run_cnt, a.geo, a.n_struct, tile_refl,
              a.cap_refl, a.refl_off, a.tile_off, (const int*)a.order, a.cls_list, a.abort_flag, a.totals, a.status,
-             a.work, (const long long*)a.parts);
+             a.work, (const long long*)a.parts, (const int*)a.oparts, a.aorder);
 }
 
 void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl)

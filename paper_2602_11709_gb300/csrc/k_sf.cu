@@ -382,32 +382,6 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
     return imax;
 }
 
-// Structures by reflection count, largest first (buckets of a quarter octave), by one CTA beside the tiles of the
-// others: the profile kernels that follow give every structure a CTA and start with the largest. cnt: kCountBuckets
-// ints of shared memory. The order within a bucket is arbitrary; nothing but the load balance depends on it.
-constexpr int kCountBuckets = 128;
-__device__ void order_by_count(const SfArgs& a, int* cnt)
-{
-    for (int i = threadIdx.x; i < kCountBuckets; i += blockDim.x) cnt[i] = 0;
-    __syncthreads();
-    auto bucket = [&](int s) {
-        const int64_t R = a.refl_off[s + 1] - a.refl_off[s];
-        return R <= 0 ? 0 : min(kCountBuckets - 1, 1 + (int)(4.f * log2f((float)R)));
-    };
-    for (int s = threadIdx.x; s < a.n_struct; s += blockDim.x) atomicAdd(&cnt[bucket(s)], 1);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int b = kCountBuckets - 1; b >= 0; b--) {
-            const int c = cnt[b];
-            cnt[b] = acc;
-            acc += c;
-        }
-    }
-    __syncthreads();
-    for (int s = threadIdx.x; s < a.n_struct; s += blockDim.x) a.aorder[atomicAdd(&cnt[bucket(s)], 1)] = s;
-}
-
 // Persistent CTAs; every warp takes tiles of 32 runs (one per lane) from a
 // queue in largest-first order (tiles of the structures with the most atoms
 // first). A structure's atoms stay staged in the warp's shared memory while its
@@ -428,10 +402,6 @@ __global__ void __launch_bounds__(32 * WARPS,
     __shared__ float2 sstep[RUNS ? WARPS : 1][RUNS ? kSfChunk : 1];
     __shared__ int4 slo[PREC == XRD_FP32_PHASE64 ? WARPS : 1][PREC == XRD_FP32_PHASE64 ? kSfChunk : 1];
     extern __shared__ CoefPair scoef[];  // [zmax + 1]
-    if (a.aorder && blockIdx.x == gridDim.x - 1) {
-        __shared__ int cnt[kCountBuckets];
-        order_by_count(a, cnt);
-    }
     if (*a.abort_flag) return;
     const int ntiles = a.tile_off[a.n_struct];
     if ((int)blockIdx.x >= ntiles) return;  // the CTAs before this one already have a tile each
