@@ -271,7 +271,8 @@ typedef struct {
  * Lorentzian is summed over every grid point (no window), beyond 256 points by
  * interpolation of a run's sum (below 1e-7 of it); a reflection's
  * Gaussian is skipped only on runs of 256 consecutive grid points where it
- * stays below 2^-40 of its peak (x^2 >= 40). grid.fwhm is ignored; grid.n_pts <= 2^22
+ * stays below 2^-40 of its peak (x^2 >= 40). A structure's row does not depend on
+ * the batch it is in. grid.fwhm is ignored; grid.n_pts <= 2^22
  * and every 2-theta in [tt_min, tt_max] lies within 2^22 dt of t0.
  * opts.precision must be XRD_FP32_PHASEFIX; rel_cutoff, scaled and tt_tol do
  * not enter the result (they are validated as for xrd_pattern_batch). y is

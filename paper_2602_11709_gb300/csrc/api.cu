@@ -1259,7 +1259,6 @@ int xrd_pattern_augmented(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     profile_front(h, b, o, L, ws, cap_refl, status, totals, st, nullptr);
     xrd::AugArgs a{};
     a.n_struct = (int)n;
-    a.sms = h->sms;
     a.n_pts = grid->n_pts;
     a.t0 = grid->t0;
     a.dt = grid->dt;

@@ -276,7 +276,7 @@ struct GradArgs {
 };
 
 struct AugArgs {
-    int n_struct, n_pts, sms;
+    int n_struct, n_pts;
     double t0, dt, inv_dt;
     float l2h, l2l;  // lambda^2 / 4 as two floats
     const TTab* ttab;
