@@ -1056,6 +1056,7 @@ static xrd::GradArgs grad_args(xrd_handle* h, const xrd_batch* b, const xrd_grid
     a.n_struct = b->n_struct;
     a.n_pts = g->n_pts;
     a.W = W;
+    a.sms = h->sms;
     a.n_atoms = b->n_atoms;
     a.t0 = g->t0;
     a.dt = g->dt;

@@ -59,9 +59,47 @@ __device__ __forceinline__ double cluster_load(const double* p, int rank)
 // loads). The cells themselves come from the structure-factor kernel, whose FP64 unit is free, where 13 FP64 operations
 // a reflection bound this one. 512 cells of 8 to 128 atoms on 4096 points: 127 us with 256 threads a structure, the
 // permutation and the cells formed here, 33 us now (and 6 us more in the structure-factor kernel).
-constexpr int kBroadenThreads = 1024;
+// Threads: 1024 while the structures are few enough that the largest sets the time, up to kBroadenFew a SM; beyond,
+// 512, since the short phases between barriers of more CTAs overlap (512 cells of 8-128 atoms on 4096 points 310 us a step
+// with 1024 and 321 with 512; 1500 cells of 3 atoms on 257 points 286 and 258, 100 000 one-atom cells 6.5 and 5.9 ms).
+constexpr int kBroadenMaxThreads = 1024;
+constexpr int kBroadenFew = 4;
 
-__global__ void __launch_bounds__(kBroadenThreads) k_broaden(const GradArgs a)
+// PER consecutive points a thread, whose windows share most reflections where these are dense (16 cells of 200-2000 atoms
+// on 4096 points 14.2 ms a step with four, 14.5 with one); on a grid of fewer points than that needs, four left most
+// threads idle (3000 one-atom cells on 257 points 1.16 ms a step, 0.97 with one).
+template <int PER>
+__device__ __forceinline__ void broaden_gather(int n_pts, int W, float dt, float cg, const int* bins,
+                                               const int* __restrict__ sb, const float2* __restrict__ sda,
+                                               float* __restrict__ yo)
+{
+    for (int k0 = PER * threadIdx.x; k0 < n_pts; k0 += PER * blockDim.x) {
+        float acc[PER];
+        int lo[PER], hi[PER];
+#pragma unroll
+        for (int j = 0; j < PER; j++) {
+            const int k = min(k0 + j, n_pts - 1);
+            acc[j] = 0.f;
+            lo[j] = k ? bins[k - 1] : 0;
+            hi[j] = bins[k + 2 * W + 1];  // cells c = b + W + 1 of k .. k + 2 W + 1
+        }
+        for (int i = lo[0]; i < hi[PER - 1]; i++) {
+            const float2 v = sda[i];
+            const int b = sb[i];
+#pragma unroll
+            for (int j = 0; j < PER; j++) {
+                const float u = ((float)(k0 + j - b) - v.x) * dt;
+                const float t = fmaf(v.y, ex2_approx(-u * u * cg), acc[j]);
+                if (i >= lo[j] && i < hi[j]) acc[j] = t;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < PER; j++)
+            if (k0 + j < n_pts) yo[k0 + j] = acc[j];
+    }
+}
+
+__global__ void __launch_bounds__(kBroadenMaxThreads) k_broaden(const GradArgs a)
 {
     pdl_enter();
     extern __shared__ int bins[];  // cell counts, then offsets; cells c = b + W + 1 in [0, nb)
@@ -116,31 +154,8 @@ __global__ void __launch_bounds__(kBroadenThreads) k_broaden(const GradArgs a)
     __syncthreads();
     // gather: grid point k sees the reflections of cells b in [k - W - 1, k + W]
     const float dt = (float)a.dt;
-    constexpr int kPer = 4;  // consecutive points a thread takes: their windows share most reflections
-    for (int k0 = kPer * threadIdx.x; k0 < a.n_pts; k0 += kPer * blockDim.x) {
-        float acc[kPer];
-        int lo[kPer], hi[kPer];
-#pragma unroll
-        for (int j = 0; j < kPer; j++) {
-            const int k = min(k0 + j, a.n_pts - 1);
-            acc[j] = 0.f;
-            lo[j] = k ? bins[k - 1] : 0;
-            hi[j] = bins[k + 2 * W + 1];  // cells c = b + W + 1 of k .. k + 2 W + 1
-        }
-        for (int i = lo[0]; i < hi[kPer - 1]; i++) {
-            const float2 v = sda[i];
-            const int b = sb[i];
-#pragma unroll
-            for (int j = 0; j < kPer; j++) {
-                const float u = ((float)(k0 + j - b) - v.x) * dt;
-                const float t = fmaf(v.y, ex2_approx(-u * u * cg), acc[j]);
-                if (i >= lo[j] && i < hi[j]) acc[j] = t;
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < kPer; j++)
-            if (k0 + j < a.n_pts) yo[k0 + j] = acc[j];
-    }
+    if (a.n_pts >= 4 * (int)blockDim.x) broaden_gather<4>(a.n_pts, W, dt, cg, bins, sb, sda, yo);
+    else broaden_gather<1>(a.n_pts, W, dt, cg, bins, sb, sda, yo);
 }
 
 // ---------------------------------------------------------------- backward: per reflection + lattice
@@ -274,7 +289,7 @@ __global__ void __launch_bounds__(kReflThreads) k_grad_refl(const GradArgs a)
 // P = 2 and up to 1300 terms in a row. So the four warps form the terms of a stage of reflections side by side, two to a packed FP32
 // operation, into shared memory, and then add them in order, a warp per component x, y, z, B: six instructions a term
 // on the chain instead of 55. 512 cells of 8 to 128 atoms: one 256-thread CTA a structure, a thread a sum, 203 us; a
-// warp a CTA forming its own terms 160 us; 123 us now. The sums are the same bits in each form.
+// warp a CTA forming its own terms 160 us; 123 us now. The sums are the same bits in each form (k_grad_atoms_few too).
 constexpr int kAtomCluster = 4;
 constexpr int kAtomWarps = 8;
 constexpr int kAtomCtaSums = 64;  // four warps for each 32
@@ -399,6 +414,98 @@ __global__ void __launch_bounds__(32 * kAtomWarps, 4) k_grad_atoms(const GradArg
     }
 }
 
+// The same sums for batches of few atoms a structure (kAtomFew on average): one CTA per structure, a thread a sum, which
+// forms its own terms. With few atoms a structure's 256 sums are of few terms each, and what a cluster shares (staging by
+// every CTA, three barriers a stage, the exchange) outweighs the shorter sums: a step of 3000 cells of 8 atoms on 1000
+// points 556 us with clusters and 442 here, of one atom 1026 and 710, 50 000 cells of 4 atoms 4.65 and 2.91 ms; at 16
+// cells of 8 atoms, or one, equal; 512 cells of 8 to 128 atoms 311 us with clusters and 411 here, 5000 cells of 27 atoms on
+// average and up to 500 1.33 and 1.57 ms.
+constexpr int kAtomFew = 8;
+
+__global__ void __launch_bounds__(kAtomSums) k_grad_atoms_few(const GradArgs a)
+{
+    pdl_enter();
+    __shared__ uint32_t skey[kAtomChunkRefl];
+    __shared__ float ss2[kAtomChunkRefl], sU[kAtomChunkRefl], sV[kAtomChunkRefl];
+    __shared__ float4 red[kAtomSums];
+    const int s = a.order[blockIdx.x], t = threadIdx.x;
+    const int64_t j0 = a.atom_off[s], j1 = a.atom_off[s + 1];
+    const int N = (int)(j1 - j0);
+    const bool ok = !*a.abort_flag && a.geo[s].status == XRD_OK;
+    if (!ok) {
+        if (j0 < 0 || j1 > a.n_atoms || N < 0) return;  // invalid atom offsets: touch nothing
+        for (int i = t; i < N; i += kAtomSums) {
+            a.d_frac[3 * (j0 + i)] = a.d_frac[3 * (j0 + i) + 1] = a.d_frac[3 * (j0 + i) + 2] = 0.f;
+            a.d_B[j0 + i] = 0.f;
+        }
+        return;
+    }
+    const int64_t rb = a.refl_off[s];
+    const int nr = (int)(a.refl_off[s + 1] - rb);
+    const int Nc = min(N, kAtomSums);
+    if (Nc == 0) return;
+    const int P = kAtomSums / Nc, Pn = min(P, nr);
+    const int rho = t / Nc, al = t % Nc;
+    for (int ac0 = 0; ac0 < N; ac0 += Nc) {
+        const int at_i = ac0 + al;
+        const bool valid = rho < P && at_i < N;
+        Atom32 at{};
+        Coef32 c{};
+        if (valid) {
+            at = a.atom32[j0 + at_i];
+            c = a.coef32[at.z];
+        }
+        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int r0 = 0; r0 < nr; r0 += kAtomChunkRefl) {
+            const int nc = min(kAtomChunkRefl, nr - r0);
+            __syncthreads();
+            for (int i = t; i < nc; i += kAtomSums) {
+                skey[i] = a.key[rb + r0 + i];
+                ss2[i] = d2f_pos(a.q[rb + r0 + i]) * 0.25f;
+                sU[i] = a.U[rb + r0 + i];
+                sV[i] = a.V[rb + r0 + i];
+            }
+            __syncthreads();
+            for (int i = valid ? rho : nc; i < nc; i += P) {
+                const uint32_t key = skey[i];
+                const int h = hkl_h(key), k = hkl_k(key), l = hkl_l(key);
+                const uint32_t Ph = (uint32_t)h * at.X + (uint32_t)k * at.Y + (uint32_t)l * at.Z;
+                float sn, cs;
+                __sincosf((float)(int32_t)Ph * 1.4629180792671596e-09f, &sn, &cs);
+                const float s2 = ss2[i], U = sU[i], V = sV[i];
+                const float e0 = ex2_approx(c.bl[0] * s2), e1 = ex2_approx(c.bl[1] * s2);
+                const float e2 = ex2_approx(c.bl[2] * s2), e3 = ex2_approx(c.bl[3] * s2);
+                const float f = fmaf(s2, fmaf(c.a[0], e0, fmaf(c.a[1], e1, fmaf(c.a[2], e2, c.a[3] * e3))), at.zf);
+                const float wt = f * ex2_approx(fmaf(at.nb, s2, at.lo));
+                const float t1 = wt * fmaf(V, cs, -U * sn), t2 = wt * fmaf(U, cs, V * sn);
+                g.x = fmaf((float)h, t1, g.x);
+                g.y = fmaf((float)k, t1, g.y);
+                g.z = fmaf((float)l, t1, g.z);
+                g.w = fmaf(s2, t2, g.w);
+            }
+        }
+        red[t] = g;
+        __syncthreads();
+        if (rho == 0 && at_i < N) {
+            float sx = 0.f, sy = 0.f, sz = 0.f, sb = 0.f;
+            for (int p = 0; p < Pn; p++) {
+                const float4 v = red[p * Nc + al];
+                sx += v.x;
+                sy += v.y;
+                sz += v.z;
+                sb += v.w;
+            }
+            const int64_t o = j0 + at.src;
+            const float fourpi = (float)(4.0 * kPi);
+            a.d_frac[3 * o] = fourpi * sx;
+            a.d_frac[3 * o + 1] = fourpi * sy;
+            a.d_frac[3 * o + 2] = fourpi * sz;
+            a.d_B[o] = -2.f * sb;
+        }
+        __syncthreads();
+    }
+}
+
 size_t broaden_smem_bytes(int n_pts, int W) { return sizeof(int) * (size_t)(n_pts + 2 * W + 3); }
 
 void launch_broaden(const GradArgs& a, cudaStream_t st)
@@ -406,7 +513,7 @@ void launch_broaden(const GradArgs& a, cudaStream_t st)
     if (a.n_struct <= 0) return;
     const size_t smem = broaden_smem_bytes(a.n_pts, a.W);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_broaden, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(k_broaden, a.n_struct, kBroadenThreads, smem, st, a);
+    launch_pdl(k_broaden, a.n_struct, a.n_struct <= kBroadenFew * a.sms ? kBroadenMaxThreads : kBroadenMaxThreads / 2, smem, st, a);
 }
 
 template <typename K>
@@ -431,7 +538,8 @@ void launch_grad(const GradArgs& a, cudaStream_t st)
 {
     if (a.n_struct <= 0) return;
     launch_clusters(k_grad_refl, a, kReflCluster, kReflThreads, false, st);
-    launch_clusters(k_grad_atoms, a, kAtomCluster, 32 * kAtomWarps, true, st);
+    if (a.n_atoms <= (int64_t)kAtomFew * a.n_struct) launch_pdl(k_grad_atoms_few, a.n_struct, kAtomSums, 0, st, a);
+    else launch_clusters(k_grad_atoms, a, kAtomCluster, 32 * kAtomWarps, true, st);
 }
 
 }  // namespace xrd

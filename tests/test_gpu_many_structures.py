@@ -27,8 +27,8 @@ def _profiles(xrd, h, b):
     out = [new(N, 3), new(N), new(n, 6)]
     h.pattern_grad(db, co, cg, g, *out, ws)
     assert not status.any()
-    per = N // n
-    return [t.cpu().numpy().reshape(n, -1) for t in (ya, y, out[0].reshape(n, 3 * per), out[1].reshape(n, per), out[2])]
+    split = lambda v: [v[b.atom_off[s]:b.atom_off[s + 1]] for s in range(n)]  # noqa: E731
+    return [ya.cpu().numpy(), y.cpu().numpy(), split(out[0].cpu().numpy()), split(out[1].cpu().numpy()), out[2].cpu().numpy()]
 
 
 @pytest.mark.parametrize("n", [300, 3000, 9000])
@@ -46,7 +46,26 @@ def test_rows_of_a_large_batch(gpu_lib, n, atoms):
         rows = np.concatenate([np.arange(0, 40), np.arange(n - 60, n)])
         part = _profiles(gpu_lib, h, b.subset(rows))
         for w, p in zip(whole, part):
-            assert np.isfinite(w).all()
-            assert np.array_equal(w[rows], p)
+            assert all(np.isfinite(v).all() for v in w)
+            assert all(np.array_equal(w[s], v) for s, v in zip(rows, p))
+    finally:
+        h.close()
+
+
+def test_few_atoms_on_average(gpu_lib):
+    """Batches of up to 8 atoms a structure on average form the atoms' sums in one CTA, others in clusters: the same bits, for
+    structures of any size among them."""
+    rng = np.random.default_rng(11)
+    counts = [1, 2, 5, 8, 9, 31, 64, 65, 128, 200, 256, 257, 300]
+    cells = [synth.random_cell(rng, c, edge=(3.0, 8.0)) for c in counts]
+    cells.append(synth.random_cell(rng, 3, edge=(0.5, 0.6)))  # no reflections
+    many = synth.concat(cells + [synth.random_cell(rng, 1, edge=(3.0, 5.0)) for _ in range(300)])
+    assert many.n_atoms <= 8 * many.n_struct
+    h = gpu_lib.Handle(0)
+    try:
+        whole = _profiles(gpu_lib, h, many)
+        part = _profiles(gpu_lib, h, many.subset(np.arange(len(cells))))
+        for w, p in zip(whole, part):
+            assert all(np.array_equal(w[s], v) for s, v in enumerate(p))
     finally:
         h.close()
