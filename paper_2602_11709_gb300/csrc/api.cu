@@ -48,7 +48,7 @@ constexpr int kRunsPerTileHost = xrd::kRunsPerTile;  // structure-factor tile: 3
 constexpr int kFlagBytes = 256;
 constexpr int kWorkOffset = 64;
 constexpr int kRefinedOffset = 96;
-constexpr int kQueryParts = 16384;  // enumeration parts of a reflection count outside a call
+constexpr int kQueryParts = 65536;  // enumeration parts of a reflection count outside a call
 constexpr int kStages = 9;
 constexpr int kSfStage = 5;      // index of the structure-factor stage
 constexpr int kRefineStage = 6;  // index of the re-evaluation stage
@@ -296,6 +296,9 @@ void radii(const xrd_opts* o, double& r2min, double& r2max, double& rmax)
     rmax = std::sqrt(r2max);
 }
 
+// enumeration parts that a free part of the workspace holds (16 bytes each)
+int part_room(size_t bytes) { return (int)std::min<size_t>(bytes / 16, (size_t)1 << 29); }
+
 xrd::GeomArgs geom_args(const xrd_batch* b, const xrd_opts* o, const Layout& L, char* ws, int64_t cap_refl,
                         int64_t* totals, int32_t* status, int rb)
 {
@@ -330,9 +333,11 @@ xrd::GeomArgs geom_args(const xrd_batch* b, const xrd_opts* o, const Layout& L, 
     g.cls_list = (int*)(ws + L.cls_list);
     g.abort_flag = (int*)(ws + L.flags);
     g.enum_ctr = g.abort_flag + 26;
-    g.part_tab = (int2*)(ws + L.st_q);  // free until the post-processing
-    g.part_cnt = (int2*)(ws + L.st_I);
-    g.part_cap = (int)std::min<int64_t>(cap_refl, INT32_MAX / 2);
+    // everything between the intensities and the staging is free until the structure factor: room for four parts a
+    // reflection (a shell of few reflections has many columns)
+    g.part_cap = part_room(L.parts - L.I);
+    g.part_tab = (int2*)(ws + L.I);
+    g.part_cnt = g.part_tab + g.part_cap;
     g.totals = totals;
     g.status = status;
     g.q = (double*)(ws + L.q);
@@ -1136,9 +1141,9 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.tile_tab = (int2*)(ws + L.tile_tab);
     ga.abort_flag = (int*)(ws + L.flags);
     ga.enum_ctr = ga.abort_flag + 26;
-    ga.part_tab = (int2*)(ws + L.Fx);  // 16 bytes a reflection, free until the structure factor
-    ga.part_cnt = ga.part_tab + cap_refl;
-    ga.part_cap = (int)std::min<int64_t>(cap_refl, INT32_MAX / 2);
+    ga.part_cap = part_room(L.aorder - L.Fx);  // free until the structure factor
+    ga.part_tab = (int2*)(ws + L.Fx);
+    ga.part_cnt = ga.part_tab + ga.part_cap;
     ga.totals = totals;
     ga.status = status;
     ga.q = (double*)(ws + L.q);

@@ -145,8 +145,6 @@ __global__ void k_prep(const double* __restrict__ lattice, int n, double rmax, G
 // 8 lanes per structure up to this many structures (latency-bound), one above (throughput-bound)
 constexpr int kPrepWideMax = 8192;
 
-static int enum_part_cols(int n_struct);
-
 // f(s) coefficients in the form the FP32 loops use (exp2 with the scale folded
 // in) and, for the accurate re-evaluation, (a_i, b_i) as two floats each
 // (cdd[4 z + i] = (a hi, a lo, b hi, b lo); skipped when cdd is null).
@@ -493,14 +491,23 @@ __device__ __forceinline__ int warp_sum_int(int v)
 // about the time of part_cols / 32 steps of 32 columns, so a batch of few large cells, or one cell, fills the part.
 // Measured with one warp or one CTA a structure before: the 50 A cell of 679 000 reflections 0.25 ms to count and
 // 1.53 ms to emit, 256 cells of 15-40 A 0.13 and 1.37 ms; now 6 and 32 us, 17 and 106 us. 100 000 mixed cells in parts of
-// 512 columns 0.21 and 0.72 ms, of 128 columns 0.19 and 0.55 ms; 5000 of them 45 and 153 us, and 20 and 64 us.
-// Items are claimed from a counter, the parts first: kClaim structures (or one part) at a time.
+// 512 columns 0.21 and 0.72 ms, of 128 columns 0.19 and 0.55 ms; 5000 of them 45 and 153 us, and 20 and 64 us. Thin shells
+// are where room runs out: 3000 cells of 20-30 A, 0.01 degrees of 2-theta, 12 000 reflections, 200 us a call with a warp a
+// structure, 262 with room for a part a reflection, 173 with room for four; 2047 of them 177, 202 with narrow parts for some
+// of them, 143 with wide ones for all.
+// Items are claimed from a counter, the parts first: kClaimWide structures (or one part) at a time.
 constexpr int kEnumMaxThreads = 1024;
-constexpr int kClaimWide = 2;         // structures a claim takes in a batch of at least kWideBatch structures
+constexpr int kClaimWide = 2;         // structures a claim takes in a batch of at least kClaimBatch, many for every warp
+constexpr int kClaimBatch = 32768;    // (below, a warp with two structures that found no room is the last one to end)
 constexpr int kWideBatch = 2048;      // enough structures to fill the GPU by themselves: parts of four chunks, which
 constexpr int kPartColsWide = 128;    // bound the tail; below, every chunk of 32 columns is an item, since a warp's chunks
 constexpr int kPartColsNarrow = 32;   // are a serial chain of about 5 us each
-static int enum_part_cols(int n_struct) { return n_struct >= kWideBatch ? kPartColsWide : kPartColsNarrow; }
+constexpr int kPartRoom = 64;         // unless there is room for fewer parts a structure: wide ones then, since a structure
+                                      // that finds no room is one item, and the last one to end
+static int enum_part_cols(int n_struct, int part_cap)
+{
+    return n_struct >= kWideBatch || part_cap < (int64_t)kPartRoom * n_struct ? kPartColsWide : kPartColsNarrow;
+}
 
 struct EnumItems {
     int nparts, n_struct, claim;
@@ -524,7 +531,7 @@ struct EnumItems {
 
 __device__ __forceinline__ EnumItems enum_items(int n_struct, const int* part_ctr, int part_cap, int* ctr)
 {
-    return EnumItems{min(*part_ctr, part_cap), n_struct, n_struct >= kWideBatch ? kClaimWide : 1, ctr};
+    return EnumItems{min(*part_ctr, part_cap), n_struct, n_struct >= kClaimBatch ? kClaimWide : 1, ctr};
 }
 
 // The structure and the columns [c0, c1) of an item (none where bad says so); false where there is nothing to do (a structure that its
@@ -1295,7 +1302,7 @@ static void launch_k(bool pdl, void (*k)(P...), dim3 grid, dim3 block, cudaStrea
 
 static EnumParts enum_parts(const GeomArgs& a)
 {
-    return EnumParts{a.enum_ctr + kPartCtr, enum_part_cols(a.n_struct), a.part_cap, a.part_tab, a.refl_cnt, a.run_cnt};
+    return EnumParts{a.enum_ctr + kPartCtr, enum_part_cols(a.n_struct, a.part_cap), a.part_cap, a.part_tab, a.refl_cnt, a.run_cnt};
 }
 
 static void prep_launch(bool pdl, const GeomArgs& a, cudaStream_t st)
@@ -1422,7 +1429,7 @@ static void count_launch(const GeomArgs& a, const ScanArgs& sa, cudaStream_t st,
     auto go = [&](auto launch) {
         launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.refl_cnt,
                a.run_cnt, a.enum_ctr, (const int*)(a.enum_ctr + kPartCtr), (const int2*)a.part_tab, a.part_cnt,
-               a.part_cap, enum_part_cols(a.n_struct), sa, last ? a.enum_ctr + kDoneCtr : (int*)nullptr, sa.bad);
+               a.part_cap, enum_part_cols(a.n_struct, a.part_cap), sa, last ? a.enum_ctr + kDoneCtr : (int*)nullptr, sa.bad);
     };
     if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });
     else go([&](auto... v) { k<<<grid, a.enum_threads, smem, st>>>(v...); });
@@ -1473,7 +1480,7 @@ void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl)
         launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, 32 * a.rb,
                (const int64_t*)a.refl_off, (const int64_t*)a.run_cnt, (const int*)a.abort_flag, a.q, a.key, a.runs,
                (const int*)a.tile_off, a.tile_tab, a.enum_ctr + 1, (const int*)(a.enum_ctr + kPartCtr),
-               (const int2*)a.part_tab, (const int2*)a.part_cnt, a.part_cap, enum_part_cols(a.n_struct));
+               (const int2*)a.part_tab, (const int2*)a.part_cnt, a.part_cap, enum_part_cols(a.n_struct, a.part_cap));
     };
     if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });
     else go([&](auto... v) { k<<<grid, a.enum_threads, smem, st>>>(v...); });
