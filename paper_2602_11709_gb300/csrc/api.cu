@@ -43,7 +43,7 @@ namespace {
 constexpr int kRunsPerTileHost = xrd::kRunsPerTile;  // structure-factor tile: 32 runs (one per lane)
 // flags area, zeroed at the start of every call: flag words (see GeomArgs::abort_flag), the
 // structure-factor work counters (3 x 64 bit) at byte kWorkOffset, the re-evaluation's
-// reflection count (64 bit) at kRefinedOffset, the enumeration's counters at ints 26 to 29 and the post
+// reflection count (64 bit) at kRefinedOffset, the enumeration's counters at ints 26 to 30 and the post
 // class counts and work counters at ints kFlagClsCnt and kFlagClsNext
 constexpr int kFlagBytes = 256;
 constexpr int kWorkOffset = 64;
@@ -477,7 +477,7 @@ static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* 
                              int64_t* sums, int tile_refl)
 {
     const int64_t n = b->n_struct;
-    const size_t need = al(sizeof(xrd::Geo) * n) + al(8 * n) + al(16) + 2 * al(8 * kQueryParts);
+    const size_t need = al(sizeof(xrd::Geo) * n) + al(8 * n) + al(32) + 2 * al(8 * kQueryParts);
     if (h->qbuf_bytes < need) {
         if (h->qbuf) cudaFree(h->qbuf);
         h->qbuf = nullptr;
@@ -496,12 +496,12 @@ static int count_reflections(xrd_handle* h, const xrd_batch* b, const xrd_opts* 
     a.geo = (xrd::Geo*)((char*)h->qbuf + L.geo);
     a.refl_cnt = (int64_t*)((char*)h->qbuf + L.refl_cnt);
     a.enum_ctr = (int*)((char*)h->qbuf + L.refl_cnt + al(8 * n));  // the counting kernel's claim counter
-    a.part_tab = (int2*)((char*)a.enum_ctr + al(16));
+    a.part_tab = (int2*)((char*)a.enum_ctr + al(32));
     a.part_cnt = (int2*)((char*)a.part_tab + al(8 * kQueryParts));
     a.part_cap = kQueryParts;
     a.enum_threads = 256;
     a.sms = h->sms;
-    cudaMemsetAsync(a.enum_ctr, 0, 16, st);
+    cudaMemsetAsync(a.enum_ctr, 0, 32, st);
     xrd::launch_count_only(a, cnt ? nullptr : h->wbuf + 4, tile_refl, st);
     cudaError_t e = cnt ? cudaMemcpyAsync(cnt, a.refl_cnt, 8 * n, cudaMemcpyDeviceToHost, st)
                         : cudaMemcpyAsync(sums, h->wbuf + 4, 32, cudaMemcpyDeviceToHost, st);

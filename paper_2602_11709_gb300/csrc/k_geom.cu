@@ -120,10 +120,12 @@ __device__ __forceinline__ void prep_thread(int t, const double* __restrict__ la
             int pbase = -1;
             const int ncol = H < 0 ? 0 : (K + 1) + H * (2 * K + 1);
             if (ncol > ep.cols) {
-                const int np = (ncol + ep.cols - 1) / ep.cols, b = atomicAdd(ep.ctr, np);
-                const bool room = b >= 0 && b <= ep.cap - np;
-                if (room) pbase = b;
-                for (int i = 0; i < np && b >= 0 && b + i < ep.cap; i++) ep.tab[b + i] = make_int2(room ? s : -1, i);
+                const int np = (ncol + ep.cols - 1) / ep.cols;
+                // 64 bits: up to 4088 parts a structure, room or not
+                const long long b = (long long)atomicAdd(ep.ctr, (unsigned long long)np);
+                const bool room = b <= ep.cap - np;
+                if (room) pbase = (int)b;
+                for (int i = 0; i < np && b + i < ep.cap; i++) ep.tab[b + i] = make_int2(room ? s : -1, i);
                 if (room) {
                     ep.cnt[s] = 0;
                     if (ep.run_cnt) ep.run_cnt[s] = 0;
@@ -529,9 +531,9 @@ struct EnumItems {
     }
 };
 
-__device__ __forceinline__ EnumItems enum_items(int n_struct, const int* part_ctr, int part_cap, int* ctr)
+__device__ __forceinline__ EnumItems enum_items(int n_struct, const unsigned long long* part_ctr, int part_cap, int* ctr)
 {
-    return EnumItems{min(*part_ctr, part_cap), n_struct, n_struct >= kClaimBatch ? kClaimWide : 1, ctr};
+    return EnumItems{(int)min(*part_ctr, (unsigned long long)part_cap), n_struct, n_struct >= kClaimBatch ? kClaimWide : 1, ctr};
 }
 
 // The structure and the columns [c0, c1) of an item (none where bad says so); false where there is nothing to do (a structure that its
@@ -623,7 +625,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_emit(const Geo* __restrict_
                                                           const int* __restrict__ abort_flag, double* __restrict__ q,
                                                           uint32_t* __restrict__ key, int* __restrict__ runs,
                                                           const int* __restrict__ tile_off, int2* __restrict__ tile_tab,
-                                                          int* __restrict__ ctr, const int* __restrict__ part_ctr,
+                                                          int* __restrict__ ctr, const unsigned long long* __restrict__ part_ctr,
                                                           const int2* __restrict__ part_tab,
                                                           const int2* __restrict__ part_cnt, int part_cap, int part_cols)
 {
@@ -918,7 +920,7 @@ template <bool RUNS>
 __global__ void __launch_bounds__(kEnumMaxThreads) k_count(Geo* geo, int n_struct, double r2min,
                                                            double r2max, float r2minf, float r2maxf,
                                                            int64_t* __restrict__ cnt, int64_t* __restrict__ run_cnt,
-                                                           int* __restrict__ ctr, const int* __restrict__ part_ctr,
+                                                           int* __restrict__ ctr, const unsigned long long* __restrict__ part_ctr,
                                                            const int2* __restrict__ part_tab,
                                                            int2* __restrict__ part_cnt, int part_cap, int part_cols,
                                                            const ScanArgs scan, int* __restrict__ done,
@@ -1302,7 +1304,7 @@ static void launch_k(bool pdl, void (*k)(P...), dim3 grid, dim3 block, cudaStrea
 
 static EnumParts enum_parts(const GeomArgs& a)
 {
-    return EnumParts{a.enum_ctr + kPartCtr, enum_part_cols(a.n_struct, a.part_cap), a.part_cap, a.part_tab, a.refl_cnt, a.run_cnt};
+    return EnumParts{(unsigned long long*)(a.enum_ctr + kPartCtr), enum_part_cols(a.n_struct, a.part_cap), a.part_cap, a.part_tab, a.refl_cnt, a.run_cnt};
 }
 
 static void prep_launch(bool pdl, const GeomArgs& a, cudaStream_t st)
@@ -1428,7 +1430,7 @@ static void count_launch(const GeomArgs& a, const ScanArgs& sa, cudaStream_t st,
     const int grid = enum_grid(a, (const void*)k, smem);
     auto go = [&](auto launch) {
         launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, a.refl_cnt,
-               a.run_cnt, a.enum_ctr, (const int*)(a.enum_ctr + kPartCtr), (const int2*)a.part_tab, a.part_cnt,
+               a.run_cnt, a.enum_ctr, (const unsigned long long*)(a.enum_ctr + kPartCtr), (const int2*)a.part_tab, a.part_cnt,
                a.part_cap, enum_part_cols(a.n_struct, a.part_cap), sa, last ? a.enum_ctr + kDoneCtr : (int*)nullptr, sa.bad);
     };
     if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });
@@ -1479,7 +1481,7 @@ void launch_emit(const GeomArgs& a, cudaStream_t st, bool pdl)
     auto go = [&](auto launch) {
         launch(a.geo, a.n_struct, a.r2min, a.r2max, (float)a.r2min, (float)a.r2max, 32 * a.rb,
                (const int64_t*)a.refl_off, (const int64_t*)a.run_cnt, (const int*)a.abort_flag, a.q, a.key, a.runs,
-               (const int*)a.tile_off, a.tile_tab, a.enum_ctr + 1, (const int*)(a.enum_ctr + kPartCtr),
+               (const int*)a.tile_off, a.tile_tab, a.enum_ctr + 1, (const unsigned long long*)(a.enum_ctr + kPartCtr),
                (const int2*)a.part_tab, (const int2*)a.part_cnt, a.part_cap, enum_part_cols(a.n_struct, a.part_cap));
     };
     if (pdl) go([&](auto... v) { launch_pdl(k, grid, a.enum_threads, smem, st, v...); });

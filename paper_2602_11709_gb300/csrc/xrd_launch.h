@@ -49,7 +49,7 @@ struct GeomArgs {
     uint32_t* key;
     long long* parts;  // chunk sums of the multi-block scan (nullptr: single-block scan)
     int* oparts;       // [chunks][4096] bin counts of the multi-block order (nullptr: one-block order)
-    int* enum_ctr;     // flags[26..29]: claims of counting and of emission, parts listed (kPartCtr), CTAs of counting done
+    int* enum_ctr;     // flags[26..30]: claims of counting and of emission, parts listed (kPartCtr, 64 bits), CTAs of counting done
     int2* part_tab;    // [part_cap] (structure, part) of each enumeration part, by k_prep
     int2* part_cnt;    // [part_cap] its reflections and runs, by k_count
     int part_cap;
@@ -60,11 +60,11 @@ struct GeomArgs {
     AtomR* atomr;      // [atoms] records of the accurate re-evaluation, by k_atoms (or nullptr)
 };
 
-constexpr int kPartCtr = 2, kDoneCtr = 3;  // indices within enum_ctr
+constexpr int kPartCtr = 2, kDoneCtr = 4;  // indices within enum_ctr
 
 // What k_prep needs to list the enumeration parts of the structures with more than `cols` columns.
 struct EnumParts {
-    int* ctr;
+    unsigned long long* ctr;
     int cols, cap;
     int2* tab;
     int64_t* cnt;      // reflection and run counts: zeroed for the structures in parts
