@@ -10,6 +10,8 @@
 // |g|^2 is evaluated in one fixed order with every product and sum rounded on
 // its own (no fused multiply-add), so the set of reflections on the sphere
 // boundary is decided exactly as a plain FP64 evaluation of the same order.
+#include <algorithm>
+
 #include "xrd_dd.cuh"
 #include "xrd_fx.cuh"
 #include "xrd_internal.cuh"
@@ -1407,14 +1409,17 @@ size_t order_parts_bytes(int64_t n)
     return nch > 2 ? (size_t)4 * kOrderBins * nch : 0;
 }
 
-// CTAs of the enumeration: what fits on the SMs at once, or fewer where even one part per 32 columns and one
-// structure per warp would leave CTAs without an item
+// CTAs of the enumeration: what fits on the SMs at once, or fewer where one item per warp would leave CTAs without one.
+// The parts are estimated by the reflections and 256 a structure: idle CTAs hold back the structure factor's, which then
+// share SMs (one small cell in FP64 86 us a call, 102 with CTAs for all the parts that there is room for).
 static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
 {
     const int nt = a.enum_threads;
     const int per_sm = resident_ctas(kernel, nt, smem);
-    const int64_t most = ((int64_t)a.n_struct + a.part_cap + nt / 32 - 1) / (nt / 32);
-    return (int)min((int64_t)a.sms * per_sm, max(most, (int64_t)1));
+    const int64_t n = a.n_struct;
+    const int64_t parts = a.cap_refl ? std::min<int64_t>(a.part_cap, std::max(a.cap_refl, 256 * n)) : a.part_cap;
+    const int64_t most = (n + parts + nt / 32 - 1) / (nt / 32);
+    return (int)std::min<int64_t>((int64_t)a.sms * per_sm, std::max<int64_t>(most, 1));
 }
 
 static ScanArgs scan_args(const GeomArgs& a)
