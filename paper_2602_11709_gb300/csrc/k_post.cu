@@ -35,6 +35,37 @@ __host__ __device__ constexpr size_t post_smem_of(size_t c)
 
 size_t post_smem_bytes(int cap) { return post_smem_of((size_t)cap); }
 
+// The shared memory of a structure of up to CAP reflections
+struct PostMem {
+    double* q;
+    uint32_t* key;
+    uint16_t* perm;
+    int* bkt;
+    uint8_t* flag;
+    int* pst;
+    double* psum;
+    int* fcnt;
+    float* I;  // the FP32 variants' intensities, in the second half of psum
+};
+template <int CAP>
+__device__ __forceinline__ PostMem post_mem()
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const size_t c = (size_t)CAP;
+    PostMem m;
+    unsigned char* p = smem;
+    m.q = (double*)p; p += align16(c * 8);
+    m.key = (uint32_t*)p; p += align16(c * 4);
+    m.perm = (uint16_t*)p; p += align16(c * 2);
+    m.bkt = (int*)p; p += align16((c + 1) * 4);
+    m.flag = (uint8_t*)p; p += align16(c);
+    m.pst = (int*)p; p += align16(c * 4);
+    m.psum = (double*)p; p += align16(c * 8);
+    m.fcnt = (int*)p;
+    m.I = (float*)m.psum + c;
+    return m;
+}
+
 // CTAs per SM that the shared memory of a class allows (228 KB per SM; about
 // 2 KB more per CTA for the static arrays and the per-CTA reservation), at most
 // 1024 threads: the launch bounds ask the compiler to fit that many CTAs in the
@@ -238,7 +269,6 @@ __device__ __noinline__ int merged_peak_large(FK fk, double* q, uint32_t* key, c
     return merged_peak_body<kWarpPeak / 32, PermT, FI>(fk, q, key, perm, i0, m, Is, I, sum);
 }
 
-// A peak of more than kWarpPeak members (out of line: rare): its number of families, and their staging at family offset f0.
 template <typename PermT>
 struct FamilyKeys {  // family key of the member at merge position i
     const unsigned long long* fkg;
@@ -250,41 +280,98 @@ struct FamilyKeys {  // family key of the member at merge position i
         return fkg ? fkg[perm[i]] : family_key(key[perm[i]], hex);
     }
 };
-template <typename PermT>
-__device__ __noinline__ int large_count(const unsigned long long* fkg, const uint32_t* key, const PermT* perm, bool hex,
-                                        int i0, int i1)
+// The same for a peak of any number of members (rare, by tolerances far above a line's width): each member's
+// representative (0 unless it is the first of its family) and family size go through trep and tcnt, m words each of the
+// structure's output staging, which is free until the peaks are done. A thread each, which compares every member with
+// every family of the peak and again for the ranks, took 4.4 s on 30 small cells at a tolerance of 5 degrees; now 1 ms.
+template <typename PermT, bool FI, typename T>
+__device__ __forceinline__ int merged_peak_any(FamilyKeys<PermT> fk, double* q, uint32_t* key, const PermT* perm, int i0, int m,
+                                            const float* Is, const double* I, uint32_t* trep, int* tcnt, T& sum)
 {
-    return count_families(FamilyKeys<PermT>{fkg, key, perm, hex}, i0, i1);
-}
-template <typename PermT>
-__device__ __noinline__ void large_families(const PostArgs& a, int64_t base, const uint32_t* key, const PermT* perm,
-                                            bool hex, int i0, int i1, int f0)
-{
-    const FamilyKeys<PermT> fk{a.fkg ? a.fkg + base : nullptr, key, perm, hex};
-    // leaders are first members of each family; rank by descending representative
-    for (int i = i0; i < i1; i++) {
-        const unsigned long long fi = fk(i);
-        bool lead = true;
-        for (int j = i0; j < i && lead; j++) lead = fk(j) != fi;
-        if (!lead) continue;
-        uint32_t rep = 0;
-        int cnt = 0;
-        for (int j = i0; j < i1; j++)
-            if (fk(j) == fi) { rep = max(rep, key[perm[j]]); cnt++; }
-        int rank = 0;
-        for (int m = i0; m < i1; m++) {  // other leaders with a larger representative
-            const unsigned long long fm = fk(m);
-            if (fm == fi) continue;
-            bool lm = true;
-            for (int j = i0; j < m && lm; j++) lm = fk(j) != fm;
-            if (!lm) continue;
-            uint32_t rm = 0;
-            for (int j = i0; j < i1; j++)
-                if (fk(j) == fm) rm = max(rm, key[perm[j]]);
-            rank += rm > rep;
+    constexpr int C = kWarpPeak / 32;
+    const int lane = threadIdx.x & 31;
+    sum = (T)0;
+    for (int j0 = 0; j0 < m; j0 += 32) {
+        const int v = perm[i0 + min(j0 + lane, m - 1)];
+        T Iv;
+        if constexpr (FI) Iv = Is[v];
+        else Iv = I[v];
+        for (int j = 0; j < min(32, m - j0); j++) sum = peak_add(sum, __shfl_sync(0xffffffffu, Iv, j), j0 + j == 0);
+    }
+    int nf = 0;
+    for (int b0 = 0; b0 < m; b0 += 32 * C) {
+        unsigned long long k[C];
+        uint32_t rep[C];
+        int cnt[C];
+        bool lead[C];
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            const int i = b0 + 32 * c + lane;
+            k[c] = fk(i0 + min(i, m - 1));
+            rep[c] = 0;
+            cnt[c] = 0;
+            lead[c] = i < m;
         }
-        a.st_key[base + f0 + rank] = rep;
-        a.st_mult[base + f0 + rank] = 2 * cnt;
+        for (int j0 = 0; j0 < m; j0 += 32) {
+            const int at = i0 + min(j0 + lane, m - 1);
+            const unsigned long long kl = fk(at);
+            const uint32_t kvl = key[perm[at]];
+            for (int j = 0; j < min(32, m - j0); j++) {
+                const unsigned long long kj = __shfl_sync(0xffffffffu, kl, j);
+                const uint32_t kvj = __shfl_sync(0xffffffffu, kvl, j);
+#pragma unroll
+                for (int c = 0; c < C; c++)
+                    if (kj == k[c]) {
+                        cnt[c]++;
+                        rep[c] = max(rep[c], kvj);
+                        lead[c] = lead[c] && j0 + j >= b0 + 32 * c + lane;
+                    }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            const int i = b0 + 32 * c + lane;
+            if (i < m) {
+                trep[i] = lead[c] ? rep[c] : 0u;
+                tcnt[i] = cnt[c];
+            }
+            nf += __popc(__ballot_sync(0xffffffffu, lead[c]));
+        }
+    }
+    __syncwarp();  // every key is read, trep and tcnt are written
+    for (int b0 = 0; b0 < m; b0 += 32) {
+        const int i = b0 + lane;
+        const uint32_t r = i < m ? trep[i] : 0u;
+        int rank = 0;
+        if (!__ballot_sync(0xffffffffu, r != 0u)) continue;
+        for (int j0 = 0; j0 < m; j0 += 32) {
+            const uint32_t rl = j0 + lane < m ? trep[j0 + lane] : 0u;
+            for (int j = 0; j < 32; j++) rank += __shfl_sync(0xffffffffu, rl, j) > r;
+        }
+        if (r != 0u) {
+            const int slot = perm[i0 + rank];
+            key[slot] = r;
+            if (rank > 0) q[slot] = __longlong_as_double(tcnt[i]);
+        }
+    }
+    return nf;
+}
+// all of them, listed at the end of m.pst (n: the structure's reflections)
+template <int CAP, bool FI>
+__device__ __noinline__ void merged_peaks_any(const PostArgs& a, int64_t base, bool hex, int n, int nlist)
+{
+    using T = typename std::conditional<FI, float, double>::type;
+    const PostMem m = post_mem<CAP>();
+    const FamilyKeys<uint16_t> fk{a.fkg ? a.fkg + base : nullptr, m.key, m.perm, hex};
+    for (int li = threadIdx.x >> 5; li < nlist; li += blockDim.x >> 5) {
+        const int p = m.pst[n - 1 - li], i0 = m.bkt[p], mp = m.bkt[p + 1] - i0;
+        T sum;
+        const int nf = merged_peak_any<uint16_t, FI>(fk, m.q, m.key, m.perm, i0, mp, m.I, FI ? nullptr : a.I + base,
+                                                     a.st_key + base + i0, a.st_mult + base + i0, sum);
+        if ((threadIdx.x & 31) == 0) {
+            ((T*)m.psum)[p] = sum;
+            m.fcnt[p] = nf;
+        }
     }
 }
 
@@ -297,7 +384,7 @@ __device__ __noinline__ void large_families(const PostArgs& a, int64_t base, con
 // out of the scans themselves, and the next structure is claimed meanwhile (16 barriers a structure; with a pass for
 // each of these, 25 barriers and the claim in the open, 100 000 mixed cells took 7.06 ms a call, now 6.89; 20 000 at
 // Mo K-alpha 6.31, now 6.17).
-template <typename PermT, bool FI, typename Ahead>
+template <int CAP, typename PermT, bool FI, typename Ahead>
 __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, bool hex, double* q, uint32_t* key,
                                float* Is, PermT* perm, int* bkt, uint8_t* flag, int* pst, double* psum, int* fcnt,
                                int* tmp, double* dtmp, Ahead ahead)
@@ -401,11 +488,11 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, bo
     });
     if (tid == 0) {
         bkt[np] = n;
-        bkt[np + 1] = 0;  // merged peaks of 2 to kWarpPeak members (np < n here)
+        bkt[np + 1] = 0;  // merged peaks of more than one member (np < n here)
     }
     __syncthreads();
     // ---- per peak: merged intensity (each half-space reflection stands for g and -g) and families ----
-    // A peak of one member is its thread's; one of 2 to kWarpPeak members goes to a list (pst is free until the cutoff)
+    // A peak of one member is its thread's; one of more goes to a list (pst is free until the cutoff)
     // that the warps work off (merged_peak). One thread a peak took most of the structure's time where peaks have many
     // members: rock salt (293 reflections, peaks of up to 36) 62 000 of 105 000 cycles, and 13 000 more in the staging.
     // Peak sums are >= 0, so their maximum is taken through the bit patterns.
@@ -421,30 +508,39 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, bo
     };
     unsigned long long lmax = 0;
     for (int p = tid; p < np; p += nt) {
-        const int i0 = bkt[p], i1 = bkt[p + 1], m = i1 - i0;
-        if (m > 1 && m <= kWarpPeak) {
-            pst[atomicAdd(&bkt[np + 1], 1)] = p;
+        const int i0 = bkt[p], m = bkt[p + 1] - i0;
+        if (m > kWarpPeak) {  // from the list's end, counted in the upper half
+            pst[n - 1 - (atomicAdd(&bkt[np + 1], 1 << 16) >> 16)] = p;
             continue;
         }
-        T sum = peak_add((T)0, member_I(perm[i0]), true);
-        for (int i = i0 + 1; i < i1; i++) sum = peak_add(sum, member_I(perm[i]), false);
+        if (m > 1) {
+            pst[atomicAdd(&bkt[np + 1], 1) & 0xffff] = p;
+            continue;
+        }
+        const T sum = peak_add((T)0, member_I(perm[i0]), true);
         ps[p] = sum;
-        fcnt[p] = m == 1 ? 1 : large_count<PermT>(fk.fkg, key, perm, hex, i0, i1);
+        fcnt[p] = 1;
         lmax = max(lmax, bits_of(sum));
     }
     __syncthreads();
-    const int nmulti = bkt[np + 1];
+    const int nmulti = bkt[np + 1] & 0xffff, nlarge = bkt[np + 1] >> 16;
+    const double* const Id = FI ? nullptr : a.I + base;
     for (int li = tid >> 5; li < nmulti; li += nt >> 5) {
         const int p = pst[li], i0 = bkt[p], m = bkt[p + 1] - i0;
         T sum;
         int nf;
-        if (m <= 32) nf = merged_peak_body<1, PermT, FI>(fk, q, key, perm, i0, m, Is, FI ? nullptr : a.I + base, sum);
-        else nf = merged_peak_large<PermT, FI>(fk, q, key, perm, i0, m, Is, FI ? nullptr : a.I + base, sum);
+        if (m <= 32) nf = merged_peak_body<1, PermT, FI>(fk, q, key, perm, i0, m, Is, Id, sum);
+        else nf = merged_peak_large<PermT, FI>(fk, q, key, perm, i0, m, Is, Id, sum);
         if ((tid & 31) == 0) {
             ps[p] = sum;
             fcnt[p] = nf;
             lmax = max(lmax, bits_of(sum));
         }
+    }
+    if (nlarge) {
+        merged_peaks_any<CAP, FI>(a, base, hex, n, nlarge);
+        __syncthreads();
+        for (int li = tid; li < nlarge; li += nt) lmax = max(lmax, bits_of(ps[pst[n - 1 - li]]));
     }
     const unsigned long long mbits = post_max<FI>(lmax, (unsigned long long*)dtmp);
     T imax, inv_imax;
@@ -477,10 +573,6 @@ __device__ void post_structure(const PostArgs& a, int s, int64_t base, int n, bo
         const T v = ps[p];        // the largest peak maps to exactly 100
         ((T*)a.st_I)[o] = (a.scaled && imax > (T)0) ? (v == imax ? (T)100 : (T)100 * (v * inv_imax)) : v;
         a.st_foff[o] = f0;
-        if (m > kWarpPeak) {
-            large_families<PermT>(a, base, key, perm, hex, i0, i0 + m, f0);
-            continue;
-        }
         const int nfp = fcnt[p];
         int first = m;  // members of the first family: those of no other
         for (int r = nfp - 1; r >= 0; r--) {
@@ -522,7 +614,6 @@ __global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const Pos
 {
     static_assert(CAP > 0, "the largest class runs as the flat passes");
     pdl_chain_enter(first);
-    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int tmp[32];
     __shared__ double dtmp[33];
     __shared__ PostClaim claims[2];
@@ -578,19 +669,9 @@ __global__ void __launch_bounds__(NT, post_min_blocks(CAP, NT)) k_post(const Pos
             ahead(0);
             ahead(1);
         } else {
-            const size_t c = (size_t)CAP;
-            unsigned char* p = smem;
-            double* sq = (double*)p; p += align16(c * 8);
-            uint32_t* sk = (uint32_t*)p; p += align16(c * 4);
-            uint16_t* perm = (uint16_t*)p; p += align16(c * 2);
-            int* bkt = (int*)p; p += align16((c + 1) * 4);
-            uint8_t* flag = (uint8_t*)p; p += align16(c);
-            int* pst = (int*)p; p += align16(c * 4);
-            double* psum = (double*)p; p += align16(c * 8);
-            int* fcnt = (int*)p;
-            float* sI = (float*)psum + c;
-            post_structure<uint16_t, FI>(a, s, base, n, cl.hex != 0, sq, sk, sI, perm, bkt, flag, pst, psum, fcnt, tmp,
-                                         dtmp, ahead);
+            const PostMem m = post_mem<CAP>();
+            post_structure<CAP, uint16_t, FI>(a, s, base, n, cl.hex != 0, m.q, m.key, m.I, m.perm, m.bkt, m.flag, m.pst,
+                                              m.psum, m.fcnt, tmp, dtmp, ahead);
         }
         if (threadIdx.x == 0) copy_async_wait();
     }

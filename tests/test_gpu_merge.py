@@ -75,3 +75,20 @@ def test_flat_passes_any_counts(gpu_lib, prec, n):
     ref = oracle.pattern_batch(b, o)
     assert got["sizes"]["n_refl"] > 6144 * n
     compare_batch(got, ref, prec, o.rel_cutoff, o.scaled)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_phasefix"])
+@pytest.mark.parametrize("tol", [1.0, 8.0, 200.0])
+@pytest.mark.parametrize("group", [None, "mmm"])
+def test_peaks_of_hundreds_and_thousands(gpu_lib, prec, tol, group):
+    """Peaks beyond what a warp holds in registers: families, sums and the largest peak, up to one peak of all reflections."""
+    b = _cells()
+    rng = np.random.default_rng(6)
+    b = synth.concat([b, synth.random_cell(rng, 3, edge=(12.0, 13.0)), synth.random_cell(rng, 2, edge=(3.0, 3.5))])
+    o = synth.Opts(tt_max=100.0, tt_tol=tol, rel_cutoff=1e-4)
+    if group:
+        o.point_group = adapter.laue_group_ops(group)
+    ref = oracle.pattern_batch(b, o)
+    members = [int(m.sum()) // 2 for m in ref["fam_mult"]]
+    assert max(members) <= 6144 and max(m / max(len(p), 1) for m, p in zip(members, ref["peak_tt"])) > 30
+    compare_batch(gpu_lib.compute(b, o, prec), ref, prec, o.rel_cutoff, o.scaled)
