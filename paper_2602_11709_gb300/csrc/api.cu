@@ -1066,7 +1066,6 @@ static xrd::GradArgs grad_args(xrd_handle* h, const xrd_batch* b, const xrd_grid
     a.t0 = g->t0;
     a.dt = g->dt;
     a.inv_dt = 1.0 / g->dt;
-    a.sigma = sigma;
     a.cg = (float)(1.4426950408889634f / (2.0 * sigma * sigma));
     a.inv_s2 = (float)(1.0 / (sigma * sigma));
     a.l2d = o->lambda * o->lambda * 0.25;

@@ -526,19 +526,6 @@ __device__ __forceinline__ void chunk_scan(long long (&v)[kScanItems], long long
     __syncthreads();
 }
 
-__device__ __forceinline__ double block_max_double(double v, double* tmp)
-{
-    const int nw = (blockDim.x + 31) >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (lane == 0) tmp[w] = v;
-    __syncthreads();
-    double r = tmp[0];
-    for (int i = 1; i < nw; i++) r = fmax(r, tmp[i]);
-    __syncthreads();
-    return r;
-}
-
 __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v, unsigned long long* tmp)
 {
     const int nw = (blockDim.x + 31) >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -548,19 +535,6 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
     __syncthreads();
     unsigned long long r = tmp[0];
     for (int i = 1; i < nw; i++) r = max(r, tmp[i]);
-    __syncthreads();
-    return r;
-}
-
-__device__ __forceinline__ int block_sum_int(int v, int* tmp)
-{
-    const int nw = (blockDim.x + 31) >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) tmp[w] = v;
-    __syncthreads();
-    int r = 0;
-    for (int i = 0; i < nw; i++) r += tmp[i];
     __syncthreads();
     return r;
 }

@@ -244,7 +244,7 @@ struct CompactArgs {
 struct GradArgs {
     int n_struct, n_pts, W, sms;
     int64_t n_atoms;
-    double t0, dt, inv_dt, sigma, l2d;
+    double t0, dt, inv_dt, l2d;
     float cg, inv_s2;  // log2(e) / (2 sigma^2) and 1 / sigma^2, formed in FP64 (a division per thread costs ten FP64 operations)
     float l2h, l2l;  // lambda^2 / 4 as two floats
     const TTab* ttab;
