@@ -48,7 +48,7 @@ constexpr int kRunsPerTileHost = xrd::kRunsPerTile;  // structure-factor tile: 3
 constexpr int kFlagBytes = 256;
 constexpr int kWorkOffset = 64;
 constexpr int kRefinedOffset = 96;
-constexpr int kQueryParts = 65536;  // enumeration parts of a reflection count outside a call
+constexpr int kQueryParts = 32768;  // enumeration parts of a reflection count outside a call
 constexpr int kStages = 9;
 constexpr int kSfStage = 5;      // index of the structure-factor stage
 constexpr int kRefineStage = 6;  // index of the re-evaluation stage
@@ -1134,7 +1134,8 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.refl_off = (int64_t*)(ws + L.refl_off);
     ga.tile_off = (int*)(ws + L.tile_off);
     ga.order = (int*)(ws + L.order);
-    ga.aorder = (int*)(ws + L.aorder);
+    const bool fused = n > 0 && xrd::front_fused((int)n, b->n_atoms);
+    ga.aorder = fused ? nullptr : (int*)(ws + L.aorder);
     ga.atom_bad = (int*)(ws + L.atom_bad);
     ga.atoms_set_geo = 1;  // a structure with an invalid atom has no reflections here
     ga.tile_tab = (int2*)(ws + L.tile_tab);
@@ -1150,7 +1151,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     ga.parts = (long long*)(ws + L.parts);
     ga.oparts = xrd::order_parts_bytes(n) ? (int*)(ws + L.oparts) : nullptr;
     cudaMemsetAsync(ws + L.flags, 0, kFlagBytes, st);
-    if (n > 0 && xrd::front_fused((int)n, b->n_atoms)) {
+    if (fused) {
         xrd::launch_front(ga, st);
         xrd::launch_count(ga, st, true, true);  // structures with an invalid atom lose their status there
     } else {
@@ -1188,6 +1189,7 @@ static void profile_front(xrd_handle* h, const xrd_batch* b, const xrd_opts* o, 
     sa.atomx = ga.atomx;
     sa.q = ga.q;
     sa.key = ga.key;
+    sa.aorder = fused ? (int*)(ws + L.aorder) : nullptr;
     if (grad) {
         sa.Fx = (float4*)(ws + L.Fx);
         sa.Ig = (float*)(ws + L.Ig);

@@ -7,7 +7,7 @@
 //   PV(u) = eta (2 / (pi w)) / (1 + x^2) + (1 - eta) (2 / w) sqrt(ln 2 / pi) 2^(-x^2),  x = 2 u / w
 //   then y_k += sigma sqrt(max(y_k, 0)) z_k.
 //
-// The structures come in order of their reflection count, largest first (aorder, by the scan of the counts).
+// The structures come in order of their reflection count, largest first (aorder).
 // k_aug_sum gives each warp 256 grid points of one structure (kAugPts
 // consecutive points per thread) and streams all of the structure's reflections
 // through shared memory, turning each into a record as it is staged: its grid

@@ -797,6 +797,8 @@ __device__ __forceinline__ void scan_count_bins(int* bins)
 
 // buf: kScanItems * blockDim long longs of shared memory. The counts are read past the L1 cache: the CTA that runs
 // this may be one of the kernel that wrote them.
+// ORDER: also the order by reflection count, if sa.aorder.
+template <bool ORDER>
 __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restrict__ geo, int n,
                                                 const ScanArgs& sa, ScanShared& sh, long long* buf)
 {
@@ -814,7 +816,7 @@ __device__ __forceinline__ void scan_refl_block(const int64_t* cnt, Geo* __restr
     long long* const ws = sh.ws;
     int* const ccnt = sh.ccnt;
     const int nt = blockDim.x, tid = threadIdx.x, CH = kScanItems * nt;
-    int* const aorder = sa.aorder;
+    int* const aorder = ORDER ? sa.aorder : nullptr;
     int* const bins = sh.bins;
     long long tot;
     if (aorder) {
@@ -913,7 +915,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_refl(const int64_t* __res
     pdl_enter();
     __shared__ ScanShared sh;
     __shared__ __align__(16) long long buf[kScanItems * kScanThreads];
-    scan_refl_block(cnt, geo, n, sa, sh, buf);
+    scan_refl_block<true>(cnt, geo, n, sa, sh, buf);
 }
 
 // Reflection (and, with RUNS, run) counts per structure, and of every part (k_prep has zeroed the counts of a
@@ -989,7 +991,7 @@ __global__ void __launch_bounds__(kEnumMaxThreads) k_count(Geo* geo, int n_struc
         if (threadIdx.x == 0) scan.sums[1] = m;
         return;
     }
-    scan_refl_block(cnt, geo, n_struct, scan, sh, scan_buf);
+    scan_refl_block<false>(cnt, geo, n_struct, scan, sh, scan_buf);
 }
 
 // Multi-block form of k_scan_refl for batches of more than two chunks (one

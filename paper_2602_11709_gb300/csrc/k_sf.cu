@@ -382,6 +382,45 @@ __device__ float sf_tile_fp32(const SfArgs& a, int s, int64_t first, int len, in
     return imax;
 }
 
+// Structures by reflection count, largest first (buckets of a quarter octave), by one CTA beside the tiles of the
+// others: the profile kernels that follow give every structure a CTA and start with the largest. cnt: kCountBuckets
+// ints of shared memory. The order within a bucket is arbitrary; nothing but the load balance depends on it. For the small
+// batches of the one-launch front, where it ends before the tiles do; in the scan of the counts, which orders the others, it
+// lengthened the chain of launches (1024 small cells 190.8 -> 194.4 us a call).
+constexpr int kCountBuckets = 128;
+__device__ void order_by_count(const SfArgs& a, int* cnt)
+{
+    for (int i = threadIdx.x; i < kCountBuckets; i += blockDim.x) cnt[i] = 0;
+    __syncthreads();
+    // f(s, bucket) of every structure, the counts of four read together
+    auto each = [&](auto f) {
+        for (int s0 = threadIdx.x; s0 < a.n_struct; s0 += 4 * blockDim.x) {
+            int64_t R[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int s = min(s0 + u * (int)blockDim.x, a.n_struct - 1);
+                R[u] = a.refl_off[s + 1] - a.refl_off[s];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (s0 + u * (int)blockDim.x < a.n_struct)
+                    f(s0 + u * (int)blockDim.x, R[u] <= 0 ? 0 : min(kCountBuckets - 1, 1 + (int)(4.f * log2f((float)R[u]))));
+        }
+    };
+    each([&](int, int b) { atomicAdd(&cnt[b], 1); });
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int acc = 0;
+        for (int b = kCountBuckets - 1; b >= 0; b--) {
+            const int c = cnt[b];
+            cnt[b] = acc;
+            acc += c;
+        }
+    }
+    __syncthreads();
+    each([&](int s, int b) { a.aorder[atomicAdd(&cnt[b], 1)] = s; });
+}
+
 // Persistent CTAs; every warp takes tiles of 32 runs (one per lane) from a
 // queue in largest-first order (tiles of the structures with the most atoms
 // first). A structure's atoms stay staged in the warp's shared memory while its
@@ -402,6 +441,10 @@ __global__ void __launch_bounds__(32 * WARPS,
     __shared__ float2 sstep[RUNS ? WARPS : 1][RUNS ? kSfChunk : 1];
     __shared__ int4 slo[PREC == XRD_FP32_PHASE64 ? WARPS : 1][PREC == XRD_FP32_PHASE64 ? kSfChunk : 1];
     extern __shared__ CoefPair scoef[];  // [zmax + 1]
+    if (a.aorder && blockIdx.x == gridDim.x - 1) {
+        __shared__ int cnt[kCountBuckets];
+        order_by_count(a, cnt);
+    }
     if (*a.abort_flag) return;
     const int ntiles = a.tile_off[a.n_struct];
     if ((int)blockIdx.x >= ntiles) return;  // the CTAs before this one already have a tile each

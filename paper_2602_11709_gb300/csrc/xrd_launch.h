@@ -35,7 +35,8 @@ struct GeomArgs {
     int64_t* refl_off;
     int* tile_off;   // [n_struct + 1] first structure-factor tile of each structure; [n_struct] = tiles
     int* order;      // [n_struct] structures by atom count, largest first
-    int* aorder;     // [n_struct] and by reflection count, for the profile kernels (or nullptr)
+    int* aorder;     // [n_struct] and by reflection count, for the profile kernels (or nullptr; by the scan of the counts,
+                     // after the one-launch front by the structure factor: SfArgs::aorder)
     int2* tile_tab;  // [tiles] (structure, first reflection) of each structure-factor tile
     int* atom_bad;   // [n_struct] 1 where an atom of the structure is invalid
     int atoms_set_geo;  // such structures become invalid in geo before the enumeration: by k_atoms, or after
@@ -114,6 +115,7 @@ struct SfArgs {
     int* Es;     // the structure of each reflection whose bound exceeds tau times its intensity (others: unset)
     float eps_k; // K times the relative error of one FP32 term (the bound of |dF| / sqrt(sum a_j^2))
     float tau;
+    int* aorder;     // [n_struct] structures by reflection count, largest first, for the profile kernels (or nullptr)
     unsigned* imax;  // FP32 pattern variants: [n_struct] bits of the largest reflection intensity (zeroed by k_prep)
 };
 
