@@ -87,7 +87,7 @@ void init_fx_tables(cudaStream_t st) { k_fx_init<<<(kFxExpN + kFxScN + 1 + 31) /
 // or huge b, denormal a, not finite); f is then formed in FP64 with the library's exp.
 struct CoefX {
     uint64_t bm[4];
-    int64_t am[4];
+    uint64_t am[4];
     int16_t be[4], ae[4];
     int slow, pad;
 };

@@ -116,13 +116,13 @@ XRD_HD FxNum fx_log2e(double b)
     return FxNum{(hi << 1) | (lo >> 63), n.e};
 }
 
-// exp(-b s2) for bl2 = b log2(e) and s2, as (m, n): the value is m 2^(-64 - n), m in [2^63, 2^64), or m = 0 where it is
-// below 2^-1021. tab: kFxExpN entries.
+// exp(-b s2) for bl2 = b log2(e) and s2, as (m, n): the value is m 2^(-64 - n), m in [2^63, 2^64), or m = 0 (and n >= 1021)
+// where it is below 2^-1021. tab: kFxExpN entries.
 XRD_HD uint64_t fx_exp2_neg(uint64_t bm, int be, uint64_t sm, int se, const uint64_t* __restrict__ tab, int& n)
 {
     const uint64_t P = fx_mulhi64(bm, sm);
     const int sh = 9 - be - se;  // T = b s2 log2(e) with 53 fractional bits
-    n = 0;
+    n = 2048;
     if (sh < 0) return 0ull;
     const uint64_t T = sh == 0 ? P : (sh <= 64 ? ((P >> (sh - 1)) + 1ull) >> 1 : 0ull);
     n = (int)(T >> 53);
@@ -151,44 +151,43 @@ XRD_HD double fx_exp_double(uint64_t m, int n)
     return fx_as_double(((uint64_t)(1021 - n) << 52) + (m >> 11) + ((m >> 10) & 1ull));
 }
 
-// A normal double as am 2^(e - 60), |am| in [2^60, 2^61); zero has am = 0.
-XRD_HD int64_t fx_signed(double v, int& e)
+// A normal double as (-1)^(e & 1) am 2^((e >> 1) - 60), am in [2^60, 2^61); zero has am = 0 and an exponent below any other's.
+XRD_HD uint64_t fx_signed(double v, int& e)
 {
     const FxNum n = fx_num(v < 0.0 ? -v : v);
-    e = n.e;
-    const int64_t am = (int64_t)(n.m >> 3);
-    return v < 0.0 ? -am : am;
+    e = 2 * n.e + (v < 0.0);
+    return n.m >> 3;
 }
 
-// sum of four am_i 2^(ae_i - 60) exp(-b_i s2), the exponentials as in fx_exp2_neg, to 2^-58 of the largest term: terms
-// are aligned to that one, not to the largest coefficient, whose term may have decayed.
-XRD_HD double fx_exp_sum(const int64_t* am, const int16_t* ae, const uint64_t* bm, const int16_t* be, FxNum S,
+// sum of four such numbers (am, ae) times exp(-b_i s2), the exponentials as in fx_exp2_neg, to 2^-58 of the largest term:
+// terms are aligned to that one, not to the largest coefficient, whose term may have decayed.
+XRD_HD double fx_exp_sum(const uint64_t* am, const int16_t* ae, const uint64_t* bm, const int16_t* be, FxNum S,
                          const uint64_t* __restrict__ tab)
 {
     uint64_t v[4];
-    int e[4], top = -(1 << 20);
+    int e[4];
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         int n;
         const uint64_t m = fx_exp2_neg(bm[i], be[i], S.m, S.e, tab, n);
-        v[i] = fx_mulhi64(am[i] < 0 ? 0ull - (uint64_t)am[i] : (uint64_t)am[i], m);  // v 2^(ae - n - 60), below 2^61
-        e[i] = ae[i] - n;
-        if (v[i] != 0ull && e[i] > top) top = e[i];
+        v[i] = fx_mulhi64(am[i], m);  // v 2^(e - 60), below 2^61
+        e[i] = (ae[i] >> 1) - n;
     }
+    const int t0 = e[0] > e[1] ? e[0] : e[1], t1 = e[2] > e[3] ? e[2] : e[3], top = t0 > t1 ? t0 : t1;
     int64_t sum = 0;
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         const int sh = top - e[i];
-        const int64_t w = v[i] != 0ull && sh < 64 ? (int64_t)(v[i] >> sh) : 0;
-        sum += am[i] < 0 ? -w : w;
+        const int64_t w = (int64_t)(v[i] >> (sh < 63 ? sh : 63)), neg = -(int64_t)(ae[i] & 1);
+        sum += (w ^ neg) - neg;
     }
-    if (sum == 0) return 0.0;
+    const uint64_t sign = (uint64_t)sum & 0x8000000000000000ull;
     const uint64_t a = sum < 0 ? 0ull - (uint64_t)sum : (uint64_t)sum;
-    const int z = fx_clz64(a);
+    const int z = fx_clz64(a | 1ull);
     const int f = 1023 + 62 + top - 60 - z;  // exponent field less one: the significand's top bit carries into it
-    if (f < 0) return 0.0;                   // below 2^-1022
     const uint64_t m = a << z;
-    return fx_as_double((sum < 0 ? 0x8000000000000000ull : 0ull) | (((uint64_t)f << 52) + (m >> 11) + ((m >> 10) & 1ull)));
+    if (a == 0ull || f < 0) return 0.0;  // below 2^-1022
+    return fx_as_double(sign | (((uint64_t)f << 52) + (m >> 11) + ((m >> 10) & 1ull)));
 }
 
 // A signed fixed-point number with F fractional bits as a double (rounded to nearest)

@@ -27,8 +27,7 @@ extern "C" void host_exp(int n, const double* b, const double* s2, const uint64_
 extern "C" void host_exp_sum(int n, const double* ab, const double* s2, const uint64_t* tab, double* out)
 {
     for (int i = 0; i < n; i++) {
-        int64_t am[4];
-        uint64_t bm[4];
+        uint64_t am[4], bm[4];
         int16_t ae[4], be[4];
         for (int j = 0; j < 4; j++) {
             int e;
