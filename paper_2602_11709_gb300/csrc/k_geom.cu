@@ -11,6 +11,7 @@
 // its own (no fused multiply-add), so the set of reflections on the sphere
 // boundary is decided exactly as a plain FP64 evaluation of the same order.
 #include <algorithm>
+#include <cmath>
 
 #include "xrd_dd.cuh"
 #include "xrd_fx.cuh"
@@ -1412,15 +1413,16 @@ size_t order_parts_bytes(int64_t n)
 }
 
 // CTAs of the enumeration: what fits on the SMs at once, or fewer where one item per warp would leave CTAs without one.
-// The parts are estimated by the reflections and 256 a structure: idle CTAs hold back the structure factor's, which then
-// share SMs (one small cell in FP64 86 us a call, 102 with CTAs for all the parts that there is room for).
+// A sphere has fewer parts than reflections; a shell's are estimated by those of the sphere that it is the rim of. Idle
+// CTAs hold back the structure factor's, which then share SMs (one small cell in FP64 86 us a call, 102 with CTAs for all
+// the parts that there is room for).
 static int enum_grid(const GeomArgs& a, const void* kernel, size_t smem)
 {
     const int nt = a.enum_threads;
     const int per_sm = resident_ctas(kernel, nt, smem);
-    const int64_t n = a.n_struct;
-    const int64_t parts = a.cap_refl ? std::min<int64_t>(a.part_cap, std::max(a.cap_refl, 256 * n)) : a.part_cap;
-    const int64_t most = (n + parts + nt / 32 - 1) / (nt / 32);
+    double parts = a.part_cap;
+    if (a.cap_refl) parts = std::min(parts, (double)a.cap_refl / std::max(1.0 - std::pow(a.r2min / a.r2max, 1.5), 1e-12));
+    const int64_t most = (a.n_struct + (int64_t)parts + nt / 32 - 1) / (nt / 32);
     return (int)std::min<int64_t>((int64_t)a.sms * per_sm, std::max<int64_t>(most, 1));
 }
 
