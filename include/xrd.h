@@ -41,7 +41,8 @@ extern "C" {
 #define XRD_ETIMEOUT 4  /* a bounded device-side wait ran out */
 
 /* Precision of the structure-factor sum (Sec. 2, the structure-factor sum). */
-#define XRD_FP64 0          /* FP64 throughout; phases, sin, cos and exponentials in 64-bit fixed point, to FP64's accuracy */
+#define XRD_FP64 0          /* FP64 throughout; phases, sin, cos, exponentials and the sum of f(s) in 64-bit fixed point,
+                               to the accuracy that FP64 gives them in the sum */
 #define XRD_FP32_PHASE64 1  /* phase h.x+k.y+l.z formed and reduced mod 1 to 53 fractional bits, the rest in FP32 */
 #define XRD_FP32_PHASEFIX 2 /* coordinates in 32-bit fixed point, phase reduced mod 1 exactly in integers, the rest in FP32 */
 
@@ -86,7 +87,8 @@ typedef struct {
 typedef struct {
     int64_t n_refl;       /* Friedel-unique reflections of the whole batch (each stands for g and -g) */
     int64_t max_refl;     /* largest Friedel-unique count of one structure */
-    int64_t n_tiles;      /* structure-factor tiles at the tile size a call with ws_bytes takes (runs along l: as if strided) */
+    int64_t n_tiles;      /* structure-factor tiles at the tile size a call with ws_bytes takes (runs along
+                             l: as if strided) */
     size_t ws_bytes;      /* workspace bytes xrd_pattern_batch needs for this batch and these options */
     size_t ws_grad_bytes; /* workspace bytes xrd_pattern_broadened + xrd_pattern_grad need */
 } xrd_sizes;
@@ -395,8 +397,11 @@ void xrd_graph_destroy(void* graph);
  * stage durations in milliseconds (order: prep, atoms, count, scan, emit,
  * structure factor, refine, post, compact, profile sum; in mode 2 every stage but the
  * structure factor reads 0; after an xrd_pattern_augmented call, in either
- * mode, only the profile sum -- the two kernels after the structure factors --
- * is timed and the others read 0) and returns the count. */
+ * mode, only the profile sum -- the kernel after the structure factors --
+ * is timed and the others read 0) and returns the count. The atoms are packed
+ * beside the enumeration, or in batches of up to 2048 structures as part of prep:
+ * "atoms" reads an empty pair of events. In those batches the scan is part of
+ * count, and "scan" is empty too. */
 int xrd_set_profiling(xrd_handle* h, int enabled);
 int xrd_stage_times(xrd_handle* h, float* ms, int n);
 

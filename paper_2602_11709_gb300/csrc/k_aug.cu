@@ -24,7 +24,7 @@
 // What bounds it: instruction issue and the reciprocals, 2.2 instructions a clock (the CTAs also wait at the barriers
 // around the staging): per reflection and warp about 2.5 instructions for a far one, 36 for a near Lorentzian and 30 for
 // a Gaussian. 1024 cells of 1 to 64 atoms, 4096 points: 755 us with every (point, reflection) pair evaluated by
-// itself, 282 us now; summing the tails once per node instead of in every point's long sum also took the error of the
+// itself, 275 us now; summing the tails once per node instead of in every point's long sum also took the error of the
 // patterns from 4.6e-6 to 2e-7 of their norm.
 //
 // Precision: x = (k - b) s - d s with k - b an exact integer in FP32 (|k|, |b| <

